@@ -6,6 +6,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -31,6 +32,8 @@ constexpr int64_t kPairsDefaultIons = 65536;
 // in FP64), which beats the per-level tile kernel at every size measured;
 // the bound keeps the FP64 partial-row pool within a few GB
 constexpr int64_t kPairsDefaultIonsCudaCore = 262144;
+// partial rows of one batch of the FP64 M2L beyond that many ions
+constexpr int64_t kF64PoolBytes = (int64_t)4 << 30;
 
 struct GraphKey {
     int D = -1;
@@ -138,7 +141,8 @@ struct OpSet {
     void* T_l2l = nullptr;
     void* T_m2l = nullptr;
     void* T_m2l_tc = nullptr;
-    void* T_rot = nullptr;   // rotation-based M2L operators (CUDA-core precisions)
+    void* T_rot = nullptr;   // rotation-based M2L operators (CUDA-core precisions), once asked for
+    void* T_f64 = nullptr;   // FP64 operator digits of the tensor-core translations
 };
 std::mutex g_ops_mu;
 std::map<std::tuple<int, int, int>, OpSet> g_ops;
@@ -153,6 +157,7 @@ void release_ops(fmm_plan_s* pl) {
         cudaFree(it->second.T_m2l);
         if (it->second.T_m2l_tc) cudaFree(it->second.T_m2l_tc);
         if (it->second.T_rot) cudaFree(it->second.T_rot);
+        if (it->second.T_f64) cudaFree(it->second.T_f64);
         g_ops.erase(it);
     }
     pl->ops_held = false;
@@ -241,28 +246,7 @@ int build_operators(fmm_plan_s* pl) {
     cudaError_t e = pl->ws.fp64 ? upload_ops<double>(pl, m2m, l2l, m2l)
                                 : upload_ops<float>(pl, m2m, l2l, m2l);
     if (e != cudaSuccess) return status_from(e);
-    if (pl->ws.T_rot) {
-        // rotation-based M2L operators of every offset index (neighbours zero)
-        const int nv = pl->ws.rot_op_vals;
-        std::vector<double> rot((size_t)343 * nv, 0.0);
-        for (int ox = -3; ox <= 3; ++ox)
-            for (int oy = -3; oy <= 3; ++oy)
-                for (int oz = -3; oz <= 3; ++oz) {
-                    if (ox >= -1 && ox <= 1 && oy >= -1 && oy <= 1 && oz >= -1 && oz <= 1) continue;
-                    const int idx = (ox + 3) * 49 + (oy + 3) * 7 + (oz + 3);
-                    if (!ops::build_m2l_rotation(p, ox, oy, oz, &rot[(size_t)idx * nv]))
-                        return PT_ERR_CUDA;
-                }
-        if (pl->ws.fp64) {
-            e = cudaMemcpy(pl->ws.T_rot, rot.data(), rot.size() * sizeof(double),
-                           cudaMemcpyHostToDevice);
-        } else {
-            std::vector<float> rf(rot.begin(), rot.end());
-            e = cudaMemcpy(pl->ws.T_rot, rf.data(), rf.size() * sizeof(float),
-                           cudaMemcpyHostToDevice);
-        }
-        if (e != cudaSuccess) return status_from(e);
-    }
+    if (pl->ws.fp64 && (e = m2l_f64_pack(pl->ws)) != cudaSuccess) return status_from(e);
     if (is_tc(pl->precision)) {
         const bool bf16 = pl->precision == PT_MIXED_BF16X3;
         std::vector<unsigned char> packed(m2l_tc_operand_bytes(p, bf16));
@@ -271,6 +255,29 @@ int build_operators(fmm_plan_s* pl) {
         if (e != cudaSuccess) return status_from(e);
     }
     return PT_OK;
+}
+
+// Rotation-based M2L operators of every offset index (neighbours zero) into
+// ws.T_rot.
+int build_rotation_operators(fmm_plan_s* pl) {
+    const int p = pl->p, nv = pl->ws.rot_op_vals;
+    cudaError_t e;
+    std::vector<double> rot((size_t)343 * nv, 0.0);
+    for (int ox = -3; ox <= 3; ++ox)
+        for (int oy = -3; oy <= 3; ++oy)
+            for (int oz = -3; oz <= 3; ++oz) {
+                if (ox >= -1 && ox <= 1 && oy >= -1 && oy <= 1 && oz >= -1 && oz <= 1) continue;
+                const int idx = (ox + 3) * 49 + (oy + 3) * 7 + (oz + 3);
+                if (!ops::build_m2l_rotation(p, ox, oy, oz, &rot[(size_t)idx * nv]))
+                    return PT_ERR_CUDA;
+            }
+    if (pl->ws.fp64) {
+        e = cudaMemcpy(pl->ws.T_rot, rot.data(), rot.size() * sizeof(double), cudaMemcpyHostToDevice);
+    } else {
+        std::vector<float> rf(rot.begin(), rot.end());
+        e = cudaMemcpy(pl->ws.T_rot, rf.data(), rf.size() * sizeof(float), cudaMemcpyHostToDevice);
+    }
+    return status_from(e);
 }
 
 // Rotation-based M2L operators: CUDA-core precisions whose operators fit the
@@ -294,31 +301,28 @@ int acquire_ops(fmm_plan_s* pl, size_t op_bytes) {
     if (it == g_ops.end()) {
         OpSet o;
         const size_t tc = is_tc(pl->precision) ? m2l_tc_operand_bytes(pl->p, ws.tc_bf16 != 0) : 0;
-        const size_t rot = rot_operator_bytes(pl);
+        const size_t f64 = ws.fp64 ? m2l_f64_operator_bytes(pl->p) : 0;
+        auto drop = [&]() {
+            for (void* v : {o.T_m2m, o.T_l2l, o.T_m2l, o.T_m2l_tc, o.T_f64})
+                if (v) cudaFree(v);
+            ws.T_m2m = ws.T_l2l = ws.T_m2l = ws.T_m2l_tc = ws.T_f64 = nullptr;
+        };
         if (cudaMalloc(&o.T_m2m, 8 * op_bytes) != cudaSuccess ||
             cudaMalloc(&o.T_l2l, 8 * op_bytes) != cudaSuccess ||
             cudaMalloc(&o.T_m2l, 343 * op_bytes) != cudaSuccess ||
             (tc && cudaMalloc(&o.T_m2l_tc, tc) != cudaSuccess) ||
-            (rot && cudaMalloc(&o.T_rot, rot) != cudaSuccess)) {
-            cudaFree(o.T_m2m);
-            cudaFree(o.T_l2l);
-            cudaFree(o.T_m2l);
-            cudaFree(o.T_m2l_tc);
+            (f64 && cudaMalloc(&o.T_f64, f64) != cudaSuccess)) {
+            drop();
             return PT_ERR_OOM;
         }
         ws.T_m2m = o.T_m2m;
         ws.T_l2l = o.T_l2l;
         ws.T_m2l = o.T_m2l;
         ws.T_m2l_tc = o.T_m2l_tc;
-        ws.T_rot = o.T_rot;
+        ws.T_f64 = o.T_f64;
         int r = build_operators(pl);
         if (r != PT_OK) {
-            cudaFree(o.T_m2m);
-            cudaFree(o.T_l2l);
-            cudaFree(o.T_m2l);
-            if (o.T_m2l_tc) cudaFree(o.T_m2l_tc);
-            if (o.T_rot) cudaFree(o.T_rot);
-            ws.T_m2m = ws.T_l2l = ws.T_m2l = ws.T_m2l_tc = ws.T_rot = nullptr;
+            drop();
             return r;
         }
         it = g_ops.emplace(key, o).first;
@@ -329,7 +333,32 @@ int acquire_ops(fmm_plan_s* pl, size_t op_bytes) {
     ws.T_m2l = it->second.T_m2l;
     ws.T_m2l_tc = it->second.T_m2l_tc;
     ws.T_rot = it->second.T_rot;
+    ws.T_f64 = it->second.T_f64;
     pl->ops_held = true;
+    return PT_OK;
+}
+
+// The rotation operators of the plan's shared set, built when a plan first
+// selects the rotation schedule.
+int acquire_rotation(fmm_plan_s* pl) {
+    Workspace& ws = pl->ws;
+    if (ws.T_rot) return PT_OK;
+    std::lock_guard<std::mutex> g(g_ops_mu);
+    OpSet& o = g_ops.find(std::make_tuple(pl->device, pl->p, pl->precision))->second;
+    if (!o.T_rot) {
+        if (cudaMalloc(&ws.T_rot, rot_operator_bytes(pl)) != cudaSuccess) {
+            ws.T_rot = nullptr;
+            return PT_ERR_OOM;
+        }
+        const int r = build_rotation_operators(pl);
+        if (r != PT_OK) {
+            cudaFree(ws.T_rot);
+            ws.T_rot = nullptr;
+            return r;
+        }
+        o.T_rot = ws.T_rot;
+    }
+    ws.T_rot = o.T_rot;
     return PT_OK;
 }
 
@@ -378,10 +407,12 @@ static int alloc_pairs(fmm_plan_s* pl) {
     const int dcap = pl->depth >= 0 ? pl->depth : ws.depth_max;
     int64_t exact = 0;
     for (int l = 2; l <= dcap; ++l) exact += 189 * (pow8(l) < pl->n_max ? pow8(l) : pl->n_max);
+    // batches: every pair a batch of targets can have
+    if (ws.f64_batch > 0) exact = std::min<int64_t>(exact, 189 * ws.f64_batch);
     // initial pool: the exact bound, or about twelve pairs per ion if less
     // (the 10,000-ion spheroid has ten); the first call counts its pairs and
     // every later call checks the count of the last step (ensure_pairs)
-    int64_t cap = std::min<int64_t>(exact, 12 * pl->n_max + 4096);
+    int64_t cap = ws.f64_batch > 0 ? exact : std::min<int64_t>(exact, 12 * pl->n_max + 4096);
     ws.pp_slot_cap = cap > 0 ? cap : 1;
     ws.pp_rows_cap = ws.pp_slot_cap + 343 * 128;
     ws.pp_item_cap = ws.pp_slot_cap / 128 + 344;
@@ -619,7 +650,8 @@ GraphKey make_key(const fmm_plan_s* plan, const pt_state* st, const PushParams& 
     key.laser = lz;
     key.profile = plan->profile;
     key.expand = plan->ws.expand;
-    key.sched = plan->ws.m2l_pairs + 2 * plan->ws.m2l_rot + 4 * plan->ws.pp_mirror;
+    key.sched = plan->ws.m2l_pairs + 2 * plan->ws.m2l_rot + 4 * plan->ws.pp_mirror +
+                8 * plan->ws.f64_tc;
     key.ctas = plan->ws.m2l_ctas;
     key.pool = plan->ws.pp_gen;
     return key;
@@ -774,12 +806,21 @@ int fmm_plan_set_m2l_schedule(fmm_plan plan, int schedule) {
     if (!plan || (schedule != PT_M2L_TILES && schedule != PT_M2L_PAIRS &&
                   schedule != PT_M2L_ROTATION))
         return PT_ERR_ARG;
-    if (schedule == PT_M2L_ROTATION && (is_tc(plan->precision) || !plan->ws.T_rot))
+    if (schedule == PT_M2L_ROTATION && (is_tc(plan->precision) || plan->ws.rot_op_vals == 0))
         return PT_ERR_UNSUPPORTED;
     if (cudaSetDevice(plan->device) != cudaSuccess) return PT_ERR_CUDA;
     int r = schedule != PT_M2L_TILES ? alloc_pairs(plan)
             : is_tc(plan->precision) ? alloc_tile_slabs(plan) : PT_OK;
+    if (r == PT_OK && schedule == PT_M2L_ROTATION) r = acquire_rotation(plan);
     if (r != PT_OK) return r;
+    // a schedule that was asked for runs as it is defined: FP64 plans leave
+    // the tensor-core translations for the CUDA-core ones
+    plan->ws.f64_tc = 0;
+    if (plan->ws.f64_batch > 0 && schedule != PT_M2L_TILES) {
+        // the batches' pool was sized for a part of the targets
+        plan->ws.f64_batch = 0;
+        plan->pp_counted = false;
+    }
     plan->ws.m2l_pairs = schedule != PT_M2L_TILES ? 1 : 0;
     plan->ws.m2l_rot = schedule == PT_M2L_ROTATION ? 1 : 0;
     return PT_OK;
@@ -856,7 +897,7 @@ static int plan_create_impl(int64_t n_max, int p, int leaf_max, int depth, int p
     ws.fp64 = (precision == PT_FP64);
     ws.tc_bf16 = (precision == PT_MIXED_BF16X3) ? 1 : 0;
     ws.pp_mirror = ws.tc_bf16;  // offset mirroring: the BF16x3 pair products only
-    ws.ld = ws.fp64 ? pl->P : ((pl->P + 31) / 32) * 32;
+    ws.ld = ws.fp64 ? ((pl->P + 3) / 4) * 4 : ((pl->P + 31) / 32) * 32;
     ws.rot_op_vals = rot_operator_bytes(pl) > 0 ? ops::rot_op_vals(p) : 0;
     if (depth >= 0) {
         ws.depth_max = depth;
@@ -891,7 +932,7 @@ static int plan_create_impl(int64_t n_max, int p, int leaf_max, int depth, int p
         std::lock_guard<std::mutex> g(g_tables_mu);
         if (!g_tables_dev.count(pl->device)) {
             if (upload_harmonic_tables() != cudaSuccess || m2l_tc_init() != cudaSuccess ||
-                m2l_rot_init() != cudaSuccess) {
+                m2l_f64_init() != cudaSuccess || m2l_rot_init() != cudaSuccess) {
                 free_plan(pl);
                 return PT_ERR_CUDA;
             }
@@ -945,11 +986,21 @@ static int plan_create_impl(int64_t n_max, int p, int leaf_max, int depth, int p
         ws.m2l_pairs = ok ? 1 : 0;
         ws.m2l_rot = ok && ws.fp64 && ws.rot_op_vals > 0 ? 1 : 0;
     }
+    if (ok && ws.fp64) {
+        ok = dalloc(pl, ws.f64_dig, m2l_f64_digit_bytes(p, cells)) &&
+             dalloc(pl, ws.f64_rexp, sizeof(int) * cells);
+        ws.f64_tc = 1;
+        if (ok && !ws.m2l_pairs) {
+            // beyond kPairsDefaultIonsCudaCore the M2L runs in batches
+            ws.f64_batch = std::max<int64_t>(1, kF64PoolBytes / (189 * 8 * (int64_t)ws.ld));
+            ok = alloc_pairs(pl) == PT_OK;
+        }
+    }
     if (dry) {
         *dry_bytes = (int64_t)pl->dry_bytes;
         *op_bytes = (int64_t)(tsz * (8 + 8 + 343) * PP +
                               (is_tc(precision) ? m2l_tc_operand_bytes(p, ws.tc_bf16 != 0) : 0) +
-                              rot_operator_bytes(pl));
+                              (ws.fp64 ? m2l_f64_operator_bytes(p) : 0));
         delete pl;
         return PT_OK;
     }
@@ -964,6 +1015,9 @@ static int plan_create_impl(int64_t n_max, int p, int leaf_max, int depth, int p
         (ws.M_pieces &&
          cudaMemset(ws.M_pieces, 0, sizeof(uint16_t) * kPieceRows * ws.ld * cells) != cudaSuccess) ||
         cudaMemset(ws.L, 0, tsz * ws.ld * cells) != cudaSuccess ||
+        // digit zero is stored as 128: the padding beyond column P stays zero
+        (ws.f64_dig &&
+         cudaMemset(ws.f64_dig, 128, m2l_f64_digit_bytes(p, cells)) != cudaSuccess) ||
         cudaMemset(ws.ticket, 0, sizeof(unsigned)) != cudaSuccess ||
         cudaMemset(ws.bbox_acc, 0, sizeof(unsigned long long) * 8) != cudaSuccess ||
         cudaMemset(ws.err, 0, sizeof(int)) != cudaSuccess ||

@@ -1166,6 +1166,10 @@ static cudaError_t run_fmm(int64_t n, int D, int phases, Workspace& ws, bool use
     // the M2L work list: the tensor-core schedules, and the pair-packed
     // schedule of the CUDA-core paths
     const bool pairs_simt = far && !use_tc && ws.m2l_pairs;
+    // FP64: M2M, M2L and L2L on the tensor cores (m2l_f64.cu), the M2L over
+    // the pair work list of all targets or of one batch of them after another
+    const bool f64 = far && ws.fp64 && ws.f64_tc;
+    const bool f64_batched = f64 && ws.f64_batch > 0;
     if (far && (use_tc || pairs_simt)) {
         if ((e = use_tc ? launch_m2l_tc_worklist(n, D, ws, sn)
                         : launch_m2l_pairs_worklist(n, D, ws, sn)) != cudaSuccess)
@@ -1229,6 +1233,7 @@ static cudaError_t run_fmm(int64_t n, int D, int phases, Workspace& ws, bool use
         if ((e = launch_near(false)) != cudaSuccess) return e;
     }
     const bool near_late = fork && use_tc && !near_early;
+    if (f64 && (e = launch_f64_slice(n, D, (const double*)ws.M, ws, s)) != cudaSuccess) return e;
     if (nf && !near_late && !near_early) {
         if (fork && (e = cudaEventRecord(ws.ev_p2m, s)) != cudaSuccess) return e;
         if ((e = launch_near(true)) != cudaSuccess) return e;
@@ -1239,6 +1244,10 @@ static cudaError_t run_fmm(int64_t n, int D, int phases, Workspace& ws, bool use
                 e = level_cap(n, l) <= kShiftSmallM2M ? launch_shift_small(0, n, D, l, ws, s)
                                                       : launch_m2m_tc(n, D, l, ws, s);
                 if (e != cudaSuccess) return e;
+                continue;
+            }
+            if (f64) {
+                if ((e = launch_f64_m2m(n, D, l, ws, s)) != cudaSuccess) return e;
                 continue;
             }
             int64_t cl = (int64_t)1 << (3 * l);
@@ -1260,6 +1269,23 @@ static cudaError_t run_fmm(int64_t n, int D, int phases, Workspace& ws, bool use
                                    near_late ? ws.ev_p2m : nullptr)) != cudaSuccess)
             return e;
         if (nf && near_late && (e = launch_near(true)) != cudaSuccess) return e;
+    } else if (f64) {
+        if (pairs_simt && fork && (e = cudaStreamWaitEvent(s, ws.ev_items, 0)) != cudaSuccess)
+            return e;
+        if (ws.kev[0] && (e = record_timing(ws.kev[0], s)) != cudaSuccess) return e;
+        const int64_t tb = target_cells_bound(n, D), step = f64_batched ? ws.f64_batch : tb;
+        for (int64_t t0 = 0; t0 < tb; t0 += step) {
+            const int b0 = (int)t0, b1 = f64_batched ? (int)(t0 + step) : kAllTargets;
+            if (f64_batched && (e = launch_m2l_pairs_worklist(n, D, ws, s, b0, b1)) != cudaSuccess)
+                return e;
+            if ((e = launch_f64_m2l(ws, s)) != cudaSuccess) return e;
+            if (!f64_batched && ws.kev[1] && (e = record_timing(ws.kev[1], s)) != cudaSuccess)
+                return e;
+            if ((e = launch_m2l_pairs_reduce(n, D, ws, ws.ld, s, b0, b1)) != cudaSuccess) return e;
+        }
+        if (f64_batched && ws.kev[1] && (e = record_timing(ws.kev[1], s)) != cudaSuccess) return e;
+        for (int l = 3; l <= D; ++l)
+            if ((e = launch_f64_l2l(n, D, l, ws, s)) != cudaSuccess) return e;
     } else if (pairs_simt) {
         if (fork && (e = cudaStreamWaitEvent(s, ws.ev_items, 0)) != cudaSuccess) return e;
         // M2L products of the work list, the per-target sums, L2L down to

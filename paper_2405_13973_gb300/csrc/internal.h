@@ -101,7 +101,7 @@ struct Workspace {
     int64_t n_max = 0;
     int depth_max = 0;
     int p = 0, P = 0;
-    int ld = 0;                 // row stride of M and L (P for FP64, P rounded up to 32 for FP32)
+    int ld = 0;                 // row stride of M and L (P rounded up to 4 for FP64, to 32 for FP32)
     bool fp64 = true;
     int64_t cells_max = 0;      // capacity of the compact cell arrays
     int sms = 152;              // multiprocessors of the plan's device
@@ -176,6 +176,16 @@ struct Workspace {
     int pp_mirror = 0;
     void* T_rot = nullptr;
     int rot_op_vals = 0;
+    // FP64 translations on the tensor cores (m2l_f64.cu), the default of FP64
+    // plans until a schedule is set: operator digits and their exponents, the
+    // digits [cell][7][lda] and exponents of every cell's M (L in the downward
+    // pass).  f64_batch > 0: the M2L in batches of that many targets, whose
+    // pairs the pool holds whatever the tree
+    int f64_tc = 0;
+    int64_t f64_batch = 0;
+    void* T_f64 = nullptr;
+    uint8_t* f64_dig = nullptr;
+    int* f64_rexp = nullptr;
     // kernel timing (profiled steps only, else null): recorded right before
     // and after the M2L kernel(s) [0, 1] and the near-field kernel [2, 3]
     cudaEvent_t kev[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -246,11 +256,17 @@ size_t m2l_tc_work_bytes(int64_t tiles_cap, int64_t slab_cap);
 // pp_item_cap and pp_stride
 size_t m2l_pp_work_bytes(const Workspace& ws);
 size_t m2l_pp_part_bytes(const Workspace& ws);
-// the work list of the current tree (reads the tree only)
-cudaError_t launch_m2l_pairs_worklist(int64_t n, int D, Workspace& ws, cudaStream_t s);
-// L of every cell of levels 2..D = the sum of its pairs' partial rows
-// (`width` columns)
-cudaError_t launch_m2l_pairs_reduce(int64_t n, int D, Workspace& ws, int width, cudaStream_t s);
+// the work list of the current tree (reads the tree only), of the target
+// cells t0 <= t < t1 in the order of the levels 2..D
+constexpr int kAllTargets = 0x7fffffff;
+cudaError_t launch_m2l_pairs_worklist(int64_t n, int D, Workspace& ws, cudaStream_t s, int t0 = 0,
+                                      int t1 = kAllTargets);
+// L of those cells = the sum of their pairs' partial rows (`width` columns;
+// FP64: ld)
+cudaError_t launch_m2l_pairs_reduce(int64_t n, int D, Workspace& ws, int width, cudaStream_t s,
+                                    int t0 = 0, int t1 = kAllTargets);
+// target cells of levels 2..D at most
+int64_t target_cells_bound(int64_t n, int D);
 // CUDA-core paths: the M2L products of the work list, the reduction and the
 // L2L shifts into levels 3 .. l2l_last
 cudaError_t launch_m2l_pairs_simt(int64_t n, int D, Workspace& ws, int l2l_last, cudaStream_t s);
@@ -260,6 +276,22 @@ cudaError_t m2l_pairs_stats(const Workspace& ws, int64_t* out, cudaStream_t s);
 // this order do not fit), per-device kernel set-up
 int m2l_rot_tile(const Workspace& ws);
 cudaError_t m2l_rot_init();
+// ---- FP64 translations on the tensor cores (m2l_f64.cu) -------------------------
+// digit row stride (bytes), digit bytes of `cells` cells, operator bytes
+int m2l_f64_lda(int p);
+size_t m2l_f64_digit_bytes(int p, int64_t cells);
+size_t m2l_f64_operator_bytes(int p);
+cudaError_t m2l_f64_init();
+// operator digits from the FP64 operators of ws (synchronous)
+cudaError_t m2l_f64_pack(const Workspace& ws);
+// digits of the rows of Y (M or L) of level l's cells
+cudaError_t launch_f64_slice(int64_t n, int l, const double* Y, Workspace& ws, cudaStream_t s);
+// M and its digits at level l from the digits at level l + 1 (L is scratch)
+cudaError_t launch_f64_m2m(int64_t n, int D, int l, Workspace& ws, cudaStream_t s);
+// L at level l += the shift of L at level l - 1
+cudaError_t launch_f64_l2l(int64_t n, int D, int l, Workspace& ws, cudaStream_t s);
+// the partial rows of the pair work list
+cudaError_t launch_f64_m2l(Workspace& ws, cudaStream_t s);
 // the tensor-core partial-row width (P rounded up to 16)
 int m2l_tc_npad(int p);
 // (re)builds ws.pp_map for the current pp_part / pp_rows_cap (BF16 tensor-core

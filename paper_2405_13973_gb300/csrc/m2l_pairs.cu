@@ -30,6 +30,7 @@ namespace {
 struct PpArgs {
     int D;
     int mirror;  // pairs of -o in the runs of o (kPairMirror)
+    int t0, t1;  // the targets t0 <= t < t1 of this list (a batch, or all)
     const LevelInfo* linfo;
     const uint32_t* code;
     const int32_t* cid;
@@ -57,6 +58,12 @@ __device__ __forceinline__ int pp_level(const LevelInfo& li, int D, int g) {
     return l;
 }
 
+// past the last target cell of the list
+__device__ __forceinline__ int pp_end(const LevelInfo& li, const PpArgs& a) {
+    const int g1 = li.gbase[a.D + 1];
+    return g1 - li.gbase[2] > a.t1 ? li.gbase[2] + a.t1 : g1;
+}
+
 // source of candidate c of the target at (x, y, z) of level l, or -1
 __device__ __forceinline__ int pp_source(const PpArgs& a, int l, int x, int y, int z, int c,
                                          int* op) {
@@ -79,7 +86,7 @@ __global__ void __launch_bounds__(kPpThreads) k_pp_count(PpArgs a, uint32_t* tma
     for (int i = threadIdx.x; i < 343; i += blockDim.x) hist[i] = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31;
-    const int g0 = li.gbase[2], g1 = li.gbase[a.D + 1];
+    const int g0 = li.gbase[2] + a.t0, g1 = pp_end(li, a);
     const int wpb = blockDim.x >> 5;
     for (int g = g0 + blockIdx.x * wpb + (threadIdx.x >> 5); g < g1; g += gridDim.x * wpb) {
         const int l = pp_level(li, a.D, g);
@@ -107,7 +114,8 @@ __global__ void __launch_bounds__(kPpThreads) k_pp_count(PpArgs a, uint32_t* tma
 // has n_targets + 1 entries), pair bases of the offsets, and the work items
 // (each offset's pairs in runs of 128, offsets in increasing order).
 constexpr int kPpScanThreads = 1024;
-__global__ void __launch_bounds__(kPpScanThreads) k_pp_scan(int D, const LevelInfo* linfo,
+__global__ void __launch_bounds__(kPpScanThreads) k_pp_scan(int D, int t0, int t1,
+                                                             const LevelInfo* linfo,
                                                              int64_t slot_cap, int64_t rows_cap,
                                                              int item_cap,
                                                              const int* tcount, int* tbase,
@@ -119,7 +127,7 @@ __global__ void __launch_bounds__(kPpScanThreads) k_pp_scan(int D, const LevelIn
     __shared__ int s_carry;
     __shared__ int s_ibase[344];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int nt = linfo->gbase[D + 1] - linfo->gbase[2];
+    const int nt = max(0, min(linfo->gbase[D + 1] - linfo->gbase[2], t1) - t0);
     if (tid == 0) s_carry = 0;
     __syncthreads();
     for (int c0 = 0; c0 < nt; c0 += kPpScanThreads) {
@@ -255,7 +263,7 @@ __global__ void __launch_bounds__(kPpThreads) k_pp_fill(PpArgs a, const uint32_t
     __syncthreads();
     if (hdr->overflow) return;
     const int lane = threadIdx.x & 31;
-    const int g0 = li.gbase[2], g1 = li.gbase[a.D + 1];
+    const int g0 = li.gbase[2] + a.t0, g1 = pp_end(li, a);
     const int wpb = blockDim.x >> 5;
     for (int g = g0 + blockIdx.x * wpb + (threadIdx.x >> 5); g < g1; g += gridDim.x * wpb) {
         const int t = g - g0;
@@ -354,6 +362,63 @@ __global__ void __launch_bounds__(256) k_pp_reduce_f4(int D, int ld, int stride,
                 v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
             }
             *reinterpret_cast<float4*>(L + (int64_t)(g0 + t) * ld + 4 * u) = v;
+        }
+        __syncthreads();
+    }
+}
+
+// FP64 rows (ld and stride multiples of 4): a block per target, 4 x ld / 4
+// threads; thread (j, u) sums the four columns u of the j-th quarter of the
+// target's slots in slot order, four rows in flight, and the quarters are
+// added in order (deterministic).  Bound by the rows' reads and by the FP64
+// adds (one per value at two lanes a clock).
+__global__ void __launch_bounds__(320) k_pp_reduce_d4(int D, int t0, int t1, int ld, int stride,
+                                                       const LevelInfo* linfo, const M2lPairHdr* hdr,
+                                                       const int* tbase,
+                                                       const int* __restrict__ tpair,
+                                                       const double* __restrict__ part, double* L) {
+    pdl_wait();
+    __shared__ double4_32a s_part[kRedParts][(kMaxOrder + 1) * (kMaxOrder + 1) / 4 + 1];
+    const int g0 = linfo->gbase[2] + t0, nt = max(0, min(linfo->gbase[D + 1] - linfo->gbase[2], t1) - t0);
+    const bool over = hdr->overflow != 0;
+    const int w4 = ld / 4, j = threadIdx.x / w4, u = threadIdx.x - j * w4;
+    for (int t = blockIdx.x; t < nt; t += gridDim.x) {
+        const int b0 = tbase[t], b1 = over ? b0 : tbase[t + 1];
+        const int cs = (b1 - b0 + kRedParts - 1) / kRedParts;
+        const int s0 = min(b0 + j * cs, b1), s1 = min(s0 + cs, b1);
+        double4_32a v = make_double4_32a(0, 0, 0, 0);
+        int rw[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) rw[k] = s0 + k < s1 ? tpair[s0 + k] : 0;
+        for (int s = s0; s < s1; s += 4) {
+            double4_32a q[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (s + k < s1)
+                    q[k] = *reinterpret_cast<const double4_32a*>(part + (int64_t)rw[k] * stride + 4 * u);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) rw[k] = s + 4 + k < s1 ? tpair[s + 4 + k] : 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (s + k < s1) {
+                    v.x += q[k].x;
+                    v.y += q[k].y;
+                    v.z += q[k].z;
+                    v.w += q[k].w;
+                }
+        }
+        s_part[j][u] = v;
+        __syncthreads();
+        if (j == 0) {
+#pragma unroll
+            for (int k = 1; k < kRedParts; ++k) {
+                const double4_32a w = s_part[k][u];
+                v.x += w.x;
+                v.y += w.y;
+                v.z += w.z;
+                v.w += w.w;
+            }
+            *reinterpret_cast<double4_32a*>(L + (int64_t)(g0 + t) * ld + 4 * u) = v;
         }
         __syncthreads();
     }
@@ -630,7 +695,7 @@ size_t m2l_pp_part_bytes(const Workspace& ws) {
     return (size_t)ws.pp_rows_cap * ws.pp_stride * (ws.fp64 ? sizeof(double) : sizeof(float));
 }
 
-static int64_t target_cells_bound(int64_t n, int D) {
+int64_t target_cells_bound(int64_t n, int D) {
     int64_t t = 0;
     for (int l = 2; l <= D; ++l) {
         const int64_t cl = (int64_t)1 << (3 * l);
@@ -639,10 +704,13 @@ static int64_t target_cells_bound(int64_t n, int D) {
     return t > 0 ? t : 1;
 }
 
-cudaError_t launch_m2l_pairs_worklist(int64_t n, int D, Workspace& ws, cudaStream_t s) {
+cudaError_t launch_m2l_pairs_worklist(int64_t n, int D, Workspace& ws, cudaStream_t s, int t0,
+                                      int t1) {
     if (D < 2) return cudaSuccess;
     PpArgs a;
     a.D = D;
+    a.t0 = t0;
+    a.t1 = t1;
     // only the BF16x3 tensor-core product reads mirrored pairs (its A rows
     // from the mirrored multipole pieces)
     a.mirror = ws.tc_bf16 && ws.pp_mirror ? 1 : 0;
@@ -655,12 +723,12 @@ cudaError_t launch_m2l_pairs_worklist(int64_t n, int D, Workspace& ws, cudaStrea
     cudaError_t e;
     // the offset counts and fill counters are zero here: zeroed at allocation
     // and by k_pp_scan after use
-    const int64_t tb = target_cells_bound(n, D);
+    const int64_t tb = std::min<int64_t>(target_cells_bound(n, D), (int64_t)t1 - t0);
     const int64_t warps = kPpThreads / 32;
     const unsigned gc = (unsigned)std::min<int64_t>((tb + warps - 1) / warps, 152 * 8);
     k_pp_count<<<gc, kPpThreads, 0, s>>>(a, L.tmask, L.tcount, L.ocnt);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = launch_pdl(k_pp_scan, dim3(1), dim3(kPpScanThreads), 0, s, D,
+    if ((e = launch_pdl(k_pp_scan, dim3(1), dim3(kPpScanThreads), 0, s, D, t0, t1,
                         (const LevelInfo*)ws.linfo, (int64_t)ws.pp_slot_cap,
                         (int64_t)ws.pp_rows_cap, (int)ws.pp_item_cap, (const int*)L.tcount,
                         L.tbase, L.ocnt, L.ofill, L.obase, L.hdr, (M2lPairHdr*)ws.h_pp_hdr,
@@ -673,15 +741,18 @@ cudaError_t launch_m2l_pairs_worklist(int64_t n, int D, Workspace& ws, cudaStrea
 
 
 
-cudaError_t launch_m2l_pairs_reduce(int64_t n, int D, Workspace& ws, int width, cudaStream_t s) {
+cudaError_t launch_m2l_pairs_reduce(int64_t n, int D, Workspace& ws, int width, cudaStream_t s,
+                                    int t0, int t1) {
     if (D < 2) return cudaSuccess;
     PairList L = pair_list(ws);
-    const int64_t tb = target_cells_bound(n, D);
+    const int64_t tb = std::min<int64_t>(target_cells_bound(n, D), (int64_t)t1 - t0);
     const unsigned gr = (unsigned)std::min<int64_t>((tb + 7) / 8, 152 * 16);
     if (ws.fp64) {
-        k_pp_reduce<double><<<gr, 256, 0, s>>>(D, ws.ld, ws.pp_stride, width, ws.linfo, L.hdr,
-                                               L.tbase, L.tpair, (const double*)ws.pp_part,
-                                               (double*)ws.L);
+        const unsigned g4 = (unsigned)std::min<int64_t>(tb, 152 * 32);
+        return launch_pdl(k_pp_reduce_d4, dim3(g4), dim3(kRedParts * (ws.ld / 4)), 0, s, D, t0, t1,
+                          ws.ld, ws.pp_stride, (const LevelInfo*)ws.linfo, (const M2lPairHdr*)L.hdr,
+                          (const int*)L.tbase, (const int*)L.tpair, (const double*)ws.pp_part,
+                          (double*)ws.L);
     } else if (width % 4 == 0 && width <= 256 && ws.pp_stride % 4 == 0 && ws.ld % 4 == 0) {
         const unsigned g4 = (unsigned)std::min<int64_t>(tb, 152 * 32);
         return launch_pdl(k_pp_reduce_f4, dim3(g4), dim3(kRedParts * (width / 4)), 0, s, D,
