@@ -484,6 +484,43 @@ __device__ __forceinline__ void epi_unpark(uint32_t trow, int n, unsigned char* 
     }
 }
 
+// The products of one 32-wide K chunk (A pieces at shared address ah, B
+// pieces after them); MORE = 0: the first product of each accumulator
+// overwrites it.
+template <int BF16, int MORE>
+__device__ __forceinline__ void tc_products(uint32_t d0, uint32_t d1, uint32_t ah, int a_bytes,
+                                            int b_bytes, uint32_t idesc) {
+    if (BF16) {
+        // pieces hi, mid, lo of A then of B; 2 K-steps of 16 values
+        const uint32_t am = ah + a_bytes, al = am + a_bytes;
+        const uint32_t bh = ah + 3 * a_bytes, bm = bh + b_bytes, bl = bm + b_bytes;
+#pragma unroll
+        for (int kk = 0; kk < 2; ++kk) {
+            const uint32_t o = 32 * kk;
+            if (kk == 0) mma_bf16<MORE>(d1, sdesc64(am + o), sdesc64(bm + o), idesc);
+            else mma_bf16<1>(d1, sdesc64(am + o), sdesc64(bm + o), idesc);
+            mma_bf16<1>(d1, sdesc64(ah + o), sdesc64(bl + o), idesc);
+            mma_bf16<1>(d1, sdesc64(al + o), sdesc64(bh + o), idesc);
+            mma_bf16<1>(d1, sdesc64(ah + o), sdesc64(bm + o), idesc);
+            mma_bf16<1>(d1, sdesc64(am + o), sdesc64(bh + o), idesc);
+            if (kk == 0) mma_bf16<MORE>(d0, sdesc64(ah + o), sdesc64(bh + o), idesc);
+            else mma_bf16<1>(d0, sdesc64(ah + o), sdesc64(bh + o), idesc);
+        }
+    } else {
+        const uint32_t al = ah + a_bytes;
+        const uint32_t bh = ah + 2 * a_bytes, bl = bh + b_bytes;
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+            const uint32_t o = 32 * kk;
+            if (kk == 0) mma_tf32<MORE>(d1, sdesc(ah + o), sdesc(bl + o), idesc);
+            else mma_tf32<1>(d1, sdesc(ah + o), sdesc(bl + o), idesc);
+            mma_tf32<1>(d1, sdesc(al + o), sdesc(bh + o), idesc);
+            if (kk == 0) mma_tf32<MORE>(d0, sdesc(ah + o), sdesc(bh + o), idesc);
+            else mma_tf32<1>(d0, sdesc(ah + o), sdesc(bh + o), idesc);
+        }
+    }
+}
+
 // One instantiation per mode and operand format (MODE == MODE, BF16 == BF16):
 // each kernel carries only its own paths.
 template <int MODE, int BF16>
@@ -499,7 +536,8 @@ __global__ void __launch_bounds__((TcLayout<MODE, BF16>::kThreads), 1)
     __shared__ LevelInfo li;
     volatile int* abort_v = &abort_sh;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform to the compiler
     unsigned char* base = (unsigned char*)(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
     const int a_bytes = a.a_bytes, b_bytes = a.b_bytes, pieces = a.pieces;
     const int stage_bytes = pieces * (a_bytes + b_bytes);
@@ -578,68 +616,52 @@ __global__ void __launch_bounds__((TcLayout<MODE, BF16>::kThreads), 1)
             }
         }
     } else if (warp == L::kWarpMma) {
-        // ---- MMA issuer
-        if (lane == 0) {
-            int g = 0, jacc = 0;
-            for (int idx = first; idx < count && !*abort_v; idx += stride) {
-                TcWork w;
-                if (!tc_work<MODE>(a, li, idx, w)) continue;
-                const int n_it = (w.end - w.begin) * a.kchunks;
-                if (n_it == 0) continue;
-                // the epilogue of the previous item has read the accumulators
-                if (jacc > 0 && !mbar_wait_or_abort(&acce_bar, (jacc - 1) & 1, abort_v)) {
-                    *abort_v = 1;
-                    break;
-                }
+        // ---- MMA issuer.  The whole warp runs the loops on warp-uniform
+        // values and one elected lane issues (mbar_wait_warp): issued from a
+        // one-lane branch, the operands of every product were moved to
+        // uniform registers anew and a product of N = 176 took 132 cycles
+        // instead of the tensor core's 88
+        const uint32_t d0 = __shfl_sync(0xffffffffu, tmem, 0);
+        // accumulator 0 takes only the leading products hi x hi, the
+        // rest (2^-8 / 2^-11 of them and smaller) go to accumulator 1
+        const uint32_t d1 = d0 + (uint32_t)a.acc_cols;
+        const uint32_t sbase = smem_addr(base);
+        const int last = __shfl_sync(0xffffffffu, count, 0);
+        int st = 0, ph = 0, pacc = 1;  // stage and its phase, accumulator phase
+        bool ok = true;
+        for (int idx = first; ok && idx < last; idx += stride) {
+            TcWork w;
+            const bool any = tc_work<MODE>(a, li, idx, w);
+            const int n_it = __shfl_sync(0xffffffffu, any ? (w.end - w.begin) * a.kchunks : 0, 0);
+            if (n_it == 0) continue;
+            // the epilogue of the previous item has read the accumulators
+            // (the first wait finds the barrier's initial phase complete)
+            ok = mbar_wait_warp(&acce_bar, pacc, abort_v);
+            pacc ^= 1;
+            if (!ok) break;
+            for (int it = 0; it < n_it; ++it) {
+                ok = mbar_wait_warp(&fullB_bar[st], ph, abort_v) &&
+                     mbar_wait_warp(&fullA_bar[st], ph, abort_v);
+                if (!ok) break;
+                // pre-split A rows arrive by cp.async (generic proxy): order
+                // them before the tensor core's reads
+                if ((MODE == MODE_M2L || MODE == MODE_PAIR) && BF16) fence_proxy_async();
                 tc_fence_after();
-                // accumulator 0 takes only the leading products hi x hi, the
-                // rest (2^-8 / 2^-11 of them and smaller) go to accumulator 1
-                const uint32_t d0 = tmem, d1 = tmem + (uint32_t)a.acc_cols;
-                for (int it = 0; it < n_it; ++it, ++g) {
-                    const int st = g % NS, use = g / NS;
-                    if (!mbar_wait_or_abort(&fullB_bar[st], use & 1, abort_v) ||
-                        !mbar_wait_or_abort(&fullA_bar[st], use & 1, abort_v)) {
-                        *abort_v = 1;
-                        break;
-                    }
-                    // pre-split A rows arrive by cp.async (generic proxy): order
-                    // them before the tensor core's reads
-                    if ((MODE == MODE_M2L || MODE == MODE_PAIR) && BF16) fence_proxy_async();
-                    tc_fence_after();
-                    const uint32_t ah = smem_addr(base + st * stage_bytes);
-                    if (BF16) {
-                        // pieces hi, mid, lo of A then of B; 2 K-steps of 16 values
-                        const uint32_t am = ah + a_bytes, al = am + a_bytes;
-                        const uint32_t bh = ah + 3 * a_bytes, bm = bh + b_bytes, bl = bm + b_bytes;
-#pragma unroll
-                        for (int kk = 0; kk < 2; ++kk) {
-                            const uint32_t acc = (it > 0 || kk > 0) ? 1u : 0u;
-                            const uint32_t o = 32 * kk;
-                            mma_bf16(d1, sdesc64(am + o), sdesc64(bm + o), a.idesc, acc);
-                            mma_bf16(d1, sdesc64(ah + o), sdesc64(bl + o), a.idesc, 1u);
-                            mma_bf16(d1, sdesc64(al + o), sdesc64(bh + o), a.idesc, 1u);
-                            mma_bf16(d1, sdesc64(ah + o), sdesc64(bm + o), a.idesc, 1u);
-                            mma_bf16(d1, sdesc64(am + o), sdesc64(bh + o), a.idesc, 1u);
-                            mma_bf16(d0, sdesc64(ah + o), sdesc64(bh + o), a.idesc, acc);
-                        }
-                    } else {
-                        const uint32_t al = ah + a_bytes;
-                        const uint32_t bh = ah + 2 * a_bytes, bl = bh + b_bytes;
-#pragma unroll
-                        for (int kk = 0; kk < 4; ++kk) {
-                            const uint32_t acc = (it > 0 || kk > 0) ? 1u : 0u;
-                            mma_tf32(d1, sdesc(ah + 32 * kk), sdesc(bl + 32 * kk), a.idesc, acc);
-                            mma_tf32(d1, sdesc(al + 32 * kk), sdesc(bh + 32 * kk), a.idesc, 1u);
-                            mma_tf32(d0, sdesc(ah + 32 * kk), sdesc(bh + 32 * kk), a.idesc, acc);
-                        }
-                    }
+                const uint32_t ah = sbase + (uint32_t)(st * stage_bytes);
+                if (elect_one()) {
+                    if (it == 0) tc_products<BF16, 0>(d0, d1, ah, a_bytes, b_bytes, a.idesc);
+                    else tc_products<BF16, 1>(d0, d1, ah, a_bytes, b_bytes, a.idesc);
                     mma_commit(&empty_bar[st]);  // frees the stage once these MMAs finish
+                    if (it + 1 == n_it) mma_commit(&accf_bar);  // the item's accumulators are complete
                 }
-                if (*abort_v) break;
-                mma_commit(&accf_bar);  // this item's accumulators are complete
-                ++jacc;
+                __syncwarp();
+                if (++st == NS) {
+                    st = 0;
+                    ph ^= 1;
+                }
             }
         }
+        if (!ok) *abort_v = 1;
     } else if (warp >= L::kWarpA0 && warp < L::kWarpA0 + L::kAWarps) {
         if ((MODE == MODE_M2L || MODE == MODE_PAIR) && BF16) {
             // ---- A producers, BF16x3 M2L: the sources' M rows are already

@@ -127,21 +127,17 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int N, int M) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
            ((uint32_t)(M >> 4) << 24);
 }
-__device__ __forceinline__ void mma_tf32(uint32_t dtmem, uint64_t ad, uint64_t bd, uint32_t idesc,
-                                         uint32_t accum) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}" ::"r"(dtmem),
-        "l"(ad), "l"(bd), "r"(idesc), "r"(accum)
-        : "memory");
+template <int ACC>
+__device__ __forceinline__ void mma_tf32(uint32_t dtmem, uint64_t ad, uint64_t bd, uint32_t idesc) {
+    asm volatile("tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, %4;" ::"r"(dtmem), "l"(ad),
+                 "l"(bd), "r"(idesc), "n"(ACC)
+                 : "memory");
 }
-__device__ __forceinline__ void mma_bf16(uint32_t dtmem, uint64_t ad, uint64_t bd, uint32_t idesc,
-                                         uint32_t accum) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(dtmem),
-        "l"(ad), "l"(bd), "r"(idesc), "r"(accum)
-        : "memory");
+template <int ACC>
+__device__ __forceinline__ void mma_bf16(uint32_t dtmem, uint64_t ad, uint64_t bd, uint32_t idesc) {
+    asm volatile("tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, %4;" ::"r"(dtmem), "l"(ad),
+                 "l"(bd), "r"(idesc), "n"(ACC)
+                 : "memory");
 }
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
     asm volatile(
@@ -241,6 +237,12 @@ __device__ __forceinline__ void tmem_wait_st() {
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
+// one elected lane of the converged warp
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(r));
+    return r != 0;
+}
 __device__ __forceinline__ bool mbar_wait_or_abort(uint64_t* bar, uint32_t parity,
                                                    volatile int* abort_flag) {
     if (mbar_try_wait(bar, parity)) return true;
@@ -251,6 +253,15 @@ __device__ __forceinline__ bool mbar_wait_or_abort(uint64_t* bar, uint32_t parit
         if (*abort_flag) return false;
         if (globaltimer_ns() - t0 > kWaitLimitNs) return false;
     }
+}
+
+// the same for a whole warp, with one answer for all lanes: control flow that
+// depends on it stays warp-uniform (tcgen05.mma takes its operands from
+// uniform registers, and in code that the compiler has to treat as divergent
+// every operand is moved there anew for every instruction)
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity,
+                                               volatile int* abort_flag) {
+    return __all_sync(0xffffffffu, mbar_wait_or_abort(bar, parity, abort_flag)) != 0;
 }
 
 }  // namespace pt
