@@ -62,9 +62,11 @@ namespace {
 constexpr int kDig = 7;                 // digits per coefficient
 constexpr int kChunk = 48;              // output columns per chunk (at most)
 constexpr int kF64Rows = 128;
+constexpr int kSegBytes = kDig * 32;    // digits of one row in a 32-wide K segment
+constexpr int kMaxRing = 5;             // ring slots of digit rows
 constexpr int kAStages = 3;             // K steps of A in tensor memory
 constexpr int kACol0 = kDig * kChunk;   // their first TMEM column
-constexpr int kBStages = 4;             // 32-wide K chunks of B in shared memory
+constexpr int kBStages = 4;             // 32-wide K chunks of B in shared memory (at most)
 constexpr int kF64Threads = 448;
 constexpr int kF64Ops = 359;            // 343 M2L offsets, 8 M2M, 8 L2L octants
 constexpr int kF64M2M = 343, kF64L2L = 351;
@@ -74,9 +76,11 @@ enum F64Mode { F64_PAIR = 0, F64_M2M = 1, F64_L2L = 2 };
 
 struct F64Args {
     int P, ld, lda;            // coefficients, row stride of M, L and partial rows, digit row stride
-    int npad, ksteps, kst32, nch, level, sms;
+    int npad, ksteps, kst32, nch, level;
+    int ring, gsegs, resident, bst;  // A ring slots, K segments in each, items resident, B stages
+    int64_t zero_cell;         // a cell whose digits are all zero
     int64_t out_stride, op_bytes;
-    const uint8_t* dig;        // [cell][kDig][lda]
+    const uint8_t* dig;        // [cell][kst32][kDig][32]
     const int* rexp;           // [cell]
     const unsigned char* ops;  // [kF64Ops][chunk][kst32][kDig][columns][64 B]
     const int16_t* oexp;       // [kF64Ops][npad]
@@ -95,13 +99,29 @@ struct F64Args {
 __device__ __forceinline__ uint32_t idesc_f16(int N) {
     return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kF64Rows >> 4) << 24);
 }
-__device__ __forceinline__ void mma_f16_ts(uint32_t dtmem, uint32_t atmem, uint64_t bd,
-                                           uint32_t idesc, uint32_t accum) {
+template <int ACC>
+__device__ __forceinline__ void mma_f16_ts(uint32_t dtmem, uint32_t atmem, uint32_t blo,
+                                           uint32_t bhi, uint32_t idesc) {
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(dtmem),
-        "r"(atmem), "l"(bd), "r"(idesc), "r"(accum)
+        "{\n .reg .b64 b;\n mov.b64 b, {%2, %3};\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %4, %5;\n}" ::"r"(dtmem),
+        "r"(atmem), "r"(blo), "r"(bhi), "r"(idesc), "n"(ACC)
         : "memory");
+}
+// the 28 products of a K step; MORE = 0: the first of an accumulator
+// overwrites it
+template <int MORE>
+__device__ __forceinline__ void f64_products(uint32_t tm, uint32_t at, uint32_t blo, uint32_t bhi,
+                                             uint32_t bstep, uint32_t id) {
+#pragma unroll
+    for (int j = 0; j < kDig; ++j)
+        mma_f16_ts<MORE>(tm + (uint32_t)(j * kChunk), at, blo + bstep * (uint32_t)j, bhi, id);
+#pragma unroll
+    for (int i = 1; i < kDig; ++i)
+#pragma unroll
+        for (int j = 0; j + i < kDig; ++j)
+            mma_f16_ts<1>(tm + (uint32_t)((i + j) * kChunk), at + (uint32_t)(8 * i),
+                          blo + bstep * (uint32_t)j, bhi, id);
 }
 __device__ __forceinline__ void tmem_ld8_nw(uint32_t taddr, uint32_t (&r)[8]) {
     asm volatile(
@@ -131,6 +151,22 @@ __device__ __forceinline__ void expand16(const uint4& v, uint32_t (&h)[8]) {
         h[2 * q] = *reinterpret_cast<const uint32_t*>(&a);
         h[2 * q + 1] = *reinterpret_cast<const uint32_t*>(&b);
     }
+}
+
+__device__ __forceinline__ void tmem_ld1(uint32_t taddr, uint32_t (&r)[1]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r[0]) : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+// sum_d s_d 2^(8 (5 - d)), the last term rounded to an integer, from the bits
+// v_d of s_d + 1.5 2^23 (|s_d| < 2^22): neighbours joined in 32 bits
+// (|256 s + s'| < 2^31), the biases taken off modulo 2^32
+__device__ __forceinline__ long long f64_join(const uint32_t (&v)[kDig]) {
+    constexpr uint32_t B = 0x4B400000u, B2 = 257u * B;
+    const int u = (int)(v[0] * 256u + v[1] - B2);
+    const int w = (int)(v[2] * 256u + v[3] - B2);
+    const int x = (int)(v[4] * 256u + v[5] - B2) + (((int)(v[6] - B) + 128) >> 8);
+    return ((long long)u << 32) + ((long long)w * 65536 + (long long)x);
 }
 
 // I 2^e as a double, rounded to nearest, without the FP64 units
@@ -200,12 +236,13 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
     extern __shared__ unsigned char smem_dyn[];
     pdl_wait();
     __shared__ __align__(8) uint64_t fullA[kAStages], emptyA[kAStages], fullB[kBStages],
-        emptyB[kBStages], accf, acce, drain_bar;
+        emptyB[kBStages], fullR[kMaxRing], accf, acce, drain_bar;
     __shared__ uint32_t tmem_base_sh;
     __shared__ int abort_sh;
     __shared__ LevelInfo li;
     volatile int* abort_v = &abort_sh;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform to the compiler
     unsigned char* base = (unsigned char*)(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
     const int b_stage = kDig * min(kChunk, a.npad) * 64;
     if (MODE != F64_PAIR) {
@@ -223,6 +260,7 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
             mbar_init(&fullB[s], 1);
             mbar_init(&emptyB[s], 1);
         }
+        for (int s = 0; s < kMaxRing; ++s) mbar_init(&fullR[s], 128);
         mbar_init(&accf, 1);
         mbar_init(&acce, 256);
         mbar_init(&drain_bar, 1);
@@ -243,6 +281,7 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_base_sh;
+    int r_issued = 0;     // A producers: digit copies issued
     int b_par[kBStages];  // operator producer: parity of the last copy per stage
 #pragma unroll
     for (int s = 0; s < kBStages; ++s) b_par[s] = -1;
@@ -257,7 +296,7 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
                 for (int c = 0; c < a.nch; ++c) {
                     const uint32_t bytes = (uint32_t)(kDig * min(kChunk, a.npad - c * kChunk) * 64);
                     for (int k = 0; k < a.kst32; ++k, ++g) {
-                        const int st = g % kBStages, use = g / kBStages;
+                        const int st = g % a.bst, use = g / a.bst;
                         if (!mbar_wait_or_abort(&emptyB[st], (use & 1) ^ 1, abort_v)) {
                             *abort_v = 1;
                             break;
@@ -274,119 +313,135 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
             }
         }
     } else if (warp == 9) {
-        // ---- MMA issuer
-        if (lane == 0) {
-            int ga = 0, gb = 0, jacc = 0;
-            F64Work w;
-            for (int idx = first; f64_work<MODE>(a, li, idx, count, w) && !*abort_v; idx += stride) {
-                for (int c = 0; c < a.nch && !*abort_v; ++c, ++jacc) {
-                    const int N = min(kChunk, a.npad - c * kChunk);
-                    const uint32_t id = idesc_f16(N);
-                    const uint64_t bstep = (uint64_t)((N * 64) >> 4);  // one digit of B
-                    // the epilogue has read the previous chunk's accumulators
-                    if (jacc > 0 && !mbar_wait_or_abort(&acce, (jacc - 1) & 1, abort_v)) {
-                        *abort_v = 1;
-                        break;
-                    }
-                    for (int ks = 0; ks < a.ksteps; ++ks, ++ga) {
-                        const int sb = gb % kBStages, ub = gb / kBStages;
-                        const int sa = ga % kAStages, ua = ga / kAStages;
-                        if (!(ks & 1) && !mbar_wait_or_abort(&fullB[sb], ub & 1, abort_v)) {
-                            *abort_v = 1;
-                            break;
-                        }
-                        if (!mbar_wait_or_abort(&fullA[sa], ua & 1, abort_v)) {
-                            *abort_v = 1;
-                            break;
-                        }
-                        tc_fence_after();
-                        const uint64_t bd = sdesc64(smem_addr(base + sb * b_stage) + 32u * (ks & 1));
-                        const uint32_t at = tmem + (uint32_t)(kACol0 + sa * kDig * 8);
-                        const uint32_t more = ks > 0 ? 1u : 0u;
-#pragma unroll
-                        for (int i = 0; i < kDig; ++i)
-#pragma unroll
-                            for (int j = 0; j + i < kDig; ++j)
-                                mma_f16_ts(tmem + (uint32_t)((i + j) * kChunk), at + (uint32_t)(8 * i),
-                                           bd + bstep * (uint64_t)j, id, i > 0 ? 1u : more);
+        // ---- MMA issuer.  The whole warp runs the loops on warp-uniform
+        // values and one elected lane issues (mbar_wait_warp)
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+        const int items = __shfl_sync(0xffffffffu, (count - first + stride - 1) / stride, 0);
+        int sa = 0, pa = 0, sb = 0, pb = 0, pacc = 1;  // stages and phases
+        bool ok = true;
+        for (int t = 0; ok && t < items; ++t) {
+            for (int c = 0; ok && c < a.nch; ++c) {
+                const int N = min(kChunk, a.npad - c * kChunk);
+                const uint32_t id = idesc_f16(N);
+                const uint32_t bstep = (uint32_t)(N * 64) >> 4;  // one digit of B
+                // the epilogue has read the previous chunk's accumulators
+                // (the first wait finds the barrier's initial phase complete)
+                ok = mbar_wait_warp(&acce, pacc, abort_v);
+                pacc ^= 1;
+                if (!ok) break;
+                for (int ks = 0; ks < a.ksteps; ++ks) {
+                    if (!(ks & 1)) ok = mbar_wait_warp(&fullB[sb], pb, abort_v);
+                    ok = ok && mbar_wait_warp(&fullA[sa], pa, abort_v);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint64_t bd = sdesc64(smem_addr(base) + (uint32_t)(sb * b_stage) + 32u * (ks & 1));
+                    const uint32_t blo = (uint32_t)bd, bhi = (uint32_t)(bd >> 32);
+                    const uint32_t at = tm + (uint32_t)(kACol0 + sa * kDig * 8);
+                    const bool last = (ks & 1) || ks + 1 == a.ksteps;
+                    if (elect_one()) {
+                        if (ks == 0) f64_products<0>(tm, at, blo, bhi, bstep, id);
+                        else f64_products<1>(tm, at, blo, bhi, bstep, id);
                         mma_commit(&emptyA[sa]);
-                        if ((ks & 1) || ks + 1 == a.ksteps) {
-                            mma_commit(&emptyB[sb]);
-                            ++gb;
-                        }
+                        if (last) mma_commit(&emptyB[sb]);
+                        if (ks + 1 == a.ksteps) mma_commit(&accf);
                     }
-                    if (*abort_v) break;
-                    mma_commit(&accf);
+                    __syncwarp();
+                    if (++sa == kAStages) {
+                        sa = 0;
+                        pa ^= 1;
+                    }
+                    if (last && ++sb == a.bst) {
+                        sb = 0;
+                        pb ^= 1;
+                    }
                 }
             }
         }
+        if (!ok) *abort_v = 1;
     } else if (warp >= 10) {
-        // ---- A producers: thread = row; a K step's seven digit groups (16
-        // bytes each) are loaded two steps ahead of their expansion
+        // ---- A producers, thread = row.  Each thread brings its own row's
+        // digits (contiguous in memory) by bulk copies of a.gsegs K segments
+        // into its part of a ring slot, reads them back and expands them; it
+        // alone reads and refills that part, so the rows need no barrier but
+        // the slot's transaction count.  When an item's slots fit
+        // (a.resident) they are loaded once and read by every column chunk,
+        // and a slot is refilled for a later item while the last chunk runs;
+        // else each chunk streams them.
         const int quad = warp & 3, row = quad * 32 + lane;
         const uint32_t tq = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)kACol0;
         const int64_t cell_bytes = (int64_t)kDig * a.lda;
-        int idx = first, c = 0, k = 0;  // the next step to load
+        const int row_bytes = a.gsegs * kSegBytes + 16;  // 16: no bank conflicts
+        unsigned char* ring = base + a.bst * b_stage + row * row_bytes;
+        const int groups = (a.kst32 + a.gsegs - 1) / a.gsegs;
+        const int loads = a.resident ? groups : a.nch * groups;  // per item
         F64Work w;
-        bool more = f64_work<MODE>(a, li, idx, count, w);
-        int src = more ? f64_source<MODE>(a, w, row) : -1, nsrc = -1;
-        if (f64_work<MODE>(a, li, idx + stride, count, w)) nsrc = f64_source<MODE>(a, w, row);
-        auto load = [&](uint4 (&b)[kDig]) {
-            if (!more) return;
-            const uint8_t* p = a.dig + (int64_t)(src < 0 ? 0 : src) * cell_bytes + 16 * k;
+        // the loading side: item lidx, its load lo; the source of the item
+        // after it waits in a register
+        int lidx = first, lo = 0, lslot = 0, issued = 0, freed = 0;
+        int src = f64_work<MODE>(a, li, lidx, count, w) ? f64_source<MODE>(a, w, row) : -1, nsrc = -1;
+        if (f64_work<MODE>(a, li, lidx + stride, count, w)) nsrc = f64_source<MODE>(a, w, row);
+        auto issue = [&]() {
+            if (lidx >= count || issued - freed >= a.ring) return;
+            const int grp = lo % groups;
+            const uint32_t bytes = (uint32_t)(min(a.gsegs, a.kst32 - grp * a.gsegs) * kSegBytes);
+            mbar_arrive_expect_tx(&fullR[lslot], bytes);
+            bulk_g2s(ring + lslot * kF64Rows * row_bytes,
+                     a.dig + (int64_t)(src < 0 ? a.zero_cell : src) * cell_bytes +
+                         (int64_t)grp * a.gsegs * kSegBytes,
+                     bytes, &fullR[lslot]);
+            if (++lslot == a.ring) lslot = 0;
+            r_issued = ++issued;
+            if (++lo == loads) {
+                lo = 0;
+                lidx += stride;
+                src = nsrc;
+                nsrc = -1;
+                if (f64_work<MODE>(a, li, lidx + stride, count, w)) nsrc = f64_source<MODE>(a, w, row);
+            }
+        };
+        for (int k = 0; k < a.ring; ++k) issue();
+        int sa = 0, pa = 1, used = 0;  // A stage and phase, the item's first load
+        bool ok = true;
+        for (int idx = first; ok && idx < count; idx += stride, used += loads) {
+            for (int c = 0; ok && c < a.nch; ++c) {
+                for (int grp = 0; ok && grp < groups; ++grp) {
+                    const int id = used + (a.resident ? grp : c * groups + grp);
+                    const int slot = id % a.ring;
+                    ok = mbar_wait_warp(&fullR[slot], (id / a.ring) & 1, abort_v);
+                    const unsigned char* mine = ring + slot * kF64Rows * row_bytes;
+                    const int ks0 = grp * a.gsegs * 2, ks1 = min(a.ksteps, ks0 + a.gsegs * 2);
+#pragma unroll 1
+                    for (int ks = ks0; ok && ks < ks1; ++ks) {
+                        const unsigned char* at = mine + ((ks - ks0) >> 1) * kSegBytes + (ks & 1) * 16;
+                        uint4 b[kDig];
 #pragma unroll
-            for (int i = 0; i < kDig; ++i)
-                b[i] = src >= 0 ? __ldg(reinterpret_cast<const uint4*>(p + i * a.lda))
-                                : make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
-            if (++k == a.ksteps) {
-                k = 0;
-                if (++c == a.nch) {
-                    c = 0;
-                    idx += stride;
-                    more = idx < count;
-                    src = nsrc;
-                    nsrc = -1;
-                    if (f64_work<MODE>(a, li, idx + stride, count, w))
-                        nsrc = f64_source<MODE>(a, w, row);
+                        for (int i = 0; i < kDig; ++i)
+                            b[i] = *reinterpret_cast<const uint4*>(at + i * 32);
+                        ok = mbar_wait_warp(&emptyA[sa], pa, abort_v);
+                        if (!ok) break;
+                        tc_fence_after();
+#pragma unroll
+                        for (int i = 0; i < kDig; ++i) {
+                            uint32_t h[8];
+                            expand16(b[i], h);
+                            tmem_st8(tq + (uint32_t)(sa * kDig * 8 + 8 * i), h);
+                        }
+                        tmem_wait_st();
+                        tc_fence_before();
+                        mbar_arrive(&fullA[sa]);
+                        if (++sa == kAStages) {
+                            sa = 0;
+                            pa ^= 1;
+                        }
+                    }
+                    if (!a.resident || c + 1 == a.nch) {
+                        ++freed;
+                        issue();
+                    }
                 }
             }
-        };
-        int g = 0;
-        auto store = [&](const uint4 (&b)[kDig]) -> bool {
-            const int st = g % kAStages, use = g / kAStages;
-            ++g;
-            int ok = 1;
-            if (lane == 0) ok = mbar_wait_or_abort(&emptyA[st], (use & 1) ^ 1, abort_v) ? 1 : 0;
-            ok = __shfl_sync(0xffffffffu, ok, 0);
-            if (!ok) {
-                *abort_v = 1;
-                return false;
-            }
-            tc_fence_after();
-#pragma unroll
-            for (int i = 0; i < kDig; ++i) {
-                uint32_t h[8];
-                expand16(b[i], h);
-                tmem_st8(tq + (uint32_t)(st * kDig * 8 + 8 * i), h);
-            }
-            tmem_wait_st();
-            tc_fence_before();
-            mbar_arrive(&fullA[st]);
-            return true;
-        };
-        uint4 b0[kDig], b1[kDig];
-        bool h0 = more;
-        load(b0);
-        bool h1 = more;
-        load(b1);
-        while (h0) {
-            if (!store(b0)) break;
-            h0 = more;
-            load(b0);
-            if (!h1 || !store(b1)) break;
-            h1 = more;
-            load(b1);
         }
+        if (!ok) *abort_v = 1;
     } else {
         // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 (row =
         // lane), warps 0..3 the first half of a chunk's columns, 4..7 the rest
@@ -418,6 +473,7 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
                 }
                 tc_fence_after();
                 long long I[3][8];
+                uint32_t big = 0;  // bits 23 and up set by a sum of 2^22 or more
 #pragma unroll
                 for (int q = 0; q < 3; ++q) {
                     if (q >= ng) break;  // uniform
@@ -428,15 +484,36 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
                     tmem_wait_ld();
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
-                        int v[kDig];
+                        // s + 1.5 2^23 holds the integer s in its low bits
+                        // while |s| < 2^22 (crystals stay below 2^20); the
+                        // conversion instruction runs at 16 a clock, the add at 128
+                        uint32_t v[kDig];
 #pragma unroll
-                        for (int d = 0; d < kDig; ++d) v[d] = __float2int_rn(__uint_as_float(s[d][j]));
-                        const long long hi = (long long)v[0] * (1 << 24) +
-                                             ((long long)v[1] * (1 << 16) +
-                                              ((long long)v[2] * (1 << 8) + (long long)v[3]));
-                        const long long lo = (long long)v[4] * (1 << 16) +
-                                             ((long long)v[5] * (1 << 8) + (long long)v[6]);
-                        I[q][j] = (hi << 16) + ((lo + 128) >> 8);
+                        for (int d = 0; d < kDig; ++d) {
+                            v[d] = __float_as_uint(__uint_as_float(s[d][j]) + 12582912.f);
+                            big |= v[d] ^ 0x4B400000u;
+                        }
+                        I[q][j] = f64_join(v);
+                    }
+                    if (__any_sync(0xffffffffu, big >> 23)) {
+                        // (uniform, rare) sums up to 2^24 by conversion
+#pragma unroll 1
+                        for (int j = 0; j < 8; ++j) {
+                            long long S = 0;
+#pragma unroll 1
+                            for (int d = 0; d < kDig - 1; ++d) {
+                                uint32_t x[1];
+                                tmem_ld1(tq + (uint32_t)(d * kChunk + c0 + 8 * q + j), x);
+                                S += (long long)__float2int_rn(__uint_as_float(x[0])) << (40 - 8 * d);
+                            }
+                            uint32_t x[1];
+                            tmem_ld1(tq + (uint32_t)((kDig - 1) * kChunk + c0 + 8 * q + j), x);
+                            S += ((long long)__float2int_rn(__uint_as_float(x[0])) + 128) >> 8;
+#pragma unroll
+                            for (int jj = 0; jj < 8; ++jj)
+                                if (jj == j) I[q][jj] = S;
+                        }
+                        big = 0;
                     }
                 }
                 tc_fence_before();
@@ -486,6 +563,9 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
                 if (b_par[s] >= 0) mbar_wait(&fullB[s], (uint32_t)b_par[s]);
             atomicOr(a.err, ERR_TIMEOUT);
         }
+        if (warp >= 10)
+            for (int k = max(0, r_issued - a.ring); k < r_issued; ++k)
+                mbar_wait(&fullR[k % a.ring], (uint32_t)((k / a.ring) & 1));
     }
     tc_fence_before();
     __syncthreads();
@@ -518,7 +598,7 @@ constexpr int kSliceThreads = 256;
 constexpr int kSliceRegs = ((kMaxOrder + 1) * (kMaxOrder + 1) + 31) / 32;
 
 // a warp writes the digits of one row, lane l holding coefficients l + 32 r
-__device__ __forceinline__ void store_digits(const double (&v)[kSliceRegs], int P, int lane, int lda,
+__device__ __forceinline__ void store_digits(const double (&v)[kSliceRegs], int P, int lane,
                                              uint8_t* dig, int* rexp) {
     int emax = 0;
 #pragma unroll
@@ -531,13 +611,14 @@ __device__ __forceinline__ void store_digits(const double (&v)[kSliceRegs], int 
         const int k = lane + 32 * r;
         if (k >= P) break;
         long long X = emax == 0x7ff ? 0ll : fixed54(v[r], emax);
+        uint8_t* d = dig + (k >> 5) * kSegBytes + lane;  // [k / 32][digit][k % 32]
 #pragma unroll
         for (int s = kDig - 1; s > 0; --s) {
             const long long t = X + 128;
-            dig[s * lda + k] = (uint8_t)(t & 255);
+            d[s * 32] = (uint8_t)(t & 255);
             X = t >> 8;
         }
-        dig[k] = (uint8_t)(X + 128);
+        d[0] = (uint8_t)(X + 128);
     }
 }
 
@@ -555,7 +636,7 @@ __global__ void __launch_bounds__(kSliceThreads) k_f64_slice(int level, int P, i
 #pragma unroll
         for (int r = 0; r < kSliceRegs; ++r)
             v[r] = lane + 32 * r < P ? Y[(int64_t)g * ld + lane + 32 * r] : 0.0;
-        store_digits(v, P, lane, lda, dig + (int64_t)g * kDig * lda, rexp + g);
+        store_digits(v, P, lane, dig + (int64_t)g * kDig * lda, rexp + g);
     }
 }
 
@@ -584,7 +665,7 @@ __global__ void __launch_bounds__(kSliceThreads) k_f64_parents(
 #pragma unroll
         for (int r = 0; r < kSliceRegs; ++r)
             if (lane + 32 * r < P) M[(int64_t)g * ld + lane + 32 * r] = v[r];
-        store_digits(v, P, lane, lda, dig + (int64_t)g * kDig * lda, rexp + g);
+        store_digits(v, P, lane, dig + (int64_t)g * kDig * lda, rexp + g);
     }
 }
 
@@ -635,6 +716,43 @@ __global__ void __launch_bounds__(256) k_f64_pack(int op0, int nops, int P, int 
     }
 }
 
+// bytes of a ring slot of g K segments
+int f64_slot(int g) { return kF64Rows * (g * kSegBytes + 16); }
+constexpr int kF64SmemMax = 227 * 1024 - 3 * 1024;
+
+int f64_smem(const F64Args& a) {
+    return a.bst * kDig * std::min(kChunk, a.npad) * 64 + f64_slot(a.gsegs) * a.ring + 1024;
+}
+
+// Shared memory: an item's digits resident in two (or a multiple of) slots
+// where they fit beside two B stages (p <= 12), else five one-segment slots
+// streamed; the rest to B stages.
+void f64_rings(F64Args& a) {
+    const int half = (a.kst32 + 1) / 2, groups = (a.kst32 + half - 1) / half;
+    a.gsegs = half;
+    a.bst = 2;
+    a.ring = groups;
+    a.resident = f64_smem(a) <= kF64SmemMax ? 1 : 0;
+    if (!a.resident) {
+        a.gsegs = 1;
+        a.ring = kMaxRing;
+    }
+    while (a.bst < kBStages) {
+        ++a.bst;
+        if (f64_smem(a) > kF64SmemMax) {
+            --a.bst;
+            break;
+        }
+    }
+    while (a.resident && a.ring + groups < kMaxRing) {
+        a.ring += groups;
+        if (f64_smem(a) > kF64SmemMax) {
+            a.ring -= groups;
+            break;
+        }
+    }
+}
+
 F64Args f64_args(const Workspace& ws) {
     F64Args a;
     memset(&a, 0, sizeof a);
@@ -646,6 +764,8 @@ F64Args f64_args(const Workspace& ws) {
     a.kst32 = (ws.P + 31) / 32;
     a.nch = (a.npad + kChunk - 1) / kChunk;
     a.op_bytes = (int64_t)a.kst32 * kDig * a.npad * 64;
+    f64_rings(a);
+    a.zero_cell = ws.cells_max;
     a.dig = ws.f64_dig;
     a.rexp = ws.f64_rexp;
     a.ops = (const unsigned char*)ws.T_f64;
@@ -656,8 +776,6 @@ F64Args f64_args(const Workspace& ws) {
     a.err = ws.err;
     return a;
 }
-
-int f64_smem(int npad) { return kBStages * kDig * std::min(kChunk, npad) * 64 + 1024; }
 
 unsigned f64_grid(const Workspace& ws, int64_t items) {
     int64_t g = ws.m2l_ctas > 0 ? std::min(ws.m2l_ctas, ws.sms) : ws.sms;
@@ -673,7 +791,9 @@ unsigned slice_grid(int64_t rows) {
 
 int m2l_f64_lda(int p) { return ((p + 1) * (p + 1) + 31) / 32 * 32; }
 
-size_t m2l_f64_digit_bytes(int p, int64_t cells) { return (size_t)cells * kDig * m2l_f64_lda(p); }
+size_t m2l_f64_digit_bytes(int p, int64_t cells) {
+    return (size_t)(cells + 1) * kDig * m2l_f64_lda(p);  // and one cell of zeros
+}
 
 size_t m2l_f64_operator_bytes(int p) {
     const int64_t P = (p + 1) * (p + 1), npad = (P + 15) / 16 * 16, k32 = (P + 31) / 32;
@@ -681,14 +801,10 @@ size_t m2l_f64_operator_bytes(int p) {
 }
 
 cudaError_t m2l_f64_init() {
-    const int smem = f64_smem(kChunk);
-    // the rest of the SM's memory as L1: the digit rows are read once per chunk
-    const int carve = 45;
     for (const void* f : {(const void*)k_f64_mma<F64_PAIR>, (const void*)k_f64_mma<F64_M2M>,
                           (const void*)k_f64_mma<F64_L2L>}) {
-        cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, carve);
+        cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             kF64SmemMax);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -724,7 +840,7 @@ cudaError_t launch_f64_m2m(int64_t n, int D, int l, Workspace& ws, cudaStream_t 
     a.out_stride = ws.ld;
     const int64_t items = level_cap(n, l + 1) / kF64Rows + 8;
     cudaError_t e = launch_pdl(k_f64_mma<F64_M2M>, dim3(f64_grid(ws, items)), dim3(kF64Threads),
-                               f64_smem(a.npad), s, a);
+                               f64_smem(a), s, a);
     if (e != cudaSuccess) return e;
     return launch_pdl(k_f64_parents, dim3(slice_grid(level_cap(n, l))), dim3(kSliceThreads), 0, s, l,
                       ws.P, ws.ld, a.lda, (const LevelInfo*)ws.linfo, (const uint32_t*)ws.code,
@@ -742,7 +858,7 @@ cudaError_t launch_f64_l2l(int64_t n, int D, int l, Workspace& ws, cudaStream_t 
     a.out_stride = ws.ld;
     const int64_t items = level_cap(n, l) / kF64Rows + 8;
     return launch_pdl(k_f64_mma<F64_L2L>, dim3(f64_grid(ws, items)), dim3(kF64Threads),
-                      f64_smem(a.npad), s, a);
+                      f64_smem(a), s, a);
 }
 
 cudaError_t launch_f64_m2l(Workspace& ws, cudaStream_t s) {
@@ -753,7 +869,7 @@ cudaError_t launch_f64_m2l(Workspace& ws, cudaStream_t s) {
     a.pairs = L.pairs;
     a.out = (double*)ws.pp_part;
     a.out_stride = ws.pp_stride;
-    k_f64_mma<F64_PAIR><<<f64_grid(ws, ws.pp_item_cap), kF64Threads, f64_smem(a.npad), s>>>(a);
+    k_f64_mma<F64_PAIR><<<f64_grid(ws, ws.pp_item_cap), kF64Threads, f64_smem(a), s>>>(a);
     return cudaGetLastError();
 }
 
