@@ -1419,6 +1419,10 @@ int pt_set_damping(fmm_plan plan, double gamma) {
 namespace {
 // scratch of the temperature reduction: {T_par, T_perp} and per-block partials
 static __device__ __align__(256) double g_diag_scratch[2 + 2 * 256];
+// scratch of pt_mh_scans up to kMhStaticIons ions: a call's cudaMalloc and
+// cudaFree cost as much as a scan of 1,000 ions
+constexpr int64_t kMhStaticIons = 4096;
+static __device__ __align__(256) double g_mh_scratch[mh_scratch_doubles(kMhStaticIons)];
 std::mutex g_diag_mu;
 }  // namespace
 
@@ -1462,18 +1466,26 @@ int pt_mh_scans(const pt_state* st, const pt_trap* trap, double temperature, dou
     std::lock_guard<std::mutex> g(g_diag_mu);
     double* d = nullptr;
     double* scratch = nullptr;
+    double* own = nullptr;
+    int dev = 0, sms = 0;
     cudaError_t e = cudaGetSymbolAddress((void**)&d, g_diag_scratch);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaStream_t s = (cudaStream_t)stream;
-    const size_t sb = mh_scratch_bytes(st->n);
-    if (e == cudaSuccess && sb > 0 && cudaMalloc((void**)&scratch, sb) != cudaSuccess)
-        return PT_ERR_OOM;
+    if (e == cudaSuccess && st->n <= kMhStaticIons)
+        e = cudaGetSymbolAddress((void**)&scratch, g_mh_scratch);
+    else if (e == cudaSuccess) {
+        if (cudaMalloc((void**)&own, sizeof(double) * mh_scratch_doubles(st->n)) != cudaSuccess)
+            return PT_ERR_OOM;
+        scratch = own;
+    }
     if (e == cudaSuccess)
         e = launch_mh_scans(st->n, st->x, st->y, st->z, st->q, mp, scan0, n_scans,
-                            (unsigned long long*)d, d + 1, scratch, s);
+                            (unsigned long long*)d, d + 1, scratch, sms, s);
     double h[2] = {0, 0};
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, d, sizeof h, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (scratch) cudaFree(scratch);
+    if (own) cudaFree(own);
     if (e != cudaSuccess) return status_from(e);
     unsigned long long a;
     memcpy(&a, &h[0], sizeof a);

@@ -347,11 +347,16 @@ struct MhParams {
     double temp, dx;        // temperature (K), largest displacement (m)
     uint64_t seed;
 };
-// scratch: mh_scratch_bytes(n) of device memory (none needed for large n)
-size_t mh_scratch_bytes(int64_t n);
+constexpr int kMhBatch = 128;      // moves summed at once
+constexpr int kMhMaxChunks = 64;   // source ranges per move
+constexpr int kMhProp = 7;         // per ion: b, U(b) - U(a), the window of dE, the accept uniform
+// doubles of device scratch
+constexpr size_t mh_scratch_doubles(int64_t n) {
+    return (size_t)kMhProp * n + kMhBatch * kMhMaxChunks + kMhBatch * kMhBatch;
+}
 cudaError_t launch_mh_scans(int64_t n, double* x, double* y, double* z, const double* q,
                             const MhParams& mp, int64_t scan0, int64_t n_scans,
-                            unsigned long long* acc_out, double* de_out, double* scratch,
+                            unsigned long long* acc_out, double* de_out, double* scratch, int sms,
                             cudaStream_t s);
 
 cudaError_t launch_drift_bbox(int64_t n, double* x, double* y, double* z, double* vx, double* vy,

@@ -17,22 +17,39 @@
 // Marsaglia's disc pick of the direction.  The distance depends on |b - a|
 // only: the proposal is symmetric.
 //
-// Crystals of up to 4096 ions run on a cluster of 8 CTAs (below), larger ones
-// on one 1024-thread block: thread 0 draws the proposal and takes the
-// decision, all threads sum the Coulomb change over their share of the other
-// ions (FP64), combined by a fixed tree (deterministic).  Compiled with
-// -fmad=false like the push, so the proposal and U are the literal IEEE
-// sequence; the pair sum (its order, and rsqrt on the cluster path) differs
-// from the sequential 1/sqrt sum only in the last bits of dE.
-#include <cooperative_groups.h>
+// The chain is sequential, but only through the moves that were kept: a
+// batch of kMhBatch consecutive moves is summed against the positions at its
+// start on the whole GPU, together with what each kept move j of the batch
+// adds to the energy change of each later one k,
+//   C_jk = k_e q_k q_j [(1/|b_k - b_j| - 1/|a_k - b_j|) - (1/|b_k - a_j| - 1/|a_k - a_j|)],
+// and one warp then takes the decisions in order, adding row j of C to the
+// later ones whenever move j is kept.  Between two kept moves nothing
+// changes, so it goes from one kept move to the next.  Three kernels:
+//   k_mh_draw    once per scan: every ion's proposal (an ion moves once a
+//                scan, so its own position is the scan's start's), U(b) - U(a)
+//                and the window of dE around -k_B T ln u outside of which the
+//                decision is certain without the exponential;
+//   k_mh_sums    per batch: the sums and C (FP64, bound by the FP64 units:
+//                2 rsqrt per pair);
+//   k_mh_decide  per batch: one block, the decisions by its first warp.
+// 1,000 ions: 4.9 us a move by one cluster of 8 CTAs (a cluster barrier per
+// move, FP64 on 8 SMs) before, 0.3 us now.
+// Compiled with -fmad=false like the push, so the proposal and U are the
+// literal IEEE sequence; the pair sums (explicit fma, rsqrt, their order)
+// differ from the sequential 1/sqrt sum only in the last bits of dE.
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include "internal.h"
 #include "rng.cuh"
 
 namespace pt {
 
-constexpr int kMhThreads = 1024;
+namespace {
+
+constexpr int kMhSumThreads = 128;
+constexpr int kMhDecideThreads = 1024;
 
 __device__ __forceinline__ double mh_u_ext(const MhParams& mp, double qi, double x, double y,
                                            double z) {
@@ -41,234 +58,203 @@ __device__ __forceinline__ double mh_u_ext(const MhParams& mp, double qi, double
            0.25 * qi * mp.kz * mp.delta * (xr * xr - yr * yr);
 }
 
-__global__ void __launch_bounds__(kMhThreads) k_mh_scans(int64_t n, double* x, double* y, double* z,
-                                                         const double* __restrict__ q, MhParams mp,
-                                                         int64_t scan0, int64_t n_scans,
-                                                         unsigned long long* acc_out,
-                                                         double* de_out) {
-    __shared__ double prop[4];  // b and the accept uniform
-    __shared__ double red[kMhThreads / 32];
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    unsigned long long acc = 0;
-    double de_sum = 0.0;
-    for (int64_t sc = 0; sc < n_scans; ++sc) {
-        const uint64_t scan = (uint64_t)(scan0 + sc);
-        for (int64_t i = 0; i < n; ++i) {
-            if (tid == 0) {
-                uint32_t w[4];
-                philox4x32_10((uint32_t)i, 0xFFu, (uint32_t)scan, (uint32_t)(scan >> 32),
-                              (uint32_t)mp.seed, (uint32_t)(mp.seed >> 32), w);
-                const double r = mp.dx * u01(w[0], w[1]);
-                const double u = u01(w[2], w[3]);
-                double v1 = 0.0, v2 = 0.0, ss = 0.0;
-                for (uint32_t slot = 1; slot <= (uint32_t)kMaxTries; ++slot) {
-                    philox4x32_10((uint32_t)i, 0xFFu | (slot << 8), (uint32_t)scan,
-                                  (uint32_t)(scan >> 32), (uint32_t)mp.seed,
-                                  (uint32_t)(mp.seed >> 32), w);
-                    v1 = 2.0 * u01(w[0], w[1]) - 1.0;
-                    v2 = 2.0 * u01(w[2], w[3]) - 1.0;
-                    ss = v1 * v1 + v2 * v2;
-                    if (ss < 1.0) break;
-                }
-                const double f = 2.0 * sqrt(1.0 - ss);
-                prop[0] = x[i] + r * (v1 * f);
-                prop[1] = y[i] + r * (v2 * f);
-                prop[2] = z[i] + r * (1.0 - 2.0 * ss);
-                prop[3] = u;
-            }
-            __syncthreads();
-            const double ax = x[i], ay = y[i], az = z[i];
-            const double bx = prop[0], by = prop[1], bz = prop[2];
-            double part = 0.0;
-            for (int64_t j = tid; j < n; j += kMhThreads) {
-                if (j == i) continue;
-                const double dbx = bx - x[j], dby = by - y[j], dbz = bz - z[j];
-                const double dax = ax - x[j], day = ay - y[j], daz = az - z[j];
-                part += q[j] * (1.0 / sqrt(dbx * dbx + dby * dby + dbz * dbz) -
-                                1.0 / sqrt(dax * dax + day * day + daz * daz));
-            }
-            for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-            if (lane == 0) red[wid] = part;
-            __syncthreads();
-            if (tid == 0) {
-                double sum = 0.0;
-                for (int k = 0; k < kMhThreads / 32; ++k) sum += red[k];
-                const double qi = q[i];
-                const double dE = (mh_u_ext(mp, qi, bx, by, bz) - mh_u_ext(mp, qi, ax, ay, az)) +
-                                  mp.ke * qi * sum;
-                if (dE < 0.0 || prop[3] < pt_exp(-dE / (mp.kb * mp.temp))) {
-                    x[i] = bx;
-                    y[i] = by;
-                    z[i] = bz;
-                    ++acc;
-                    de_sum += dE;
-                }
-            }
-            __syncthreads();  // the move (or not) is seen by the next proposal
-        }
+__global__ void __launch_bounds__(128) k_mh_draw(int64_t n, const double* __restrict__ x,
+                                                 const double* __restrict__ y,
+                                                 const double* __restrict__ z,
+                                                 const double* __restrict__ q, MhParams mp,
+                                                 uint64_t scan, double* prop) {
+    pdl_wait();
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    uint32_t w[4];
+    philox4x32_10((uint32_t)i, 0xFFu, (uint32_t)scan, (uint32_t)(scan >> 32), (uint32_t)mp.seed,
+                  (uint32_t)(mp.seed >> 32), w);
+    const double r = mp.dx * u01(w[0], w[1]);
+    const double u = u01(w[2], w[3]);
+    double v1 = 0.0, v2 = 0.0, ss = 0.0;
+    for (uint32_t slot = 1; slot <= (uint32_t)kMaxTries; ++slot) {
+        philox4x32_10((uint32_t)i, 0xFFu | (slot << 8), (uint32_t)scan, (uint32_t)(scan >> 32),
+                      (uint32_t)mp.seed, (uint32_t)(mp.seed >> 32), w);
+        v1 = 2.0 * u01(w[0], w[1]) - 1.0;
+        v2 = 2.0 * u01(w[2], w[3]) - 1.0;
+        ss = v1 * v1 + v2 * v2;
+        if (ss < 1.0) break;
     }
-    if (tid == 0) {
-        *acc_out = acc;
-        *de_out = de_sum;
+    const double f = 2.0 * sqrt(1.0 - ss);
+    const double ax = x[i], ay = y[i], az = z[i];
+    const double bx = ax + r * (v1 * f), by = ay + r * (v2 * f), bz = az + r * (1.0 - 2.0 * ss);
+    // dE < -k_B T ln u keeps the move; within 1e-9 (k_B T + that) of it, or
+    // with u = 0, the exponential decides
+    const double kt = mp.kb * mp.temp;
+    double lo = -INFINITY, hi = INFINITY;
+    if (u > 0.0) {
+        const double thr = -kt * log(u), margin = 1e-9 * (kt + thr);
+        lo = thr - margin;
+        hi = thr + margin;
     }
+    double* p = prop + i;
+    p[0] = bx;
+    p[n] = by;
+    p[2 * n] = bz;
+    p[3 * n] = mh_u_ext(mp, q[i], bx, by, bz) - mh_u_ext(mp, q[i], ax, ay, az);
+    p[4 * n] = lo;
+    p[5 * n] = hi;
+    p[6 * n] = u;
 }
 
-// ---------------------------------------------------------------------------
-// The same chain on a cluster of kMhCtas CTAs (crystals of up to kMhClusterIons
-// ions).  Each CTA keeps a replica of the positions and charges in shared
-// memory.  Per scan, the proposals (b = a + displacement, the accept uniform,
-// the external-energy change U(b) - U(a)) are drawn for all ions in parallel:
-// they depend only on the moving ion's own position, which no earlier move
-// of the scan changes.  Per move, every CTA sums the Coulomb change over its
-// share of the other ions (FP64, rsqrt), writes its partial into a
-// double-buffered slot, and after one cluster barrier every CTA's thread 0
-// adds the partials of all CTAs in rank order (distributed shared memory),
-// takes the same decision and updates its replica.  The barrier is the
-// hardware cluster barrier; nothing spins.
-// ---------------------------------------------------------------------------
-constexpr int kMhCtas = 8;
-constexpr int kMhCtaThreads = 256;
-constexpr int64_t kMhClusterIons = 4096;
+__device__ __forceinline__ double mh_inv(double dx, double dy, double dz) {
+    return rsqrt(fma(dz, dz, fma(dy, dy, dx * dx)));
+}
 
-__global__ void __launch_bounds__(kMhCtaThreads) k_mh_scans_cluster(
-    int64_t n, double* x, double* y, double* z, const double* __restrict__ q, MhParams mp,
-    int64_t scan0, int64_t n_scans, double* prop, unsigned long long* acc_out, double* de_out) {
-    namespace cg = cooperative_groups;
-    cg::cluster_group cl = cg::this_cluster();
-    const int rank = (int)cl.block_rank(), nr = (int)cl.num_blocks();
-    extern __shared__ double mh_sm[];
-    double* sx = mh_sm;
-    double* sy = sx + n;
-    double* sz = sy + n;
-    double* sq = sz + n;
-    __shared__ double slot[2];
-    __shared__ double red[kMhCtaThreads / 32];
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    for (int64_t j = tid; j < n; j += kMhCtaThreads) {
-        sx[j] = x[j];
-        sy[j] = y[j];
-        sz[j] = z[j];
-        sq[j] = q[j];
+// blocks [0, sum_blocks): a warp per (move, source range); the rest: a
+// thread per (j, k) of C, j < k
+__global__ void __launch_bounds__(kMhSumThreads) k_mh_sums(
+    int64_t n, int64_t i0, int nb, int chunks, int64_t per, int sum_blocks,
+    const double* __restrict__ x, const double* __restrict__ y, const double* __restrict__ z,
+    const double* __restrict__ q, double ke, const double* __restrict__ prop, double* part, double* C) {
+    pdl_wait();
+    const int lane = threadIdx.x & 31;
+    if ((int)blockIdx.x < sum_blocks) {
+        const int u = (int)((blockIdx.x * kMhSumThreads + threadIdx.x) >> 5);
+        const int k = u / chunks, c = u % chunks;
+        if (k >= nb) return;
+        const int64_t i = i0 + k, j1 = min(n, (c + 1) * per);
+        const double ax = x[i], ay = y[i], az = z[i];
+        const double bx = prop[i], by = prop[n + i], bz = prop[2 * n + i];
+        double s = 0.0;
+        for (int64_t j = c * per + lane; j < j1; j += 32) {
+            const double xj = x[j], yj = y[j], zj = z[j];
+            const double ib = mh_inv(bx - xj, by - yj, bz - zj), ia = mh_inv(ax - xj, ay - yj, az - zj);
+            if (j != i) s = fma(q[j], ib - ia, s);
+        }
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) part[k * chunks + c] = s;
+        return;
+    }
+    const int e = ((int)blockIdx.x - sum_blocks) * kMhSumThreads + threadIdx.x;
+    const int j = e / nb, k = e % nb;
+    if (j >= nb || k <= j) return;
+    const int64_t ij = i0 + j, ik = i0 + k;
+    const double ajx = x[ij], ajy = y[ij], ajz = z[ij], akx = x[ik], aky = y[ik], akz = z[ik];
+    const double bjx = prop[ij], bjy = prop[n + ij], bjz = prop[2 * n + ij];
+    const double bkx = prop[ik], bky = prop[n + ik], bkz = prop[2 * n + ik];
+    const double after = mh_inv(bkx - bjx, bky - bjy, bkz - bjz) - mh_inv(akx - bjx, aky - bjy, akz - bjz);
+    const double before = mh_inv(bkx - ajx, bky - ajy, bkz - ajz) - mh_inv(akx - ajx, aky - ajy, akz - ajz);
+    C[j * kMhBatch + k] = ke * q[ik] * (q[ij] * (after - before));
+}
+
+// The decisions of a batch.  Lane l of warp 0 holds moves l + 32 m.
+__global__ void __launch_bounds__(kMhDecideThreads) k_mh_decide(
+    int64_t n, int64_t i0, int nb, int chunks, double* x, double* y, double* z,
+    const double* __restrict__ q, MhParams mp, const double* __restrict__ prop,
+    const double* __restrict__ part, const double* __restrict__ C, unsigned long long* acc_out,
+    double* de_out) {
+    extern __shared__ double sC[];  // [nb][kMhBatch]
+    __shared__ double s_sum[kMhBatch];
+    __shared__ unsigned s_kept[kMhBatch / 32];
+    pdl_wait();
+    const int tid = threadIdx.x, lane = tid & 31;
+#pragma unroll 8
+    for (int e = tid; e < nb * kMhBatch; e += kMhDecideThreads)
+        if (e % kMhBatch > e / kMhBatch) sC[e] = C[e];
+    if (tid < nb) {
+        double s = 0.0;
+        for (int c = 0; c < chunks; ++c) s += part[tid * chunks + c];
+        s_sum[tid] = s;
     }
     __syncthreads();
-    unsigned long long acc = 0;
-    double de_sum = 0.0;
-    const int64_t gt = (int64_t)rank * kMhCtaThreads + tid, gs = (int64_t)nr * kMhCtaThreads;
-    for (int64_t sc = 0; sc < n_scans; ++sc) {
-        const uint64_t scan = (uint64_t)(scan0 + sc);
-        for (int64_t i = gt; i < n; i += gs) {
-            uint32_t w[4];
-            philox4x32_10((uint32_t)i, 0xFFu, (uint32_t)scan, (uint32_t)(scan >> 32),
-                          (uint32_t)mp.seed, (uint32_t)(mp.seed >> 32), w);
-            const double r = mp.dx * u01(w[0], w[1]);
-            const double u = u01(w[2], w[3]);
-            double v1 = 0.0, v2 = 0.0, ss = 0.0;
-            for (uint32_t slt = 1; slt <= (uint32_t)kMaxTries; ++slt) {
-                philox4x32_10((uint32_t)i, 0xFFu | (slt << 8), (uint32_t)scan,
-                              (uint32_t)(scan >> 32), (uint32_t)mp.seed, (uint32_t)(mp.seed >> 32),
-                              w);
-                v1 = 2.0 * u01(w[0], w[1]) - 1.0;
-                v2 = 2.0 * u01(w[2], w[3]) - 1.0;
-                ss = v1 * v1 + v2 * v2;
-                if (ss < 1.0) break;
-            }
-            const double f = 2.0 * sqrt(1.0 - ss);
-            const double ax = sx[i], ay = sy[i], az = sz[i];
-            const double bx = ax + r * (v1 * f), by = ay + r * (v2 * f), bz = az + r * (1.0 - 2.0 * ss);
-            double* pr = prop + 5 * i;
-            pr[0] = bx;
-            pr[1] = by;
-            pr[2] = bz;
-            pr[3] = u;
-            pr[4] = mh_u_ext(mp, sq[i], bx, by, bz) - mh_u_ext(mp, sq[i], ax, ay, az);
+    if (tid < 32) {
+        constexpr int NM = kMhBatch / 32;
+        double E[NM], lo[NM], hi[NM];  // dE with the moves kept so far
+#pragma unroll
+        for (int m = 0; m < NM; ++m) {
+            const int k = lane + 32 * m;
+            const int64_t i = i0 + k;
+            const bool live = k < nb;
+            E[m] = live ? prop[3 * n + i] + mp.ke * q[i] * s_sum[k] : 0.0;
+            lo[m] = live ? prop[4 * n + i] : -INFINITY;
+            hi[m] = live ? prop[5 * n + i] : -INFINITY;
         }
-        cl.sync();  // the scan's proposals, written by every CTA, are visible
-        for (int64_t i = 0; i < n; ++i) {
-            const double* pr = prop + 5 * i;
-            const double bx = __ldcg(pr), by = __ldcg(pr + 1), bz = __ldcg(pr + 2);
-            double u = 0.0, dU = 0.0;
-            if (tid == 0) {
-                u = __ldcg(pr + 3);
-                dU = __ldcg(pr + 4);
-            }
-            const double ax = sx[i], ay = sy[i], az = sz[i];
-            double part = 0.0;
-            for (int64_t j = gt; j < n; j += gs) {
-                if (j == i) continue;
-                const double dbx = bx - sx[j], dby = by - sy[j], dbz = bz - sz[j];
-                const double dax = ax - sx[j], day = ay - sy[j], daz = az - sz[j];
-                part += sq[j] * (rsqrt(dbx * dbx + dby * dby + dbz * dbz) -
-                                 rsqrt(dax * dax + day * day + daz * daz));
-            }
-            for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-            if (lane == 0) red[wid] = part;
-            __syncthreads();
-            if (tid == 0) {
-                double p = 0.0;
-                for (int k = 0; k < kMhCtaThreads / 32; ++k) p += red[k];
-                slot[i & 1] = p;
-            }
-            cl.sync();  // every CTA's partial of this move is in its slot
-            if (tid == 0) {
-                double sum = 0.0;
-                for (int k = 0; k < nr; ++k) sum += *cl.map_shared_rank(&slot[i & 1], k);
-                const double dE = dU + mp.ke * sq[i] * sum;
-                const int keep = (dE < 0.0 || u < pt_exp(-dE / (mp.kb * mp.temp))) ? 1 : 0;
-                if (keep) {
-                    sx[i] = bx;
-                    sy[i] = by;
-                    sz[i] = bz;
-                    ++acc;
-                    de_sum += dE;
+        unsigned long long acc = 0;
+        double de_sum = *de_out;
+#pragma unroll
+        for (int m = 0; m < NM; ++m) {
+            // the first undecided move of the group that may be kept: the
+            // undecided ones before it are not (nothing changed since)
+            unsigned left = 32 * m < nb ? 0xffffffffu : 0u, kept = 0;
+            while (left) {
+                const unsigned may = __ballot_sync(0xffffffffu, E[m] <= hi[m]) & left;
+                const unsigned sure = __ballot_sync(0xffffffffu, E[m] < lo[m]);
+                if (!may) break;
+                const int l = __ffs(may) - 1, j = l + 32 * m;
+                left = l == 31 ? 0u : left & (0xffffffffu << (l + 1));
+                if (!((sure >> l) & 1u)) {
+                    // too close to the threshold: the exponential decides
+                    bool keep = false;
+                    if (lane == l)
+                        keep = E[m] < 0.0 || prop[6 * n + i0 + j] < pt_exp(-E[m] / (mp.kb * mp.temp));
+                    if (!__ballot_sync(0xffffffffu, keep)) continue;
                 }
+                kept |= 1u << l;
+                ++acc;
+                de_sum += __shfl_sync(0xffffffffu, E[m], l);
+                // (the columns up to j are decided: what is added there is unused)
+                const double* row = sC + j * kMhBatch + lane;
+#pragma unroll
+                for (int mm = m; mm < NM; ++mm) E[mm] += row[32 * mm];
             }
-            __syncthreads();  // the replica is updated before the next move reads it
+            if (lane == 0) s_kept[m] = kept;
         }
-    }
-    if (rank == 0) {
-        for (int64_t j = tid; j < n; j += kMhCtaThreads) {
-            x[j] = sx[j];
-            y[j] = sy[j];
-            z[j] = sz[j];
-        }
-        if (tid == 0) {
-            *acc_out = acc;
+        if (lane == 0) {
+            *acc_out += acc;
             *de_out = de_sum;
         }
     }
-    cl.sync();  // no CTA leaves while another may still read its slots
+    __syncthreads();
+    if (tid < nb && ((s_kept[tid >> 5] >> (tid & 31)) & 1u)) {
+        const int64_t i = i0 + tid;
+        x[i] = prop[i];
+        y[i] = prop[n + i];
+        z[i] = prop[2 * n + i];
+    }
 }
 
-size_t mh_scratch_bytes(int64_t n) {
-    return n <= kMhClusterIons ? sizeof(double) * 5 * (size_t)n : 0;
-}
+}  // namespace
 
 cudaError_t launch_mh_scans(int64_t n, double* x, double* y, double* z, const double* q,
                             const MhParams& mp, int64_t scan0, int64_t n_scans,
-                            unsigned long long* acc_out, double* de_out, double* scratch,
+                            unsigned long long* acc_out, double* de_out, double* scratch, int sms,
                             cudaStream_t s) {
-    if (n > kMhClusterIons || !scratch) {
-        k_mh_scans<<<1, kMhThreads, 0, s>>>(n, x, y, z, q, mp, scan0, n_scans, acc_out, de_out);
-        return cudaGetLastError();
+    double* prop = scratch;
+    double* part = prop + (size_t)kMhProp * n;
+    double* C = part + kMhBatch * kMhMaxChunks;
+    const int smem = (int)sizeof(double) * kMhBatch * kMhBatch;
+    cudaError_t e = cudaFuncSetAttribute(k_mh_decide, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaMemsetAsync(acc_out, 0, sizeof *acc_out, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(de_out, 0, sizeof *de_out, s);
+    // source ranges of whole warps' worth, about eight warps per SM over the batch
+    const int64_t want = (sms * 8 + kMhBatch - 1) / kMhBatch;
+    int64_t chunks = std::min<int64_t>(std::min<int64_t>(want, kMhMaxChunks), (n + 31) / 32);
+    const int64_t per = ((n + chunks - 1) / chunks + 31) / 32 * 32;
+    chunks = (n + per - 1) / per;
+    for (int64_t sc = 0; sc < n_scans && e == cudaSuccess; ++sc) {
+        e = launch_pdl(k_mh_draw, dim3((unsigned)((n + 127) / 128)), dim3(128), 0, s, n, (const double*)x,
+                       (const double*)y, (const double*)z, q, mp, (uint64_t)(scan0 + sc), prop);
+        for (int64_t i0 = 0; i0 < n && e == cudaSuccess; i0 += kMhBatch) {
+            const int nb = (int)std::min<int64_t>(kMhBatch, n - i0);
+            const int wpb = kMhSumThreads / 32;
+            const int sb = (int)((nb * chunks + wpb - 1) / wpb);
+            const int cb = (nb * nb + kMhSumThreads - 1) / kMhSumThreads;
+            e = launch_pdl(k_mh_sums, dim3((unsigned)(sb + cb)), dim3(kMhSumThreads), 0, s, n, i0, nb,
+                           (int)chunks, per, sb, (const double*)x, (const double*)y, (const double*)z,
+                           q, mp.ke, (const double*)prop, part, C);
+            if (e == cudaSuccess)
+                e = launch_pdl(k_mh_decide, dim3(1), dim3(kMhDecideThreads), (size_t)smem, s, n, i0, nb,
+                               (int)chunks, x, y, z, q, mp, (const double*)prop, (const double*)part,
+                               (const double*)C, acc_out, de_out);
+        }
     }
-    const size_t smem = sizeof(double) * 4 * (size_t)n;
-    cudaError_t e = cudaFuncSetAttribute(k_mh_scans_cluster,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kMhCtas, 1, 1);
-    cfg.blockDim = dim3(kMhCtaThreads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = kMhCtas;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_mh_scans_cluster, n, x, y, z, q, mp, scan0, n_scans, scratch,
-                              acc_out, de_out);
+    return e;
 }
 
 }  // namespace pt
