@@ -143,6 +143,7 @@ struct OpSet {
     void* T_m2l_tc = nullptr;
     void* T_rot = nullptr;   // rotation-based M2L operators (CUDA-core precisions), once asked for
     void* T_f64 = nullptr;   // FP64 operator digits of the tensor-core translations
+    void* T_f32 = nullptr;   // FP32 plans: transposed operators
 };
 std::mutex g_ops_mu;
 std::map<std::tuple<int, int, int>, OpSet> g_ops;
@@ -158,6 +159,7 @@ void release_ops(fmm_plan_s* pl) {
         if (it->second.T_m2l_tc) cudaFree(it->second.T_m2l_tc);
         if (it->second.T_rot) cudaFree(it->second.T_rot);
         if (it->second.T_f64) cudaFree(it->second.T_f64);
+        if (it->second.T_f32) cudaFree(it->second.T_f32);
         g_ops.erase(it);
     }
     pl->ops_held = false;
@@ -247,6 +249,7 @@ int build_operators(fmm_plan_s* pl) {
                                 : upload_ops<float>(pl, m2m, l2l, m2l);
     if (e != cudaSuccess) return status_from(e);
     if (pl->ws.fp64 && (e = m2l_f64_pack(pl->ws)) != cudaSuccess) return status_from(e);
+    if (pl->precision == PT_FP32 && (e = m2l_f32_pack(pl->ws)) != cudaSuccess) return status_from(e);
     if (is_tc(pl->precision)) {
         const bool bf16 = pl->precision == PT_MIXED_BF16X3;
         std::vector<unsigned char> packed(m2l_tc_operand_bytes(p, bf16));
@@ -302,16 +305,18 @@ int acquire_ops(fmm_plan_s* pl, size_t op_bytes) {
         OpSet o;
         const size_t tc = is_tc(pl->precision) ? m2l_tc_operand_bytes(pl->p, ws.tc_bf16 != 0) : 0;
         const size_t f64 = ws.fp64 ? m2l_f64_operator_bytes(pl->p) : 0;
+        const size_t f32 = pl->precision == PT_FP32 ? m2l_f32_operator_bytes(pl->p) : 0;
         auto drop = [&]() {
-            for (void* v : {o.T_m2m, o.T_l2l, o.T_m2l, o.T_m2l_tc, o.T_f64})
+            for (void* v : {o.T_m2m, o.T_l2l, o.T_m2l, o.T_m2l_tc, o.T_f64, o.T_f32})
                 if (v) cudaFree(v);
-            ws.T_m2m = ws.T_l2l = ws.T_m2l = ws.T_m2l_tc = ws.T_f64 = nullptr;
+            ws.T_m2m = ws.T_l2l = ws.T_m2l = ws.T_m2l_tc = ws.T_f64 = ws.T_f32 = nullptr;
         };
         if (cudaMalloc(&o.T_m2m, 8 * op_bytes) != cudaSuccess ||
             cudaMalloc(&o.T_l2l, 8 * op_bytes) != cudaSuccess ||
             cudaMalloc(&o.T_m2l, 343 * op_bytes) != cudaSuccess ||
             (tc && cudaMalloc(&o.T_m2l_tc, tc) != cudaSuccess) ||
-            (f64 && cudaMalloc(&o.T_f64, f64) != cudaSuccess)) {
+            (f64 && cudaMalloc(&o.T_f64, f64) != cudaSuccess) ||
+            (f32 && cudaMalloc(&o.T_f32, f32) != cudaSuccess)) {
             drop();
             return PT_ERR_OOM;
         }
@@ -320,6 +325,7 @@ int acquire_ops(fmm_plan_s* pl, size_t op_bytes) {
         ws.T_m2l = o.T_m2l;
         ws.T_m2l_tc = o.T_m2l_tc;
         ws.T_f64 = o.T_f64;
+        ws.T_f32 = o.T_f32;
         int r = build_operators(pl);
         if (r != PT_OK) {
             drop();
@@ -334,6 +340,7 @@ int acquire_ops(fmm_plan_s* pl, size_t op_bytes) {
     ws.T_m2l_tc = it->second.T_m2l_tc;
     ws.T_rot = it->second.T_rot;
     ws.T_f64 = it->second.T_f64;
+    ws.T_f32 = it->second.T_f32;
     pl->ops_held = true;
     return PT_OK;
 }
@@ -932,7 +939,8 @@ static int plan_create_impl(int64_t n_max, int p, int leaf_max, int depth, int p
         std::lock_guard<std::mutex> g(g_tables_mu);
         if (!g_tables_dev.count(pl->device)) {
             if (upload_harmonic_tables() != cudaSuccess || m2l_tc_init() != cudaSuccess ||
-                m2l_f64_init() != cudaSuccess || m2l_rot_init() != cudaSuccess) {
+                m2l_f64_init() != cudaSuccess || m2l_f32_init() != cudaSuccess ||
+                m2l_rot_init() != cudaSuccess) {
                 free_plan(pl);
                 return PT_ERR_CUDA;
             }
@@ -1000,7 +1008,8 @@ static int plan_create_impl(int64_t n_max, int p, int leaf_max, int depth, int p
         *dry_bytes = (int64_t)pl->dry_bytes;
         *op_bytes = (int64_t)(tsz * (8 + 8 + 343) * PP +
                               (is_tc(precision) ? m2l_tc_operand_bytes(p, ws.tc_bf16 != 0) : 0) +
-                              (ws.fp64 ? m2l_f64_operator_bytes(p) : 0));
+                              (ws.fp64 ? m2l_f64_operator_bytes(p) : 0) +
+                              (precision == PT_FP32 ? m2l_f32_operator_bytes(p) : 0));
         delete pl;
         return PT_OK;
     }

@@ -1417,12 +1417,16 @@ static cudaError_t run_fmm(int64_t n, int D, int phases, Workspace& ws, bool use
                 if ((e = launch_f64_m2m(n, D, l, ws, s)) != cudaSuccess) return e;
                 continue;
             }
-            int64_t cl = (int64_t)1 << (3 * l);
-            int cells = (int)(n < cl ? n : cl);
-            int g = (cells + 3) / 4;
-            if (g > 152 * 16) g = 152 * 16;
-            k_m2m<T><<<g, 128, 4 * P * sizeof(T), s>>>(l, P, ws.ld, ws.linfo, ws.code, ws.cid,
-                                                       dl.off[l + 1], (const T*)ws.T_m2m, M);
+            if constexpr (sizeof(T) == 4) {
+                if ((e = launch_f32_m2m(n, D, l, ws, s)) != cudaSuccess) return e;
+            } else {
+                int64_t cl = (int64_t)1 << (3 * l);
+                int cells = (int)(n < cl ? n : cl);
+                int g = (cells + 3) / 4;
+                if (g > 152 * 16) g = 152 * 16;
+                k_m2m<T><<<g, 128, 4 * P * sizeof(T), s>>>(l, P, ws.ld, ws.linfo, ws.code, ws.cid,
+                                                           dl.off[l + 1], (const T*)ws.T_m2m, M);
+            }
         }
     }
     if (ev && (e = record_timing(ev[0], s)) != cudaSuccess)
@@ -1463,12 +1467,16 @@ static cudaError_t run_fmm(int64_t n, int D, int phases, Workspace& ws, bool use
                              cudaSuccess)
             return e;
         for (int l = 2; l <= D; ++l) {
-            int64_t cl = (int64_t)1 << (3 * l);
-            int cells = (int)(n < cl ? n : cl);
-            dim3 grid((cells + kNT - 1) / kNT + 8, (P + kRT - 1) / kRT);
-            k_m2l_simt<T><<<grid, 256, 0, s>>>(l, P, ws.ld, ws.linfo, ws.code, ws.cid, dl.off[l],
-                                               l >= 3 ? dl.off[l - 1] : 0, M, L,
-                                               (const T*)ws.T_m2l, (const T*)ws.T_l2l);
+            if constexpr (sizeof(T) == 4) {
+                if ((e = launch_f32_tiles(n, D, l, ws, s)) != cudaSuccess) return e;
+            } else {
+                int64_t cl = (int64_t)1 << (3 * l);
+                int cells = (int)(n < cl ? n : cl);
+                dim3 grid((cells + kNT - 1) / kNT + 8, (P + kRT - 1) / kRT);
+                k_m2l_simt<T><<<grid, 256, 0, s>>>(l, P, ws.ld, ws.linfo, ws.code, ws.cid, dl.off[l],
+                                                   l >= 3 ? dl.off[l - 1] : 0, M, L,
+                                                   (const T*)ws.T_m2l, (const T*)ws.T_l2l);
+            }
         }
         if (ws.kev[1] && (e = record_timing(ws.kev[1], s)) !=
                              cudaSuccess)

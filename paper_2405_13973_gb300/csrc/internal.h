@@ -184,6 +184,7 @@ struct Workspace {
     int f64_tc = 0;
     int64_t f64_batch = 0;
     void* T_f64 = nullptr;
+    void* T_f32 = nullptr;      // FP32 plans: transposed operators of m2l_f32.cu
     uint8_t* f64_dig = nullptr;
     int* f64_rexp = nullptr;
     // kernel timing (profiled steps only, else null): recorded right before
@@ -276,6 +277,17 @@ cudaError_t m2l_pairs_stats(const Workspace& ws, int64_t* out, cudaStream_t s);
 // this order do not fit), per-device kernel set-up
 int m2l_rot_tile(const Workspace& ws);
 cudaError_t m2l_rot_init();
+// ---- FP32 translations on the CUDA cores (m2l_f32.cu) ---------------------------
+size_t m2l_f32_operator_bytes(int p);
+cudaError_t m2l_f32_init();
+// transposed operators from the FP32 operators of ws (synchronous)
+cudaError_t m2l_f32_pack(const Workspace& ws);
+// the partial rows of the pair work list; M2L (+ L2L) of level l by target
+// tiles; M at level l; L at level l += its parents' shift
+cudaError_t launch_f32_pairs(Workspace& ws, cudaStream_t s);
+cudaError_t launch_f32_tiles(int64_t n, int D, int l, Workspace& ws, cudaStream_t s);
+cudaError_t launch_f32_m2m(int64_t n, int D, int l, Workspace& ws, cudaStream_t s);
+cudaError_t launch_f32_l2l(int64_t n, int D, int l, Workspace& ws, cudaStream_t s);
 // ---- FP64 translations on the tensor cores (m2l_f64.cu) -------------------------
 // digit row stride (bytes), digit bytes of `cells` cells, operator bytes
 int m2l_f64_lda(int p);

@@ -298,7 +298,7 @@ __global__ void __launch_bounds__(kPpThreads) k_pp_fill(PpArgs a, const uint32_t
 // offset); `width` columns are written.  Targets without pairs get zeros.  On
 // a pool overflow nothing is summed (the call reports it).  FP32 rows with
 // width a multiple of 4 (k_pp_reduce_f4): a block per target, the slots in
-// four ordered parts; otherwise (k_pp_reduce) a warp per target in slot
+// four ordered parts; otherwise (k_pp_reduce_seq) a group of threads per target in slot
 // order, lanes over columns.
 constexpr int kRedParts = 4;  // slot-range parts per (target, column group)
 __global__ void __launch_bounds__(256) k_pp_reduce_f4(int D, int ld, int stride, int width,
@@ -424,26 +424,50 @@ __global__ void __launch_bounds__(320) k_pp_reduce_d4(int D, int t0, int t1, int
     }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) k_pp_reduce(int D, int ld, int stride, int width,
-                                                    const LevelInfo* linfo, const M2lPairHdr* hdr,
-                                                    const int* tbase, const int* __restrict__ tpair,
-                                                    const T* __restrict__ part, T* L) {
-    const int lane = threadIdx.x & 31;
+// FP32 rows of the CUDA-core path: a group of ld / 4 threads per target, four
+// columns a thread, the rows added in slot order (the sums' order is part of
+// the path's results), eight rows in flight.
+__global__ void __launch_bounds__(320) k_pp_reduce_seq(int D, int ld, int stride, int width,
+                                                        const LevelInfo* linfo, const M2lPairHdr* hdr,
+                                                        const int* tbase,
+                                                        const int* __restrict__ tpair,
+                                                        const float* __restrict__ part, float* L) {
+    pdl_wait();
+    const int w4 = (width + 3) / 4, per = blockDim.x / w4;
+    const int j = threadIdx.x / w4, u = threadIdx.x - j * w4;
     const int g0 = linfo->gbase[2], nt = linfo->gbase[D + 1] - g0;
     const bool over = hdr->overflow != 0;
-    for (int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < nt;
-         t += gridDim.x * (blockDim.x >> 5)) {
+    if (j >= per) return;
+    for (int t = blockIdx.x * per + j; t < nt; t += gridDim.x * per) {
         const int s0 = tbase[t], s1 = over ? s0 : tbase[t + 1];
-        for (int u = lane; u < width; u += 32) {
-            T v = T(0);
-            const bool odd = coef_degree(u) & 1;
-            for (int s = s0; s < s1; ++s) {
-                const int r = tpair[s];
-                const T x = part[(int64_t)(r < 0 ? ~r : r) * stride + u];
-                v += r < 0 && odd ? -x : x;  // mirrored row: odd degrees negated
-            }
-            L[(int64_t)(g0 + t) * ld + u] = v;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        int rw[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) rw[k] = s0 + k < s1 ? tpair[s0 + k] : 0;
+        for (int s = s0; s < s1; s += 8) {
+            float4 q[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (s + k < s1)
+                    q[k] = __ldcs(reinterpret_cast<const float4*>(part + (int64_t)rw[k] * stride + 4 * u));
+#pragma unroll
+            for (int k = 0; k < 8; ++k) rw[k] = s + 8 + k < s1 ? tpair[s + 8 + k] : 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (s + k < s1) {
+                    v.x += q[k].x;
+                    v.y += q[k].y;
+                    v.z += q[k].z;
+                    v.w += q[k].w;
+                }
+        }
+        float* o = L + (int64_t)(g0 + t) * ld + 4 * u;
+        if (4 * u + 4 <= width) {
+            *reinterpret_cast<float4*>(o) = v;
+        } else {  // the padding columns stay zero
+            o[0] = v.x;
+            if (4 * u + 1 < width) o[1] = v.y;
+            if (4 * u + 2 < width) o[2] = v.z;
         }
     }
 }
@@ -746,7 +770,6 @@ cudaError_t launch_m2l_pairs_reduce(int64_t n, int D, Workspace& ws, int width, 
     if (D < 2) return cudaSuccess;
     PairList L = pair_list(ws);
     const int64_t tb = std::min<int64_t>(target_cells_bound(n, D), (int64_t)t1 - t0);
-    const unsigned gr = (unsigned)std::min<int64_t>((tb + 7) / 8, 152 * 16);
     if (ws.fp64) {
         const unsigned g4 = (unsigned)std::min<int64_t>(tb, 152 * 32);
         return launch_pdl(k_pp_reduce_d4, dim3(g4), dim3(kRedParts * (ws.ld / 4)), 0, s, D, t0, t1,
@@ -760,11 +783,13 @@ cudaError_t launch_m2l_pairs_reduce(int64_t n, int D, Workspace& ws, int width, 
                           (const M2lPairHdr*)L.hdr, (const int*)L.tbase, (const int*)L.tpair,
                           (const float4*)ws.pp_part, (float*)ws.L);
     } else {
-        k_pp_reduce<float><<<gr, 256, 0, s>>>(D, ws.ld, ws.pp_stride, width, ws.linfo, L.hdr,
-                                              L.tbase, L.tpair, (const float*)ws.pp_part,
-                                              (float*)ws.L);
+        const int w4 = (width + 3) / 4, per = 256 / w4 > 0 ? 256 / w4 : 1;
+        const unsigned gr = (unsigned)std::min<int64_t>((tb + per - 1) / per, 152 * 16);
+        return launch_pdl(k_pp_reduce_seq, dim3(gr), dim3((unsigned)(w4 * per)), 0, s, D, ws.ld,
+                          ws.pp_stride, width, (const LevelInfo*)ws.linfo, (const M2lPairHdr*)L.hdr,
+                          (const int*)L.tbase, (const int*)L.tpair, (const float*)ws.pp_part,
+                          (float*)ws.L);
     }
-    return cudaGetLastError();
 }
 
 // shared-memory bytes of k_m2l_rot for np pairs per tile
@@ -813,6 +838,8 @@ static cudaError_t simt_pairs(int64_t n, int D, Workspace& ws, int l2l_last, cud
         return e;
     if (ws.m2l_rot) {
         if ((e = rot_pairs<T>(n, D, ws, s)) != cudaSuccess) return e;
+    } else if constexpr (sizeof(T) == 4) {
+        if ((e = launch_f32_pairs(ws, s)) != cudaSuccess) return e;
     } else {
         const int64_t units = ws.pp_item_cap * 2 * ((P + kSimtCols - 1) / kSimtCols);
         const unsigned grid = (unsigned)std::min<int64_t>(units, 152 * 8);
@@ -827,6 +854,10 @@ static cudaError_t simt_pairs(int64_t n, int D, Workspace& ws, int l2l_last, cud
     if ((e = launch_m2l_pairs_reduce(n, D, ws, P, s)) != cudaSuccess) return e;
     const DenseLayout dl = dense_layout(D);
     for (int l = 3; l <= l2l_last && l <= D; ++l) {
+        if constexpr (sizeof(T) == 4) {
+            if ((e = launch_f32_l2l(n, D, l, ws, s)) != cudaSuccess) return e;
+            continue;
+        }
         const int64_t cl = (int64_t)1 << (3 * l);
         const int64_t cells = n < cl ? n : cl;
         const unsigned g = (unsigned)std::min<int64_t>((cells + 3) / 4, 152 * 16);
