@@ -158,6 +158,7 @@ __device__ __forceinline__ void ion_in_ancestor(const Ion<double>::rec& r, int s
     q = r.w;
 }
 
+constexpr int kPmax = (kMaxOrder + 1) * (kMaxOrder + 1);
 constexpr int kP2mThreads = 128;
 constexpr int kP2mIons = 32;
 
@@ -211,6 +212,89 @@ __global__ void __launch_bounds__(kP2mThreads) k_p2m(int D, int p, int ld, const
             if (c < P) {
                 M[(int64_t)g * ld + c] = acc[r];
                 if (Mp) store_pieces(Mp, g, ld, c, (float)acc[r]);  // BF16x3 operand
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// P2M and L2P in FP64.  The FP64 units serve two lanes a clock, and a warp
+// instruction occupies them as long with seven live lanes as with 32, so the
+// lanes hold the ions of several leaves: a block takes the leaves that begin
+// in its window of kSlotWindow sorted slots, and a thread evaluates all
+// (p + 1)^2 harmonics of one ion (tables from constant memory, every lane at
+// the same (n, m)).  With a block per leaf (5 to 10 ions), P2M kept 7 of 32
+// lanes busy, and L2P spent its lanes on recurrences shared by eight of them.
+// ---------------------------------------------------------------------------
+constexpr int kSlotThreads = 64, kSlotWindow = 48;
+// below these ion counts a thread per ion leaves most of the FP64 units idle
+// and its chain of recurrences is the time, so a block per leaf is faster
+// (P2M, p = 8 / 12: 8,000 ions 44 / 71 us by windows, 32 / 64 by leaves,
+// 16,000 ions 46 / 82 and 69 / 136; L2P: 4,000 ions 46 / 91 and 44 / 62, 8,000
+// ions 45 / 89 and 73 / 100)
+constexpr int64_t kP2mSlotIons = 10240, kL2pSlotIons = 7168;
+
+// the slots [s0, s1) of the leaves that begin in window b; false if none does
+__device__ __forceinline__ bool slot_window(int64_t n, int b, const int32_t* __restrict__ leaf_of,
+                                            const int32_t* __restrict__ cstart,
+                                            const int32_t* __restrict__ ccount, int& s0, int& s1) {
+    const int w0 = b * kSlotWindow, w1 = (int)min(n, (int64_t)w0 + kSlotWindow);
+    const int gf = leaf_of[w0], gl = leaf_of[w1 - 1];
+    s0 = cstart[gf];
+    if (s0 < w0) s0 += ccount[gf];
+    s1 = cstart[gl] + ccount[gl];
+    return s0 < w1;
+}
+
+// row stride of one ion's terms: odd, so that a column of rows has no bank conflicts
+__host__ __device__ inline int p2m_f64_stride(int P) { return P | 1; }
+
+__global__ void __launch_bounds__(kSlotThreads) k_p2m_f64(
+    int64_t n, int p, int ld, const int32_t* __restrict__ leaf_of,
+    const int32_t* __restrict__ cstart, const int32_t* __restrict__ ccount,
+    const Ion<double>::rec* __restrict__ sorted, double* __restrict__ M) {
+    extern __shared__ double slot_smem[];  // [kSlotThreads][stride]
+    __shared__ int s_leaf[kSlotThreads + 1];
+    const int P = (p + 1) * (p + 1), S = p2m_f64_stride(P), tid = threadIdx.x;
+    pdl_wait();
+    int s0, s1;
+    if (!slot_window(n, blockIdx.x, leaf_of, cstart, ccount, s0, s1)) return;  // uniform
+    constexpr int NA = (kPmax + kSlotThreads - 1) / kSlotThreads;
+    double acc[NA];
+#pragma unroll
+    for (int r = 0; r < NA; ++r) acc[r] = 0.0;
+    for (int p0 = s0; p0 < s1; p0 += kSlotThreads) {
+        const int ni = min(kSlotThreads, s1 - p0);
+        __syncthreads();
+        if (tid < ni) {
+            s_leaf[tid] = leaf_of[p0 + tid];
+            double x, y, z, q;
+            Ion<double>::get(sorted[p0 + tid], x, y, z, q);
+            double* row = slot_smem + tid * S;
+            for_each_ups<double>(p, x, y, z, c_tab_d, [&](int nn, int m, double re, double im) {
+                const int idx = re_idx(nn, m);
+                row[idx] = q * re;
+                if (m > 0) row[idx + 1] = -q * im;
+            });
+        }
+        if (tid == 0) s_leaf[ni] = p0 + ni < s1 ? leaf_of[p0 + ni] : -1;
+        __syncthreads();
+        // each thread its coefficients, ion after ion; a leaf ends where the
+        // next slot belongs to another
+        for (int i = 0; i < ni; ++i) {
+#pragma unroll
+            for (int r = 0; r < NA; ++r) {
+                const int c = tid + r * kSlotThreads;
+                if (c < P) acc[r] += slot_smem[i * S + c];
+            }
+            const int g = s_leaf[i];
+            if (s_leaf[i + 1] != g) {
+#pragma unroll
+                for (int r = 0; r < NA; ++r) {
+                    const int c = tid + r * kSlotThreads;
+                    if (c < P) M[(int64_t)g * ld + c] = acc[r];
+                    acc[r] = 0.0;
+                }
             }
         }
     }
@@ -750,17 +834,20 @@ __global__ void __launch_bounds__(kNfThreads) k_p2p(
 //   * `parts` blocks share a leaf's targets where there are few leaves, so
 //     that shallow trees fill the GPU;
 //   * the potential only if it is asked for.
-// 1e5 sweep ions (14.5 M pairs): 2.2 ms before; the pair sums' floor is 0.44.
+// 1e5 sweep ions (14.5 M pairs): 2.2 ms before, 0.66 now; 1e6 ions 17.4 and
+// 7.6 ms; the pair sums alone (19 instructions a pair) are 0.44 and 5.7 ms.
+constexpr int kNfSrc64 = 256;  // staged sources per pass; the partials reuse their room
 template <bool PHI>
-__global__ void __launch_bounds__(kNfThreads) k_p2p_f64(
+__global__ void __launch_bounds__(kNfThreads, 8) k_p2p_f64(
     int D, int parts, const LevelInfo* linfo, const Ion<double>::rec* __restrict__ sorted,
     const uint32_t* __restrict__ code, const int32_t* __restrict__ cid_leaf,
     const int32_t* __restrict__ cstart, const int32_t* __restrict__ ccount,
     double* __restrict__ near) {
     using R = Ion<double>::rec;
-    __shared__ R src[kNfSrc];
+    static_assert(kNfSrc64 >= kNfThreads, "the partials lie over the sources");
+    __shared__ R src[kNfSrc64];
     __shared__ int nb_start[27], nb_pre[28];
-    __shared__ R part[kNfThreads];
+    R* part = src;
     const int tid = threadIdx.x, lane = tid & 31;
     const int lim = 1 << D;
     const int g0 = linfo->gbase[D], units = (linfo->gbase[D + 1] - g0) * parts;
@@ -804,8 +891,8 @@ __global__ void __launch_bounds__(kNfThreads) k_p2p_f64(
             const R me = sorted[ts + t0 + ti];
             double ex = 0, ey = 0, ez = 0, ph = 0, cex = 0, cey = 0, cez = 0, cph = 0;
             bool first = true;
-            for (int s0 = 0; s0 < ns; s0 += kNfSrc) {    // sources in passes of kNfSrc
-                const int nsb = min(kNfSrc, ns - s0);
+            for (int s0 = 0; s0 < ns; s0 += kNfSrc64) {    // sources in passes
+                const int nsb = min(kNfSrc64, ns - s0);
                 __syncthreads();
                 for (int j = tid; j < nsb; j += kNfThreads) {
                     const int v = s0 + j;
@@ -851,12 +938,13 @@ __global__ void __launch_bounds__(kNfThreads) k_p2p_f64(
                     }
                 }
             }
-            if (ns > 64 * nch) {  // more than one block of sources somewhere
+            if (ns > 64 * nch || ns > kNfSrc64) {  // more than one block of sources somewhere
                 ex += cex;
                 ey += cey;
                 ez += cez;
                 ph += cph;
             }
+            __syncthreads();  // the sources are read
             part[tid] = make_double4_32a(ex, ey, ez, ph);
             // pairwise over the chunks: a fixed tree (deterministic)
             int live = nch;
@@ -897,7 +985,6 @@ __global__ void __launch_bounds__(kNfThreads) k_p2p_f64(
 // The near field (if any) is added and the field written in the original ion
 // order scaled to SI (k_e / s^2 for E, k_e / s for phi, s = leaf side).
 constexpr int kL2pThreads = 128;
-constexpr int kPmax = (kMaxOrder + 1) * (kMaxOrder + 1);
 
 
 // the derived expansions of one local expansion Lr (see k_l2p) into D4[4][P]
@@ -1189,6 +1276,136 @@ __global__ void __launch_bounds__(kL2pThreads) k_l2p(
     }
 }
 
+// L2P in FP64 (see k_p2m_f64): a thread per ion, the derived expansions of
+// up to `lmax` leaves in shared memory (leaf strides odd in 8-byte units: the
+// leaves of a warp read different banks).  PHI: the potential too.
+constexpr int kL2pLeaves = 16;
+// leaves whose expansions (derived 4 x, local 1 x) fit about 100 KB
+inline int l2p_f64_leaves(int P) {
+    const int l = 100 * 1024 / (5 * P * 8 + 8);
+    return l < 4 ? 4 : (l > kL2pLeaves ? kL2pLeaves : l);
+}
+inline size_t l2p_f64_smem(int P) { return sizeof(double) * (size_t)l2p_f64_leaves(P) * (5 * P + 1); }
+
+template <bool PHI>
+__global__ void __launch_bounds__(kSlotThreads) k_l2p_f64(
+    int64_t n, int D, int p, int ld, int lmax, const RootCube* root,
+    const int32_t* __restrict__ leaf_of, const int32_t* __restrict__ cstart,
+    const int32_t* __restrict__ ccount, const Ion<double>::rec* __restrict__ sorted,
+    const int32_t* __restrict__ perm, const double* __restrict__ L,
+    const double* __restrict__ near, double* E, double* phi) {
+    extern __shared__ double slot_smem[];  // derived [lmax][4 P + 1], local [lmax][P]
+    __shared__ int s_g[kL2pLeaves], s_cnt[2], s_new[2];
+    __shared__ uint16_t s_nm[(kMaxOrder + 1) * (kMaxOrder + 2) / 2];
+    __shared__ double s_f[2];
+    const int P = (p + 1) * (p + 1), DS = 4 * P + 1, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    double* sD = slot_smem;
+    double* sL = slot_smem + lmax * DS;
+    const int NT = (p + 1) * (p + 2) / 2;
+    for (int nn = tid; nn <= p; nn += kSlotThreads)
+        for (int m = 0; m <= nn; ++m) s_nm[nn * (nn + 1) / 2 + m] = (uint16_t)(nn << 8 | m);
+    pdl_wait();
+    int s0, s1;
+    if (!slot_window(n, blockIdx.x, leaf_of, cstart, ccount, s0, s1)) return;  // uniform
+    if (tid == 0) {
+        const double inv = 1.0 / (root->side / (double)(1 << D));
+        s_f[0] = kCoulomb * (inv * inv);
+        s_f[1] = kCoulomb * inv;
+    }
+    for (int p0 = s0; p0 < s1;) {
+        // the pass: slots p0 .. p0 + ni - 1, at most 64 and of at most lmax leaves
+        const bool live = p0 + tid < s1;
+        const int g = live ? leaf_of[p0 + tid] : -1;
+        const bool head = live && (tid == 0 || leaf_of[p0 + tid - 1] != g);
+        const unsigned bal = __ballot_sync(0xffffffffu, head);
+        __syncthreads();  // the previous pass is done with the shared arrays
+        if (lane == 0) s_new[wid] = __popc(bal);
+        __syncthreads();
+        const int ord = (wid ? s_new[0] : 0) + __popc(bal & (0xffffffffu >> (31 - lane))) - 1;
+        const bool in = live && ord < lmax;
+        if (head && in) s_g[ord] = g;
+        const unsigned inb = __ballot_sync(0xffffffffu, in);
+        if (lane == 0) s_cnt[wid] = __popc(inb);
+        __syncthreads();
+        const int ni = s_cnt[0] + s_cnt[1], nl = min(lmax, s_new[0] + s_new[1]);
+        for (int l = 0; l < nl; ++l)
+            for (int c = tid; c < P; c += kSlotThreads) sL[l * P + c] = L[(int64_t)s_g[l] * ld + c];
+        __syncthreads();
+        // derived expansions, as l2p_derive
+        for (int u = tid; u < nl * NT; u += kSlotThreads) {
+            const int l = u / NT, nm = s_nm[u - l * NT], nn = nm >> 8, mm = nm & 255;
+            const double* Lr = sL + l * P;
+            double* D4 = sD + l * DS;
+            const int k = re_idx(nn, mm);
+            const double w = mm > 0 ? 2.0 : 1.0;
+            double dxr = 0, dxi = 0, dyr = 0, dyi = 0, dzr = 0, dzi = 0;
+            if (nn + 1 <= p) {
+                const int k1 = re_idx(nn + 1, mm), k2 = re_idx(nn + 1, mm + 1);
+                const double e = w * g_tab_d.e[nn][mm], f = g_tab_d.f[nn][mm];
+                const double l2r = Lr[k2], l2i = Lr[k2 + 1];
+                dzr = e * Lr[k1];
+                if (mm > 0) dzi = e * Lr[k1 + 1];
+                dxr = f * l2r;
+                dxi = f * l2i;
+                dyr = dxi;
+                dyi = -dxr;
+                if (mm >= 1) {
+                    const int k3 = re_idx(nn + 1, mm - 1);
+                    const double gg = g_tab_d.g[nn][mm], gr = gg * Lr[k3];
+                    const double gi = mm > 1 ? gg * Lr[k3 + 1] : 0.0;
+                    dxr -= gr;
+                    dxi -= gi;
+                    dyr += gi;
+                    dyi -= gr;
+                }
+            }
+            D4[k] = w * Lr[k];
+            D4[P + k] = dxr;
+            D4[2 * P + k] = dyr;
+            D4[3 * P + k] = dzr;
+            if (mm > 0) {
+                D4[k + 1] = w * Lr[k + 1];
+                D4[P + k + 1] = dxi;
+                D4[2 * P + k + 1] = dyi;
+                D4[3 * P + k + 1] = dzi;
+            }
+        }
+        __syncthreads();
+        if (in) {
+            const double* D4 = sD + ord * DS;
+            double x, y, z, q, ph = 0, ax = 0, ay = 0, az = 0;
+            Ion<double>::get(sorted[p0 + tid], x, y, z, q);
+            for_each_ups<double>(p, x, y, z, c_tab_d, [&](int nn, int m, double yr, double yi) {
+                const double* d = D4 + re_idx(nn, m);
+                if (PHI) ph += d[0] * yr;
+                ax += d[P] * yr;
+                ay += d[2 * P] * yr;
+                az += d[3 * P] * yr;
+                if (m > 0) {
+                    if (PHI) ph += d[1] * yi;
+                    ax += d[P + 1] * yi;
+                    ay += d[2 * P + 1] * yi;
+                    az += d[3 * P + 1] * yi;
+                }
+            });
+            double ex = -ax, ey = -ay, ez = -az;
+            if (near) {
+                const Ion<double>::rec o = *reinterpret_cast<const Ion<double>::rec*>(near + 4 * (int64_t)(p0 + tid));
+                ex += o.x;
+                ey += o.y;
+                ez += o.z;
+                if (PHI) ph += o.w;
+            }
+            const int i = perm[p0 + tid];
+            E[i] = s_f[0] * ex;
+            E[n + i] = s_f[0] * ey;
+            E[2 * n + i] = s_f[0] * ez;
+            if (PHI) phi[i] = s_f[1] * ph;
+        }
+        p0 += ni;
+    }
+}
+
 // Direct ancestor local expansions (PT_EXPAND_DIRECT): as k_l2p, but every
 // thread evaluates its columns of the M2L-only local expansions of the
 // target's cells at levels lmin..D, each at the ion in that cell's frame,
@@ -1293,9 +1510,12 @@ void launch_p2p<float>(int D, int64_t leaves, int grid, bool phi, Workspace& ws,
 template <>
 void launch_p2p<double>(int D, int64_t leaves, int grid, bool phi, Workspace& ws,
                         const int32_t* cid_leaf, double* near, cudaStream_t s) {
-    // four blocks per SM at least: 1,000 ions at depth 2 (63 leaves) took
-    // 223 us with a block per leaf
-    const int64_t want = 4 * (int64_t)ws.sms;
+    // few leaves: several blocks share a leaf's targets, so that a shallow
+    // tree (1,000 ions at depth 2: 63 leaves, 223 us with a block per leaf)
+    // fills the GPU.  (One or two blocks per SM, to run beside the
+    // translations' CTAs: the FP64 latencies then show, 50 and 42 ms against
+    // 35 for the evaluation of 1e6 ions at p = 8.)
+    const int64_t want = (int64_t)ws.sms * 4;
     const int parts = (int)(leaves >= want ? 1 : (want + leaves - 1) / leaves);
     const int64_t units = leaves * parts, cap = 152 * 16;
     grid = (int)(units < cap ? units : cap);
@@ -1366,9 +1586,15 @@ static cudaError_t run_fmm(int64_t n, int D, int phases, Workspace& ws, bool use
                             (const int32_t*)ws.leaf_of, (const typename Ion<T>::rec*)ws.sorted,
                             M, Mp)) != cudaSuccess)
             return e;
+    } else if (far && sizeof(T) == 8 && n >= kP2mSlotIons) {
+        if ((e = launch_pdl(k_p2m_f64, dim3((unsigned)((n + kSlotWindow - 1) / kSlotWindow)),
+                            dim3(kSlotThreads), sizeof(double) * kSlotThreads * p2m_f64_stride(P), s, n,
+                            p, ws.ld, (const int32_t*)ws.leaf_of, (const int32_t*)ws.cstart,
+                            (const int32_t*)ws.ccount, (const Ion<double>::rec*)ws.sorted,
+                            (double*)ws.M)) != cudaSuccess)
+            return e;
     } else if (far) {
-        int grid = leaf_grid;
-        k_p2m<T><<<grid, kP2mThreads, kP2mIons * P * sizeof(T), s>>>(
+        k_p2m<T><<<leaf_grid, kP2mThreads, kP2mIons * P * sizeof(T), s>>>(
             D, p, ws.ld, ws.linfo, ws.cstart, ws.ccount, (const typename Ion<T>::rec*)ws.sorted, M,
             Mp);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -1378,7 +1604,9 @@ static cudaError_t run_fmm(int64_t n, int D, int phases, Workspace& ws, bool use
     // SM, beside the slab reduction and the L2L launches, which use few
     // On the tensor-core paths the near field takes a third stream from the
     // fork, beside the upward pass and the work list (both latency-bound).
-    const bool near_early = fork && use_tc && ws.side2 != nullptr;
+    // So it does on the FP64 path with the tensor-core translations (10k-ion
+    // step 0.77 against 0.71 ms; 1e5-ion evaluation 8.39 against 8.29 ms).
+    const bool near_early = fork && (use_tc || f64) && ws.side2 != nullptr;
     cudaStream_t snf = near_early ? ws.side2 : sn;
     auto launch_near = [&](bool after_event) -> cudaError_t {
         cudaError_t r;
@@ -1490,6 +1718,14 @@ static cudaError_t run_fmm(int64_t n, int D, int phases, Workspace& ws, bool use
             n, D, 2, p, ws.ld, ws.root, ws.linfo, ws.code, ws.cid,
             (const typename Ion<T>::rec*)ws.sorted, ws.perm, ws.cstart, ws.ccount, L,
             nf ? near : nullptr, E, phi);
+    else if (far && sizeof(T) == 8 && n >= kL2pSlotIons)
+        e = launch_pdl(phi ? k_l2p_f64<true> : k_l2p_f64<false>,
+                       dim3((unsigned)((n + kSlotWindow - 1) / kSlotWindow)), dim3(kSlotThreads),
+                       l2p_f64_smem(P), s, n, D, p, ws.ld, l2p_f64_leaves(P), (const RootCube*)ws.root,
+                       (const int32_t*)ws.leaf_of, (const int32_t*)ws.cstart,
+                       (const int32_t*)ws.ccount, (const Ion<double>::rec*)ws.sorted,
+                       (const int32_t*)ws.perm, (const double*)ws.L,
+                       (const double*)(nf ? ws.near : nullptr), E, phi);
     else
         e = launch_pdl(p <= 15 ? k_l2p<T, 8> : k_l2p<T, 16>, dim3(leaf_grid), dim3(kL2pThreads),
                        0, s, n, D, p, ws.ld, far,
@@ -1685,6 +1921,13 @@ cudaError_t upload_harmonic_tables() {
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_p2m<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  kP2mIons * pmax * (int)sizeof(double));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_p2m_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kSlotThreads * p2m_f64_stride(pmax) * (int)sizeof(double));
+    // (the largest over the orders: fewer leaves above the order where 16 fit)
+    for (auto f : {k_l2p_f64<true>, k_l2p_f64<false>})
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 104 * 1024);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_p2m<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  kP2mIons * pmax * (int)sizeof(float));

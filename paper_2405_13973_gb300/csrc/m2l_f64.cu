@@ -169,29 +169,56 @@ __device__ __forceinline__ long long f64_join(const uint32_t (&v)[kDig]) {
     return ((long long)u << 32) + ((long long)w * 65536 + (long long)x);
 }
 
-// I 2^e as a double, rounded to nearest, without the FP64 units
+// I 2^e as a double, rounded to nearest, in integer instructions, for
+// exponents well inside the normal range (|e| <= kExpFast; |I| < 2^62)
+constexpr int kExpFast = 900;
 __device__ __forceinline__ double fixed_to_double(long long I, int e) {
-    if (I == 0) return 0.0;
+    const uint32_t sign = (uint32_t)((unsigned long long)I >> 32) & 0x80000000u;
     const unsigned long long a = I < 0 ? 0ull - (unsigned long long)I : (unsigned long long)I;
-    const int lz = __clzll((long long)a);
-    const unsigned long long m = a << lz;
-    const int be = e + 63 - lz + 1022;  // exponent field before the hidden bit is added
-    if (be < 1 || be > 2044) return ldexp((double)I, e);
-    const unsigned long long r = ((unsigned long long)be << 52) + (m >> 11) + ((m >> 10) & 1ull);
-    return __longlong_as_double((long long)(r | ((unsigned long long)I & 0x8000000000000000ull)));
+    uint32_t h = (uint32_t)(a >> 32), l = (uint32_t)a;
+    int be = e + 63 + 1022;  // exponent field before the leading one is added
+    if (h == 0) {
+        h = l;
+        l = 0;
+        be -= 32;
+    }
+    if (h == 0) return 0.0;
+    const int lz = __clz((int)h);
+    const uint32_t mh = __funnelshift_l(l, h, lz), ml = l << lz;
+    const unsigned long long r = ((unsigned long long)((mh >> 11) + ((uint32_t)(be - lz) << 20)) << 32) +
+                                 (unsigned long long)__funnelshift_r(ml, mh, 11) + ((ml >> 10) & 1u);
+    return __longlong_as_double((long long)(r | ((unsigned long long)sign << 32)));
+}
+// the rest: rows of subnormal or huge values, NaN rows
+__device__ __noinline__ double fixed_to_double_slow(long long I, int er, int fn) {
+    if (er == kRowNan) return __longlong_as_double(0x7ff8000000000000ll);
+    return ldexp((double)I, er + fn);
 }
 
-// work item idx: operator, rows, and for M2M / L2L the first target cell
+// work unit idx: operator, rows, for M2M / L2L the first target cell, and the
+// column chunks [c0, c1).  A unit is a whole item, or one chunk of it where
+// there are few items (see k_f64_mma).
 struct F64Work {
-    int op, rows, base;
+    int op, rows, base, c0, c1;
 };
+// Chunks are units of their own while the items alone would not fill the
+// CTAs: an M2M or L2L launch of a few items then takes a chunk's time and not
+// an item's (10k ions, p = 12: 38 -> 17 us and 43 -> 20 us each); with more
+// items (316 M2L offsets of a 63-leaf tree) the units' own start costs more.
 template <int MODE>
 __device__ __forceinline__ bool f64_work(const F64Args& a, const LevelInfo& li, int idx, int count,
-                                         F64Work& w) {
+                                         int split, F64Work& w) {
     w.rows = 0;
     w.op = 0;
     w.base = 0;
+    w.c0 = 0;
+    w.c1 = a.nch;
     if (idx >= count) return false;
+    if (split > 1) {
+        w.c0 = idx % split;
+        w.c1 = w.c0 + 1;
+        idx /= split;
+    }
     if (MODE == F64_PAIR) {
         const M2lPairItem it = a.items[idx];
         w.op = it.op;
@@ -267,7 +294,9 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    const int count = f64_count<MODE>(a, li);
+    const int items = f64_count<MODE>(a, li);
+    const int split = items <= (int)gridDim.x ? a.nch : 1;
+    const int count = items * split;
     const int first = blockIdx.x, stride = gridDim.x;
     if (first >= count) return;  // uniform across the block
     if (warp == 0) {
@@ -291,9 +320,10 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
         if (lane == 0) {
             int g = 0;
             F64Work w;
-            for (int idx = first; f64_work<MODE>(a, li, idx, count, w) && !*abort_v; idx += stride) {
-                const unsigned char* src = a.ops + (int64_t)w.op * a.op_bytes;
-                for (int c = 0; c < a.nch; ++c) {
+            for (int idx = first; f64_work<MODE>(a, li, idx, count, split, w) && !*abort_v; idx += stride) {
+                const unsigned char* src = a.ops + (int64_t)w.op * a.op_bytes +
+                                           (int64_t)a.kst32 * kDig * 64 * (w.c0 * kChunk);
+                for (int c = w.c0; c < w.c1; ++c) {
                     const uint32_t bytes = (uint32_t)(kDig * min(kChunk, a.npad - c * kChunk) * 64);
                     for (int k = 0; k < a.kst32; ++k, ++g) {
                         const int st = g % a.bst, use = g / a.bst;
@@ -316,11 +346,12 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
         // ---- MMA issuer.  The whole warp runs the loops on warp-uniform
         // values and one elected lane issues (mbar_wait_warp)
         const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
-        const int items = __shfl_sync(0xffffffffu, (count - first + stride - 1) / stride, 0);
+        const int last = __shfl_sync(0xffffffffu, count, 0), sp = __shfl_sync(0xffffffffu, split, 0);
         int sa = 0, pa = 0, sb = 0, pb = 0, pacc = 1;  // stages and phases
         bool ok = true;
-        for (int t = 0; ok && t < items; ++t) {
-            for (int c = 0; ok && c < a.nch; ++c) {
+        for (int t = first; ok && t < last; t += stride) {
+            const int c0 = sp > 1 ? t % sp : 0, c1 = sp > 1 ? c0 + 1 : a.nch;
+            for (int c = c0; ok && c < c1; ++c) {
                 const int N = min(kChunk, a.npad - c * kChunk);
                 const uint32_t id = idesc_f16(N);
                 const uint32_t bstep = (uint32_t)(N * 64) >> 4;  // one digit of B
@@ -337,12 +368,12 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
                     const uint64_t bd = sdesc64(smem_addr(base) + (uint32_t)(sb * b_stage) + 32u * (ks & 1));
                     const uint32_t blo = (uint32_t)bd, bhi = (uint32_t)(bd >> 32);
                     const uint32_t at = tm + (uint32_t)(kACol0 + sa * kDig * 8);
-                    const bool last = (ks & 1) || ks + 1 == a.ksteps;
+                    const bool endb = (ks & 1) || ks + 1 == a.ksteps;
                     if (elect_one()) {
                         if (ks == 0) f64_products<0>(tm, at, blo, bhi, bstep, id);
                         else f64_products<1>(tm, at, blo, bhi, bstep, id);
                         mma_commit(&emptyA[sa]);
-                        if (last) mma_commit(&emptyB[sb]);
+                        if (endb) mma_commit(&emptyB[sb]);
                         if (ks + 1 == a.ksteps) mma_commit(&accf);
                     }
                     __syncwarp();
@@ -350,7 +381,7 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
                         sa = 0;
                         pa ^= 1;
                     }
-                    if (last && ++sb == a.bst) {
+                    if (endb && ++sb == a.bst) {
                         sb = 0;
                         pb ^= 1;
                     }
@@ -373,13 +404,14 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
         const int row_bytes = a.gsegs * kSegBytes + 16;  // 16: no bank conflicts
         unsigned char* ring = base + a.bst * b_stage + row * row_bytes;
         const int groups = (a.kst32 + a.gsegs - 1) / a.gsegs;
-        const int loads = a.resident ? groups : a.nch * groups;  // per item
+        const int nch = split > 1 ? 1 : a.nch;                   // chunks per unit
+        const int loads = a.resident ? groups : nch * groups;    // per unit
         F64Work w;
         // the loading side: item lidx, its load lo; the source of the item
         // after it waits in a register
         int lidx = first, lo = 0, lslot = 0, issued = 0, freed = 0;
-        int src = f64_work<MODE>(a, li, lidx, count, w) ? f64_source<MODE>(a, w, row) : -1, nsrc = -1;
-        if (f64_work<MODE>(a, li, lidx + stride, count, w)) nsrc = f64_source<MODE>(a, w, row);
+        int src = f64_work<MODE>(a, li, lidx, count, split, w) ? f64_source<MODE>(a, w, row) : -1, nsrc = -1;
+        if (f64_work<MODE>(a, li, lidx + stride, count, split, w)) nsrc = f64_source<MODE>(a, w, row);
         auto issue = [&]() {
             if (lidx >= count || issued - freed >= a.ring) return;
             const int grp = lo % groups;
@@ -396,14 +428,14 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
                 lidx += stride;
                 src = nsrc;
                 nsrc = -1;
-                if (f64_work<MODE>(a, li, lidx + stride, count, w)) nsrc = f64_source<MODE>(a, w, row);
+                if (f64_work<MODE>(a, li, lidx + stride, count, split, w)) nsrc = f64_source<MODE>(a, w, row);
             }
         };
         for (int k = 0; k < a.ring; ++k) issue();
         int sa = 0, pa = 1, used = 0;  // A stage and phase, the item's first load
         bool ok = true;
         for (int idx = first; ok && idx < count; idx += stride, used += loads) {
-            for (int c = 0; ok && c < a.nch; ++c) {
+            for (int c = 0; ok && c < nch; ++c) {
                 for (int grp = 0; ok && grp < groups; ++grp) {
                     const int id = used + (a.resident ? grp : c * groups + grp);
                     const int slot = id % a.ring;
@@ -434,7 +466,7 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
                             pa ^= 1;
                         }
                     }
-                    if (!a.resident || c + 1 == a.nch) {
+                    if (!a.resident || c + 1 == nch) {
                         ++freed;
                         issue();
                     }
@@ -450,11 +482,12 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
         int jacc = 0;
         F64Work w;
         bool stop = false;
-        for (int idx = first; !stop && f64_work<MODE>(a, li, idx, count, w); idx += stride) {
+        for (int idx = first; !stop && f64_work<MODE>(a, li, idx, count, split, w); idx += stride) {
             const int src = f64_source<MODE>(a, w, row);
             const int er = src >= 0 ? a.rexp[src] : 0;
+            const bool fast = abs(er) <= kExpFast - 150;  // operator exponents lie within +-100
             double* orow = a.out + (int64_t)(w.base + row) * a.out_stride;
-            for (int c = 0; c < a.nch; ++c, ++jacc) {
+            for (int c = w.c0; c < w.c1; ++c, ++jacc) {
                 const int N = min(kChunk, a.npad - c * kChunk);
                 const int ng = N / 16, c0 = half * (N / 2);  // groups of 8 columns
                 const int n0 = c * kChunk + c0;
@@ -524,11 +557,18 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
                     if (row >= w.rows) continue;
                     const int fw[4] = {f[q].x, f[q].y, f[q].z, f[q].w};
                     double v[8];
+                    if (fast) {
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const int fn = j & 1 ? fw[j >> 1] >> 16 : (int)(int16_t)(fw[j >> 1] & 0xffff);
-                        v[j] = er == kRowNan ? __longlong_as_double(0x7ff8000000000000ll)
-                                             : fixed_to_double(I[q][j], er + fn - 50);
+                        for (int j = 0; j < 8; ++j) {
+                            const int fn = j & 1 ? fw[j >> 1] >> 16 : (int)(int16_t)(fw[j >> 1] & 0xffff);
+                            v[j] = fixed_to_double(I[q][j], er + fn - 50);
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            const int fn = j & 1 ? fw[j >> 1] >> 16 : (int)(int16_t)(fw[j >> 1] & 0xffff);
+                            v[j] = fixed_to_double_slow(I[q][j], er, fn - 50);
+                        }
                     }
                     // rows are multiples of 4 doubles apart: whole 32-byte units
 #pragma unroll
@@ -838,7 +878,7 @@ cudaError_t launch_f64_m2m(int64_t n, int D, int l, Workspace& ws, cudaStream_t 
     a.level = l + 1;  // the children, each row its own shifted multipole in L
     a.out = (double*)ws.L;
     a.out_stride = ws.ld;
-    const int64_t items = level_cap(n, l + 1) / kF64Rows + 8;
+    const int64_t items = (level_cap(n, l + 1) / kF64Rows + 8) * a.nch;
     cudaError_t e = launch_pdl(k_f64_mma<F64_M2M>, dim3(f64_grid(ws, items)), dim3(kF64Threads),
                                f64_smem(a), s, a);
     if (e != cudaSuccess) return e;
@@ -856,7 +896,7 @@ cudaError_t launch_f64_l2l(int64_t n, int D, int l, Workspace& ws, cudaStream_t 
     a.off_parent = dense_layout(D).off[l - 1];
     a.out = (double*)ws.L;
     a.out_stride = ws.ld;
-    const int64_t items = level_cap(n, l) / kF64Rows + 8;
+    const int64_t items = (level_cap(n, l) / kF64Rows + 8) * a.nch;
     return launch_pdl(k_f64_mma<F64_L2L>, dim3(f64_grid(ws, items)), dim3(kF64Threads),
                       f64_smem(a), s, a);
 }
@@ -869,7 +909,7 @@ cudaError_t launch_f64_m2l(Workspace& ws, cudaStream_t s) {
     a.pairs = L.pairs;
     a.out = (double*)ws.pp_part;
     a.out_stride = ws.pp_stride;
-    k_f64_mma<F64_PAIR><<<f64_grid(ws, ws.pp_item_cap), kF64Threads, f64_smem(a), s>>>(a);
+    k_f64_mma<F64_PAIR><<<f64_grid(ws, ws.pp_item_cap * a.nch), kF64Threads, f64_smem(a), s>>>(a);
     return cudaGetLastError();
 }
 
