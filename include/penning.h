@@ -501,7 +501,9 @@ int pt_ensemble_create(int n_members, const fmm_plan* plans, pt_ensemble* out);
  * members that use the BF16x3 pair-packed schedule (Eq. FMM_local) are
  * replaced in that graph by one launch over all of their work items, which
  * waits for every such member's multipoles and precedes every member's
- * reduction (see pt_ensemble_set_joined_m2l).  A member's result equals
+ * reduction (see pt_ensemble_set_joined_m2l).  With that switch on, the
+ * members' other launches are joined kernel by kernel as well (unless a
+ * member is being profiled).  A member's result equals
  * the same plan stepped alone by pt_step, bit for bit.  Asynchronous like
  * pt_step_async: automatic-depth plans keep the depth chosen at their first
  * step; device errors are latched and returned by pt_ensemble_sync.

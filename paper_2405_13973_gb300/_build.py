@@ -19,7 +19,7 @@ LIB = os.path.join(HERE, "libpenning.so")
 BUILD = os.path.join(HERE, "_build")
 
 SOURCES = ["abi.cu", "tree.cu", "fmm.cu", "push.cu", "m2l_tc.cu", "m2l_pairs.cu", "m2l_f64.cu", "m2l_f32.cu",
-           "energy_noalloc.cu", "mh.cu"]
+           "energy_noalloc.cu", "mh.cu", "join.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 COMMON = ["-O3", "-lineinfo", "-std=c++17", "--expt-relaxed-constexpr",
           "-Xcompiler", "-fPIC,-ffp-contract=off,-O2", "-I", CSRC,

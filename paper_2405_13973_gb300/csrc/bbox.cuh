@@ -53,13 +53,13 @@ struct BboxAcc {
     }
 };
 
-// Folds every thread's extremes into acc[] (all threads of the block call
-// it); the last block writes the root cube exactly as
+// Folds every thread's extremes into acc[] (all threads of the `blocks`
+// blocks call it); the last block writes the root cube exactly as
 //   side = max_a (max_a - min_a) (1 if zero); lo_a = (min_a+max_a)/2 - side/2
 // and clears acc[] and the ticket.  Returns true in the one thread that
 // finalised the cube.
-__device__ __forceinline__ bool bbox_commit(BboxAcc& t, unsigned long long* acc, unsigned* ticket,
-                                            RootCube* root, int* err) {
+__device__ __forceinline__ bool bbox_commit(BboxAcc& t, unsigned blocks, unsigned long long* acc,
+                                            unsigned* ticket, RootCube* root, int* err) {
     __shared__ bool last;
     const int lane = threadIdx.x & 31;
 #pragma unroll
@@ -76,7 +76,7 @@ __device__ __forceinline__ bool bbox_commit(BboxAcc& t, unsigned long long* acc,
     __syncthreads();
     if (threadIdx.x == 0) {
         const unsigned tk = atomicAdd(ticket, 1u);
-        last = (tk == gridDim.x - 1);
+        last = (tk == blocks - 1);
     }
     __syncthreads();
     if (!last || threadIdx.x != 0) return false;

@@ -24,6 +24,7 @@
 #include "fmm_math.cuh"
 #include "harmonics.cuh"
 #include "internal.h"
+#include "join.cuh"
 
 namespace pt {
 
@@ -169,7 +170,7 @@ constexpr int kP2mIons = 32;
 // (deterministic).  Leaves with more ions than kP2mIons are done in passes.
 // ---------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(kP2mThreads) k_p2m(int D, int p, int ld, const LevelInfo* linfo,
+__device__ __forceinline__ void k_p2m_body(const BlockId& blk, int D, int p, int ld, const LevelInfo* linfo,
                                                      const int32_t* __restrict__ cstart,
                                                      const int32_t* __restrict__ ccount,
                                                      const typename Ion<T>::rec* __restrict__ sorted,
@@ -179,7 +180,7 @@ __global__ void __launch_bounds__(kP2mThreads) k_p2m(int D, int p, int ld, const
     T* terms = reinterpret_cast<T*>(p2m_smem);  // [kP2mIons][P]
     const HarmTables<T>& t = tab<T>();
     const int g0 = linfo->gbase[D], g1 = linfo->gbase[D + 1];
-    for (int g = g0 + blockIdx.x; g < g1; g += gridDim.x) {
+    for (int g = g0 + (int)blk.x; g < g1; g += (int)blk.nx) {
         const int s = cstart[g], k = ccount[g];
         T acc[(kMaxOrder + 1) * (kMaxOrder + 1) / kP2mThreads + 1];
         constexpr int NA = (kMaxOrder + 1) * (kMaxOrder + 1) / kP2mThreads + 1;
@@ -215,6 +216,14 @@ __global__ void __launch_bounds__(kP2mThreads) k_p2m(int D, int p, int ld, const
             }
         }
     }
+}
+template <typename T>
+__global__ void __launch_bounds__(kP2mThreads) k_p2m(int D, int p, int ld, const LevelInfo* linfo,
+                                                     const int32_t* __restrict__ cstart,
+                                                     const int32_t* __restrict__ ccount,
+                                                     const typename Ion<T>::rec* __restrict__ sorted,
+                                                     T* __restrict__ M, uint16_t* Mp) {
+    k_p2m_body<T>(solo_block(), D, p, ld, linfo, cstart, ccount, sorted, M, Mp);
 }
 
 // ---------------------------------------------------------------------------
@@ -311,8 +320,7 @@ __global__ void __launch_bounds__(kSlotThreads) k_p2m_f64(
 constexpr int kP2mAncIons = 64;
 
 template <typename T>
-__global__ void __launch_bounds__(kP2mThreads) k_p2m_anc(
-    int D, int lmin, int p, int ld, const LevelInfo* linfo, const uint32_t* __restrict__ code,
+__device__ __forceinline__ void k_p2m_anc_body(const BlockId& blk, int D, int lmin, int p, int ld, const LevelInfo* linfo, const uint32_t* __restrict__ code,
     const int32_t* __restrict__ leaf_start, const int32_t* __restrict__ leaf_of,
     const typename Ion<T>::rec* __restrict__ sorted, T* __restrict__ M, uint16_t* Mp) {
     extern __shared__ unsigned char p2m_smem[];
@@ -321,7 +329,7 @@ __global__ void __launch_bounds__(kP2mThreads) k_p2m_anc(
     T* terms = reinterpret_cast<T*>(p2m_smem);  // [kP2mAncIons][P]
     const HarmTables<T>& t = tab<T>();
     const int g0 = linfo->gbase[lmin], g1 = linfo->gbase[D + 1];
-    for (int g = g0 + blockIdx.x; g < g1; g += gridDim.x) {
+    for (int g = g0 + (int)blk.x; g < g1; g += (int)blk.nx) {
         int l = lmin;
         while (l < D && g >= linfo->gbase[l + 1]) ++l;
         const int sh = D - l, mask = (1 << sh) - 1;
@@ -366,6 +374,12 @@ __global__ void __launch_bounds__(kP2mThreads) k_p2m_anc(
             }
         }
     }
+}
+template <typename T>
+__global__ void __launch_bounds__(kP2mThreads) k_p2m_anc(int D, int lmin, int p, int ld, const LevelInfo* linfo, const uint32_t* __restrict__ code,
+    const int32_t* __restrict__ leaf_start, const int32_t* __restrict__ leaf_of,
+    const typename Ion<T>::rec* __restrict__ sorted, T* __restrict__ M, uint16_t* Mp) {
+    k_p2m_anc_body<T>(solo_block(), D, lmin, p, ld, linfo, code, leaf_start, leaf_of, sorted, M, Mp);
 }
 
 // ---------------------------------------------------------------------------
@@ -454,7 +468,7 @@ size_t shift_rows_smem(int P) {
 }
 
 template <typename T, int MODE>
-__global__ void __launch_bounds__(kShThreads) k_shift_rows(int l, int P, int ld,
+__device__ __forceinline__ void k_shift_rows_body(const BlockId& blk, int l, int P, int ld,
                                                            const LevelInfo* linfo,
                                                            const uint32_t* __restrict__ code,
                                                            const int32_t* __restrict__ cid,
@@ -469,8 +483,8 @@ __global__ void __launch_bounds__(kShThreads) k_shift_rows(int l, int P, int ld,
     T* sOp = reinterpret_cast<T*>(smem_raw);  // [kShRows][S]
     T* sX = sOp + kShRows * S;                // [CG][K]
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-    const int r0 = blockIdx.x * kShRows;
-    const int oct = MODE == 1 ? (int)blockIdx.y : 0;
+    const int r0 = (int)blk.x * kShRows;
+    const int oct = MODE == 1 ? (int)(int)blk.y : 0;
     if (MODE == 0) {
         // Op = T_m2m transposed, [o][c][r]: element (r, t = o P + c) at t P + r
         for (int e = tid; e < K * kShRows; e += kShThreads) {
@@ -495,8 +509,8 @@ __global__ void __launch_bounds__(kShThreads) k_shift_rows(int l, int P, int ld,
         g1 = linfo->oct_start[l][oct + 1];
     }
     const int nch = (g1 - g0 + CG - 1) / CG;
-    const int ch0 = MODE == 0 ? (int)blockIdx.y : (int)blockIdx.z;
-    const int chs = MODE == 0 ? (int)gridDim.y : (int)gridDim.z;
+    const int ch0 = MODE == 0 ? (int)(int)blk.y : (int)(int)blk.z;
+    const int chs = MODE == 0 ? (int)(int)blk.ny : (int)(int)blk.nz;
     const T* op0 = sOp + w * S;
     const T* op1 = sOp + (w + 8) * S;
     for (int ch = ch0; ch < nch; ch += chs) {
@@ -561,6 +575,16 @@ __global__ void __launch_bounds__(kShThreads) k_shift_rows(int l, int P, int ld,
             }
         }
     }
+}
+template <typename T, int MODE>
+__global__ void __launch_bounds__(kShThreads) k_shift_rows(int l, int P, int ld,
+                                                           const LevelInfo* linfo,
+                                                           const uint32_t* __restrict__ code,
+                                                           const int32_t* __restrict__ cid,
+                                                           int64_t off_nb,
+                                                           const T* __restrict__ Op, T* Y,
+                                                           uint16_t* Mp) {
+    k_shift_rows_body<T, MODE>(solo_block(), l, P, ld, linfo, code, cid, off_nb, Op, Y, Mp);
 }
 
 // ---------------------------------------------------------------------------
@@ -707,8 +731,7 @@ constexpr int kNfThreads = 128;
 constexpr int kNfSrc = 1024;   // staged sources per pass
 
 template <typename T>
-__global__ void __launch_bounds__(kNfThreads) k_p2p(
-    int D, const LevelInfo* linfo, const typename Ion<T>::rec* __restrict__ sorted,
+__device__ __forceinline__ void k_p2p_body(const BlockId& blk, int D, const LevelInfo* linfo, const typename Ion<T>::rec* __restrict__ sorted,
     const uint32_t* __restrict__ code, const int32_t* __restrict__ cid_leaf,
     const int32_t* __restrict__ cstart, const int32_t* __restrict__ ccount, T* __restrict__ near) {
     using R = typename Ion<T>::rec;
@@ -718,7 +741,7 @@ __global__ void __launch_bounds__(kNfThreads) k_p2p(
     const int tid = threadIdx.x;
     const int lim = 1 << D;
     const int g0 = linfo->gbase[D], g1 = linfo->gbase[D + 1];
-    for (int g = g0 + blockIdx.x; g < g1; g += gridDim.x) {
+    for (int g = g0 + (int)blk.x; g < g1; g += (int)blk.nx) {
         const int ts = cstart[g], nt = ccount[g];
         int ix, iy, iz;
         demorton3(code[g], ix, iy, iz);
@@ -820,6 +843,12 @@ __global__ void __launch_bounds__(kNfThreads) k_p2p(
         }
         __syncthreads();
     }
+}
+template <typename T>
+__global__ void __launch_bounds__(kNfThreads) k_p2p(int D, const LevelInfo* linfo, const typename Ion<T>::rec* __restrict__ sorted,
+    const uint32_t* __restrict__ code, const int32_t* __restrict__ cid_leaf,
+    const int32_t* __restrict__ cstart, const int32_t* __restrict__ ccount, T* __restrict__ near) {
+    k_p2p_body<T>(solo_block(), D, linfo, sorted, code, cid_leaf, cstart, ccount, near);
 }
 
 // The same in FP64.  The FP64 units serve two lanes a clock, a warp
@@ -1178,15 +1207,14 @@ __device__ __forceinline__ void l2p_columns8(int p, int j, unsigned gmask, T x, 
 // (equal to the L2L shift into the leaf, which shifts a truncated expansion
 // exactly), saving the last L2L launch.
 template <typename T, int G>
-__global__ void __launch_bounds__(kL2pThreads) k_l2p(
-    int64_t n, int D, int p, int ld, bool far, int nlev, const RootCube* root,
+__device__ __forceinline__ void k_l2p_body(const BlockId& blk, int64_t n, int D, int p, int ld, bool far, int nlev, const RootCube* root,
     const LevelInfo* linfo, const uint32_t* __restrict__ code, const int32_t* __restrict__ cid,
     const typename Ion<T>::rec* __restrict__ sorted, const int32_t* __restrict__ perm,
     const int32_t* __restrict__ cstart, const int32_t* __restrict__ ccount,
     const T* __restrict__ L, const T* __restrict__ near, double* E, double* phi) {
     pdl_wait();
     const int g0 = linfo->gbase[D], g1 = linfo->gbase[D + 1];
-    if (g0 + (int)blockIdx.x >= g1) return;  // no leaf for this block
+    if (g0 + (int)(int)blk.x >= g1) return;  // no leaf for this block
     constexpr int NL = sizeof(T) == 4 ? 3 : 2;  // levels evaluated at most (shared memory)
     __shared__ T sL[NL][kPmax];
     __shared__ T sD[NL][4][kPmax];  // derived expansions: phi, grad x, grad y, grad z
@@ -1214,7 +1242,7 @@ __global__ void __launch_bounds__(kL2pThreads) k_l2p(
     const unsigned hw_mask = (G == 8 ? 0xffu : 0xffffu) << (lane & (32 - G));
     const int P = (p + 1) * (p + 1);
     const int levs = far ? (nlev < NL ? nlev : NL) : 0;
-    for (int g = g0 + blockIdx.x; g < g1; g += gridDim.x) {
+    for (int g = g0 + (int)blk.x; g < g1; g += (int)blk.nx) {
         const int ts = cstart[g], nt = ccount[g];
         const uint32_t cl = code[g];
         int ix, iy, iz;
@@ -1274,6 +1302,14 @@ __global__ void __launch_bounds__(kL2pThreads) k_l2p(
             }
         }
     }
+}
+template <typename T, int G>
+__global__ void __launch_bounds__(kL2pThreads) k_l2p(int64_t n, int D, int p, int ld, bool far, int nlev, const RootCube* root,
+    const LevelInfo* linfo, const uint32_t* __restrict__ code, const int32_t* __restrict__ cid,
+    const typename Ion<T>::rec* __restrict__ sorted, const int32_t* __restrict__ perm,
+    const int32_t* __restrict__ cstart, const int32_t* __restrict__ ccount,
+    const T* __restrict__ L, const T* __restrict__ near, double* E, double* phi) {
+    k_l2p_body<T, G>(solo_block(), n, D, p, ld, far, nlev, root, linfo, code, cid, sorted, perm, cstart, ccount, L, near, E, phi);
 }
 
 // L2P in FP64 (see k_p2m_f64): a thread per ion, the derived expansions of
@@ -1945,6 +1981,44 @@ cudaError_t upload_harmonic_tables() {
         e = cudaFuncSetAttribute(k_shift_rows<float, 1>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)shift_rows_smem<float, 1>(pmax));
+    return e;
+}
+
+// ---------------------------------------------------------------------------
+// Joined ensemble launches (join.cuh) of the FP32 stages of the tensor-core
+// and CUDA-core precisions.
+// ---------------------------------------------------------------------------
+struct P2mJoin {
+    template <class... A>
+    __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const { k_p2m_body<float>(b, a...); }
+};
+struct P2mAncJoin {
+    template <class... A>
+    __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const { k_p2m_anc_body<float>(b, a...); }
+};
+struct ShiftJoin {
+    template <class... A>
+    __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const {
+        k_shift_rows_body<float, 0>(b, a...);
+    }
+};
+struct P2pJoin {
+    template <class... A>
+    __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const { k_p2p_body<float>(b, a...); }
+};
+struct L2pJoin {
+    template <class... A>
+    __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const {
+        k_l2p_body<float, 8>(b, a...);
+    }
+};
+
+cudaError_t join_fmm(JoinCtx& c) {
+    cudaError_t e = join_kernel<P2mJoin, kP2mThreads, 3>(c, k_p2m<float>);
+    if (e == cudaSuccess) e = join_kernel<P2mAncJoin, kP2mThreads, 4>(c, k_p2m_anc<float>);
+    if (e == cudaSuccess) e = join_kernel<ShiftJoin, kShThreads, 3>(c, k_shift_rows<float, 0>);
+    if (e == cudaSuccess) e = join_kernel<P2pJoin, kNfThreads, 1>(c, k_p2p<float>);
+    if (e == cudaSuccess) e = join_kernel<L2pJoin, kL2pThreads, 7>(c, k_l2p<float, 8>);
     return e;
 }
 

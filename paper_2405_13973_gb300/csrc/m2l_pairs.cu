@@ -21,6 +21,7 @@
 
 #include "bf16split.cuh"
 #include "harmonics.cuh"
+#include "join.cuh"
 #include "m2l_pairs.h"
 
 namespace pt {
@@ -78,7 +79,7 @@ __device__ __forceinline__ int pp_source(const PpArgs& a, int l, int x, int y, i
 // One warp per target: presence words of its 216 candidates, its pair count,
 // and the per-offset pair counts (block histogram, then global).
 constexpr int kPpThreads = 256;
-__global__ void __launch_bounds__(kPpThreads) k_pp_count(PpArgs a, uint32_t* tmask, int* tcount,
+__device__ __forceinline__ void k_pp_count_body(const BlockId& blk, PpArgs a, uint32_t* tmask, int* tcount,
                                                          int* ocnt) {
     __shared__ int hist[343];
     __shared__ LevelInfo li;
@@ -88,7 +89,7 @@ __global__ void __launch_bounds__(kPpThreads) k_pp_count(PpArgs a, uint32_t* tma
     const int lane = threadIdx.x & 31;
     const int g0 = li.gbase[2] + a.t0, g1 = pp_end(li, a);
     const int wpb = blockDim.x >> 5;
-    for (int g = g0 + blockIdx.x * wpb + (threadIdx.x >> 5); g < g1; g += gridDim.x * wpb) {
+    for (int g = g0 + (int)blk.x * wpb + (threadIdx.x >> 5); g < g1; g += (int)blk.nx * wpb) {
         const int l = pp_level(li, a.D, g);
         int x, y, z;
         demorton3(a.code[g], x, y, z);
@@ -109,12 +110,16 @@ __global__ void __launch_bounds__(kPpThreads) k_pp_count(PpArgs a, uint32_t* tma
     for (int i = threadIdx.x; i < 343; i += blockDim.x)
         if (hist[i]) atomicAdd(&ocnt[i], hist[i]);
 }
+__global__ void __launch_bounds__(kPpThreads) k_pp_count(PpArgs a, uint32_t* tmask, int* tcount,
+                                                         int* ocnt) {
+    k_pp_count_body(solo_block(), a, tmask, tcount, ocnt);
+}
 
 // One block: slot bases of the targets (exclusive scan of their counts; tbase
 // has n_targets + 1 entries), pair bases of the offsets, and the work items
 // (each offset's pairs in runs of 128, offsets in increasing order).
 constexpr int kPpScanThreads = 1024;
-__global__ void __launch_bounds__(kPpScanThreads) k_pp_scan(int D, int t0, int t1,
+__device__ __forceinline__ void k_pp_scan_body(const BlockId& blk, int D, int t0, int t1,
                                                              const LevelInfo* linfo,
                                                              int64_t slot_cap, int64_t rows_cap,
                                                              int item_cap,
@@ -247,13 +252,23 @@ __global__ void __launch_bounds__(kPpScanThreads) k_pp_scan(int D, int t0, int t
         ofill[o] = 0;
     }
 }
+__global__ void __launch_bounds__(kPpScanThreads) k_pp_scan(int D, int t0, int t1,
+                                                             const LevelInfo* linfo,
+                                                             int64_t slot_cap, int64_t rows_cap,
+                                                             int item_cap,
+                                                             const int* tcount, int* tbase,
+                                                             int* ocnt, int* ofill, int* obase,
+                                                             M2lPairHdr* hdr, M2lPairHdr* host_hdr,
+                                                             M2lPairItem* items, int* err) {
+    k_pp_scan_body(solo_block(), D, t0, t1, linfo, slot_cap, rows_cap, item_cap, tcount, tbase, ocnt, ofill, obase, hdr, host_hdr, items, err);
+}
 
 // One warp per target: each present offset takes the next position of that
 // offset's list (an atomic counter: the order of the pairs inside an
 // offset's list does not change any result, every product row being
 // computed alone), with its source and its slot (the target's slot base plus
 // the rank of the offset among the target's present ones).
-__global__ void __launch_bounds__(kPpThreads) k_pp_fill(PpArgs a, const uint32_t* tmask,
+__device__ __forceinline__ void k_pp_fill_body(const BlockId& blk, PpArgs a, const uint32_t* tmask,
                                                          const int* tbase, const int* obase,
                                                          int* ofill, const M2lPairHdr* hdr,
                                                          M2lPair* pairs, int* tpair) {
@@ -265,7 +280,7 @@ __global__ void __launch_bounds__(kPpThreads) k_pp_fill(PpArgs a, const uint32_t
     const int lane = threadIdx.x & 31;
     const int g0 = li.gbase[2] + a.t0, g1 = pp_end(li, a);
     const int wpb = blockDim.x >> 5;
-    for (int g = g0 + blockIdx.x * wpb + (threadIdx.x >> 5); g < g1; g += gridDim.x * wpb) {
+    for (int g = g0 + (int)blk.x * wpb + (threadIdx.x >> 5); g < g1; g += (int)blk.nx * wpb) {
         const int t = g - g0;
         const int l = pp_level(li, a.D, g);
         int x, y, z;
@@ -293,6 +308,12 @@ __global__ void __launch_bounds__(kPpThreads) k_pp_fill(PpArgs a, const uint32_t
         }
     }
 }
+__global__ void __launch_bounds__(kPpThreads) k_pp_fill(PpArgs a, const uint32_t* tmask,
+                                                         const int* tbase, const int* obase,
+                                                         int* ofill, const M2lPairHdr* hdr,
+                                                         M2lPair* pairs, int* tpair) {
+    k_pp_fill_body(solo_block(), a, tmask, tbase, obase, ofill, hdr, pairs, tpair);
+}
 
 // L of every target = the sum of its partial rows over its slots (increasing
 // offset); `width` columns are written.  Targets without pairs get zeros.  On
@@ -301,7 +322,7 @@ __global__ void __launch_bounds__(kPpThreads) k_pp_fill(PpArgs a, const uint32_t
 // four ordered parts; otherwise (k_pp_reduce_seq) a group of threads per target in slot
 // order, lanes over columns.
 constexpr int kRedParts = 4;  // slot-range parts per (target, column group)
-__global__ void __launch_bounds__(256) k_pp_reduce_f4(int D, int ld, int stride, int width,
+__device__ __forceinline__ void k_pp_reduce_f4_body(const BlockId& blk, int D, int ld, int stride, int width,
                                                        const LevelInfo* linfo,
                                                        const M2lPairHdr* hdr, const int* tbase,
                                                        const int* __restrict__ tpair,
@@ -324,7 +345,7 @@ __global__ void __launch_bounds__(256) k_pp_reduce_f4(int D, int ld, int stride,
     odd.y = (coef_degree(4 * u + 1) & 1) ? 0x80000000u : 0u;
     odd.z = (coef_degree(4 * u + 2) & 1) ? 0x80000000u : 0u;
     odd.w = (coef_degree(4 * u + 3) & 1) ? 0x80000000u : 0u;
-    for (int t = blockIdx.x; t < nt; t += gridDim.x) {
+    for (int t = (int)blk.x; t < nt; t += (int)blk.nx) {
         const int b0 = tbase[t], b1 = over ? b0 : tbase[t + 1];
         const int cs = (b1 - b0 + kRedParts - 1) / kRedParts;
         const int s0 = min(b0 + j * cs, b1), s1 = min(s0 + cs, b1);
@@ -365,6 +386,13 @@ __global__ void __launch_bounds__(256) k_pp_reduce_f4(int D, int ld, int stride,
         }
         __syncthreads();
     }
+}
+__global__ void __launch_bounds__(256) k_pp_reduce_f4(int D, int ld, int stride, int width,
+                                                       const LevelInfo* linfo,
+                                                       const M2lPairHdr* hdr, const int* tbase,
+                                                       const int* __restrict__ tpair,
+                                                       const float4* __restrict__ part, float* L) {
+    k_pp_reduce_f4_body(solo_block(), D, ld, stride, width, linfo, hdr, tbase, tpair, part, L);
 }
 
 // FP64 rows (ld and stride multiples of 4): a block per target, 4 x ld / 4
@@ -887,6 +915,32 @@ cudaError_t m2l_pairs_stats(const Workspace& ws, int64_t* out, cudaStream_t s) {
     out[2] = h.n_items;
     out[3] = h.n_pairs;
     return cudaSuccess;
+}
+
+// Joined ensemble launches (join.cuh).
+struct PpCountJoin {
+    template <class... A>
+    __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const { k_pp_count_body(b, a...); }
+};
+struct PpScanJoin {
+    template <class... A>
+    __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const { k_pp_scan_body(b, a...); }
+};
+struct PpFillJoin {
+    template <class... A>
+    __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const { k_pp_fill_body(b, a...); }
+};
+struct PpReduceJoin {
+    template <class... A>
+    __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const { k_pp_reduce_f4_body(b, a...); }
+};
+
+cudaError_t join_pairs(JoinCtx& c) {
+    cudaError_t e = join_kernel<PpCountJoin, kPpThreads, 1>(c, k_pp_count);
+    if (e == cudaSuccess) e = join_kernel<PpScanJoin, kPpScanThreads, 3>(c, k_pp_scan);
+    if (e == cudaSuccess) e = join_kernel<PpFillJoin, kPpThreads, 1>(c, k_pp_fill);
+    if (e == cudaSuccess) e = join_kernel<PpReduceJoin, 256, 4>(c, k_pp_reduce_f4);
+    return e;
 }
 
 }  // namespace pt

@@ -14,6 +14,7 @@
 
 #include "bbox.cuh"
 #include "internal.h"
+#include "join.cuh"
 #include "rng.cuh"
 
 namespace pt {
@@ -121,7 +122,7 @@ __device__ __forceinline__ void gyrate(const PushParams& pp, double& x, double& 
 
 // First half-drift of a step, fused with the bounding cube of the midpoint
 // positions; the finalising thread also advances the step counter.
-__global__ void __launch_bounds__(kBboxThreads) k_drift_bbox(int64_t n, int64_t per, double* x,
+__device__ __forceinline__ void k_drift_bbox_body(const BlockId& blk, int64_t n, int64_t per, double* x,
                                                              double* y, double* z, double* vx,
                                                              double* vy, const double* vz,
                                                              PushParams pp,
@@ -129,7 +130,7 @@ __global__ void __launch_bounds__(kBboxThreads) k_drift_bbox(int64_t n, int64_t 
                                                              unsigned* ticket, RootCube* root,
                                                              int* err, StepCounter* steps) {
     BboxAcc t;
-    const int64_t i0 = blockIdx.x * per, i1 = min(n, i0 + per);
+    const int64_t i0 = (int)blk.x * per, i1 = min(n, i0 + per);
     for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
         double px = x[i], py = y[i], pz = z[i], ux = vx[i], uy = vy[i];
         gyrate(pp, px, py, pz, ux, uy, vz[i]);
@@ -140,10 +141,19 @@ __global__ void __launch_bounds__(kBboxThreads) k_drift_bbox(int64_t n, int64_t 
         vy[i] = uy;
         t.add(px, py, pz);
     }
-    if (bbox_commit(t, acc, ticket, root, err)) {
+    if (bbox_commit(t, blk.nx, acc, ticket, root, err)) {
         steps->cur = steps->next;
         steps->next = steps->next + 1;
     }
+}
+__global__ void __launch_bounds__(kBboxThreads) k_drift_bbox(int64_t n, int64_t per, double* x,
+                                                             double* y, double* z, double* vx,
+                                                             double* vy, const double* vz,
+                                                             PushParams pp,
+                                                             unsigned long long* acc,
+                                                             unsigned* ticket, RootCube* root,
+                                                             int* err, StepCounter* steps) {
+    k_drift_bbox_body(solo_block(), n, per, x, y, z, vx, vy, vz, pp, acc, ticket, root, err, steps);
 }
 
 // Kick (Eq. velocity_kick with the laser kicks of Eq. laser_kick) and the
@@ -155,9 +165,8 @@ __global__ void __launch_bounds__(kBboxThreads) k_drift_bbox(int64_t n, int64_t 
 // beams in order, kicks and drifts, exactly the sequence of laser_ion.
 constexpr int kKickIons = 128;
 constexpr int kKickThreads = 256;
-__global__ void __launch_bounds__(kKickThreads) k_kick_drift(
-    int64_t n, int64_t per, double* x, double* y, double* z, double* vx, double* vy, double* vz,
-    const double* __restrict__ q, const double* __restrict__ E, PushParams pp, pt_laser laser,
+__device__ __forceinline__ void k_kick_drift_body(const BlockId& blk, int64_t n, int64_t per, double* x, double* y, double* z, double* vx, double* vy, double* vz,
+    const double* __restrict__ q, const double* __restrict__ E, const PushParams& pp, const pt_laser& laser,
     const StepCounter* steps, const double* __restrict__ wall_cs) {
     pdl_wait();
     __shared__ int s_cnt[PT_MAX_BEAMS][kKickIons];
@@ -167,7 +176,7 @@ __global__ void __launch_bounds__(kKickThreads) k_kick_drift(
     const int64_t widx = step - steps->base;
     const double c = wall_cs[2 * widx], s = wall_cs[2 * widx + 1];
     const double kw = 0.5 * pp.kz * pp.delta;
-    const int64_t b0 = blockIdx.x * per, b1 = min(n, b0 + per);
+    const int64_t b0 = (int)blk.x * per, b1 = min(n, b0 + per);
     for (int64_t r0 = b0; r0 < b1; r0 += kKickIons) {
         const int nr = (int)min((int64_t)kKickIons, b1 - r0);
         if (lasers) {
@@ -212,6 +221,11 @@ __global__ void __launch_bounds__(kKickThreads) k_kick_drift(
         }
         if (lasers) __syncthreads();  // s_cnt is rewritten for the next run
     }
+}
+__global__ void __launch_bounds__(kKickThreads) k_kick_drift(int64_t n, int64_t per, double* x, double* y, double* z, double* vx, double* vy, double* vz,
+    const double* __restrict__ q, const double* __restrict__ E, const __grid_constant__ PushParams pp, const __grid_constant__ pt_laser laser,
+    const StepCounter* steps, const double* __restrict__ wall_cs) {
+    k_kick_drift_body(solo_block(), n, per, x, y, z, vx, vy, vz, q, E, pp, laser, steps, wall_cs);
 }
 
 __global__ void k_laser_kicks(pt_laser laser, double rk, int64_t n, const double* x,
@@ -400,6 +414,22 @@ cudaError_t launch_rms_displacement(int64_t n, const double* acc, int64_t sample
                                     cudaStream_t s) {
     k_rms_displacement<<<grid_for(n, 256), 256, 0, s>>>(n, acc, 1.0 / (double)samples, out);
     return cudaGetLastError();
+}
+
+// Joined ensemble launches (join.cuh).
+struct DriftJoin {
+    template <class... A>
+    __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const { k_drift_bbox_body(b, a...); }
+};
+struct KickJoin {
+    template <class... A>
+    __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const { k_kick_drift_body(b, a...); }
+};
+
+cudaError_t join_push(JoinCtx& c) {
+    cudaError_t e = join_kernel<DriftJoin, kBboxThreads, 9>(c, k_drift_bbox);
+    if (e == cudaSuccess) e = join_kernel<KickJoin, kKickThreads, 2>(c, k_kick_drift);
+    return e;
 }
 
 }  // namespace pt

@@ -17,6 +17,7 @@
 
 #include "harmonics.cuh"
 #include "internal.h"
+#include "join.cuh"
 #include "bbox.cuh"
 
 namespace pt {
@@ -45,7 +46,7 @@ __global__ void __launch_bounds__(kBboxThreads) k_bbox(const double* __restrict_
     BboxAcc t;
     const int64_t i0 = blockIdx.x * per, i1 = min(n, i0 + per);
     for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) t.add(x[i], y[i], z[i]);
-    bbox_commit(t, acc, ticket, root, err);
+    bbox_commit(t, gridDim.x, acc, ticket, root, err);
 }
 
 cudaError_t launch_bbox(const double* x, const double* y, const double* z, int64_t n,
@@ -67,14 +68,14 @@ __device__ __forceinline__ int leaf_coord(double v, double lo, double side, doub
     return (int)f;
 }
 
-__global__ void k_keys(const double* __restrict__ x, const double* __restrict__ y,
+__device__ __forceinline__ void k_keys_body(const BlockId& blk, const double* __restrict__ x, const double* __restrict__ y,
                        const double* __restrict__ z, int64_t n, int64_t per, int D,
                        const RootCube* root, uint32_t* key, uint32_t* rank, int32_t* leaf_count) {
     pdl_wait();
     const double lo0 = root->lo[0], lo1 = root->lo[1], lo2 = root->lo[2], side = root->side;
     const double scale = (double)(1 << D);
     const int m = (1 << D) - 1;
-    const int64_t i0 = blockIdx.x * per, i1 = min(n, i0 + per);
+    const int64_t i0 = (int)blk.x * per, i1 = min(n, i0 + per);
     for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
         uint32_t k = morton3(leaf_coord(x[i], lo0, side, scale, m),
                              leaf_coord(y[i], lo1, side, scale, m),
@@ -82,6 +83,11 @@ __global__ void k_keys(const double* __restrict__ x, const double* __restrict__ 
         key[i] = k;
         rank[i] = (uint32_t)atomicAdd(&leaf_count[k], 1);
     }
+}
+__global__ void k_keys(const double* __restrict__ x, const double* __restrict__ y,
+                       const double* __restrict__ z, int64_t n, int64_t per, int D,
+                       const RootCube* root, uint32_t* key, uint32_t* rank, int32_t* leaf_count) {
+    k_keys_body(solo_block(), x, y, z, n, per, D, root, key, rank, leaf_count);
 }
 
 // ---------------------------------------------------------------------------
@@ -286,13 +292,18 @@ __device__ __forceinline__ void scan_cluster_body(const Src& src, int64_t total,
 }
 
 template <class SrcA, class SrcB>
-__global__ void __launch_bounds__(kScanCtaThreads) k_scan_cluster2(SrcA a, int64_t total_a, SrcB b,
+__device__ __forceinline__ void k_scan_cluster2_body(const BlockId& blk, SrcA a, int64_t total_a, SrcB b,
                                                                   int64_t total_b) {
     __shared__ int warp_tot[kScanCtaThreads / 32];
     __shared__ int cta_tot, s_tot[kScanCtas];
     pdl_wait();
     scan_cluster_body(a, total_a, warp_tot, &cta_tot, s_tot);
     scan_cluster_body(b, total_b, warp_tot, &cta_tot, s_tot);
+}
+template <class SrcA, class SrcB>
+__global__ void __launch_bounds__(kScanCtaThreads) k_scan_cluster2(SrcA a, int64_t total_a, SrcB b,
+                                                                  int64_t total_b) {
+    k_scan_cluster2_body<SrcA, SrcB>(solo_block(), a, total_a, b, total_b);
 }
 
 // a cluster launch of kScanCtas CTAs, programmatic (see launch_pdl)
@@ -414,12 +425,16 @@ struct CellCompaction {
 // ---------------------------------------------------------------------------
 // 4./6. scatter and per-leaf ordering + gather
 // ---------------------------------------------------------------------------
-__global__ void k_scatter(const uint32_t* __restrict__ key, const uint32_t* __restrict__ rank,
+__device__ __forceinline__ void k_scatter_body(const BlockId& blk, const uint32_t* __restrict__ key, const uint32_t* __restrict__ rank,
                           const int32_t* __restrict__ leaf_start, int64_t n, int32_t* perm_tmp) {
     pdl_wait();
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
+    for (int64_t i = (int)blk.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)(int)blk.nx * blockDim.x)
         perm_tmp[leaf_start[key[i]] + rank[i]] = (int32_t)i;
+}
+__global__ void k_scatter(const uint32_t* __restrict__ key, const uint32_t* __restrict__ rank,
+                          const int32_t* __restrict__ leaf_start, int64_t n, int32_t* perm_tmp) {
+    k_scatter_body(solo_block(), key, rank, leaf_start, n, perm_tmp);
 }
 
 // Sorted ion record: FP64 path (u_x, u_y, u_z, q) in double; FP32 paths
@@ -448,7 +463,7 @@ __device__ __forceinline__ double4_32a make4<double4_32a>(double a, double b, do
 // of k_keys); the leaf's ions are read from the few cache lines the
 // neighbouring threads share.
 template <typename T4>
-__global__ void k_leaf_gather(const double* __restrict__ x, const double* __restrict__ y,
+__device__ __forceinline__ void k_leaf_gather_body(const BlockId& blk, const double* __restrict__ x, const double* __restrict__ y,
                               const double* __restrict__ z, const double* __restrict__ q, int64_t n,
                               int64_t per, int D, const RootCube* root,
                               const uint32_t* __restrict__ key,
@@ -459,7 +474,7 @@ __global__ void k_leaf_gather(const double* __restrict__ x, const double* __rest
     pdl_wait();
     const double lo0 = root->lo[0], lo1 = root->lo[1], lo2 = root->lo[2], side = root->side;
     const double scale = (double)(1 << D);
-    const int64_t i0 = blockIdx.x * per, i1 = min(n, i0 + per);
+    const int64_t i0 = (int)blk.x * per, i1 = min(n, i0 + per);
     for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
         const int idx = perm_tmp[i];
         const uint32_t c = key[idx];
@@ -477,6 +492,17 @@ __global__ void k_leaf_gather(const double* __restrict__ x, const double* __rest
         const double uz = (z[idx] - lo2) / side * scale - (iz + 0.5);
         sorted[slot] = make4<T4>(ux, uy, uz, q[idx]);
     }
+}
+template <typename T4>
+__global__ void k_leaf_gather(const double* __restrict__ x, const double* __restrict__ y,
+                              const double* __restrict__ z, const double* __restrict__ q, int64_t n,
+                              int64_t per, int D, const RootCube* root,
+                              const uint32_t* __restrict__ key,
+                              const int32_t* __restrict__ leaf_start,
+                              const int32_t* __restrict__ cid_leaf,
+                              const int32_t* __restrict__ perm_tmp, int32_t* perm,
+                              int32_t* slot_of, int32_t* leaf_of, T4* sorted) {
+    k_leaf_gather_body<T4>(solo_block(), x, y, z, q, n, per, D, root, key, leaf_start, cid_leaf, perm_tmp, perm, slot_of, leaf_of, sorted);
 }
 
 cudaError_t launch_tree(int64_t n, const double* x, const double* y, const double* z,
@@ -580,6 +606,42 @@ cudaError_t launch_level_counts(int64_t n, const double* x, const double* y, con
                              cudaMemcpyDeviceToHost, s)) != cudaSuccess)
         return e;
     return cudaStreamSynchronize(s);
+}
+
+// ---------------------------------------------------------------------------
+// Joined ensemble launches (join.cuh).
+// ---------------------------------------------------------------------------
+struct KeysJoin {
+    template <class... A>
+    __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const { k_keys_body(b, a...); }
+};
+struct ScanJoin {
+    template <class... A>
+    __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const {
+        k_scan_cluster2_body<LeafCountScan, CellCompaction>(b, a...);
+    }
+};
+struct ScatterJoin {
+    template <class... A>
+    __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const { k_scatter_body(b, a...); }
+};
+template <typename T4>
+struct GatherJoin {
+    template <class... A>
+    __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const {
+        k_leaf_gather_body<T4>(b, a...);
+    }
+};
+
+cudaError_t join_tree(JoinCtx& c) {
+    cudaError_t e = join_kernel<KeysJoin, 128, 8>(c, k_keys);
+    if (e == cudaSuccess)
+        e = join_kernel<ScanJoin, kScanCtaThreads, 0>(c, k_scan_cluster2<LeafCountScan, CellCompaction>,
+                                                      kScanCtas);
+    if (e == cudaSuccess) e = join_kernel<ScatterJoin, 256, 4>(c, k_scatter);
+    if (e == cudaSuccess) e = join_kernel<GatherJoin<int4>, 128, 12>(c, k_leaf_gather<int4>);
+    if (e == cudaSuccess) e = join_kernel<GatherJoin<double4_32a>, 128, 12>(c, k_leaf_gather<double4_32a>);
+    return e;
 }
 
 }  // namespace pt
