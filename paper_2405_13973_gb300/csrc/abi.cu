@@ -75,6 +75,7 @@ struct fmm_plan_s {
     cudaGraphExec_t graph = nullptr;
     GraphKey gkey;
     int* h_err = nullptr;      // pinned
+    int32_t* h_counts = nullptr;  // pinned: cells per level (kMaxDepth + 1, after h_err)
     // pinned host ring for the per-chunk wall-phase tables and step counters
     // (asynchronous steps may have several chunks in flight)
     static constexpr int kSlots = 8;
@@ -192,7 +193,7 @@ void free_plan(fmm_plan_s* pl) {
     Workspace& ws = pl->ws;
     if (ws.side) cudaStreamDestroy(ws.side);
     if (ws.side2) cudaStreamDestroy(ws.side2);
-    for (cudaEvent_t ev : {ws.ev_fork, ws.ev_p2m, ws.ev_items, ws.ev_near})
+    for (cudaEvent_t ev : {ws.ev_fork, ws.ev_p2m, ws.ev_items, ws.ev_near, ws.ev_drift, ws.ev_photons})
         if (ev) cudaEventDestroy(ev);
     for (int k = 0; k < fmm_plan_s::kSlots; ++k) {
         if (pl->h_wall[k]) cudaFreeHost(pl->h_wall[k]);
@@ -397,7 +398,7 @@ int choose_depth(fmm_plan_s* pl, int64_t n, const double* x, const double* y, co
         *D = pl->depth;
         return PT_OK;
     }
-    int32_t counts[kMaxDepth + 1] = {0};
+    int32_t* counts = pl->h_counts;
     cudaError_t e = launch_level_counts(n, x, y, z, pl->ws.depth_max, pl->ws, counts, s);
     if (e != cudaSuccess) return status_from(e);
     int r = check_err(pl, s);
@@ -550,8 +551,13 @@ int forces_impl(fmm_plan_s* pl, int64_t n, const double* x, const double* y, con
     if (r != PT_OK) return r;
     // with profiling on, the M2L and near-field kernels are timed as in a step
     for (int k = 0; k < 4; ++k) pl->ws.kev[k] = pl->profile ? pl->k_ev[k] : nullptr;
-    cudaError_t e = launch_bbox(x, y, z, n, pl->ws, s);
-    if (e == cudaSuccess) e = launch_tree(n, x, y, z, q, D, pl->ws, s);
+    cudaError_t e = cudaSuccess;
+    if (small_tree_fits(n, D)) {
+        e = launch_small_tree(n, x, y, z, q, D, pl->ws, s);
+    } else {
+        e = launch_bbox(x, y, z, n, pl->ws, s);
+        if (e == cudaSuccess) e = launch_tree(n, x, y, z, q, D, pl->ws, s);
+    }
     if (e == cudaSuccess)
         e = launch_fmm(n, D, pl->phases, pl->ws, is_tc(pl->precision), E, phi, s);
     for (int k = 0; k < 4; ++k) pl->ws.kev[k] = nullptr;
@@ -562,8 +568,10 @@ int forces_impl(fmm_plan_s* pl, int64_t n, const double* x, const double* y, con
 
 // One time step: drift + cube, tree, FMM, kick + drift.  With profiling on,
 // event records between the phases are captured too.
+// alone: not a member of an ensemble (whose launches are joined kernel by
+// kernel instead).
 cudaError_t enqueue_step(fmm_plan_s* pl, const pt_state& st, const PushParams& pp,
-                         const pt_laser& laser, int D, cudaStream_t s) {
+                         const pt_laser& laser, int D, bool alone, cudaStream_t s) {
     Workspace& ws = pl->ws;
     const int64_t n = st.n;
     for (int k = 0; k < 4; ++k) ws.kev[k] = pl->profile ? pl->k_ev[k] : nullptr;
@@ -572,15 +580,30 @@ cudaError_t enqueue_step(fmm_plan_s* pl, const pt_state& st, const PushParams& p
                            : cudaSuccess;
     };
     cudaError_t e = mark(0);
-    if (e == cudaSuccess) e = launch_drift_bbox(n, st.x, st.y, st.z, st.vx, st.vy, st.vz, pp, ws, s);
+    // profiling times the drift apart from the tree
+    const bool front = alone && !pl->profile && small_tree_fits(n, D);
+    if (e == cudaSuccess)
+        e = front ? launch_small_front(n, st.x, st.y, st.z, st.vx, st.vy, st.vz, st.q, pp, D, ws, s)
+                  : launch_drift_bbox(n, st.x, st.y, st.z, st.vx, st.vy, st.vz, pp, ws, s);
+    // the photon kicks run on a side stream up to the kick
+    const bool lasers = laser.enabled && laser.n_beams > 0;
+    if (lasers) {
+        if (e == cudaSuccess) e = cudaEventRecord(ws.ev_drift, s);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(ws.side2, ws.ev_drift, 0);
+        if (e == cudaSuccess)
+            e = launch_photons(n, st.y, st.z, st.vx, st.vy, st.vz, pp, laser, ws, ws.side2);
+        if (e == cudaSuccess) e = cudaEventRecord(ws.ev_photons, ws.side2);
+    }
     if (e == cudaSuccess) e = mark(1);
-    if (e == cudaSuccess) e = launch_tree(n, st.x, st.y, st.z, st.q, D, ws, s);
+    if (e == cudaSuccess && !front) e = launch_tree(n, st.x, st.y, st.z, st.q, D, ws, s);
     if (e == cudaSuccess) e = mark(2);
     if (e == cudaSuccess)
         e = launch_fmm_phased(n, D, PT_PHASE_ALL, ws, is_tc(pl->precision), ws.E,
                               nullptr, s, pl->profile ? pl->ph_ev + 3 : nullptr);
+    if (lasers && e == cudaSuccess) e = cudaStreamWaitEvent(s, ws.ev_photons, 0);
     if (e == cudaSuccess)
-        e = launch_kick_drift(n, st.x, st.y, st.z, st.vx, st.vy, st.vz, st.q, ws.E, pp, laser, ws, s);
+        e = launch_kick_drift(n, st.x, st.y, st.z, st.vx, st.vy, st.vz, st.q, ws.E, pp,
+                              lasers ? ws.dv : nullptr, ws, s);
     if (e == cudaSuccess) e = mark(6);
     for (int k = 0; k < 4; ++k) ws.kev[k] = nullptr;
     return e;
@@ -718,7 +741,7 @@ int step_impl(fmm_plan_s* plan, pt_state* st, const pt_trap* trap, const pt_lase
             cudaGraph_t g = nullptr;
             e = cudaStreamBeginCapture(plan->cap_stream, cudaStreamCaptureModeThreadLocal);
             if (e != cudaSuccess) return status_from(e);
-            cudaError_t e2 = enqueue_step(plan, *st, pp, lz, D, plan->cap_stream);
+            cudaError_t e2 = enqueue_step(plan, *st, pp, lz, D, true, plan->cap_stream);
             e = cudaStreamEndCapture(plan->cap_stream, &g);
             if (e2 != cudaSuccess || e != cudaSuccess) {
                 if (g) cudaGraphDestroy(g);
@@ -999,6 +1022,7 @@ static int plan_create_impl(int64_t n_max, int p, int leaf_max, int depth, int p
          dalloc(pl, ws.cstart, sizeof(int32_t) * cells) && dalloc(pl, ws.ccount, sizeof(int32_t) * cells) &&
          dalloc(pl, ws.linfo, sizeof(LevelInfo)) && dalloc(pl, ws.M, tsz * ws.ld * cells) &&
          dalloc(pl, ws.L, tsz * ws.ld * cells) && dalloc(pl, ws.E, sizeof(double) * 3 * n_max) &&
+         dalloc(pl, ws.dv, sizeof(double) * 3 * n_max) &&
          dalloc(pl, ws.near, tsz * 4 * n_max) &&
          dalloc(pl, ws.block_sums, sizeof(int32_t) * ws.block_sums_cap) &&
          dalloc(pl, ws.root, sizeof(RootCube)) &&
@@ -1073,17 +1097,20 @@ static int plan_create_impl(int64_t n_max, int p, int leaf_max, int depth, int p
         cudaMemset(ws.bbox_acc, 0, sizeof(unsigned long long) * 8) != cudaSuccess ||
         cudaMemset(ws.err, 0, sizeof(int)) != cudaSuccess ||
         cudaMemset(ws.steps, 0, sizeof(StepCounter)) != cudaSuccess ||
-        cudaMallocHost(&pl->h_err, sizeof(int)) != cudaSuccess ||
+        cudaMallocHost(&pl->h_err, sizeof(int) * (2 + kMaxDepth)) != cudaSuccess ||
         cudaStreamCreateWithPriority(&pl->cap_stream, cudaStreamNonBlocking, prio_high()) != cudaSuccess ||
         cudaStreamCreateWithPriority(&ws.side, cudaStreamNonBlocking, prio_low()) != cudaSuccess ||
         cudaStreamCreateWithPriority(&ws.side2, cudaStreamNonBlocking, prio_low()) != cudaSuccess ||
         cudaEventCreateWithFlags(&ws.ev_fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&ws.ev_p2m, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&ws.ev_items, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ws.ev_near, cudaEventDisableTiming) != cudaSuccess) {
+        cudaEventCreateWithFlags(&ws.ev_near, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ws.ev_drift, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ws.ev_photons, cudaEventDisableTiming) != cudaSuccess) {
         free_plan(pl);
         return PT_ERR_CUDA;
     }
+    pl->h_counts = pl->h_err + 1;
     for (int k = 0; k < fmm_plan_s::kSlots; ++k) {
         if (cudaMallocHost(&pl->h_wall[k], sizeof(double) * 2 * ws.wall_cap) != cudaSuccess ||
             cudaMallocHost(&pl->h_steps[k], sizeof(StepCounter)) != cudaSuccess ||
@@ -1398,7 +1425,7 @@ int pt_ensemble_step(pt_ensemble ens, pt_state* states, const pt_trap* traps,
             for (int b = 0; e2 == cudaSuccess && b < nm; ++b) {
                 e2 = cudaStreamWaitEvent(ens->br[b], ens->fork, 0);
                 if (e2 == cudaSuccess)
-                    e2 = enqueue_step(ens->plans[b], states[b], pp[b], lz[b], D[b], ens->br[b]);
+                    e2 = enqueue_step(ens->plans[b], states[b], pp[b], lz[b], D[b], false, ens->br[b]);
                 if (e2 == cudaSuccess) e2 = cudaEventRecord(ens->join[b], ens->br[b]);
                 if (e2 == cudaSuccess) e2 = cudaStreamWaitEvent(ens->cap, ens->join[b], 0);
             }

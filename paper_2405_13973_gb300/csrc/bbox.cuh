@@ -53,6 +53,33 @@ struct BboxAcc {
     }
 };
 
+// the root cube of the reduced words; a non-finite position is latched in err
+__device__ __forceinline__ void root_of_words(const unsigned long long (&v)[7], RootCube* root,
+                                              int* err) {
+    double u[3], hi[3];
+    for (int a = 0; a < 3; ++a) {
+        u[a] = ord_val(~v[a]);
+        hi[a] = ord_val(v[3 + a]);
+    }
+    const bool b = v[6] != 0ull;
+    if (v[0] == 0ull)  // no point at all: the unit cube at the origin
+        for (int a = 0; a < 3; ++a) u[a] = hi[a] = 0.0;
+    double side = 0.0;
+    for (int a = 0; a < 3; ++a) {
+        double e = __dsub_rn(hi[a], u[a]);
+        if (e > side) side = e;
+    }
+    if (!(side > 0.0)) side = 1.0;
+    if (b || !isfinite(side)) {
+        atomicOr(err, ERR_NONFINITE);
+        side = 1.0;
+        for (int a = 0; a < 3; ++a) u[a] = hi[a] = 0.0;
+    }
+    for (int a = 0; a < 3; ++a)
+        root->lo[a] = __dsub_rn(__dmul_rn(0.5, __dadd_rn(u[a], hi[a])), __dmul_rn(0.5, side));
+    root->side = side;
+}
+
 // Folds every thread's extremes into acc[] (all threads of the `blocks`
 // blocks call it); the last block writes the root cube exactly as
 //   side = max_a (max_a - min_a) (1 if zero); lo_a = (min_a+max_a)/2 - side/2
@@ -84,28 +111,7 @@ __device__ __forceinline__ bool bbox_commit(BboxAcc& t, unsigned blocks, unsigne
     unsigned long long v[7];
 #pragma unroll
     for (int w = 0; w < 7; ++w) v[w] = atomicExch(&acc[w], 0ull);
-    double u[3], hi[3];
-    for (int a = 0; a < 3; ++a) {
-        u[a] = ord_val(~v[a]);
-        hi[a] = ord_val(v[3 + a]);
-    }
-    const bool b = v[6] != 0ull;
-    if (v[0] == 0ull)  // no point at all: the unit cube at the origin
-        for (int a = 0; a < 3; ++a) u[a] = hi[a] = 0.0;
-    double side = 0.0;
-    for (int a = 0; a < 3; ++a) {
-        double e = __dsub_rn(hi[a], u[a]);
-        if (e > side) side = e;
-    }
-    if (!(side > 0.0)) side = 1.0;
-    if (b || !isfinite(side)) {
-        atomicOr(err, ERR_NONFINITE);
-        side = 1.0;
-        for (int a = 0; a < 3; ++a) u[a] = hi[a] = 0.0;
-    }
-    for (int a = 0; a < 3; ++a)
-        root->lo[a] = __dsub_rn(__dmul_rn(0.5, __dadd_rn(u[a], hi[a])), __dmul_rn(0.5, side));
-    root->side = side;
+    root_of_words(v, root, err);
     *ticket = 0u;
     return true;
 }

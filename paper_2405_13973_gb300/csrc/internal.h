@@ -129,7 +129,9 @@ struct Workspace {
     // which overlap the main chain; events of the fork and the joins
     // (ev_p2m: when the near field may start)
     cudaStream_t side = nullptr;
-    cudaStream_t side2 = nullptr;  // the near field of the tensor-core paths
+    cudaStream_t side2 = nullptr;  // the photon kicks, then the near field of the tensor-core paths
+    double* dv = nullptr;          // [3n] recoil velocity changes of the step
+    cudaEvent_t ev_drift = nullptr, ev_photons = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_p2m = nullptr, ev_items = nullptr, ev_near = nullptr;
     int32_t* block_sums = nullptr; // scan scratch
     int64_t block_sums_cap = 0;
@@ -220,6 +222,17 @@ cudaError_t launch_bbox(const double* x, const double* y, const double* z, int64
                         Workspace& ws, cudaStream_t s);
 cudaError_t launch_tree(int64_t n, const double* x, const double* y, const double* z,
                         const double* q, int D, Workspace& ws, cudaStream_t s);
+// up to a few thousand ions: the tree (with its root cube), or a time step's
+// first half-drift, root cube and tree, in one launch
+bool small_tree_fits(int64_t n, int D);
+cudaError_t launch_small_tree(int64_t n, const double* x, const double* y, const double* z,
+                              const double* q, int D, Workspace& ws, cudaStream_t s);
+struct PushParams;
+cudaError_t launch_small_front(int64_t n, double* x, double* y, double* z, double* vx, double* vy,
+                               const double* vz, const double* q, const PushParams& pp, int D,
+                               Workspace& ws, cudaStream_t s);
+// non-empty cells of every level 0..D into host_counts (pinned; valid once s
+// is synchronised)
 cudaError_t launch_level_counts(int64_t n, const double* x, const double* y, const double* z,
                                 int D, Workspace& ws, int32_t* host_counts, cudaStream_t s);
 
@@ -373,9 +386,15 @@ cudaError_t launch_mh_scans(int64_t n, double* x, double* y, double* z, const do
 
 cudaError_t launch_drift_bbox(int64_t n, double* x, double* y, double* z, double* vx, double* vy,
                               double* vz, const PushParams& pp, Workspace& ws, cudaStream_t s);
+// recoil velocity changes of the step into ws.dv, from the state after the
+// first half-drift
+cudaError_t launch_photons(int64_t n, const double* y, const double* z, const double* vx,
+                           const double* vy, const double* vz, const PushParams& pp,
+                           const pt_laser& laser, Workspace& ws, cudaStream_t s);
+// dv: ws.dv, or null without cooling
 cudaError_t launch_kick_drift(int64_t n, double* x, double* y, double* z, double* vx, double* vy,
                               double* vz, const double* q, const double* E, const PushParams& pp,
-                              const pt_laser& laser, Workspace& ws, cudaStream_t s);
+                              const double* dv, Workspace& ws, cudaStream_t s);
 cudaError_t launch_laser_kicks(const pt_laser& laser, double rk, int64_t n, const double* x,
                                const double* y, const double* z, const double* vx,
                                const double* vy, const double* vz, int64_t step, double dt,

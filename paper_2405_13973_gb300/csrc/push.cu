@@ -13,6 +13,7 @@
 #include <cuda_runtime.h>
 
 #include "bbox.cuh"
+#include "gyrate.cuh"
 #include "internal.h"
 #include "join.cuh"
 #include "rng.cuh"
@@ -109,17 +110,6 @@ __device__ void laser_ion(const pt_laser& L, double rk, int64_t i, int64_t step,
     }
 }
 
-// Exact gyration U0(h) (Eq. U0, B along +z: clockwise velocity rotation).
-__device__ __forceinline__ void gyrate(const PushParams& pp, double& x, double& y, double& z,
-                                       double& vx, double& vy, double vz) {
-    double ux = vx, uy = vy;
-    x = x + (ux * pp.S + uy * (1.0 - pp.C)) / pp.wc;
-    y = y + (uy * pp.S - ux * (1.0 - pp.C)) / pp.wc;
-    z = z + vz * pp.h;
-    vx = ux * pp.C + uy * pp.S;
-    vy = -ux * pp.S + uy * pp.C;
-}
-
 // First half-drift of a step, fused with the bounding cube of the midpoint
 // positions; the finalising thread also advances the step counter.
 __device__ __forceinline__ void k_drift_bbox_body(const BlockId& blk, int64_t n, int64_t per, double* x,
@@ -156,76 +146,108 @@ __global__ void __launch_bounds__(kBboxThreads) k_drift_bbox(int64_t n, int64_t 
     k_drift_bbox_body(solo_block(), n, per, x, y, z, vx, vy, vz, pp, acc, ticket, root, err, steps);
 }
 
-// Kick (Eq. velocity_kick with the laser kicks of Eq. laser_kick) and the
-// second half-drift.  A block takes an equal contiguous share of the ions
-// (ion_split: FP64 is the bound, so every SM gets the same amount) in runs of
-// kKickIons: the block's threads first draw the photon counts of every
-// (beam, ion) pair of the run in parallel (the rate and Poisson draw, the
-// bulk of the FP64 work), then one thread per ion adds the recoils of the
-// beams in order, kicks and drifts, exactly the sequence of laser_ion.
+// Photon kicks of a step (Eq. laser_kick) at its midpoint state: the recoil
+// velocity change of every ion into dv (SoA 3n).  They need the first
+// half-drift only, so they run on a side stream beside the tree and the field
+// and the kick just adds them; drawn inside the kick they were half of it
+// (14.6 us of the 10,000-ion step).  A block takes an equal contiguous share of the
+// ions (ion_split: FP64 is the bound, so every SM gets the same amount) in
+// runs of kKickIons: the threads first draw the photon counts of every (beam,
+// ion) pair of the run in parallel (the rate and Poisson draw, the bulk of
+// the FP64 work), then one thread per ion adds the recoils of the beams in
+// order, exactly the sequence of laser_ion.
 constexpr int kKickIons = 128;
 constexpr int kKickThreads = 256;
-__device__ __forceinline__ void k_kick_drift_body(const BlockId& blk, int64_t n, int64_t per, double* x, double* y, double* z, double* vx, double* vy, double* vz,
-    const double* __restrict__ q, const double* __restrict__ E, const PushParams& pp, const pt_laser& laser,
-    const StepCounter* steps, const double* __restrict__ wall_cs) {
-    pdl_wait();
+__device__ __forceinline__ void k_photons_body(const BlockId& blk, int64_t n, int64_t per,
+                                               const double* y, const double* z, const double* vx,
+                                               const double* vy, const double* vz, double rk,
+                                               double dt, const pt_laser& laser,
+                                               const StepCounter* steps, double* dv) {
     __shared__ int s_cnt[PT_MAX_BEAMS][kKickIons];
-    const bool lasers = laser.enabled && laser.n_beams > 0;
-    const int nb = lasers ? laser.n_beams : 0;
+    const int nb = laser.n_beams;
     const int64_t step = steps->cur;
-    const int64_t widx = step - steps->base;
-    const double c = wall_cs[2 * widx], s = wall_cs[2 * widx + 1];
-    const double kw = 0.5 * pp.kz * pp.delta;
-    const int64_t b0 = (int)blk.x * per, b1 = min(n, b0 + per);
+    const int64_t b0 = blk.x * per, b1 = min(n, b0 + per);
     for (int64_t r0 = b0; r0 < b1; r0 += kKickIons) {
         const int nr = (int)min((int64_t)kKickIons, b1 - r0);
-        if (lasers) {
-            for (int j = threadIdx.x; j < nb * nr; j += kKickThreads) {
-                const int l = j / nr, k = j - l * nr;
-                const int64_t i = r0 + k;
-                s_cnt[l][k] = beam_count(laser, i, step, pp.dt, l, y[i], z[i], vx[i], vy[i], vz[i]);
-            }
-            __syncthreads();
+        for (int j = threadIdx.x; j < nb * nr; j += kKickThreads) {
+            const int l = j / nr, k = j - l * nr;
+            const int64_t i = r0 + k;
+            s_cnt[l][k] = beam_count(laser, i, step, dt, l, y[i], z[i], vx[i], vy[i], vz[i]);
         }
+        __syncthreads();
         for (int k = threadIdx.x; k < nr; k += kKickThreads) {
             const int64_t i = r0 + k;
-            double px = x[i], py = y[i], pz = z[i], ux = vx[i], uy = vy[i], uz = vz[i];
-            double etx = 0.5 * pp.kz * px, ety = 0.5 * pp.kz * py, etz = -pp.kz * pz;
-            double ewx = -kw * (px * c - py * s);
-            double ewy = -kw * (-py * c - px * s);
-            double Fx = etx + ewx, Fy = ety + ewy, Fz = etz;
             double dx = 0.0, dy = 0.0, dz = 0.0;
             for (int l = 0; l < nb; ++l) {
                 const int cnt = s_cnt[l][k];
-                if (cnt != 0) beam_recoil(laser, pp.rk, i, step, l, cnt, dx, dy, dz);
+                if (cnt != 0) beam_recoil(laser, rk, i, step, l, cnt, dx, dy, dz);
             }
-            double qm = q[i] / pp.mass;
-            ux = ux + qm * (E[i] + Fx) * pp.dt + dx;
-            uy = uy + qm * (E[n + i] + Fy) * pp.dt + dy;
-            uz = uz + qm * (E[2 * n + i] + Fz) * pp.dt + dz;
-            if (pp.damp != 1.0) {
-                // artificial damping: the velocity relative to the rigid rotation
-                // at this (mid-step) position shrinks by exp(-gamma dt)
-                const double rx = pp.wr * py, ry = -pp.wr * px;
-                ux = rx + pp.damp * (ux - rx);
-                uy = ry + pp.damp * (uy - ry);
-                uz = pp.damp * uz;
-            }
-            gyrate(pp, px, py, pz, ux, uy, uz);
-            x[i] = px;
-            y[i] = py;
-            z[i] = pz;
-            vx[i] = ux;
-            vy[i] = uy;
-            vz[i] = uz;
+            dv[i] = dx;
+            dv[n + i] = dy;
+            dv[2 * n + i] = dz;
         }
-        if (lasers) __syncthreads();  // s_cnt is rewritten for the next run
+        __syncthreads();  // s_cnt is rewritten for the next run
     }
 }
-__global__ void __launch_bounds__(kKickThreads) k_kick_drift(int64_t n, int64_t per, double* x, double* y, double* z, double* vx, double* vy, double* vz,
-    const double* __restrict__ q, const double* __restrict__ E, const __grid_constant__ PushParams pp, const __grid_constant__ pt_laser laser,
-    const StepCounter* steps, const double* __restrict__ wall_cs) {
-    k_kick_drift_body(solo_block(), n, per, x, y, z, vx, vy, vz, q, E, pp, laser, steps, wall_cs);
+__global__ void __launch_bounds__(kKickThreads) k_photons(int64_t n, int64_t per, const double* y,
+                                                          const double* z, const double* vx,
+                                                          const double* vy, const double* vz, double rk,
+                                                          double dt,
+                                                          const __grid_constant__ pt_laser laser,
+                                                          const StepCounter* steps, double* dv) {
+    k_photons_body(solo_block(), n, per, y, z, vx, vy, vz, rk, dt, laser, steps, dv);
+}
+
+// Kick (Eq. velocity_kick with the laser kicks dv, null without cooling) and
+// the second half-drift; a block an equal contiguous share of the ions.
+__device__ __forceinline__ void k_kick_drift_body(
+    const BlockId& blk, int64_t n, int64_t per, double* x, double* y, double* z, double* vx,
+    double* vy, double* vz, const double* __restrict__ q, const double* __restrict__ E,
+    const PushParams& pp, const double* __restrict__ dv, const StepCounter* steps,
+    const double* __restrict__ wall_cs) {
+    pdl_wait();
+    const int64_t widx = steps->cur - steps->base;
+    const double c = wall_cs[2 * widx], s = wall_cs[2 * widx + 1];
+    const double kw = 0.5 * pp.kz * pp.delta;
+    const int64_t b0 = blk.x * per, b1 = min(n, b0 + per);
+    for (int64_t i = b0 + threadIdx.x; i < b1; i += kKickIons) {
+        double px = x[i], py = y[i], pz = z[i], ux = vx[i], uy = vy[i], uz = vz[i];
+        double etx = 0.5 * pp.kz * px, ety = 0.5 * pp.kz * py, etz = -pp.kz * pz;
+        double ewx = -kw * (px * c - py * s);
+        double ewy = -kw * (-py * c - px * s);
+        double Fx = etx + ewx, Fy = ety + ewy, Fz = etz;
+        double dx = 0.0, dy = 0.0, dz = 0.0;
+        if (dv) {
+            dx = dv[i];
+            dy = dv[n + i];
+            dz = dv[2 * n + i];
+        }
+        double qm = q[i] / pp.mass;
+        ux = ux + qm * (E[i] + Fx) * pp.dt + dx;
+        uy = uy + qm * (E[n + i] + Fy) * pp.dt + dy;
+        uz = uz + qm * (E[2 * n + i] + Fz) * pp.dt + dz;
+        if (pp.damp != 1.0) {
+            // artificial damping: the velocity relative to the rigid rotation
+            // at this (mid-step) position shrinks by exp(-gamma dt)
+            const double rx = pp.wr * py, ry = -pp.wr * px;
+            ux = rx + pp.damp * (ux - rx);
+            uy = ry + pp.damp * (uy - ry);
+            uz = pp.damp * uz;
+        }
+        gyrate(pp, px, py, pz, ux, uy, uz);
+        x[i] = px;
+        y[i] = py;
+        z[i] = pz;
+        vx[i] = ux;
+        vy[i] = uy;
+        vz[i] = uz;
+    }
+}
+__global__ void __launch_bounds__(kKickIons) k_kick_drift(
+    int64_t n, int64_t per, double* x, double* y, double* z, double* vx, double* vy, double* vz,
+    const double* __restrict__ q, const double* __restrict__ E, const __grid_constant__ PushParams pp,
+    const double* __restrict__ dv, const StepCounter* steps, const double* __restrict__ wall_cs) {
+    k_kick_drift_body(solo_block(), n, per, x, y, z, vx, vy, vz, q, E, pp, dv, steps, wall_cs);
 }
 
 __global__ void k_laser_kicks(pt_laser laser, double rk, int64_t n, const double* x,
@@ -257,13 +279,21 @@ cudaError_t launch_drift_bbox(int64_t n, double* x, double* y, double* z, double
     return cudaGetLastError();
 }
 
+cudaError_t launch_photons(int64_t n, const double* y, const double* z, const double* vx,
+                           const double* vy, const double* vz, const PushParams& pp,
+                           const pt_laser& laser, Workspace& ws, cudaStream_t s) {
+    const IonSplit sp = ion_split(n, kKickIons, ws.sms, (int64_t)1 << 30);
+    k_photons<<<sp.grid, kKickThreads, 0, s>>>(n, sp.per, y, z, vx, vy, vz, pp.rk, pp.dt, laser,
+                                               ws.steps, ws.dv);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_kick_drift(int64_t n, double* x, double* y, double* z, double* vx, double* vy,
                               double* vz, const double* q, const double* E, const PushParams& pp,
-                              const pt_laser& laser, Workspace& ws, cudaStream_t s) {
+                              const double* dv, Workspace& ws, cudaStream_t s) {
     const IonSplit sp = ion_split(n, kKickIons, ws.sms, (int64_t)1 << 30);
-    return launch_pdl(k_kick_drift, dim3(sp.grid), dim3(kKickThreads), 0, s, n, sp.per, x, y, z, vx,
-                      vy, vz, q, E, pp, laser, (const StepCounter*)ws.steps,
-                      (const double*)ws.wall_cs);
+    return launch_pdl(k_kick_drift, dim3(sp.grid), dim3(kKickIons), 0, s, n, sp.per, x, y, z, vx,
+                      vy, vz, q, E, pp, dv, (const StepCounter*)ws.steps, (const double*)ws.wall_cs);
 }
 
 cudaError_t launch_laser_kicks(const pt_laser& laser, double rk, int64_t n, const double* x,
@@ -421,6 +451,10 @@ struct DriftJoin {
     template <class... A>
     __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const { k_drift_bbox_body(b, a...); }
 };
+struct PhotonsJoin {
+    template <class... A>
+    __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const { k_photons_body(b, a...); }
+};
 struct KickJoin {
     template <class... A>
     __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const { k_kick_drift_body(b, a...); }
@@ -428,7 +462,8 @@ struct KickJoin {
 
 cudaError_t join_push(JoinCtx& c) {
     cudaError_t e = join_kernel<DriftJoin, kBboxThreads, 9>(c, k_drift_bbox);
-    if (e == cudaSuccess) e = join_kernel<KickJoin, kKickThreads, 2>(c, k_kick_drift);
+    if (e == cudaSuccess) e = join_kernel<PhotonsJoin, kKickThreads, 2>(c, k_photons);
+    if (e == cudaSuccess) e = join_kernel<KickJoin, kKickIons, 2>(c, k_kick_drift);
     return e;
 }
 

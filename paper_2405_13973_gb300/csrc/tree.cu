@@ -14,11 +14,13 @@
 // the whole sequence can be captured in a CUDA graph.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
+#include <string.h>
 
 #include "harmonics.cuh"
 #include "internal.h"
 #include "join.cuh"
 #include "bbox.cuh"
+#include "gyrate.cuh"
 
 namespace pt {
 
@@ -505,6 +507,200 @@ __global__ void k_leaf_gather(const double* __restrict__ x, const double* __rest
     k_leaf_gather_body<T4>(solo_block(), x, y, z, q, n, per, D, root, key, leaf_start, cid_leaf, perm_tmp, perm, slot_of, leaf_of, sorted);
 }
 
+// ---------------------------------------------------------------------------
+// The whole front of a small evaluation in one launch: first half-drift
+// (DRIFT, a time step), root cube, keys, histogram, both scans, scatter and
+// gather, on one cluster of kScanCtas CTAs with cluster barriers between the
+// stages.  Up to kSmallTreeIons ions the five launches are all latency (300
+// ions: 23 us of kernels and their gaps); beyond, the FP64 divisions of keys
+// and gather on eight SMs take longer than the launches saved.  What another
+// CTA wrote in this launch is read through L2.  Every stage computes exactly
+// what its own kernel does.
+// ---------------------------------------------------------------------------
+constexpr int64_t kSmallTreeIons = 2048;
+
+template <typename T4>
+struct SmallTree {
+    int64_t n;
+    double *x, *y, *z, *vx, *vy;   // written with DRIFT
+    const double *vz, *q;
+    PushParams pp;
+    int D;
+    RootCube* root;
+    int* err;
+    StepCounter* steps;
+    uint32_t* key;
+    int32_t *leaf_count, *perm_tmp, *perm, *slot_of, *leaf_of;
+    const int32_t* cid_leaf;
+    T4* sorted;
+    LeafCountScan ls;
+    CellCompaction cc;
+    int64_t ncells, ntotal;
+};
+
+template <typename T4, bool DRIFT>
+__global__ void __launch_bounds__(kScanCtaThreads) k_small_tree(const __grid_constant__ SmallTree<T4> a) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    __shared__ int warp_tot[kScanCtaThreads / 32];
+    __shared__ int cta_tot, s_tot[kScanCtas];
+    __shared__ unsigned long long s_acc[kBboxWords], s_all[kBboxWords];
+    __shared__ RootCube s_root;
+    const int tid = threadIdx.x, rank = (int)cl.block_rank(), nr = (int)cl.num_blocks();
+    const int64_t per = (a.n + nr - 1) / nr, i = rank * per + tid;
+    const bool mine = tid < per && i < a.n;
+    if (tid < kBboxWords) s_acc[tid] = 0ull;
+    pdl_wait();
+    __syncthreads();
+    double px = 0, py = 0, pz = 0;
+    BboxAcc t;
+    if (mine) {
+        px = a.x[i];
+        py = a.y[i];
+        pz = a.z[i];
+        if (DRIFT) {
+            double ux = a.vx[i], uy = a.vy[i];
+            gyrate(a.pp, px, py, pz, ux, uy, a.vz[i]);
+            a.x[i] = px;
+            a.y[i] = py;
+            a.z[i] = pz;
+            a.vx[i] = ux;
+            a.vy[i] = uy;
+        }
+        t.add(px, py, pz);
+    }
+#pragma unroll
+    for (int w = 0; w < 6; ++w) {
+        for (int o = 16; o > 0; o >>= 1) t.k[w] = umax64(t.k[w], __shfl_xor_sync(0xffffffffu, t.k[w], o));
+        if ((tid & 31) == 0 && t.k[w] != 0ull) atomicMax(&s_acc[w], t.k[w]);
+    }
+    if (t.bad) s_acc[6] = 1ull;
+    cl.sync();  // every CTA's words are in its shared memory
+    if (tid < kBboxWords) {
+        unsigned long long m = 0ull;
+        for (int r = 0; r < nr; ++r) m = umax64(m, cl.map_shared_rank(s_acc, (unsigned)r)[tid]);
+        s_all[tid] = m;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        unsigned long long v[7];
+#pragma unroll
+        for (int w = 0; w < 7; ++w) v[w] = s_all[w];
+        root_of_words(v, &s_root, a.err);
+        if (rank == 0) {
+            *a.root = s_root;
+            if (DRIFT) {
+                const int64_t next = a.steps->next;
+                a.steps->cur = next;
+                a.steps->next = next + 1;
+            }
+        }
+    }
+    __syncthreads();
+    const double lo0 = s_root.lo[0], lo1 = s_root.lo[1], lo2 = s_root.lo[2], side = s_root.side;
+    const double scale = (double)(1 << a.D);
+    uint32_t k = 0;
+    int arrival = 0;
+    if (mine) {
+        const int m = (1 << a.D) - 1;
+        k = morton3(leaf_coord(px, lo0, side, scale, m), leaf_coord(py, lo1, side, scale, m),
+                    leaf_coord(pz, lo2, side, scale, m));
+        a.key[i] = k;
+        arrival = atomicAdd(&a.leaf_count[k], 1);
+    }
+    cl.sync();  // the histogram is complete (and the CTAs' words are read)
+    scan_cluster_body(a.ls, a.ncells, warp_tot, &cta_tot, s_tot);
+    scan_cluster_body(a.cc, a.ntotal, warp_tot, &cta_tot, s_tot);
+    if (mine) a.perm_tmp[__ldcg(&a.ls.start[k]) + arrival] = (int32_t)i;
+    cl.sync();  // every ion is in its leaf's slots
+    if (mine) {  // slot i
+        const int idx = __ldcg(&a.perm_tmp[i]);
+        const uint32_t c = __ldcg(&a.key[idx]);
+        const int s = __ldcg(&a.ls.start[c]), cnt = __ldcg(&a.ls.start[c + 1]) - s;
+        int r = 0;
+        for (int u = 0; u < cnt; ++u) r += (__ldcg(&a.perm_tmp[s + u]) < idx);
+        const int slot = s + r;
+        int ix, iy, iz;
+        demorton3(c, ix, iy, iz);
+        a.perm[slot] = idx;
+        a.slot_of[idx] = slot;
+        a.leaf_of[slot] = __ldcg(&a.cid_leaf[c]);
+        const double ux = (__ldcg(&a.x[idx]) - lo0) / side * scale - (ix + 0.5);
+        const double uy = (__ldcg(&a.y[idx]) - lo1) / side * scale - (iy + 0.5);
+        const double uz = (__ldcg(&a.z[idx]) - lo2) / side * scale - (iz + 0.5);
+        a.sorted[slot] = make4<T4>(ux, uy, uz, a.q[idx]);
+    }
+}
+
+static CellCompaction cell_compaction(const DenseLayout& dl, int D, const Workspace& ws) {
+    CellCompaction cc;
+    cc.leaf_start = ws.leaf_start;
+    cc.cid = ws.cid;
+    cc.code = ws.code;
+    cc.cstart = ws.cstart;
+    cc.ccount = ws.ccount;
+    cc.linfo = ws.linfo;
+    cc.D = D;
+    cc.lmin = dl.lmin;
+    for (int l = 0; l < kMaxDepth + 2; ++l) cc.off[l] = dl.off[l];
+    return cc;
+}
+
+bool small_tree_fits(int64_t n, int D) {
+    return n <= kSmallTreeIons && ((int64_t)1 << (3 * D)) <= kScan1Max && dense_layout(D).total <= kScan1Max;
+}
+
+template <typename T4, bool DRIFT>
+static cudaError_t run_small_tree(int64_t n, double* x, double* y, double* z, double* vx, double* vy,
+                                  const double* vz, const double* q, const PushParams* pp, int D,
+                                  Workspace& ws, cudaStream_t s) {
+    const DenseLayout dl = dense_layout(D);
+    SmallTree<T4> a;
+    memset(&a, 0, sizeof a);
+    a.n = n;
+    a.x = x;
+    a.y = y;
+    a.z = z;
+    a.vx = vx;
+    a.vy = vy;
+    a.vz = vz;
+    a.q = q;
+    if (pp) a.pp = *pp;
+    a.D = D;
+    a.root = ws.root;
+    a.err = ws.err;
+    a.steps = ws.steps;
+    a.key = ws.key;
+    a.leaf_count = ws.leaf_count;
+    a.perm_tmp = ws.perm_tmp;
+    a.perm = ws.perm;
+    a.slot_of = ws.slot_of;
+    a.leaf_of = ws.leaf_of;
+    a.cid_leaf = ws.cid + dl.off[D];
+    a.sorted = (T4*)ws.sorted;
+    a.ncells = (int64_t)1 << (3 * D);
+    a.ntotal = dl.total;
+    a.ls = LeafCountScan{ws.leaf_count, ws.leaf_start, a.ncells};
+    a.cc = cell_compaction(dl, D, ws);
+    return launch_scan_cluster(k_small_tree<T4, DRIFT>, s, a);
+}
+
+cudaError_t launch_small_tree(int64_t n, const double* x, const double* y, const double* z,
+                              const double* q, int D, Workspace& ws, cudaStream_t s) {
+    double *mx = const_cast<double*>(x), *my = const_cast<double*>(y), *mz = const_cast<double*>(z);
+    return ws.fp64 ? run_small_tree<double4_32a, false>(n, mx, my, mz, nullptr, nullptr, nullptr, q,
+                                                        nullptr, D, ws, s)
+                   : run_small_tree<int4, false>(n, mx, my, mz, nullptr, nullptr, nullptr, q, nullptr,
+                                                 D, ws, s);
+}
+
+cudaError_t launch_small_front(int64_t n, double* x, double* y, double* z, double* vx, double* vy,
+                               const double* vz, const double* q, const PushParams& pp, int D,
+                               Workspace& ws, cudaStream_t s) {
+    return ws.fp64 ? run_small_tree<double4_32a, true>(n, x, y, z, vx, vy, vz, q, &pp, D, ws, s)
+                   : run_small_tree<int4, true>(n, x, y, z, vx, vy, vz, q, &pp, D, ws, s);
+}
+
 cudaError_t launch_tree(int64_t n, const double* x, const double* y, const double* z,
                         const double* q, int D, Workspace& ws, cudaStream_t s) {
     const int64_t ncells = (int64_t)1 << (3 * D);
@@ -518,16 +714,7 @@ cudaError_t launch_tree(int64_t n, const double* x, const double* y, const doubl
     if (e != cudaSuccess) return e;
     LeafCountScan ls{ws.leaf_count, ws.leaf_start, ncells};
     DenseLayout dl = dense_layout(D);
-    CellCompaction cc;
-    cc.leaf_start = ws.leaf_start;
-    cc.cid = ws.cid;
-    cc.code = ws.code;
-    cc.cstart = ws.cstart;
-    cc.ccount = ws.ccount;
-    cc.linfo = ws.linfo;
-    cc.D = D;
-    cc.lmin = dl.lmin;
-    for (int l = 0; l < kMaxDepth + 2; ++l) cc.off[l] = dl.off[l];
+    const CellCompaction cc = cell_compaction(dl, D, ws);
     // the cell compaction reads only the leaf starts: both scans in one
     // cluster launch when they fit, then the scatter
     if (ncells <= kScan1Max && dl.total <= kScan1Max) {
@@ -602,10 +789,7 @@ cudaError_t launch_level_counts(int64_t n, const double* x, const double* y, con
         return e;
     k_level_nonempty<<<152 * 4, 256, 0, s>>>(ws.leaf_start, Dm, d_counts);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = cudaMemcpyAsync(host_counts, d_counts, sizeof(int32_t) * (Dm + 1),
-                             cudaMemcpyDeviceToHost, s)) != cudaSuccess)
-        return e;
-    return cudaStreamSynchronize(s);
+    return cudaMemcpyAsync(host_counts, d_counts, sizeof(int32_t) * (Dm + 1), cudaMemcpyDeviceToHost, s);
 }
 
 // ---------------------------------------------------------------------------
