@@ -242,12 +242,17 @@ constexpr int kSlotThreads = 64, kSlotWindow = 48;
 // 16,000 ions 46 / 82 and 69 / 136; L2P: 4,000 ions 46 / 91 and 44 / 62, 8,000
 // ions 45 / 89 and 73 / 100)
 constexpr int64_t kP2mSlotIons = 10240, kL2pSlotIons = 7168;
+// FP32 from which k_l2p_f32 beats k_l2p (us, k_l2p / k_l2p_f32): 5,000 ions
+// (p = 15) 16 / 19, 10,000 (p = 12) 31 / 32, 23,000 (p = 8) 42 / 22, 30,000
+// (p = 3) 21 / 12, 1e5 (p = 12) 220 / 115, 1e6 (p = 12) 1727 / 700.
+constexpr int64_t kL2pF32Ions = 16384;
 
 // the slots [s0, s1) of the leaves that begin in window b; false if none does
 __device__ __forceinline__ bool slot_window(int64_t n, int b, const int32_t* __restrict__ leaf_of,
                                             const int32_t* __restrict__ cstart,
-                                            const int32_t* __restrict__ ccount, int& s0, int& s1) {
-    const int w0 = b * kSlotWindow, w1 = (int)min(n, (int64_t)w0 + kSlotWindow);
+                                            const int32_t* __restrict__ ccount, int& s0, int& s1,
+                                            int window = kSlotWindow) {
+    const int w0 = b * window, w1 = (int)min(n, (int64_t)w0 + window);
     const int gf = leaf_of[w0], gl = leaf_of[w1 - 1];
     s0 = cstart[gf];
     if (s0 < w0) s0 += ccount[gf];
@@ -1016,47 +1021,52 @@ __global__ void __launch_bounds__(kNfThreads, 8) k_p2p_f64(
 constexpr int kL2pThreads = 128;
 
 
-// the derived expansions of one local expansion Lr (see k_l2p) into D4[4][P]
+// The derived expansions of one local expansion Lr (see k_l2p) at (nn, mm):
+// put(k, phi, grad x, grad y, grad z) for the real part and, for mm > 0, the
+// imaginary part (for mm = 0 it would meet Im Y = 0).
+template <typename T, class Put>
+__device__ __forceinline__ void l2p_derive_entry(int p, int nn, int mm, const T* Lr,
+                                                 const HarmTables<T>& t, Put put) {
+    const int k = re_idx(nn, mm);
+    const T w = mm > 0 ? T(2) : T(1);
+    T d0r = w * Lr[k], d0i = mm > 0 ? w * Lr[k + 1] : T(0);
+    T dxr = 0, dxi = 0, dyr = 0, dyi = 0, dzr = 0, dzi = 0;
+    if (nn + 1 <= p) {
+        const int k1 = re_idx(nn + 1, mm);
+        const T e = w * t.e[nn][mm];
+        dzr = e * Lr[k1];
+        dzi = mm > 0 ? e * Lr[k1 + 1] : T(0);
+        const int k2 = re_idx(nn + 1, mm + 1);
+        const T f = t.f[nn][mm], l2r = Lr[k2], l2i = Lr[k2 + 1];
+        dxr = f * l2r;
+        dxi = f * l2i;
+        dyr = f * l2i;
+        dyi = -f * l2r;
+        if (mm >= 1) {
+            const int k3 = re_idx(nn + 1, mm - 1);
+            const T gg = t.g[nn][mm], l3r = Lr[k3], l3i = mm - 1 > 0 ? Lr[k3 + 1] : T(0);
+            dxr -= gg * l3r;
+            dxi -= gg * l3i;
+            dyr += gg * l3i;
+            dyi -= gg * l3r;
+        }
+    }
+    put(k, d0r, dxr, dyr, dzr);
+    if (mm > 0) put(k + 1, d0i, dxi, dyi, dzi);
+}
+// all of them into D4[4][P], by the block's threads
 template <typename T>
 __device__ __forceinline__ void l2p_derive(int p, const T* Lr, const HarmTables<T>& t, T (*D4)[kPmax]) {
     const int C = p + 1;
     for (int q = threadIdx.x; q < C * C; q += kL2pThreads) {
         const int nn = q / C, mm = q % C;
         if (mm > nn) continue;
-        const int k = re_idx(nn, mm);
-        const T w = mm > 0 ? T(2) : T(1);
-        T d0r = w * Lr[k], d0i = mm > 0 ? w * Lr[k + 1] : T(0);
-        T dxr = 0, dxi = 0, dyr = 0, dyi = 0, dzr = 0, dzi = 0;
-        if (nn + 1 <= p) {
-            const int k1 = re_idx(nn + 1, mm);
-            const T e = w * t.e[nn][mm];
-            dzr = e * Lr[k1];
-            dzi = mm > 0 ? e * Lr[k1 + 1] : T(0);
-            const int k2 = re_idx(nn + 1, mm + 1);
-            const T f = t.f[nn][mm], l2r = Lr[k2], l2i = Lr[k2 + 1];
-            dxr = f * l2r;
-            dxi = f * l2i;
-            dyr = f * l2i;
-            dyi = -f * l2r;
-            if (mm >= 1) {
-                const int k3 = re_idx(nn + 1, mm - 1);
-                const T gg = t.g[nn][mm], l3r = Lr[k3], l3i = mm - 1 > 0 ? Lr[k3 + 1] : T(0);
-                dxr -= gg * l3r;
-                dxi -= gg * l3i;
-                dyr += gg * l3i;
-                dyi -= gg * l3r;
-            }
-        }
-        D4[0][k] = d0r;
-        D4[1][k] = dxr;
-        D4[2][k] = dyr;
-        D4[3][k] = dzr;
-        if (mm > 0) {  // for m = 0 the imaginary parts meet Im Y = 0
-            D4[0][k + 1] = d0i;
-            D4[1][k + 1] = dxi;
-            D4[2][k + 1] = dyi;
-            D4[3][k + 1] = dzi;
-        }
+        l2p_derive_entry<T>(p, nn, mm, Lr, t, [&](int k, T a, T b, T c, T d) {
+            D4[0][k] = a;
+            D4[1][k] = b;
+            D4[2][k] = c;
+            D4[3][k] = d;
+        });
     }
 }
 
@@ -1367,44 +1377,16 @@ __global__ void __launch_bounds__(kSlotThreads) k_l2p_f64(
         for (int l = 0; l < nl; ++l)
             for (int c = tid; c < P; c += kSlotThreads) sL[l * P + c] = L[(int64_t)s_g[l] * ld + c];
         __syncthreads();
-        // derived expansions, as l2p_derive
         for (int u = tid; u < nl * NT; u += kSlotThreads) {
-            const int l = u / NT, nm = s_nm[u - l * NT], nn = nm >> 8, mm = nm & 255;
-            const double* Lr = sL + l * P;
-            double* D4 = sD + l * DS;
-            const int k = re_idx(nn, mm);
-            const double w = mm > 0 ? 2.0 : 1.0;
-            double dxr = 0, dxi = 0, dyr = 0, dyi = 0, dzr = 0, dzi = 0;
-            if (nn + 1 <= p) {
-                const int k1 = re_idx(nn + 1, mm), k2 = re_idx(nn + 1, mm + 1);
-                const double e = w * g_tab_d.e[nn][mm], f = g_tab_d.f[nn][mm];
-                const double l2r = Lr[k2], l2i = Lr[k2 + 1];
-                dzr = e * Lr[k1];
-                if (mm > 0) dzi = e * Lr[k1 + 1];
-                dxr = f * l2r;
-                dxi = f * l2i;
-                dyr = dxi;
-                dyi = -dxr;
-                if (mm >= 1) {
-                    const int k3 = re_idx(nn + 1, mm - 1);
-                    const double gg = g_tab_d.g[nn][mm], gr = gg * Lr[k3];
-                    const double gi = mm > 1 ? gg * Lr[k3 + 1] : 0.0;
-                    dxr -= gr;
-                    dxi -= gi;
-                    dyr += gi;
-                    dyi -= gr;
-                }
-            }
-            D4[k] = w * Lr[k];
-            D4[P + k] = dxr;
-            D4[2 * P + k] = dyr;
-            D4[3 * P + k] = dzr;
-            if (mm > 0) {
-                D4[k + 1] = w * Lr[k + 1];
-                D4[P + k + 1] = dxi;
-                D4[2 * P + k + 1] = dyi;
-                D4[3 * P + k + 1] = dzi;
-            }
+            const int l = u / NT, nm = s_nm[u - l * NT];
+            double* d = sD + l * DS;
+            l2p_derive_entry<double>(p, nm >> 8, nm & 255, sL + l * P, g_tab_d,
+                                     [&](int k, double a, double b, double c, double e) {
+                                         d[k] = a;
+                                         d[P + k] = b;
+                                         d[2 * P + k] = c;
+                                         d[3 * P + k] = e;
+                                     });
         }
         __syncthreads();
         if (in) {
@@ -1437,6 +1419,276 @@ __global__ void __launch_bounds__(kSlotThreads) k_l2p_f64(
             E[n + i] = s_f[0] * ey;
             E[2 * n + i] = s_f[0] * ez;
             if (PHI) phi[i] = s_f[1] * ph;
+        }
+        p0 += ni;
+    }
+}
+
+// L2P in FP32 for larger crystals (p <= 15): a thread per ion as in k_l2p_f64,
+// the leaf's, its parent's and grandparent's derived expansions (nlev of them)
+// once per block for all the leaves that share them, as one float4 (phi, grad)
+// per coefficient.  With 8 lanes to an ion (k_l2p) a recurrence step served
+// four ions, each leaf derived its ancestors' expansions anew and leaves of
+// few ions left most of a block idle.  Every sum is formed as there: the
+// diagonals by the same tree of products, "lane" g = 0 .. 7 of an ion adds
+// columns g and p - g of every level in turn, and the eight sums join pairwise
+// (0 + 4, 2 + 6, ...), so the fields are the same bit for bit.
+//
+// Bound by the latency of the chains of fused multiply-adds and shared loads
+// at few warps per SM: two columns run side by side (1,500 -> 820 us at 1e6
+// ions, p = 12, with the blocks of 64 threads and 36 KB it started from), and
+// a block of 128 ions shares more ancestors than two of 64 (820 -> 700 us;
+// 72 KB a block, as at 36 KB many blocks need a second pass).  In all 1,727
+// -> 700 us at 1e6 ions, 220 -> 115 us at 1e5 (p = 12), 42 -> 22 us at 23,000
+// (p = 8).
+constexpr int kL2pExp = 64;  // expansions per pass at most
+constexpr int kL2pFThreads = 128, kL2pFWindow = 112;
+// expansions (derived 16 bytes a coefficient, local 4) that fit 72 KB
+inline int l2p_f32_exps(int P) {
+    const int l = 72 * 1024 / (20 * P);
+    return l < 8 ? 8 : (l > kL2pExp ? kL2pExp : l);
+}
+inline size_t l2p_f32_smem(int P) { return (size_t)l2p_f32_exps(P) * P * 20 + 16; }
+
+struct L2pSum {
+    float ph, ax, ay, az;
+};
+// one column's running harmonic: Y_nn^m and Y_{nn-1}^m
+struct L2pCol {
+    float yr, yi, y1r, y1i;
+    __device__ __forceinline__ void second(int m, float z) {
+        y1r = yr;
+        y1i = yi;
+        yr = z * c_tab_f.d[m] * y1r;
+        yi = z * c_tab_f.d[m] * y1i;
+    }
+    __device__ __forceinline__ void next(int nn, int m, float z, float r2) {
+        const float a = c_tab_f.a[nn][m] * z, b = c_tab_f.b[nn][m] * r2;
+        const float cr = a * yr - b * y1r, ci = a * yi - b * y1i;
+        y1r = yr;
+        y1i = yi;
+        yr = cr;
+        yi = ci;
+    }
+    __device__ __forceinline__ void add(int nn, int m, const float4* D4, L2pSum& s) const {
+        const int k = re_idx(nn, m);
+        const float4 dr = D4[k];
+        s.ph += dr.x * yr;
+        s.ax += dr.y * yr;
+        s.ay += dr.z * yr;
+        s.az += dr.w * yr;
+        if (m > 0) {
+            const float4 di = D4[k + 1];
+            s.ph += di.x * yi;
+            s.ax += di.y * yi;
+            s.ay += di.z * yi;
+            s.az += di.w * yi;
+        }
+    }
+};
+__device__ __forceinline__ void l2p_run(int p, int m, float2 diag, float z, float r2,
+                                        const float4* D4, L2pSum& s) {
+    L2pCol c{diag.x, diag.y, 0.f, 0.f};
+    c.add(m, m, D4, s);
+    if (m == p) return;
+    c.second(m, z);
+    c.add(m + 1, m, D4, s);
+    for (int nn = m + 2; nn <= p; ++nn) {
+        c.next(nn, m, z, r2);
+        c.add(nn, m, D4, s);
+    }
+}
+// columns m (into a) and m + 1 <= p (into b) side by side: two chains in flight
+__device__ __forceinline__ void l2p_run2(int p, int m, float2 da, float2 db, float z, float r2,
+                                         const float4* D4, L2pSum& a, L2pSum& b) {
+    L2pCol u{da.x, da.y, 0.f, 0.f}, v{db.x, db.y, 0.f, 0.f};
+    u.add(m, m, D4, a);
+    u.second(m, z);
+    u.add(m + 1, m, D4, a);
+    v.add(m + 1, m + 1, D4, b);
+    if (m + 2 > p) return;
+    u.next(m + 2, m, z, r2);
+    v.second(m + 1, z);
+    u.add(m + 2, m, D4, a);
+    v.add(m + 2, m + 1, D4, b);
+    for (int nn = m + 3; nn <= p; ++nn) {
+        u.next(nn, m, z, r2);
+        v.next(nn, m + 1, z, r2);
+        u.add(nn, m, D4, a);
+        v.add(nn, m + 1, D4, b);
+    }
+}
+
+__global__ void __launch_bounds__(kL2pFThreads) k_l2p_f32(
+    int64_t n, int D, int p, int ld, int nlev, int emax, const RootCube* root,
+    const uint32_t* __restrict__ code, const int32_t* __restrict__ cid,
+    const int32_t* __restrict__ leaf_of, const int32_t* __restrict__ cstart,
+    const int32_t* __restrict__ ccount, const Ion<float>::rec* __restrict__ sorted,
+    const int32_t* __restrict__ perm, const float* __restrict__ L,
+    const float* __restrict__ near, double* E, double* phi) {
+    extern __shared__ float4 l2p_smem[];  // derived [emax][P], then local [emax][P] floats
+    __shared__ int s_row[kL2pExp], s_new[3][kL2pFThreads / 32], s_cnt[kL2pFThreads / 32], s_tot[3];
+    __shared__ uint16_t s_nm[(kMaxOrder + 1) * (kMaxOrder + 2) / 2];
+    __shared__ double s_f[2];
+    const int P = (p + 1) * (p + 1), tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int NT = (p + 1) * (p + 2) / 2;
+    float4* sD = l2p_smem;
+    float* sL = reinterpret_cast<float*>(l2p_smem + emax * P);
+    for (int nn = tid; nn <= p; nn += kL2pFThreads)
+        for (int m = 0; m <= nn; ++m) s_nm[nn * (nn + 1) / 2 + m] = (uint16_t)(nn << 8 | m);
+    pdl_wait();
+    int s0, s1;
+    if (!slot_window(n, blockIdx.x, leaf_of, cstart, ccount, s0, s1, kL2pFWindow)) return;  // uniform
+    if (tid == 0) {
+        const double sl = root->side / (double)(1 << D);
+        s_f[0] = kCoulomb / (sl * sl);
+        s_f[1] = kCoulomb / sl;
+    }
+    for (int p0 = s0; p0 < s1;) {
+        // the pass: at most kL2pFThreads slots whose cells number at most emax
+        const bool live = p0 + tid < s1;
+        const int g = live ? leaf_of[p0 + tid] : -1;
+        const uint32_t cl = live ? code[g] : 0xffffffffu;
+        const uint32_t prev = tid == 0 || !live ? 0xffffffffu : code[leaf_of[p0 + tid - 1]];
+        unsigned bal[3];
+        bool head[3];
+#pragma unroll
+        for (int lv = 0; lv < 3; ++lv) {
+            head[lv] = live && lv < nlev && (tid == 0 || (prev >> (3 * lv)) != (cl >> (3 * lv)));
+            bal[lv] = __ballot_sync(0xffffffffu, head[lv]);
+        }
+        __syncthreads();  // the previous pass is done with the shared arrays
+        if (lane == 0)
+            for (int lv = 0; lv < 3; ++lv) s_new[lv][wid] = __popc(bal[lv]);
+        if (tid < 3) s_tot[tid] = 0;
+        __syncthreads();
+        int ord[3], used = 0;
+#pragma unroll
+        for (int lv = 0; lv < 3; ++lv) {
+            ord[lv] = __popc(bal[lv] & (0xffffffffu >> (31 - lane))) - 1;
+#pragma unroll
+            for (int w = 0; w < kL2pFThreads / 32 - 1; ++w) ord[lv] += w < wid ? s_new[lv][w] : 0;
+            used += ord[lv] + 1;
+        }
+        const bool in = live && used <= emax;
+        const unsigned inb = __ballot_sync(0xffffffffu, in);
+        if (lane == 0) s_cnt[wid] = __popc(inb);
+        __syncthreads();
+        int ni = 0;
+#pragma unroll
+        for (int w = 0; w < kL2pFThreads / 32; ++w) ni += s_cnt[w];
+        if (tid == ni - 1)
+            for (int lv = 0; lv < 3; ++lv) s_tot[lv] = ord[lv] + 1;
+        __syncthreads();
+        int base[3] = {0, s_tot[0], s_tot[0] + s_tot[1]};
+        const int ne = base[2] + s_tot[2];
+#pragma unroll
+        for (int lv = 0; lv < 3; ++lv)
+            if (in && head[lv])
+                // dense maps of levels 2.. concatenated: level l starts at (8^l - 64) / 7
+                s_row[base[lv] + ord[lv]] =
+                    lv == 0 ? g : cid[(((1ll << (3 * (D - lv))) - 64) / 7) + (cl >> (3 * lv))];
+        __syncthreads();
+        for (int e = 0; e < ne; ++e)
+            for (int c = tid; c < P; c += kL2pFThreads) sL[e * P + c] = L[(int64_t)s_row[e] * ld + c];
+        __syncthreads();
+        for (int u = tid; u < ne * NT; u += kL2pFThreads) {
+            const int e = u / NT, nm = s_nm[u - e * NT];
+            float4* d = sD + e * P;
+            l2p_derive_entry<float>(p, nm >> 8, nm & 255, sL + e * P, g_tab_f,
+                                    [&](int k, float a, float b, float c, float w) {
+                                        d[k] = make_float4(a, b, c, w);
+                                    });
+        }
+        __syncthreads();
+        if (in) {
+            const Ion<float>::rec me = sorted[p0 + tid];
+            int ix, iy, iz;
+            demorton3(cl, ix, iy, iz);
+            float vx[8], vy[8], vz[8], vp[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) vx[q] = vy[q] = vz[q] = vp[q] = 0.f;
+#pragma unroll 1
+            for (int lv = 0; lv < nlev; ++lv) {
+                const float4* D4 = sD + (base[lv] + ord[lv]) * P;
+                float x, y, z, qq;
+                const int am = (1 << lv) - 1;  // the leaf's position inside the ancestor
+                ion_in_ancestor(me, lv, ix & am, iy & am, iz & am, x, y, z, qq);
+                // diagonals Y_m^m, m = 0 .. 15: two prefix products of eight
+                float ar[8], ai[8], br[8], bi[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    ar[q] = br[q] = 1.f;
+                    ai[q] = bi[q] = 0.f;
+                    if (q >= 1 && q <= p) {
+                        ar[q] = x * c_tab_f.c[q];
+                        ai[q] = y * c_tab_f.c[q];
+                    }
+                    if (8 + q <= p) {
+                        br[q] = x * c_tab_f.c[8 + q];
+                        bi[q] = y * c_tab_f.c[8 + q];
+                    }
+                }
+#pragma unroll
+                for (int off = 1; off < 8; off <<= 1)
+#pragma unroll
+                    for (int q = 7; q >= off; --q) {
+                        const float oar = ar[q - off], oai = ai[q - off], obr = br[q - off], obi = bi[q - off];
+                        const float r = oar * ar[q] - oai * ai[q];
+                        ai[q] = oar * ai[q] + oai * ar[q];
+                        ar[q] = r;
+                        const float s2 = obr * br[q] - obi * bi[q];
+                        bi[q] = obr * bi[q] + obi * br[q];
+                        br[q] = s2;
+                    }
+                float2 dg[16];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    dg[q] = make_float2(ar[q], ai[q]);
+                    dg[8 + q] = make_float2(ar[7] * br[q] - ai[7] * bi[q], ar[7] * bi[q] + ai[7] * br[q]);
+                }
+                const float r2 = x * x + y * y + z * z;
+                const float fp1 = lv == 0 ? 1.f : (lv == 1 ? 0.5f : 0.25f), fe1 = fp1 * fp1;
+#pragma unroll
+                for (int q = 0; q < 8; q += 2) {
+                    const int m2 = p - q;
+                    L2pSum c0{0.f, 0.f, 0.f, 0.f}, c1{0.f, 0.f, 0.f, 0.f};
+                    if (m2 - 1 > q + 1) {
+                        l2p_run2(p, q, dg[q], dg[q + 1], z, r2, D4, c0, c1);
+                        l2p_run2(p, m2 - 1, dg[m2 - 1], dg[m2], z, r2, D4, c1, c0);
+                    } else {  // the last columns (p < 15)
+                        if (q <= m2) l2p_run(p, q, dg[q], z, r2, D4, c0);
+                        if (m2 > q) l2p_run(p, m2, dg[m2], z, r2, D4, c0);
+                        if (q + 1 <= m2 - 1) l2p_run(p, q + 1, dg[q + 1], z, r2, D4, c1);
+                    }
+                    // level units -> leaf units: phi / 2^lv, E / 4^lv (exact)
+                    vp[q] += fp1 * c0.ph;
+                    vx[q] -= fe1 * c0.ax;
+                    vy[q] -= fe1 * c0.ay;
+                    vz[q] -= fe1 * c0.az;
+                    vp[q + 1] += fp1 * c1.ph;
+                    vx[q + 1] -= fe1 * c1.ax;
+                    vy[q + 1] -= fe1 * c1.ay;
+                    vz[q + 1] -= fe1 * c1.az;
+                }
+            }
+            auto join = [](const float (&v)[8]) {
+                return ((v[0] + v[4]) + (v[2] + v[6])) + ((v[1] + v[5]) + (v[3] + v[7]));
+            };
+            float ex = join(vx), ey = join(vy), ez = join(vz), ph = join(vp);
+            if (near) {
+                const float* o = near + 4 * (int64_t)(p0 + tid);
+                ex += o[0];
+                ey += o[1];
+                ez += o[2];
+                ph += o[3];
+            }
+            const float tE = (float)s_f[0], tP = (float)s_f[1];
+            const int i = perm[p0 + tid];
+            E[i] = (double)(tE * ex);
+            E[n + i] = (double)(tE * ey);
+            E[2 * n + i] = (double)(tE * ez);
+            if (phi) phi[i] = (double)(tP * ph);
         }
         p0 += ni;
     }
@@ -1762,6 +2014,14 @@ static cudaError_t run_fmm(int64_t n, int D, int phases, Workspace& ws, bool use
                        (const int32_t*)ws.ccount, (const Ion<double>::rec*)ws.sorted,
                        (const int32_t*)ws.perm, (const double*)ws.L,
                        (const double*)(nf ? ws.near : nullptr), E, phi);
+    else if (far && sizeof(T) == 4 && p <= 15 && n >= kL2pF32Ions)
+        e = launch_pdl(k_l2p_f32, dim3((unsigned)((n + kL2pFWindow - 1) / kL2pFWindow)),
+                       dim3(kL2pFThreads), l2p_f32_smem(P), s, n, D, p, ws.ld, l2p_levels,
+                       l2p_f32_exps(P), (const RootCube*)ws.root, (const uint32_t*)ws.code,
+                       (const int32_t*)ws.cid, (const int32_t*)ws.leaf_of, (const int32_t*)ws.cstart,
+                       (const int32_t*)ws.ccount, (const Ion<float>::rec*)ws.sorted,
+                       (const int32_t*)ws.perm, (const float*)ws.L,
+                       (const float*)(nf ? ws.near : nullptr), E, phi);
     else
         e = launch_pdl(p <= 15 ? k_l2p<T, 8> : k_l2p<T, 16>, dim3(leaf_grid), dim3(kL2pThreads),
                        0, s, n, D, p, ws.ld, far,
@@ -1961,6 +2221,8 @@ cudaError_t upload_harmonic_tables() {
         e = cudaFuncSetAttribute(k_p2m_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  kSlotThreads * p2m_f64_stride(pmax) * (int)sizeof(double));
     // (the largest over the orders: fewer leaves above the order where 16 fit)
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_l2p_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
     for (auto f : {k_l2p_f64<true>, k_l2p_f64<false>})
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 104 * 1024);
