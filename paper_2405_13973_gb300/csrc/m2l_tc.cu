@@ -1133,7 +1133,10 @@ __global__ void __launch_bounds__((TcLayout<MODE, BF16>::kThreads), 1)
 // in increasing order.  Up to level kBitmapLevel the level's occupancy is a
 // bitmap of x-rows (one 64-bit word per (y, z) row) in shared memory, so an
 // (offset, target row) test is one shift and one AND; deeper levels test
-// each (offset, target) through the cell-id table.
+// each (offset, target) through the cell-id table.  The bitmaps of all levels
+// are built once (k_tc_bits) and copied: with every tile's block setting the
+// bits of its level again this took 1,040 us at 1e6 ions (p = 12) and 71 us at
+// 1e5, now 122 and 34 us.
 constexpr int kPlanThreads = 512;
 constexpr int kWaveItems = 148;
 constexpr int kBitmapLevel = 6;
@@ -1143,7 +1146,29 @@ __host__ __device__ inline int tc_plan_smem_bytes(int D) {
     return 2 * (1 << (2 * l)) * (int)sizeof(unsigned long long);
 }
 
-__global__ void __launch_bounds__(kPlanThreads) k_tc_plan(TcArgs a, TcTile* tiles) {
+// words of the levels 2 .. kBitmapLevel, level l from word (4^l - 16) / 3
+constexpr int kBitmapWords = ((1 << (2 * (kBitmapLevel + 1))) - 16) / 3;
+
+// One thread per cell of the levels 2 .. min(D, kBitmapLevel); bits zeroed before.
+__global__ void __launch_bounds__(256) k_tc_bits(int D, const LevelInfo* linfo,
+                                                 const uint32_t* __restrict__ code,
+                                                 unsigned long long* bits) {
+    __shared__ LevelInfo li;
+    stage_linfo(linfo, &li);
+    __syncthreads();
+    const int top = D < kBitmapLevel ? D : kBitmapLevel;
+    for (int c = li.gbase[2] + blockIdx.x * 256 + threadIdx.x; c < li.gbase[top + 1];
+         c += gridDim.x * 256) {
+        int l = 2;
+        while (c >= li.gbase[l + 1]) ++l;
+        int x, y, z;
+        demorton3(code[c], x, y, z);
+        atomicOr(&bits[((1 << (2 * l)) - 16) / 3 + (z << l) + y], 1ull << x);
+    }
+}
+
+__global__ void __launch_bounds__(kPlanThreads) k_tc_plan(
+    TcArgs a, TcTile* tiles, const unsigned long long* __restrict__ bits) {
     extern __shared__ unsigned long long bm[];  // occupancy rows | target rows
     __shared__ uint8_t flag[343];
     __shared__ int rowlist[kTcRows];
@@ -1166,13 +1191,11 @@ __global__ void __launch_bounds__(kPlanThreads) k_tc_plan(TcArgs a, TcTile* tile
         const int nr = side * side;
         unsigned long long* occ = bm;
         unsigned long long* tg = bm + nr;
-        for (int i = tid; i < 2 * nr; i += kPlanThreads) bm[i] = 0ull;
-        __syncthreads();
-        for (int c = li.gbase[l] + tid; c < li.gbase[l + 1]; c += kPlanThreads) {
-            int x, y, z;
-            demorton3(a.code[c], x, y, z);
-            atomicOr(&occ[z * side + y], 1ull << x);
+        for (int i = tid; i < nr; i += kPlanThreads) {
+            occ[i] = bits[(nr - 16) / 3 + i];
+            tg[i] = 0ull;
         }
+        __syncthreads();
         for (int r = tid; r < rows; r += kPlanThreads) {
             int x, y, z;
             demorton3(a.code[base + r], x, y, z);
@@ -1627,10 +1650,11 @@ __global__ void k_split_m(int lfirst, int llast, int ld, const LevelInfo* linfo,
 // The M2L work list of the current tree (tiles, their non-empty offsets,
 // the work items); it reads the tree only.
 static bool tc_worklist_layout(int64_t n, int D, Workspace& ws, int64_t& tiles, TcPlanHdr*& hdr,
-                               TcTile*& tl, TcItem*& items) {
+                               TcTile*& tl, TcItem*& items, unsigned long long*& bits) {
     tiles = 0;
     for (int l = 2; l <= D; ++l) tiles += (level_cells(n, l) + kTcRows - 1) / kTcRows + 8;
-    hdr = (TcPlanHdr*)ws.tc_work;
+    bits = (unsigned long long*)ws.tc_work;
+    hdr = (TcPlanHdr*)(bits + kBitmapWords);
     tl = (TcTile*)(hdr + 1);
     items = (TcItem*)(tl + ws.tc_tiles_cap);
     return tiles <= ws.tc_tiles_cap;
@@ -1669,14 +1693,22 @@ cudaError_t launch_m2l_tc_worklist(int64_t n, int D, Workspace& ws, cudaStream_t
     TcPlanHdr* hdr;
     TcTile* tl;
     TcItem* items;
-    if (!tc_worklist_layout(n, D, ws, tiles, hdr, tl, items)) return cudaErrorInvalidValue;
+    unsigned long long* bits;
+    if (!tc_worklist_layout(n, D, ws, tiles, hdr, tl, items, bits)) return cudaErrorInvalidValue;
     TcArgs a = base_args(n, D, ws, 1);
     a.mode = MODE_M2L;
     a.tiles = tl;
     a.items = items;
     a.hdr = hdr;
-    k_tc_plan<<<(unsigned)tiles, kPlanThreads, tc_plan_smem_bytes(D), s>>>(a, tl);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = cudaMemsetAsync(bits, 0, kBitmapWords * sizeof(*bits), s);
+    if (e != cudaSuccess) return e;
+    int64_t cells = 0;
+    for (int l = 2; l <= D && l <= kBitmapLevel; ++l) cells += level_cells(n, l);
+    k_tc_bits<<<(unsigned)std::min<int64_t>((cells + 255) / 256, 608), 256, 0, s>>>(D, ws.linfo,
+                                                                                  ws.code, bits);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    k_tc_plan<<<(unsigned)tiles, kPlanThreads, tc_plan_smem_bytes(D), s>>>(a, tl, bits);
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_tc_items<<<1, kItemThreads, 0, s>>>(D, ws.linfo, (int)tiles, (int)ws.tc_slab_cap,
                                           n > kChainLargeIons ? kChainCapLarge : kChainCap, hdr, tl,
@@ -1745,7 +1777,8 @@ cudaError_t launch_m2l_tc_run(int64_t n, int D, Workspace& ws, int l2l_last, int
     TcPlanHdr* hdr;
     TcTile* tl;
     TcItem* items;
-    if (!tc_worklist_layout(n, D, ws, tiles, hdr, tl, items)) return cudaErrorInvalidValue;
+    unsigned long long* bits;
+    if (!tc_worklist_layout(n, D, ws, tiles, hdr, tl, items, bits)) return cudaErrorInvalidValue;
     TcArgs a = base_args(n, D, ws, 1);
     a.mode = MODE_M2L;
     a.tiles = tl;
@@ -1780,13 +1813,14 @@ cudaError_t m2l_tc_work_stats(const Workspace& ws, int64_t* out, cudaStream_t s)
     for (int k = 0; k < 4; ++k) out[k] = 0;
     if (ws.m2l_pairs) return m2l_pairs_stats(ws, out, s);
     if (!ws.tc_work) return cudaSuccess;
+    const auto* hdr = (const TcPlanHdr*)((const unsigned long long*)ws.tc_work + kBitmapWords);
     TcPlanHdr h;
-    cudaError_t e = cudaMemcpyAsync(&h, ws.tc_work, sizeof h, cudaMemcpyDeviceToHost, s);
+    cudaError_t e = cudaMemcpyAsync(&h, hdr, sizeof h, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return e;
     if (h.n_tiles <= 0 || h.n_tiles > ws.tc_tiles_cap) return cudaSuccess;
     std::vector<TcTile> t((size_t)h.n_tiles);
-    e = cudaMemcpyAsync(t.data(), (const TcPlanHdr*)ws.tc_work + 1, sizeof(TcTile) * t.size(),
+    e = cudaMemcpyAsync(t.data(), hdr + 1, sizeof(TcTile) * t.size(),
                         cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return e;
@@ -1800,7 +1834,7 @@ cudaError_t m2l_tc_work_stats(const Workspace& ws, int64_t* out, cudaStream_t s)
 }
 
 size_t m2l_tc_work_bytes(int64_t tiles_cap, int64_t slab_cap) {
-    return sizeof(TcPlanHdr) + (size_t)tiles_cap * sizeof(TcTile) +
+    return kBitmapWords * sizeof(unsigned long long) + sizeof(TcPlanHdr) + (size_t)tiles_cap * sizeof(TcTile) +
            (size_t)(tiles_cap + slab_cap) * sizeof(TcItem);
 }
 
