@@ -1351,39 +1351,43 @@ __global__ void __launch_bounds__(kItemThreads) k_tc_items(int D, const LevelInf
 }
 
 // L += the partial slabs of the M2L items of rank > 0, per tile in rank
-// order; 32 blocks per tile, each a slice of its rows, eight slabs in flight.
-constexpr int kRedSlices = 32;
+// order; blocks over chunks of 256 float4 of a tile, eight slabs in flight.
+// DRAM-bound (every slab is read once).  With 32 slices of whole rows a
+// quarter to a third of a block's threads had no element (172 of 256 at p = 12), and the slabs left over from a multiple of
+// eight were read one after another: 1,211 -> 1,170 us at 1e6 ions (p = 12,
+// 6 GB of slabs), 131 -> 115 us at 1e5, 49 -> 42 us at 2e5 with p = 5.
+constexpr int kRedThreads = 256;
+inline __host__ __device__ int red_chunks(int ld) {
+    return (kTcRows * (ld / 4) + kRedThreads - 1) / kRedThreads;
+}
 
-__global__ void __launch_bounds__(256) k_tc_reduce_tiles(int ld, const TcPlanHdr* hdr,
-                                                         const TcTile* tiles,
-                                                         const float4* __restrict__ slabs,
-                                                         float4* L) {
+__global__ void __launch_bounds__(kRedThreads, 4) k_tc_reduce_tiles(
+    int ld, const TcPlanHdr* hdr, const TcTile* tiles, const float4* __restrict__ slabs, float4* L) {
     const int n_tiles = hdr->n_tiles;
-    const int w = ld / 4;
+    const int w = ld / 4, chunks = red_chunks(ld);
     const int64_t slab4 = (int64_t)kTcRows * w;
-    for (int bb = blockIdx.x; bb < n_tiles * kRedSlices; bb += gridDim.x) {
-        const int b = bb / kRedSlices, slice = bb % kRedSlices;
-        const int ns = tiles[b].nsplit, base = tiles[b].base, rows = tiles[b].rows;
+    for (int bb = blockIdx.x; bb < n_tiles * chunks; bb += gridDim.x) {
+        const int b = bb / chunks, local = (bb - b * chunks) * kRedThreads + threadIdx.x;
+        const int ns = tiles[b].nsplit;
         if (ns <= 1) continue;
         const float4* first = slabs + (int64_t)(tiles[b].item0 + 1) * slab4;
-        const int r0 = (rows * slice) / kRedSlices, r1 = (rows * (slice + 1)) / kRedSlices;
-        for (int e = threadIdx.x; e < (r1 - r0) * w; e += blockDim.x) {
-            const int64_t local = (int64_t)(r0 + e / w) * w + (e % w);
-            const int64_t idx = (int64_t)base * w + local;
+        if (local < tiles[b].rows * w) {
+            const int64_t idx = (int64_t)tiles[b].base * w + local;
             float4 v = L[idx];
             int k = 0;
-            for (; k + 8 <= ns - 1; k += 8) {
+            for (; k < ns - 1; k += 8) {
                 float4 q[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) q[u] = first[(k + u) * slab4 + local];
+                for (int u = 0; u < 8; ++u)
+                    if (k + u < ns - 1) q[u] = __ldcs(&first[(k + u) * slab4 + local]);
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    v.x += q[u].x; v.y += q[u].y; v.z += q[u].z; v.w += q[u].w;
-                }
-            }
-            for (; k < ns - 1; ++k) {
-                const float4 q = first[k * slab4 + local];
-                v.x += q.x; v.y += q.y; v.z += q.z; v.w += q.w;
+                for (int u = 0; u < 8; ++u)
+                    if (k + u < ns - 1) {
+                        v.x += q[u].x;
+                        v.y += q[u].y;
+                        v.z += q[u].z;
+                        v.w += q[u].w;
+                    }
             }
             L[idx] = v;
         }
@@ -1800,7 +1804,7 @@ cudaError_t launch_m2l_tc_run(int64_t n, int D, Workspace& ws, int l2l_last, int
                          cudaSuccess)
         return e;
     if (after_m2l && (e = cudaEventRecord(after_m2l, s)) != cudaSuccess) return e;
-    const int64_t rg = tiles * kRedSlices;
+    const int64_t rg = tiles * red_chunks(ws.ld);
     k_tc_reduce_tiles<<<(unsigned)(rg < 152 * 16 ? rg : 152 * 16), 256, 0, s>>>(
         ws.ld, hdr, tl, (const float4*)ws.tc_part, (float4*)ws.L);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
