@@ -499,7 +499,8 @@ int pt_ensemble_create(int n_members, const fmm_plan* plans, pt_ensemble* out);
  * each member's step as a parallel branch (captured once, again when a
  * member's depth, buffers or parameters change).  The M2L launches of the
  * members that use the BF16x3 pair-packed schedule (Eq. FMM_local) are
- * replaced in that graph by one launch over all of their work items, which
+ * replaced in that graph by one launch over all of their work items (the
+ * members of the most frequent order p; the others launch their own), which
  * waits for every such member's multipoles and precedes every member's
  * reduction (see pt_ensemble_set_joined_m2l).  With that switch on, the
  * members' other launches are joined kernel by kernel as well (unless a

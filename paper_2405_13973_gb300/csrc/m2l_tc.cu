@@ -59,6 +59,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <map>
 #include <vector>
 
 #include "bf16split.cuh"
@@ -1899,11 +1900,26 @@ cudaError_t m2l_join_pair_launches(cudaGraph_t g, void* d_members, int* d_prefix
         cudaKernelNodeParams kp{};
         if ((e = cudaGraphKernelNodeGetParams(x, &kp)) != cudaSuccess) return e;
         if (kp.func != fn) continue;
-        if (found.empty()) first = kp;
         found.push_back(x);
         args.push_back(*static_cast<const TcArgs*>(kp.kernelParams[0]));
     }
-    const int n = (int)found.size();
+    // one launch has one tile geometry and one set of operators: the members
+    // of the most frequent order share it, the others keep their own
+    std::map<int, int> members_of;
+    for (const TcArgs& a : args) ++members_of[a.P];
+    int P = 0;
+    for (const auto& m : members_of)
+        if (P == 0 || m.second > members_of[P]) P = m.first;
+    size_t kept = 0;
+    for (size_t k = 0; k < found.size(); ++k) {
+        if (args[k].P != P) continue;
+        found[kept] = found[k];
+        args[kept++] = args[k];
+    }
+    found.resize(kept);
+    args.resize(kept);
+    if (kept && (e = cudaGraphKernelNodeGetParams(found[0], &first)) != cudaSuccess) return e;
+    const int n = (int)kept;
     if (n < 2) return cudaSuccess;  // nothing to share
     if (n > cap) return cudaErrorInvalidValue;
     std::vector<PairMember> hm((size_t)n);
