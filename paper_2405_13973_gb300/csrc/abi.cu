@@ -33,8 +33,9 @@ constexpr int64_t kPairsDefaultIons = 65536;
 // in FP64), which beats the per-level tile kernel at every size measured;
 // the bound keeps the FP64 partial-row pool within a few GB
 constexpr int64_t kPairsDefaultIonsCudaCore = 262144;
-// partial rows of one batch of the FP64 M2L beyond that many ions
-constexpr int64_t kF64PoolBytes = (int64_t)4 << 30;
+// partial rows of one batch of the FP64 M2L beyond that many ions: at most
+// kF64PoolBytes, and no more than the plan's expansions (but kF64PoolMin)
+constexpr int64_t kF64PoolBytes = (int64_t)4 << 30, kF64PoolMin = (int64_t)512 << 20;
 
 struct GraphKey {
     int D = -1;
@@ -250,7 +251,7 @@ int build_operators(fmm_plan_s* pl) {
     cudaError_t e = pl->ws.fp64 ? upload_ops<double>(pl, m2m, l2l, m2l)
                                 : upload_ops<float>(pl, m2m, l2l, m2l);
     if (e != cudaSuccess) return status_from(e);
-    if (pl->ws.fp64 && (e = m2l_f64_pack(pl->ws)) != cudaSuccess) return status_from(e);
+    if (pl->ws.T_f64 && (e = m2l_f64_pack(pl->ws)) != cudaSuccess) return status_from(e);
     if (pl->precision == PT_FP32 && (e = m2l_f32_pack(pl->ws)) != cudaSuccess) return status_from(e);
     if (is_tc(pl->precision)) {
         const bool bf16 = pl->precision == PT_MIXED_BF16X3;
@@ -317,10 +318,14 @@ int acquire_ops(fmm_plan_s* pl, size_t op_bytes) {
             cudaMalloc(&o.T_l2l, 8 * op_bytes) != cudaSuccess ||
             cudaMalloc(&o.T_m2l, 343 * op_bytes) != cudaSuccess ||
             (tc && cudaMalloc(&o.T_m2l_tc, tc) != cudaSuccess) ||
-            (f64 && cudaMalloc(&o.T_f64, f64) != cudaSuccess) ||
             (f32 && cudaMalloc(&o.T_f32, f32) != cudaSuccess)) {
             drop();
             return PT_ERR_OOM;
+        }
+        // without the digits the plans of this set stay on the CUDA cores
+        if (f64 && cudaMalloc(&o.T_f64, f64) != cudaSuccess) {
+            cudaGetLastError();
+            o.T_f64 = nullptr;
         }
         ws.T_m2m = o.T_m2m;
         ws.T_l2l = o.T_l2l;
@@ -1061,13 +1066,25 @@ static int plan_create_impl(int64_t n_max, int p, int leaf_max, int depth, int p
         ws.m2l_rot = ok && ws.fp64 && ws.rot_op_vals > 0 ? 1 : 0;
     }
     if (ok && ws.fp64) {
-        ok = dalloc(pl, ws.f64_dig, m2l_f64_digit_bytes(p, cells)) &&
-             dalloc(pl, ws.f64_rexp, sizeof(int) * cells);
-        ws.f64_tc = 1;
-        if (ok && !ws.m2l_pairs) {
+        const size_t held = pl->allocs.size();
+        bool tc = dalloc(pl, ws.f64_dig, m2l_f64_digit_bytes(p, cells)) &&
+                  dalloc(pl, ws.f64_rexp, sizeof(int) * cells);
+        if (tc && !ws.m2l_pairs) {
             // beyond kPairsDefaultIonsCudaCore the M2L runs in batches
-            ws.f64_batch = std::max<int64_t>(1, kF64PoolBytes / (189 * 8 * (int64_t)ws.ld));
-            ok = alloc_pairs(pl) == PT_OK;
+            const int64_t expansions = (int64_t)(2 * tsz) * ws.ld * cells;
+            const int64_t pool = std::min(kF64PoolBytes, std::max(kF64PoolMin, expansions));
+            ws.f64_batch = std::max<int64_t>(1, pool / (189 * 8 * (int64_t)ws.ld));
+            tc = alloc_pairs(pl) == PT_OK;
+        }
+        ws.f64_tc = tc ? 1 : 0;
+        if (!tc) {
+            // no memory for the digits or the pool: the CUDA-core
+            // translations, which need neither
+            for (; pl->allocs.size() > held; pl->allocs.pop_back()) cudaFree(pl->allocs.back());
+            cudaGetLastError();
+            ws.f64_dig = nullptr;
+            ws.f64_rexp = nullptr;
+            ws.f64_batch = 0;
         }
     }
     if (dry) {
@@ -1132,6 +1149,11 @@ static int plan_create_impl(int64_t n_max, int p, int leaf_max, int depth, int p
         }
     }
     int r = acquire_ops(pl, tsz * PP);
+    if (r == PT_OK && !ws.T_f64) {
+        ws.f64_tc = 0;
+        ws.f64_batch = 0;
+    }
+    if (r == PT_OK && ws.m2l_rot && !ws.f64_tc) r = acquire_rotation(pl);
     if (r != PT_OK) {
         free_plan(pl);
         return r;
