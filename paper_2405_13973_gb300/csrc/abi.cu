@@ -604,7 +604,7 @@ cudaError_t enqueue_step(fmm_plan_s* pl, const pt_state& st, const PushParams& p
     if (e == cudaSuccess) e = mark(2);
     if (e == cudaSuccess)
         e = launch_fmm_phased(n, D, PT_PHASE_ALL, ws, is_tc(pl->precision), ws.E,
-                              nullptr, s, pl->profile ? pl->ph_ev + 3 : nullptr);
+                              nullptr, s, pl->profile ? pl->ph_ev + 3 : nullptr, alone);
     if (lasers && e == cudaSuccess) e = cudaStreamWaitEvent(s, ws.ev_photons, 0);
     if (e == cudaSuccess)
         e = launch_kick_drift(n, st.x, st.y, st.z, st.vx, st.vy, st.vz, st.q, ws.E, pp,

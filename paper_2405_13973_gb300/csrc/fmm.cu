@@ -242,9 +242,12 @@ constexpr int kSlotThreads = 64, kSlotWindow = 48;
 // 16,000 ions 46 / 82 and 69 / 136; L2P: 4,000 ions 46 / 91 and 44 / 62, 8,000
 // ions 45 / 89 and 73 / 100)
 constexpr int64_t kP2mSlotIons = 10240, kL2pSlotIons = 7168;
-// FP32 from which k_l2p_f32 beats k_l2p (us, k_l2p / k_l2p_f32): 5,000 ions
-// (p = 15) 16 / 19, 10,000 (p = 12) 31 / 32, 23,000 (p = 8) 42 / 22, 30,000
-// (p = 3) 21 / 12, 1e5 (p = 12) 220 / 115, 1e6 (p = 12) 1727 / 700.
+// FP32 (p <= 15): ions from which k_l2p_f32 takes one thread an ion instead of
+// four (us, k_l2p / 4 threads / 1 thread): 300 ions (p = 12) 11 / 9.7 / -,
+// 1,500 16.5 / 12.8 / -, 5,000 26 / 20 / 39, 10,000 31 / 21 / 32, 23,000
+// (p = 8) 41 / 34 / 22, 30,000 (p = 3) 21 / 20 / 12, 1e5 (p = 12)
+// 220 / 158 / 115.  Members of an ensemble share a launch and fill the chip
+// together: one thread (256 crystals, k_l2p / 1 thread: 1,700 / 726 us).
 constexpr int64_t kL2pF32Ions = 16384;
 
 // the slots [s0, s1) of the leaves that begin in window b; false if none does
@@ -1424,31 +1427,36 @@ __global__ void __launch_bounds__(kSlotThreads) k_l2p_f64(
     }
 }
 
-// L2P in FP32 for larger crystals (p <= 15): a thread per ion as in k_l2p_f64,
-// the leaf's, its parent's and grandparent's derived expansions (nlev of them)
-// once per block for all the leaves that share them, as one float4 (phi, grad)
-// per coefficient.  With 8 lanes to an ion (k_l2p) a recurrence step served
-// four ions, each leaf derived its ancestors' expansions anew and leaves of
-// few ions left most of a block idle.  Every sum is formed as there: the
-// diagonals by the same tree of products, "lane" g = 0 .. 7 of an ion adds
-// columns g and p - g of every level in turn, and the eight sums join pairwise
-// (0 + 4, 2 + 6, ...), so the fields are the same bit for bit.
+// L2P in FP32 (p <= 15): G = 1 or 4 threads per ion, a block for the ions of a
+// window of sorted slots as in k_l2p_f64; the leaf's, its parent's and
+// grandparent's derived expansions (nlev of them) once per block for all the
+// leaves that share them, as one float4 (phi, grad) per coefficient.  With 8
+// lanes to an ion and a block per leaf (k_l2p) a recurrence step served four
+// ions, each leaf derived its ancestors' expansions anew and leaves of few
+// ions left most of a block idle.  Every sum is formed as there: the diagonals
+// by the same tree of products, "lane" g = 0 .. 7 of an ion adds columns g and
+// p - g of every level in turn, and the eight sums join pairwise (0 + 4,
+// 2 + 6, ...), so the fields are the same bit for bit.
 //
 // Bound by the latency of the chains of fused multiply-adds and shared loads
 // at few warps per SM: two columns run side by side (1,500 -> 820 us at 1e6
-// ions, p = 12, with the blocks of 64 threads and 36 KB it started from), and
-// a block of 128 ions shares more ancestors than two of 64 (820 -> 700 us;
-// 72 KB a block, as at 36 KB many blocks need a second pass).  In all 1,727
-// -> 700 us at 1e6 ions, 220 -> 115 us at 1e5 (p = 12), 42 -> 22 us at 23,000
-// (p = 8).
+// ions, p = 12, with blocks of 64 threads and 36 KB), and a block of 128 ions
+// shares more ancestors than two of 64 (820 -> 700 us; 72 KB a block, as at 36
+// KB many blocks need a second pass).  In all 1,727 -> 700 us at 1e6 ions,
+// 220 -> 115 us at 1e5 (p = 12), 42 -> 22 us at 23,000 (p = 8).
+// Small crystals lack the ions to fill the chip with one thread each: four,
+// each with two of the eight sums, and blocks of 64 ions for windows of 28, so
+// that nearly all need a single pass (10,000 ions, p = 12: 31 -> 21 us; with
+// blocks of 32 ions 27, with windows of 16 33).
 constexpr int kL2pExp = 64;  // expansions per pass at most
-constexpr int kL2pFThreads = 128, kL2pFWindow = 112;
-// expansions (derived 16 bytes a coefficient, local 4) that fit 72 KB
-inline int l2p_f32_exps(int P) {
-    const int l = 72 * 1024 / (20 * P);
+__host__ __device__ inline constexpr int l2p_f32_threads(int G) { return G == 1 ? 128 : 256; }
+__host__ __device__ inline constexpr int l2p_f32_window(int G) { return G == 1 ? 112 : 28; }
+// expansions (derived 16 bytes a coefficient, local 4) that fit 72 or 56 KB
+inline int l2p_f32_exps(int P, int G) {
+    const int l = (G == 1 ? 72 : 56) * 1024 / (20 * P);
     return l < 8 ? 8 : (l > kL2pExp ? kL2pExp : l);
 }
-inline size_t l2p_f32_smem(int P) { return (size_t)l2p_f32_exps(P) * P * 20 + 16; }
+inline size_t l2p_f32_smem(int P, int G) { return (size_t)l2p_f32_exps(P, G) * P * 20 + 16; }
 
 struct L2pSum {
     float ph, ax, ay, az;
@@ -1519,42 +1527,43 @@ __device__ __forceinline__ void l2p_run2(int p, int m, float2 da, float2 db, flo
     }
 }
 
-__global__ void __launch_bounds__(kL2pFThreads) k_l2p_f32(
-    int64_t n, int D, int p, int ld, int nlev, int emax, const RootCube* root,
+template <int G>
+__device__ __forceinline__ void k_l2p_f32_body(const BlockId& blk, int64_t n, int D, int p, int ld, int nlev, int emax, const RootCube* root,
     const uint32_t* __restrict__ code, const int32_t* __restrict__ cid,
     const int32_t* __restrict__ leaf_of, const int32_t* __restrict__ cstart,
     const int32_t* __restrict__ ccount, const Ion<float>::rec* __restrict__ sorted,
     const int32_t* __restrict__ perm, const float* __restrict__ L,
     const float* __restrict__ near, double* E, double* phi) {
     extern __shared__ float4 l2p_smem[];  // derived [emax][P], then local [emax][P] floats
-    __shared__ int s_row[kL2pExp], s_new[3][kL2pFThreads / 32], s_cnt[kL2pFThreads / 32], s_tot[3];
+    __shared__ int s_row[kL2pExp], s_new[3][l2p_f32_threads(G) / 32], s_cnt[l2p_f32_threads(G) / 32], s_tot[3];
     __shared__ uint16_t s_nm[(kMaxOrder + 1) * (kMaxOrder + 2) / 2];
     __shared__ double s_f[2];
     const int P = (p + 1) * (p + 1), tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int u0 = tid / G, part = tid % G;  // the thread's ion of the pass, and its share
     const int NT = (p + 1) * (p + 2) / 2;
     float4* sD = l2p_smem;
     float* sL = reinterpret_cast<float*>(l2p_smem + emax * P);
-    for (int nn = tid; nn <= p; nn += kL2pFThreads)
+    for (int nn = tid; nn <= p; nn += l2p_f32_threads(G))
         for (int m = 0; m <= nn; ++m) s_nm[nn * (nn + 1) / 2 + m] = (uint16_t)(nn << 8 | m);
     pdl_wait();
     int s0, s1;
-    if (!slot_window(n, blockIdx.x, leaf_of, cstart, ccount, s0, s1, kL2pFWindow)) return;  // uniform
+    if (!slot_window(n, (int)blk.x, leaf_of, cstart, ccount, s0, s1, l2p_f32_window(G))) return;  // uniform
     if (tid == 0) {
         const double sl = root->side / (double)(1 << D);
         s_f[0] = kCoulomb / (sl * sl);
         s_f[1] = kCoulomb / sl;
     }
     for (int p0 = s0; p0 < s1;) {
-        // the pass: at most kL2pFThreads slots whose cells number at most emax
-        const bool live = p0 + tid < s1;
-        const int g = live ? leaf_of[p0 + tid] : -1;
+        // the pass: at most l2p_f32_threads(G) / G slots whose cells number at most emax
+        const bool live = p0 + u0 < s1;
+        const int g = live ? leaf_of[p0 + u0] : -1;
         const uint32_t cl = live ? code[g] : 0xffffffffu;
-        const uint32_t prev = tid == 0 || !live ? 0xffffffffu : code[leaf_of[p0 + tid - 1]];
+        const uint32_t prev = u0 == 0 || !live ? 0xffffffffu : code[leaf_of[p0 + u0 - 1]];
         unsigned bal[3];
         bool head[3];
 #pragma unroll
         for (int lv = 0; lv < 3; ++lv) {
-            head[lv] = live && lv < nlev && (tid == 0 || (prev >> (3 * lv)) != (cl >> (3 * lv)));
+            head[lv] = live && part == 0 && lv < nlev && (u0 == 0 || (prev >> (3 * lv)) != (cl >> (3 * lv)));
             bal[lv] = __ballot_sync(0xffffffffu, head[lv]);
         }
         __syncthreads();  // the previous pass is done with the shared arrays
@@ -1567,17 +1576,17 @@ __global__ void __launch_bounds__(kL2pFThreads) k_l2p_f32(
         for (int lv = 0; lv < 3; ++lv) {
             ord[lv] = __popc(bal[lv] & (0xffffffffu >> (31 - lane))) - 1;
 #pragma unroll
-            for (int w = 0; w < kL2pFThreads / 32 - 1; ++w) ord[lv] += w < wid ? s_new[lv][w] : 0;
+            for (int w = 0; w < l2p_f32_threads(G) / 32 - 1; ++w) ord[lv] += w < wid ? s_new[lv][w] : 0;
             used += ord[lv] + 1;
         }
         const bool in = live && used <= emax;
-        const unsigned inb = __ballot_sync(0xffffffffu, in);
+        const unsigned inb = __ballot_sync(0xffffffffu, in && part == 0);
         if (lane == 0) s_cnt[wid] = __popc(inb);
         __syncthreads();
         int ni = 0;
 #pragma unroll
-        for (int w = 0; w < kL2pFThreads / 32; ++w) ni += s_cnt[w];
-        if (tid == ni - 1)
+        for (int w = 0; w < l2p_f32_threads(G) / 32; ++w) ni += s_cnt[w];
+        if (tid == (ni - 1) * G)
             for (int lv = 0; lv < 3; ++lv) s_tot[lv] = ord[lv] + 1;
         __syncthreads();
         int base[3] = {0, s_tot[0], s_tot[0] + s_tot[1]};
@@ -1590,9 +1599,9 @@ __global__ void __launch_bounds__(kL2pFThreads) k_l2p_f32(
                     lv == 0 ? g : cid[(((1ll << (3 * (D - lv))) - 64) / 7) + (cl >> (3 * lv))];
         __syncthreads();
         for (int e = 0; e < ne; ++e)
-            for (int c = tid; c < P; c += kL2pFThreads) sL[e * P + c] = L[(int64_t)s_row[e] * ld + c];
+            for (int c = tid; c < P; c += l2p_f32_threads(G)) sL[e * P + c] = L[(int64_t)s_row[e] * ld + c];
         __syncthreads();
-        for (int u = tid; u < ne * NT; u += kL2pFThreads) {
+        for (int u = tid; u < ne * NT; u += l2p_f32_threads(G)) {
             const int e = u / NT, nm = s_nm[u - e * NT];
             float4* d = sD + e * P;
             l2p_derive_entry<float>(p, nm >> 8, nm & 255, sL + e * P, g_tab_f,
@@ -1602,12 +1611,13 @@ __global__ void __launch_bounds__(kL2pFThreads) k_l2p_f32(
         }
         __syncthreads();
         if (in) {
-            const Ion<float>::rec me = sorted[p0 + tid];
+            const Ion<float>::rec me = sorted[p0 + u0];
             int ix, iy, iz;
             demorton3(cl, ix, iy, iz);
-            float vx[8], vy[8], vz[8], vp[8];
+            constexpr int NV = 8 / G;  // of the eight partial sums: part NV .. part NV + NV - 1
+            float vx[NV], vy[NV], vz[NV], vp[NV];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) vx[q] = vy[q] = vz[q] = vp[q] = 0.f;
+            for (int q = 0; q < NV; ++q) vx[q] = vy[q] = vz[q] = vp[q] = 0.f;
 #pragma unroll 1
             for (int lv = 0; lv < nlev; ++lv) {
                 const float4* D4 = sD + (base[lv] + ord[lv]) * P;
@@ -1650,8 +1660,8 @@ __global__ void __launch_bounds__(kL2pFThreads) k_l2p_f32(
                 const float r2 = x * x + y * y + z * z;
                 const float fp1 = lv == 0 ? 1.f : (lv == 1 ? 0.5f : 0.25f), fe1 = fp1 * fp1;
 #pragma unroll
-                for (int q = 0; q < 8; q += 2) {
-                    const int m2 = p - q;
+                for (int r = 0; r < NV; r += 2) {
+                    const int q = part * NV + r, m2 = p - q;
                     L2pSum c0{0.f, 0.f, 0.f, 0.f}, c1{0.f, 0.f, 0.f, 0.f};
                     if (m2 - 1 > q + 1) {
                         l2p_run2(p, q, dg[q], dg[q + 1], z, r2, D4, c0, c1);
@@ -1662,36 +1672,64 @@ __global__ void __launch_bounds__(kL2pFThreads) k_l2p_f32(
                         if (q + 1 <= m2 - 1) l2p_run(p, q + 1, dg[q + 1], z, r2, D4, c1);
                     }
                     // level units -> leaf units: phi / 2^lv, E / 4^lv (exact)
-                    vp[q] += fp1 * c0.ph;
-                    vx[q] -= fe1 * c0.ax;
-                    vy[q] -= fe1 * c0.ay;
-                    vz[q] -= fe1 * c0.az;
-                    vp[q + 1] += fp1 * c1.ph;
-                    vx[q + 1] -= fe1 * c1.ax;
-                    vy[q + 1] -= fe1 * c1.ay;
-                    vz[q + 1] -= fe1 * c1.az;
+                    vp[r] += fp1 * c0.ph;
+                    vx[r] -= fe1 * c0.ax;
+                    vy[r] -= fe1 * c0.ay;
+                    vz[r] -= fe1 * c0.az;
+                    vp[r + 1] += fp1 * c1.ph;
+                    vx[r + 1] -= fe1 * c1.ax;
+                    vy[r + 1] -= fe1 * c1.ay;
+                    vz[r + 1] -= fe1 * c1.az;
                 }
             }
-            auto join = [](const float (&v)[8]) {
-                return ((v[0] + v[4]) + (v[2] + v[6])) + ((v[1] + v[5]) + (v[3] + v[7]));
+            // every lane of the ion gets the sum
+            auto join = [&](float (&v)[NV]) {
+                if constexpr (G == 1) {
+                    return ((v[0] + v[4]) + (v[2] + v[6])) + ((v[1] + v[5]) + (v[3] + v[7]));
+                } else {
+                    const unsigned mask = 0xfu << (lane & ~3);
+#pragma unroll
+                    for (int off = 2; off > 0; off >>= 1)
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) v[q] += __shfl_xor_sync(mask, v[q], off, 4);
+                    return v[0] + v[1];
+                }
             };
             float ex = join(vx), ey = join(vy), ez = join(vz), ph = join(vp);
             if (near) {
-                const float* o = near + 4 * (int64_t)(p0 + tid);
+                const float* o = near + 4 * (int64_t)(p0 + u0);
                 ex += o[0];
                 ey += o[1];
                 ez += o[2];
                 ph += o[3];
             }
             const float tE = (float)s_f[0], tP = (float)s_f[1];
-            const int i = perm[p0 + tid];
-            E[i] = (double)(tE * ex);
-            E[n + i] = (double)(tE * ey);
-            E[2 * n + i] = (double)(tE * ez);
-            if (phi) phi[i] = (double)(tP * ph);
+            const int i = perm[p0 + u0];
+            if constexpr (G == 1) {
+                E[i] = (double)(tE * ex);
+                E[n + i] = (double)(tE * ey);
+                E[2 * n + i] = (double)(tE * ez);
+                if (phi) phi[i] = (double)(tP * ph);
+            } else {
+                const float v = part == 0 ? tE * ex : part == 1 ? tE * ey : part == 2 ? tE * ez : tP * ph;
+                double* to = part < 3 ? E + part * n : phi;
+                if (to) to[i] = (double)v;
+            }
         }
         p0 += ni;
     }
+}
+
+template <int G>
+__global__ void __launch_bounds__(l2p_f32_threads(G)) k_l2p_f32(
+    int64_t n, int D, int p, int ld, int nlev, int emax, const RootCube* root,
+    const uint32_t* __restrict__ code, const int32_t* __restrict__ cid,
+    const int32_t* __restrict__ leaf_of, const int32_t* __restrict__ cstart,
+    const int32_t* __restrict__ ccount, const Ion<float>::rec* __restrict__ sorted,
+    const int32_t* __restrict__ perm, const float* __restrict__ L,
+    const float* __restrict__ near, double* E, double* phi) {
+    k_l2p_f32_body<G>(solo_block(), n, D, p, ld, nlev, emax, root, code, cid, leaf_of, cstart, ccount,
+                      sorted, perm, L, near, E, phi);
 }
 
 // Direct ancestor local expansions (PT_EXPAND_DIRECT): as k_l2p, but every
@@ -1814,7 +1852,7 @@ void launch_p2p<double>(int D, int64_t leaves, int grid, bool phi, Workspace& ws
 
 template <typename T>
 static cudaError_t run_fmm(int64_t n, int D, int phases, Workspace& ws, bool use_tc, double* E,
-                           double* phi, cudaStream_t s, cudaEvent_t* ev) {
+                           double* phi, cudaStream_t s, cudaEvent_t* ev, bool alone) {
     const int p = ws.p, P = ws.P;
     DenseLayout dl = dense_layout(D);
     T* M = (T*)ws.M;
@@ -2014,14 +2052,16 @@ static cudaError_t run_fmm(int64_t n, int D, int phases, Workspace& ws, bool use
                        (const int32_t*)ws.ccount, (const Ion<double>::rec*)ws.sorted,
                        (const int32_t*)ws.perm, (const double*)ws.L,
                        (const double*)(nf ? ws.near : nullptr), E, phi);
-    else if (far && sizeof(T) == 4 && p <= 15 && n >= kL2pF32Ions)
-        e = launch_pdl(k_l2p_f32, dim3((unsigned)((n + kL2pFWindow - 1) / kL2pFWindow)),
-                       dim3(kL2pFThreads), l2p_f32_smem(P), s, n, D, p, ws.ld, l2p_levels,
-                       l2p_f32_exps(P), (const RootCube*)ws.root, (const uint32_t*)ws.code,
+    else if (far && sizeof(T) == 4 && p <= 15) {
+        const int G = !alone || n >= kL2pF32Ions ? 1 : 4, w = l2p_f32_window(G);
+        e = launch_pdl(G == 1 ? k_l2p_f32<1> : k_l2p_f32<4>, dim3((unsigned)((n + w - 1) / w)),
+                       dim3(l2p_f32_threads(G)), l2p_f32_smem(P, G), s, n, D, p, ws.ld, l2p_levels,
+                       l2p_f32_exps(P, G), (const RootCube*)ws.root, (const uint32_t*)ws.code,
                        (const int32_t*)ws.cid, (const int32_t*)ws.leaf_of, (const int32_t*)ws.cstart,
                        (const int32_t*)ws.ccount, (const Ion<float>::rec*)ws.sorted,
                        (const int32_t*)ws.perm, (const float*)ws.L,
                        (const float*)(nf ? ws.near : nullptr), E, phi);
+    }
     else
         e = launch_pdl(p <= 15 ? k_l2p<T, 8> : k_l2p<T, 16>, dim3(leaf_grid), dim3(kL2pThreads),
                        0, s, n, D, p, ws.ld, far,
@@ -2039,14 +2079,14 @@ static cudaError_t run_fmm(int64_t n, int D, int phases, Workspace& ws, bool use
 }
 
 cudaError_t launch_fmm_phased(int64_t n, int D, int phases, Workspace& ws, bool use_tc, double* E,
-                              double* phi, cudaStream_t s, cudaEvent_t* ev) {
-    if (ws.fp64) return run_fmm<double>(n, D, phases, ws, false, E, phi, s, ev);
-    return run_fmm<float>(n, D, phases, ws, use_tc, E, phi, s, ev);
+                              double* phi, cudaStream_t s, cudaEvent_t* ev, bool alone) {
+    if (ws.fp64) return run_fmm<double>(n, D, phases, ws, false, E, phi, s, ev, alone);
+    return run_fmm<float>(n, D, phases, ws, use_tc, E, phi, s, ev, alone);
 }
 
 cudaError_t launch_fmm(int64_t n, int D, int phases, Workspace& ws, bool use_tc, double* E,
                        double* phi, cudaStream_t s) {
-    return launch_fmm_phased(n, D, phases, ws, use_tc, E, phi, s, nullptr);
+    return launch_fmm_phased(n, D, phases, ws, use_tc, E, phi, s, nullptr, true);
 }
 
 // M2M into level l (mode 0) or L2L into level l (mode 1) of a small level of
@@ -2222,7 +2262,9 @@ cudaError_t upload_harmonic_tables() {
                                  kSlotThreads * p2m_f64_stride(pmax) * (int)sizeof(double));
     // (the largest over the orders: fewer leaves above the order where 16 fit)
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_l2p_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
+        e = cudaFuncSetAttribute(k_l2p_f32<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_l2p_f32<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
     for (auto f : {k_l2p_f64<true>, k_l2p_f64<false>})
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 104 * 1024);
@@ -2274,6 +2316,13 @@ struct L2pJoin {
         k_l2p_body<float, 8>(b, a...);
     }
 };
+template <int G>
+struct L2pSlotJoin {
+    template <class... A>
+    __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const {
+        k_l2p_f32_body<G>(b, a...);
+    }
+};
 
 cudaError_t join_fmm(JoinCtx& c) {
     cudaError_t e = join_kernel<P2mJoin, kP2mThreads, 3>(c, k_p2m<float>);
@@ -2281,6 +2330,8 @@ cudaError_t join_fmm(JoinCtx& c) {
     if (e == cudaSuccess) e = join_kernel<ShiftJoin, kShThreads, 3>(c, k_shift_rows<float, 0>);
     if (e == cudaSuccess) e = join_kernel<P2pJoin, kNfThreads, 1>(c, k_p2p<float>);
     if (e == cudaSuccess) e = join_kernel<L2pJoin, kL2pThreads, 7>(c, k_l2p<float, 8>);
+    if (e == cudaSuccess) e = join_kernel<L2pSlotJoin<4>, l2p_f32_threads(4), 6>(c, k_l2p_f32<4>);
+    if (e == cudaSuccess) e = join_kernel<L2pSlotJoin<1>, l2p_f32_threads(1), 6>(c, k_l2p_f32<1>);
     return e;
 }
 

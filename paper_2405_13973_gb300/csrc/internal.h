@@ -241,9 +241,10 @@ cudaError_t upload_harmonic_tables();
 cudaError_t launch_fmm(int64_t n, int D, int phases, Workspace& ws, bool use_tc, double* E,
                        double* phi, cudaStream_t s);
 // As launch_fmm; if ev is not null, records ev[0] after the upward pass,
-// ev[1] after M2L/L2L and ev[2] after L2P/P2P.
+// ev[1] after M2L/L2L and ev[2] after L2P/P2P.  alone: not a member of an
+// ensemble.
 cudaError_t launch_fmm_phased(int64_t n, int D, int phases, Workspace& ws, bool use_tc, double* E,
-                              double* phi, cudaStream_t s, cudaEvent_t* ev);
+                              double* phi, cudaStream_t s, cudaEvent_t* ev, bool alone);
 // Interaction counts of the last tree (synchronises s).  out[8] = {n, D,
 // leaves, cells at levels >= 2, M2L pairs, P2P pairs (ordered, i != j),
 // L2L shifts, M2M shifts}.
