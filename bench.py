@@ -146,24 +146,26 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
-def launches_per_step(depth: int, precision: str, schedule: str = "tiles") -> int:
+def launches_per_step(depth: int, precision: str, schedule: str = "tiles", n: int = 10000) -> int:
+    """Kernels of one cooled step (FP64: of the default schedule)."""
     tc = precision in ("tf32x3", "bf16x3")
-    # drift + cube, keys, scatter, leaf gather, P2P, L2P, kick; the leaf and
-    # cell scans: one launch together while both fit one block (depth <= 5),
-    # else three each
-    k = 7 + (1 if depth <= 5 else 6)
-    if depth >= 2:
-        if tc:
-            m2m = max(depth - 3, 0)          # P2M covers the leaves and their parents
-            k += 1 + 2 * m2m                 # P2M; M2M and its reduction per level
-            if schedule == "pairs":          # counts, scans, pairs, M2L, pair reduction
-                k += 5 + max(depth - 3, 0)   # (+ one memset node); L2L per level
-            else:                            # plan, items, M2L, tile reduction; L2L per level
-                k += 4 + max(depth - 3, 0)   # down to the leaves' parents
-            k += 1 if precision == "bf16x3" else 0   # split of M into bf16 pieces
-        else:
-            k += 1 + (depth - 2)             # P2M, M2M per level
-            k += depth - 1                   # M2L (+ folded L2L) per level
+    # drift + cube, keys, scans, scatter, leaf gather (up to 2,048 ions one
+    # launch; the leaf and cell scans one launch up to depth 5, else three
+    # each), then photon kicks, P2P, L2P, kick
+    k = 4 + (1 if n <= 2048 and depth <= 5 else 5 if depth <= 5 else 10)
+    if depth < 2:
+        return k
+    k += 1                                   # P2M (tensor cores: and the leaves' parents)
+    if tc:
+        m2m = max(depth - 3, 0)
+        k += m2m if m2m <= 1 else 1 + 2 * (m2m - 1)  # level 2; M2M and its reduction above
+        k += 5                               # counts, scan, pairs | bitmaps, lists, items; M2L; sums
+        k += max(depth - 4, 0)               # L2L down to the leaves' grandparents
+        k += 1 if precision == "bf16x3" and depth >= 5 else 0  # split of M into bf16 pieces
+    else:
+        k += 5 + 2 * (depth - 2)             # counts, scan, pairs, M2L, sums; M2M, L2L per level
+        if precision == "fp64":
+            k += 2 * depth - 3               # slices per level, the parents' digits
     return k
 
 
@@ -365,9 +367,10 @@ def sweep_reference(pt, torch, w, n_sample=512):
     return Eo, idx, f"FP64 oracle direct sum at {n_sample} sampled ions"
 
 
-def m2l_peak(precision, pk, pk_src):
+def m2l_peak(precision, pk, pk_src, schedule=""):
     """Roof of the M2L kernel for a precision: (peak TFLOP/s of FP32-accurate
-    (or FP64) products, bound, note)."""
+    (or FP64) products, bound, note).  schedule: chosen explicitly, which
+    keeps FP64 on the CUDA cores."""
     if precision == "tf32x3":
         return (pk["bf16_tflops"] * TF32_OVER_BF16 / 3.0, "tensor",
                 f"TF32 rate / 3 (3 products per FP32-accurate product), from {pk_src} bf16 x "
@@ -377,7 +380,10 @@ def m2l_peak(precision, pk, pk_src):
                 f"{pk_src} bf16 rate / 6 (6 products per FP32-accurate product)")
     if precision == "fp32":
         return FP32_ALU_TFLOPS, "alu", "152 SMs x 128 FP32 lanes x 2 flop x 2.07 GHz"
-    return FP64_TFLOPS, "alu", "nominal dense FP64"
+    if schedule:
+        return FP64_TFLOPS, "alu", "nominal dense FP64"
+    return (pk["bf16_tflops"] / 28.0, "tensor",
+            f"{pk_src} bf16 rate / 28 (28 products of 8-bit digits per FP64 product)")
 
 
 def force_eval_point(pt, torch, w, p, precision, steps, flush, ref=None, warmup=1, schedule=""):
@@ -422,8 +428,8 @@ def force_eval_point(pt, torch, w, p, precision, steps, flush, ref=None, warmup=
         pairs = plan.stats()["m2l_pairs"]
         if kms > 0 and pairs > 0:
             pk, pk_src = peaks()
-            peak, bound, _ = m2l_peak(precision, pk, pk_src)
-            if plan.m2l_schedule == "rotation":
+            peak, bound, _ = m2l_peak(precision, pk, pk_src, schedule)
+            if schedule == "rotation":
                 # rotate to the z axis, translate along z, rotate back:
                 # 2 sum_n (2n+1)^2 + sum_m (p+1-m)^2 (twice for m > 0) multiply-adds
                 macs = (2 * sum((2 * k + 1) ** 2 for k in range(p + 1)) +
@@ -711,7 +717,7 @@ def main():
             else "M2L kernels (k_m2l_simt, all levels)"
         roof["kernel_ms"] = kern["m2l_kernel"]
         roof["phase_achieved"] = m2l_flops / (ph["m2l"] * 1e-3) / 1e12
-        peak, bound, note = m2l_peak(args.precision, pk, pk_src)
+        peak, bound, note = m2l_peak(args.precision, pk, pk_src, args.schedule)
         roof.update(bound=bound, peak_note=note)
         roof.update(achieved=achieved, peak=peak, unit="TFLOP/s", frac=achieved / peak,
                     work=f"2 P^2 x {stats['m2l_pairs']} M2L translations per launch",
@@ -755,7 +761,7 @@ def main():
            "latency_ms": {"p50": float(np.percentile(ms, 50)), "p99": float(np.percentile(ms, 99)),
                           "max": float(max(ms))},
            "stats": stats, "roofline": roof, "clocks": clk,
-           "gpu_launches": launches_per_step(depth, args.precision, schedule) * args.steps,
+           "gpu_launches": launches_per_step(depth, args.precision, schedule, n) * args.steps,
            "wall_s_timed_region": t_wall}
 
     # the plain FP64 GPU path beside it (same workload, fewer steps)

@@ -50,7 +50,12 @@ typedef enum {
 
 /* Arithmetic of the FMM (positions, velocities and the push are FP64 in
  * every mode).
- *   PT_FP64          : every FMM stage in FP64 on the CUDA cores.
+ *   PT_FP64          : every FMM stage in FP64; M2M, M2L and L2L on the
+ *                      tensor cores as exact products of 8-bit digits (seven
+ *                      per value, scaled by the row's largest; errors of a
+ *                      few 1e-16 of a row's norm) unless a schedule is chosen
+ *                      (fmm_plan_set_m2l_schedule) or their memory is short:
+ *                      then on the CUDA cores.
  *   PT_MIXED_TF32X3  : P2M/L2P/P2P in FP32 on the CUDA cores; M2M, M2L and
  *                      L2L on the tensor cores (tcgen05, operands split into
  *                      TF32 hi + lo, three products, FP32 accumulation in
@@ -150,14 +155,17 @@ int fmm_plan_set_expansion(fmm_plan plan, int mode);
  *                    translation (7.3k instead of 28.6k at p = 12).
  * Default: PT_M2L_PAIRS for the tensor-core precisions up to n_max = 65536;
  * PT_M2L_ROTATION for FP64 and PT_M2L_PAIRS for FP32 up to n_max = 262144;
- * PT_M2L_TILES above.  Selecting another schedule allocates what it needs.
+ * PT_M2L_TILES above (the names of the CUDA-core kernels: an FP64 plan whose
+ * schedule was never chosen runs the pair work list on the tensor cores, above
+ * 262144 ions in batches of targets).  Choosing a schedule, also the default's
+ * name, runs it as described here, and allocates what it needs.
  * Errors: PT_ERR_ARG, PT_ERR_UNSUPPORTED (rotation on the tensor-core
  * precisions or beyond p = 16), PT_ERR_OOM, PT_ERR_CUDA. */
 #define PT_M2L_TILES 0
 #define PT_M2L_PAIRS 1
 #define PT_M2L_ROTATION 2
 int fmm_plan_set_m2l_schedule(fmm_plan plan, int schedule);
-/* CTAs of the plan's persistent tensor-core M2L kernel: 0 (default) one per
+/* CTAs of the plan's persistent tensor-core M2L kernel (FP64's included): 0 (default) one per
  * SM, else at most `ctas`, so that the M2L kernels of several plans stepped
  * together (an ensemble) can run side by side.  Results do not depend on it:
  * every work item is computed by one CTA whatever the grid.  Errors:
@@ -463,7 +471,8 @@ int pt_potential_temperature(fmm_plan plan, const pt_state* state, const pt_stat
  * control by memory budget.  The paper has no counterpart (a service of the
  * library, like pt_energy_noalloc).
  *   plan_bytes     : receives the plan's own workspace (octree, expansions,
- *                    work list and partial slabs), at 512-byte granularity.
+ *                    work list and partial slabs; FP64: the digits and the
+ *                    batches' pool too), at 512-byte granularity.
  *   operator_bytes : receives the translation operators, which all plans of
  *                    one (device, p, precision) share: counted once.
  * Errors: PT_ERR_ARG (as fmm_plan_create), PT_ERR_UNSUPPORTED. */

@@ -884,15 +884,15 @@ static cudaError_t simt_pairs(int64_t n, int D, Workspace& ws, int l2l_last, cud
     for (int l = 3; l <= l2l_last && l <= D; ++l) {
         if constexpr (sizeof(T) == 4) {
             if ((e = launch_f32_l2l(n, D, l, ws, s)) != cudaSuccess) return e;
-            continue;
+        } else {
+            const int64_t cl = (int64_t)1 << (3 * l);
+            const int64_t cells = n < cl ? n : cl;
+            const unsigned g = (unsigned)std::min<int64_t>((cells + 3) / 4, 152 * 16);
+            k_l2l_simt<T><<<g, 128, 4 * P * sizeof(T), s>>>(l, P, ws.ld, ws.linfo, ws.code, ws.cid,
+                                                            dl.off[l - 1], (const T*)ws.T_l2l,
+                                                            (T*)ws.L);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
-        const int64_t cl = (int64_t)1 << (3 * l);
-        const int64_t cells = n < cl ? n : cl;
-        const unsigned g = (unsigned)std::min<int64_t>((cells + 3) / 4, 152 * 16);
-        k_l2l_simt<T><<<g, 128, 4 * P * sizeof(T), s>>>(l, P, ws.ld, ws.linfo, ws.code, ws.cid,
-                                                        dl.off[l - 1], (const T*)ws.T_l2l,
-                                                        (T*)ws.L);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
