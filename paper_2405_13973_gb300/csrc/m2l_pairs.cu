@@ -65,6 +65,10 @@ __device__ __forceinline__ int pp_end(const LevelInfo& li, const PpArgs& a) {
     return g1 - li.gbase[2] > a.t1 ? li.gbase[2] + a.t1 : g1;
 }
 
+// offset index of candidate c of a target at (x, y, z)
+__device__ __forceinline__ int pp_offset(int x, int y, int z, int c) {
+    return ((x & 1) + c / 36) * 49 + ((y & 1) + (c / 6) % 6) * 7 + (z & 1) + c % 6;
+}
 // source of candidate c of the target at (x, y, z) of level l, or -1
 __device__ __forceinline__ int pp_source(const PpArgs& a, int l, int x, int y, int z, int c,
                                          int* op) {
@@ -135,10 +139,15 @@ __device__ __forceinline__ void k_pp_scan_body(const BlockId& blk, int D, int t0
     const int nt = max(0, min(linfo->gbase[D + 1] - linfo->gbase[2], t1) - t0);
     if (tid == 0) s_carry = 0;
     __syncthreads();
-    for (int c0 = 0; c0 < nt; c0 += kPpScanThreads) {
-        const int i = c0 + tid;
-        const int v = i < nt ? tcount[i] : 0;
-        int x = v;
+    for (int c0 = 0; c0 < nt; c0 += 4 * kPpScanThreads) {
+        int v[4], x = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = c0 + 4 * tid + k;
+            v[k] = i < nt ? tcount[i] : 0;
+            x += v[k];
+        }
+        const int mine = x;
         for (int o = 1; o < 32; o <<= 1) {
             const int y = __shfl_up_sync(0xffffffffu, x, o);
             if (lane >= o) x += y;
@@ -154,7 +163,13 @@ __device__ __forceinline__ void k_pp_scan_body(const BlockId& blk, int D, int t0
             wsum[lane] = w;
         }
         __syncthreads();
-        if (i < nt) tbase[i] = s_carry + (wid > 0 ? wsum[wid - 1] : 0) + x - v;
+        int at = s_carry + (wid > 0 ? wsum[wid - 1] : 0) + x - mine;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = c0 + 4 * tid + k;
+            if (i < nt) tbase[i] = at;
+            at += v[k];
+        }
         __syncthreads();
         if (tid == 0) s_carry += wsum[31];
         __syncthreads();
@@ -162,10 +177,11 @@ __device__ __forceinline__ void k_pp_scan_body(const BlockId& blk, int D, int t0
     const int total = s_carry;
     // offsets: pair bases (scan of the counts) and item bases (scan of the
     // 128-pair runs), 343 entries by the first 11 warps
-    __shared__ int s_pb[344], s_nof;
+    __shared__ int s_pb[344], s_cnt[343], s_nof;
     if (wid < 11) {
         const int o = tid;  // 0 .. 351
         const int c = o < 343 ? ocnt[o] : 0;
+        if (o < 343) s_cnt[o] = c;
         const int runs = (c + kPairRows - 1) / kPairRows;
         // each offset's pairs start on a multiple of 128 rows, so that every
         // work item covers whole 128-row blocks of the partial array
@@ -236,9 +252,9 @@ __device__ __forceinline__ void k_pp_scan_body(const BlockId& blk, int D, int t0
     __syncthreads();
     const bool over =
         (int64_t)total > slot_cap || (int64_t)s_pb[343] > rows_cap || s_ibase[343] > item_cap;
-    for (int o = tid; o < 344; o += kPpScanThreads) {
-        const int c = o < 343 ? ocnt[o] : 0;
-        for (int k = 0; !over && k * kPairRows < c; ++k) {
+    for (int o = wid; o < 343; o += kPpScanThreads / 32) {  // a warp per offset
+        const int c = s_cnt[o];
+        for (int k = lane; !over && k * kPairRows < c; k += 32) {
             M2lPairItem it;
             it.op = o;
             it.begin = s_pb[o] + k * kPairRows;
@@ -246,10 +262,12 @@ __device__ __forceinline__ void k_pp_scan_body(const BlockId& blk, int D, int t0
             it.pad = 0;
             items[s_ibase[o] + k] = it;
         }
-        // counts read: zero them and the fill counters for the next work
-        // list (zeroed once at allocation)
-        ocnt[o] = 0;
-        ofill[o] = 0;
+    }
+    // counts read: zero them and the fill counters for the next work list
+    // (zeroed once at allocation)
+    if (tid < 343) {
+        ocnt[tid] = 0;
+        ofill[tid] = 0;
     }
 }
 __global__ void __launch_bounds__(kPpScanThreads) k_pp_scan(int D, int t0, int t1,
@@ -267,19 +285,42 @@ __global__ void __launch_bounds__(kPpScanThreads) k_pp_scan(int D, int t0, int t
 // offset's list (an atomic counter: the order of the pairs inside an
 // offset's list does not change any result, every product row being
 // computed alone), with its source and its slot (the target's slot base plus
-// the rank of the offset among the target's present ones).
+// the rank of the offset among the target's present ones).  A block counts its
+// pairs per offset from the presence words first and reserves each offset's
+// run with one addition: with an addition per pair the few hundred counters
+// bounded the kernel (us, before -> after: 1e5 ions, 3.4 M pairs 226 -> 65;
+// 1e6 ions (p = 8), a batch of 4.3 M pairs 143 -> 70; 23,457 ions 29 -> 12; 10,000 ions
+// 15 -> 11; 300 ions no slower).
 __device__ __forceinline__ void k_pp_fill_body(const BlockId& blk, PpArgs a, const uint32_t* tmask,
                                                          const int* tbase, const int* obase,
                                                          int* ofill, const M2lPairHdr* hdr,
                                                          M2lPair* pairs, int* tpair) {
     pdl_wait();
     __shared__ LevelInfo li;
+    __shared__ int s_at[343];  // per offset: the block's pairs, then where its next one goes
     stage_linfo(a.linfo, &li);
+    for (int i = threadIdx.x; i < 343; i += blockDim.x) s_at[i] = 0;
     __syncthreads();
     if (hdr->overflow) return;
     const int lane = threadIdx.x & 31;
     const int g0 = li.gbase[2] + a.t0, g1 = pp_end(li, a);
     const int wpb = blockDim.x >> 5;
+    for (int g = g0 + (int)blk.x * wpb + (threadIdx.x >> 5); g < g1; g += (int)blk.nx * wpb) {
+        int x, y, z;
+        demorton3(a.code[g], x, y, z);
+#pragma unroll
+        for (int w = 0; w < kPpWords; ++w)
+            if ((tmask[(int64_t)(g - g0) * kPpWords + w] >> lane) & 1u) {
+                const int op = pp_offset(x, y, z, 32 * w + lane);
+                atomicAdd(&s_at[a.mirror && op > 171 ? 342 - op : op], 1);
+            }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 343; i += blockDim.x) {
+        const int c = s_at[i];
+        if (c > 0) s_at[i] = obase[i] + atomicAdd(&ofill[i], c);
+    }
+    __syncthreads();
     for (int g = g0 + (int)blk.x * wpb + (threadIdx.x >> 5); g < g1; g += (int)blk.nx * wpb) {
         const int t = g - g0;
         const int l = pp_level(li, a.D, g);
@@ -300,7 +341,7 @@ __device__ __forceinline__ void k_pp_fill_body(const BlockId& blk, PpArgs a, con
                     op = 342 - op;
                     pr.src |= kPairMirror;
                 }
-                const int pidx = obase[op] + atomicAdd(&ofill[op], 1);
+                const int pidx = atomicAdd(&s_at[op], 1);
                 pairs[pidx] = pr;
                 tpair[pr.slot] = mir ? ~pidx : pidx;
             }
