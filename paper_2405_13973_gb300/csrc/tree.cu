@@ -512,7 +512,7 @@ __global__ void k_leaf_gather(const double* __restrict__ x, const double* __rest
 // (DRIFT, a time step), root cube, keys, histogram, both scans, scatter and
 // gather, on one cluster of kScanCtas CTAs with cluster barriers between the
 // stages.  Up to kSmallTreeIons ions the five launches are all latency (300
-// ions: 23 us of kernels and their gaps); beyond, the FP64 divisions of keys
+// ions: 25 us with their gaps, 22.7 in one launch); beyond, the FP64 divisions of keys
 // and gather on eight SMs take longer than the launches saved.  What another
 // CTA wrote in this launch is read through L2.  Every stage computes exactly
 // what its own kernel does.
