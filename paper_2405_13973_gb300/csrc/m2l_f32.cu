@@ -220,7 +220,11 @@ __global__ void __launch_bounds__(kF32MaxThreads) k_f32_gemm(const __grid_consta
             for (int u = tid; u < ROWS * 8; u += nthr) {
                 const int r = u >> 3, q = u & 7;
                 const float* src = s_src[lbuf][r];
-                cp_async16(sA + r * kAStride + 4 * q, src ? src + lk * 32 + 4 * q : a.M, src ? 16u : 0u);
+                // zeros beyond column P: the rows' padding takes no part, whatever it
+                // holds (a row with a NaN leaves NaN there, below)
+                const int left = max(0, min(4, a.P - (lk * 32 + 4 * q)));
+                cp_async16(sA + r * kAStride + 4 * q, src ? src + lk * 32 + 4 * q : a.M,
+                           src ? 4u * (uint32_t)left : 0u);
             }
             const int rowq = a.nc / 4;  // 16-byte units per K row
             const float* B = a.ops + (int64_t)f32_op<MODE>(lw, lterm) * a.op_vals +
@@ -308,7 +312,7 @@ __global__ void __launch_bounds__(kF32MaxThreads) k_f32_gemm(const __grid_consta
             const int row = r * kRowGroups + rg;
             if (row >= w.rows) continue;
             float* o = (MODE == F32_TILE || MODE == F32_L2L ? a.L : a.out) + (int64_t)(w.row0 + row) * a.ld;
-            // columns P .. ld - 1 hold zeros (zero operator columns)
+            // columns P .. ld - 1: zeros (zero operator columns) or NaN, read by nothing
             if (n0 < a.ld) {
                 float4 v;
                 unpack2(acc[r][0], v.x, v.y);

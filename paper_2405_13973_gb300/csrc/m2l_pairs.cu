@@ -533,7 +533,7 @@ __global__ void __launch_bounds__(320) k_pp_reduce_seq(int D, int ld, int stride
         float* o = L + (int64_t)(g0 + t) * ld + 4 * u;
         if (4 * u + 4 <= width) {
             *reinterpret_cast<float4*>(o) = v;
-        } else {  // the padding columns stay zero
+        } else {  // (the padding columns are not written)
             o[0] = v.x;
             if (4 * u + 1 < width) o[1] = v.y;
             if (4 * u + 2 < width) o[2] = v.z;
