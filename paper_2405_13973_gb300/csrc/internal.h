@@ -378,7 +378,7 @@ constexpr int kMhMaxChunks = 64;   // source ranges per move
 constexpr int kMhProp = 7;         // per ion: b, U(b) - U(a), the window of dE, the accept uniform
 // doubles of device scratch
 constexpr size_t mh_scratch_doubles(int64_t n) {
-    return (size_t)kMhProp * n + kMhBatch * kMhMaxChunks + kMhBatch * kMhBatch;
+    return (size_t)kMhProp * n + kMhBatch * kMhMaxChunks + kMhBatch * kMhBatch + 1;
 }
 cudaError_t launch_mh_scans(int64_t n, double* x, double* y, double* z, const double* q,
                             const MhParams& mp, int64_t scan0, int64_t n_scans,

@@ -24,11 +24,14 @@
 //   C_jk = k_e q_k q_j [(1/|b_k - b_j| - 1/|a_k - b_j|) - (1/|b_k - a_j| - 1/|a_k - a_j|)],
 // and one warp then takes the decisions in order, adding row j of C to the
 // later ones whenever move j is kept.  Between two kept moves nothing
-// changes, so it goes from one kept move to the next.  Three kernels:
+// changes, so it goes from one kept move to the next.  A batch with a move too
+// close to its threshold for the rounding of these sums is decided move after
+// move, each summed at its turn.  Three kernels:
 //   k_mh_draw    once per scan: every ion's proposal (an ion moves once a
 //                scan, so its own position is the scan's start's), U(b) - U(a)
 //                and the window of dE around -k_B T ln u outside of which the
-//                decision is certain without the exponential;
+//                decision is certain without the exponential (inside, the
+//                batch is decided move after move);
 //   k_mh_sums    per batch: the sums and C (FP64, bound by the FP64 units:
 //                2 rsqrt per pair);
 //   k_mh_decide  per batch: one block, the decisions by its first warp.
@@ -106,12 +109,18 @@ __device__ __forceinline__ double mh_inv(double dx, double dy, double dz) {
     return rsqrt(fma(dz, dz, fma(dy, dy, dx * dx)));
 }
 
+// the high word of a magnitude: ordered as the magnitudes are
+__device__ __forceinline__ unsigned mh_high(double v) {
+    return (unsigned)__double2hiint(v) & 0x7fffffffu;
+}
+
 // blocks [0, sum_blocks): a warp per (move, source range); the rest: a
-// thread per (j, k) of C, j < k
+// thread per (j, k) of C, j < k, and the largest |C| (its high word) into *top
 __global__ void __launch_bounds__(kMhSumThreads) k_mh_sums(
     int64_t n, int64_t i0, int nb, int chunks, int64_t per, int sum_blocks,
     const double* __restrict__ x, const double* __restrict__ y, const double* __restrict__ z,
-    const double* __restrict__ q, double ke, const double* __restrict__ prop, double* part, double* C) {
+    const double* __restrict__ q, double ke, const double* __restrict__ prop, double* part, double* C,
+    unsigned* top) {
     pdl_wait();
     const int lane = threadIdx.x & 31;
     if ((int)blockIdx.x < sum_blocks) {
@@ -133,27 +142,79 @@ __global__ void __launch_bounds__(kMhSumThreads) k_mh_sums(
     }
     const int e = ((int)blockIdx.x - sum_blocks) * kMhSumThreads + threadIdx.x;
     const int j = e / nb, k = e % nb;
-    if (j >= nb || k <= j) return;
-    const int64_t ij = i0 + j, ik = i0 + k;
-    const double ajx = x[ij], ajy = y[ij], ajz = z[ij], akx = x[ik], aky = y[ik], akz = z[ik];
-    const double bjx = prop[ij], bjy = prop[n + ij], bjz = prop[2 * n + ij];
-    const double bkx = prop[ik], bky = prop[n + ik], bkz = prop[2 * n + ik];
-    const double after = mh_inv(bkx - bjx, bky - bjy, bkz - bjz) - mh_inv(akx - bjx, aky - bjy, akz - bjz);
-    const double before = mh_inv(bkx - ajx, bky - ajy, bkz - ajz) - mh_inv(akx - ajx, aky - ajy, akz - ajz);
-    C[j * kMhBatch + k] = ke * q[ik] * (q[ij] * (after - before));
+    double c = 0.0;
+    if (j < nb && k > j) {
+        const int64_t ij = i0 + j, ik = i0 + k;
+        const double ajx = x[ij], ajy = y[ij], ajz = z[ij], akx = x[ik], aky = y[ik], akz = z[ik];
+        const double bjx = prop[ij], bjy = prop[n + ij], bjz = prop[2 * n + ij];
+        const double bkx = prop[ik], bky = prop[n + ik], bkz = prop[2 * n + ik];
+        const double after = mh_inv(bkx - bjx, bky - bjy, bkz - bjz) - mh_inv(akx - bjx, aky - bjy, akz - bjz);
+        const double before = mh_inv(bkx - ajx, bky - ajy, bkz - ajz) - mh_inv(akx - ajx, aky - ajy, akz - ajz);
+        c = ke * q[ik] * (q[ij] * (after - before));
+        C[j * kMhBatch + k] = c;
+    }
+    const unsigned t = __reduce_max_sync(0xffffffffu, mh_high(c));
+    if (lane == 0 && t > 0u) atomicMax(top, t);
+}
+
+// The decisions of a batch, each move summed at its turn by the whole block:
+// the moves kept so far (marked in kept) are made.
+__device__ __noinline__ void mh_one_by_one(int64_t n, int64_t i0, int nb, const double* x,
+                                           const double* y, const double* z,
+                                           const double* __restrict__ q, const MhParams& mp,
+                                           const double* __restrict__ prop, unsigned* kept,
+                                           double* red, unsigned long long* acc_out, double* de_out) {
+    const int tid = threadIdx.x;
+    if (tid < kMhBatch / 32) kept[tid] = 0u;
+    __syncthreads();
+    for (int j = 0; j < nb; ++j) {
+        const double ax = x[i0 + j], ay = y[i0 + j], az = z[i0 + j];
+        const double bx = prop[i0 + j], by = prop[n + i0 + j], bz = prop[2 * n + i0 + j];
+        double s = 0.0;
+        for (int64_t c = tid; c < n; c += kMhDecideThreads) {
+            const int64_t k = c - i0;
+            if (k == j) continue;
+            const bool made = k >= 0 && k < j && ((kept[k >> 5] >> (k & 31)) & 1u);
+            const double xc = made ? prop[c] : x[c], yc = made ? prop[n + c] : y[c],
+                         zc = made ? prop[2 * n + c] : z[c];
+            s = fma(q[c], mh_inv(bx - xc, by - yc, bz - zc) - mh_inv(ax - xc, ay - yc, az - zc), s);
+        }
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((tid & 31) == 0) red[tid >> 5] = s;
+        __syncthreads();
+        if (tid == 0) {
+            double sum = 0.0;
+            for (int w = 0; w < kMhDecideThreads / 32; ++w) sum += red[w];
+            const int64_t i = i0 + j;
+            const double dE = prop[3 * n + i] + mp.ke * q[i] * sum;
+            if (dE < 0.0 || prop[6 * n + i] < pt_exp(-dE / (mp.kb * mp.temp))) {
+                kept[j >> 5] |= 1u << (j & 31);
+                ++*acc_out;
+                *de_out += dE;
+            }
+        }
+        __syncthreads();
+    }
 }
 
 // The decisions of a batch.  Lane l of warp 0 holds moves l + 32 m.
+// With S the largest of the batch's energy changes and of the terms C, a sum
+// of them is within 2^-38 S of the sum without rounding.  A batch with a move
+// that close to its threshold is decided one by one: at the energies of a
+// crystal (S = 1e3 k_B T) one in 1e6, and those where ions coincide or all
+// but (S infinite: infinite terms do not cancel).
 __global__ void __launch_bounds__(kMhDecideThreads) k_mh_decide(
     int64_t n, int64_t i0, int nb, int chunks, double* x, double* y, double* z,
-    const double* __restrict__ q, MhParams mp, const double* __restrict__ prop,
-    const double* __restrict__ part, const double* __restrict__ C, unsigned long long* acc_out,
-    double* de_out) {
+    const double* __restrict__ q, const __grid_constant__ MhParams mp,
+    const double* __restrict__ prop, const double* __restrict__ part,
+    const double* __restrict__ C, unsigned* top, unsigned long long* acc_out, double* de_out) {
     extern __shared__ double sC[];  // [nb][kMhBatch]
-    __shared__ double s_sum[kMhBatch];
+    __shared__ double s_sum[kMhBatch], s_red[kMhDecideThreads / 32];
     __shared__ unsigned s_kept[kMhBatch / 32];
+    __shared__ bool s_anew;
     pdl_wait();
     const int tid = threadIdx.x, lane = tid & 31;
+    const unsigned top_c = *top;
 #pragma unroll 8
     for (int e = tid; e < nb * kMhBatch; e += kMhDecideThreads)
         if (e % kMhBatch > e / kMhBatch) sC[e] = C[e];
@@ -166,39 +227,46 @@ __global__ void __launch_bounds__(kMhDecideThreads) k_mh_decide(
     if (tid < 32) {
         constexpr int NM = kMhBatch / 32;
         double E[NM], lo[NM], hi[NM];  // dE with the moves kept so far
+        unsigned t = top_c;
 #pragma unroll
         for (int m = 0; m < NM; ++m) {
             const int k = lane + 32 * m;
-            const int64_t i = i0 + k;
-            const bool live = k < nb;
-            E[m] = live ? prop[3 * n + i] + mp.ke * q[i] * s_sum[k] : 0.0;
-            lo[m] = live ? prop[4 * n + i] : -INFINITY;
-            hi[m] = live ? prop[5 * n + i] : -INFINITY;
+            E[m] = k < nb ? prop[3 * n + i0 + k] + mp.ke * q[i0 + k] * s_sum[k] : 0.0;
+            t = max(t, mh_high(E[m]));
+        }
+        t = __reduce_max_sync(0xffffffffu, t);
+        const double slack = t < 0x7ff00000u ? 0x1p-38 * __hiloint2double((int)t, -1) : (double)INFINITY;
+#pragma unroll
+        for (int m = 0; m < NM; ++m) {
+            const int64_t i = i0 + lane + 32 * m;
+            const bool live = lane + 32 * m < nb;
+            lo[m] = live ? prop[4 * n + i] - slack : 0.0;
+            hi[m] = live ? prop[5 * n + i] + slack : 0.0;
         }
         unsigned long long acc = 0;
         double de_sum = *de_out;
+        bool anew = false;
 #pragma unroll
         for (int m = 0; m < NM; ++m) {
             // the first undecided move of the group that may be kept: the
             // undecided ones before it are not (nothing changed since)
-            unsigned left = 32 * m < nb ? 0xffffffffu : 0u, kept = 0;
-            while (left) {
-                const unsigned may = __ballot_sync(0xffffffffu, E[m] <= hi[m]) & left;
+            const int nl = nb - 32 * m;  // moves left, this group's first
+            unsigned left = nl >= 32 ? 0xffffffffu : nl > 0 ? (1u << nl) - 1u : 0u, kept = 0;
+            while (left && !anew) {
+                const unsigned may = __ballot_sync(0xffffffffu, !(E[m] > hi[m])) & left;
                 const unsigned sure = __ballot_sync(0xffffffffu, E[m] < lo[m]);
                 if (!may) break;
                 const int l = __ffs(may) - 1, j = l + 32 * m;
                 left = l == 31 ? 0u : left & (0xffffffffu << (l + 1));
                 if (!((sure >> l) & 1u)) {
-                    // too close to the threshold: the exponential decides
-                    bool keep = false;
-                    if (lane == l)
-                        keep = E[m] < 0.0 || prop[6 * n + i0 + j] < pt_exp(-E[m] / (mp.kb * mp.temp));
-                    if (!__ballot_sync(0xffffffffu, keep)) continue;
+                    anew = true;
+                    break;
                 }
                 kept |= 1u << l;
                 ++acc;
                 de_sum += __shfl_sync(0xffffffffu, E[m], l);
-                // (the columns up to j are decided: what is added there is unused)
+                // (the columns up to j are decided, those from nb on are no moves:
+                // what is added there is unused)
                 const double* row = sC + j * kMhBatch + lane;
 #pragma unroll
                 for (int mm = m; mm < NM; ++mm) E[mm] += row[32 * mm];
@@ -206,11 +274,16 @@ __global__ void __launch_bounds__(kMhDecideThreads) k_mh_decide(
             if (lane == 0) s_kept[m] = kept;
         }
         if (lane == 0) {
-            *acc_out += acc;
-            *de_out = de_sum;
+            s_anew = anew;
+            *top = 0u;  // for the next batch
+            if (!anew) {
+                *acc_out += acc;
+                *de_out = de_sum;
+            }
         }
     }
     __syncthreads();
+    if (s_anew) mh_one_by_one(n, i0, nb, x, y, z, q, mp, prop, s_kept, s_red, acc_out, de_out);
     if (tid < nb && ((s_kept[tid >> 5] >> (tid & 31)) & 1u)) {
         const int64_t i = i0 + tid;
         x[i] = prop[i];
@@ -228,10 +301,12 @@ cudaError_t launch_mh_scans(int64_t n, double* x, double* y, double* z, const do
     double* prop = scratch;
     double* part = prop + (size_t)kMhProp * n;
     double* C = part + kMhBatch * kMhMaxChunks;
+    unsigned* top = reinterpret_cast<unsigned*>(C + kMhBatch * kMhBatch);
     const int smem = (int)sizeof(double) * kMhBatch * kMhBatch;
     cudaError_t e = cudaFuncSetAttribute(k_mh_decide, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = cudaMemsetAsync(acc_out, 0, sizeof *acc_out, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(de_out, 0, sizeof *de_out, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(top, 0, sizeof *top, s);
     // source ranges of whole warps' worth, about eight warps per SM over the batch
     const int64_t want = (sms * 8 + kMhBatch - 1) / kMhBatch;
     int64_t chunks = std::min<int64_t>(std::min<int64_t>(want, kMhMaxChunks), (n + 31) / 32);
@@ -247,11 +322,11 @@ cudaError_t launch_mh_scans(int64_t n, double* x, double* y, double* z, const do
             const int cb = (nb * nb + kMhSumThreads - 1) / kMhSumThreads;
             e = launch_pdl(k_mh_sums, dim3((unsigned)(sb + cb)), dim3(kMhSumThreads), 0, s, n, i0, nb,
                            (int)chunks, per, sb, (const double*)x, (const double*)y, (const double*)z,
-                           q, mp.ke, (const double*)prop, part, C);
+                           q, mp.ke, (const double*)prop, part, C, top);
             if (e == cudaSuccess)
                 e = launch_pdl(k_mh_decide, dim3(1), dim3(kMhDecideThreads), (size_t)smem, s, n, i0, nb,
                                (int)chunks, x, y, z, q, mp, (const double*)prop, (const double*)part,
-                               (const double*)C, acc_out, de_out);
+                               (const double*)C, top, acc_out, de_out);
         }
     }
     return e;
