@@ -382,8 +382,8 @@ def m2l_peak(precision, pk, pk_src, schedule=""):
         return FP32_ALU_TFLOPS, "alu", "152 SMs x 128 FP32 lanes x 2 flop x 2.07 GHz"
     if schedule:
         return FP64_TFLOPS, "alu", "nominal dense FP64"
-    return (pk["bf16_tflops"] / 28.0, "tensor",
-            f"{pk_src} bf16 rate / 28 (28 products of 8-bit digits per FP64 product)")
+    return (pk["bf16_tflops"] / 34.0, "tensor",
+            f"{pk_src} bf16 rate / 34 (34 products of 8-bit digits per FP64 product)")
 
 
 def force_eval_point(pt, torch, w, p, precision, steps, flush, ref=None, warmup=1, schedule=""):

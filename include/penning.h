@@ -51,11 +51,12 @@ typedef enum {
 /* Arithmetic of the FMM (positions, velocities and the push are FP64 in
  * every mode).
  *   PT_FP64          : every FMM stage in FP64; M2M, M2L and L2L on the
- *                      tensor cores as exact products of 8-bit digits (seven
- *                      per value, scaled by the row's largest; errors of a
- *                      few 1e-16 of a row's norm) unless a schedule is chosen
+ *                      tensor cores from 8-bit digits (seven per value, scaled
+ *                      by the row's largest; 34 of the 49 digit products,
+ *                      each exact; fields rounded no more than by FP64
+ *                      multiply-adds) unless a schedule is chosen
  *                      (fmm_plan_set_m2l_schedule) or their memory is short:
- *                      then on the CUDA cores.
+ *                      then on the CUDA cores by FP64 multiply-adds.
  *   PT_MIXED_TF32X3  : P2M/L2P/P2P in FP32 on the CUDA cores; M2M, M2L and
  *                      L2L on the tensor cores (tcgen05, operands split into
  *                      TF32 hi + lo, three products, FP32 accumulation in

@@ -14,22 +14,33 @@
 //     the largest coefficients of the row;
 //   * digits are exact in f16, digit products exact in FP32, and a sum of
 //     them is exact while it stays below 2^24.  The products of equal i + j
-//     have one weight, so they share an accumulator s_{i+j}, i + j = 0 .. 6:
-//     28 products; i + j >= 7 lies below 2^-53 of the product of the two
-//     maxima.  |s_d| <= ((d - 1) + 1) 2^14 P for d >= 1 stays below 2^24 for
-//     d <= 5 at p = 12 and d <= 3 at p = 16; beyond that bound (which needs
-//     every digit at its limit: 2^20 is what crystals reach) the last bit of
-//     s_d would be rounded, 2^-45 of the product of the maxima or less;
-//   * S = sum_d s_d 2^(8 (6 - d)) is formed in 64-bit integers (its lowest 8
-//     bits rounded away) and written as a double: the FP64 units, two lanes
-//     per clock and SM, take no part.
-// Against a long double sum the result is as good as FP64 multiply-adds
-// (2e-16 .. 2e-15 of the row's norm, p = 4 .. 16).
+//     have one weight, so they share an accumulator s_{i+j}, i + j = 0 .. 7:
+//     34 products;
+//   * S = sum_d s_d 2^(8 (7 - d)) is formed in integers (96 bits) and written
+//     as a double, rounded once: the FP64 units, two lanes per clock and SM,
+//     take no part.
+// Error of one output, in units of the product of the two rows' maxima: the
+// digits' own rounding, 2^-54 of either maximum per coefficient, and the
+// products i + j >= 8 left out, below 2^-57 per coefficient: at worst
+// P 2^-53 (1 + 1/16), the bound of P FP64 multiply-adds of values as large as
+// the maxima.  |s_d| <= d 2^14 P (d >= 1; 6 2^14 P for d = 7), so every sum is
+// exact up to p = 12; at p = 16 those from s_4 on could pass 2^24 with nearly every
+// digit at its limit, and would lose their last bit, 2^-42 (crystals reach 2^20).
+// Measured against long double, one offset's output row: 1e-16 .. 9e-16 of
+// its norm, FP64 multiply-adds 5e-16 .. 2.6e-15 (p = 4 .. 16, 1 to 100 ions a
+// cell, like and unlike charges); coefficients far below the largest of their row are less
+// exact than by multiply-adds (their error is of the row's size).  Far fields
+// of 1,000 to 60,000 ions, relative error of E: 2.4e-16 .. 7.2e-16, by
+// multiply-adds 3.0e-16 .. 8.8e-16.  Without the products i + j = 7 (28 of
+// them, 5.1 ms for the M2L below) E was off by up to 1.5e-14.
+//   * L2L: the parent's L_0, which in a large crystal is many times the rest
+//     of its row, reaches the child's L_0 only; it stays out of the digits and
+//     is added in FP64 (E at depth 4, 12,000 ions, p = 4: 6.1e-16 -> 2.6e-16).
 //
 // One CTA per SM walks the work items (one operator, up to 128 rows):
 //   D[128 rows x N] = sum over K steps of 16, i, j:  A_i[128 x 16] B_j[16 x N],
-// in column chunks of up to 48 outputs so that the seven accumulators (336
-// TMEM columns) leave room for three K steps of A in tensor memory (7 digits
+// in column chunks of up to 48 outputs so that the eight accumulators (384
+// TMEM columns) leave room for two K steps of A in tensor memory (7 digits
 // x 8 columns each).  A comes from tensor memory because with 48 columns a
 // product takes 24 cycles and reading a 4 KB A tile from shared memory 32:
 //   * warps 10..13 (one TMEM lane quarter each) load the rows' digits (one
@@ -39,14 +50,13 @@
 //     packed subtraction) and store them to tensor memory;
 //   * warp 8 brings the operator digits, packed in f16 in the swizzled
 //     K-major shared-memory image, by bulk copies of 32-wide K chunks;
-//   * warp 9 issues the 28 products of a K step;
+//   * warp 9 issues the 34 products of a K step;
 //   * warps 0..7 read the accumulators, release them once the integers are
 //     formed, and write the doubles while the next chunk's products run.
 // Every mbarrier wait is bounded as in m2l_tc.cu.
 // M2L kernel, before (CUDA cores) -> now: 1e5 ions, p = 12, 53.7 ms (rotated
-// translations) -> 5.1; 1e6 ions, p = 8, 640 ms (tiles) -> 15.1.  Bound by the
-// issue of 48-column products and the hand-over of the accumulators (tensor
-// pipe 47 % active).
+// translations) -> 6.1; a field at 1e6 ions, p = 8, 685 ms (tiles) -> 36.7.
+// Bound by the issue of 48-column products and the hand-over of the accumulators.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -68,13 +78,16 @@ constexpr int kChunk = 48;              // output columns per chunk (at most)
 constexpr int kF64Rows = 128;
 constexpr int kSegBytes = kDig * 32;    // digits of one row in a 32-wide K segment
 constexpr int kMaxRing = 5;             // ring slots of digit rows
-constexpr int kAStages = 3;             // K steps of A in tensor memory
-constexpr int kACol0 = kDig * kChunk;   // their first TMEM column
+constexpr int kAcc = kDig + 1;          // accumulators s_0 .. s_7
+constexpr int kAStages = 2;             // K steps of A in tensor memory
+constexpr int kACol0 = kAcc * kChunk;   // their first TMEM column
+static_assert(kACol0 + kAStages * kDig * 8 <= 512, "tensor memory columns");
 constexpr int kBStages = 4;             // 32-wide K chunks of B in shared memory (at most)
 constexpr int kF64Threads = 448;
 constexpr int kF64Ops = 359;            // 343 M2L offsets, 8 M2M, 8 L2L octants
 constexpr int kF64M2M = 343, kF64L2L = 351;
 constexpr int kRowNan = 0x7fffffff;     // exponent of a row with a NaN or infinity
+constexpr int kSumExp = 66;             // a sum S stands for S 2^(exponents - 66): 106 - 8 (12 - 7)
 
 enum F64Mode { F64_PAIR = 0, F64_M2M = 1, F64_L2L = 2 };
 
@@ -95,6 +108,7 @@ struct F64Args {
     const uint32_t* code;
     const int32_t* cid;
     int64_t off_parent;
+    const double* up;          // L2L: L of the parents
     double* out;
     int* err;
 };
@@ -112,8 +126,8 @@ __device__ __forceinline__ void mma_f16_ts(uint32_t dtmem, uint32_t atmem, uint3
         "r"(atmem), "r"(blo), "r"(bhi), "r"(idesc), "n"(ACC)
         : "memory");
 }
-// the 28 products of a K step; MORE = 0: the first of an accumulator
-// overwrites it
+// the 34 products i + j <= 7 of a K step; MORE = 0: the first of an
+// accumulator overwrites it
 template <int MORE>
 __device__ __forceinline__ void f64_products(uint32_t tm, uint32_t at, uint32_t blo, uint32_t bhi,
                                              uint32_t bstep, uint32_t id) {
@@ -123,16 +137,17 @@ __device__ __forceinline__ void f64_products(uint32_t tm, uint32_t at, uint32_t 
 #pragma unroll
     for (int i = 1; i < kDig; ++i)
 #pragma unroll
-        for (int j = 0; j + i < kDig; ++j)
-            mma_f16_ts<1>(tm + (uint32_t)((i + j) * kChunk), at + (uint32_t)(8 * i),
-                          blo + bstep * (uint32_t)j, bhi, id);
+        for (int j = 0; j < kDig && i + j < kAcc; ++j) {
+            const uint32_t d = tm + (uint32_t)((i + j) * kChunk), x = at + (uint32_t)(8 * i),
+                           y = blo + bstep * (uint32_t)j;
+            if (i == 1 && j == kDig - 1) mma_f16_ts<MORE>(d, x, y, bhi, id);
+            else mma_f16_ts<1>(d, x, y, bhi, id);
+        }
 }
-__device__ __forceinline__ void tmem_ld8_nw(uint32_t taddr, uint32_t (&r)[8]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7])
-        : "r"(taddr));
+__device__ __forceinline__ void tmem_ld4_nw(uint32_t taddr, uint32_t (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(taddr));
 }
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
     asm volatile(
@@ -162,41 +177,60 @@ __device__ __forceinline__ void tmem_ld1(uint32_t taddr, uint32_t (&r)[1]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// sum_d s_d 2^(8 (5 - d)), the last term rounded to an integer, from the bits
-// v_d of s_d + 1.5 2^23 (|s_d| < 2^22): neighbours joined in 32 bits
-// (|256 s + s'| < 2^31), the biases taken off modulo 2^32
-__device__ __forceinline__ long long f64_join(const uint32_t (&v)[kDig]) {
-    constexpr uint32_t B = 0x4B400000u, B2 = 257u * B;
-    const int u = (int)(v[0] * 256u + v[1] - B2);
-    const int w = (int)(v[2] * 256u + v[3] - B2);
-    const int x = (int)(v[4] * 256u + v[5] - B2) + (((int)(v[6] - B) + 128) >> 8);
-    return ((long long)u << 32) + ((long long)w * 65536 + (long long)x);
+// S = sum_d s_d 2^(8 (7 - d)) = hi 2^32 + lo (two's complement; |S| < 2^80)
+struct F64Sum {
+    long long hi;
+    uint32_t lo;
+};
+__device__ __forceinline__ F64Sum f64_sum(long long upper, long long lower) {  // upper 2^32 + lower
+    F64Sum r;
+    r.hi = upper + (lower >> 32);
+    r.lo = (uint32_t)lower;
+    return r;
+}
+// from the bits v_d of s_d + 1.5 2^23 (|s_d| < 2^22): neighbours joined in 32
+// bits (|256 s + s'| < 2^31), the biases taken off modulo 2^32
+__device__ __forceinline__ F64Sum f64_join(const uint32_t (&v)[kAcc]) {
+    constexpr uint32_t B2 = 257u * 0x4B400000u;
+    int t[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) t[k] = (int)(v[2 * k] * 256u + v[2 * k + 1] - B2);
+    return f64_sum((long long)t[0] * 65536 + (long long)t[1], (long long)t[2] * 65536 + (long long)t[3]);
 }
 
-// I 2^e as a double, rounded to nearest, in integer instructions, for
-// exponents well inside the normal range (|e| <= kExpFast; |I| < 2^62)
+// S 2^e as a double, rounded to nearest, in integer instructions, for
+// exponents well inside the normal range (|e| <= kExpFast)
 constexpr int kExpFast = 900;
-__device__ __forceinline__ double fixed_to_double(long long I, int e) {
-    const uint32_t sign = (uint32_t)((unsigned long long)I >> 32) & 0x80000000u;
-    const unsigned long long a = I < 0 ? 0ull - (unsigned long long)I : (unsigned long long)I;
-    uint32_t h = (uint32_t)(a >> 32), l = (uint32_t)a;
-    int be = e + 63 + 1022;  // exponent field before the leading one is added
-    if (h == 0) {
-        h = l;
-        l = 0;
+__device__ __forceinline__ double fixed_to_double(const F64Sum& S, int e) {
+    const uint32_t neg = (uint32_t)((unsigned long long)S.hi >> 63);
+    // magnitude in three words
+    uint32_t w0 = neg ? 0u - S.lo : S.lo;
+    unsigned long long a = (unsigned long long)S.hi;
+    if (neg) a = ~a + (S.lo == 0u ? 1ull : 0ull);
+    uint32_t w2 = (uint32_t)(a >> 32), w1 = (uint32_t)a;
+    int be = e + 95 + 1022;  // exponent field before the leading one is added
+    if (w2 == 0u) {
+        w2 = w1;
+        w1 = w0;
+        w0 = 0u;
         be -= 32;
     }
-    if (h == 0) return 0.0;
-    const int lz = __clz((int)h);
-    const uint32_t mh = __funnelshift_l(l, h, lz), ml = l << lz;
+    if (w2 == 0u) {
+        w2 = w1;
+        w1 = 0u;
+        be -= 32;
+    }
+    if (w2 == 0u) return 0.0;
+    const int lz = __clz((int)w2);
+    const uint32_t mh = __funnelshift_l(w1, w2, lz), ml = __funnelshift_l(w0, w1, lz);
     const unsigned long long r = ((unsigned long long)((mh >> 11) + ((uint32_t)(be - lz) << 20)) << 32) +
                                  (unsigned long long)__funnelshift_r(ml, mh, 11) + ((ml >> 10) & 1u);
-    return __longlong_as_double((long long)(r | ((unsigned long long)sign << 32)));
+    return __longlong_as_double((long long)(r | ((unsigned long long)neg << 63)));
 }
 // the rest: rows of subnormal or huge values, NaN rows
-__device__ __noinline__ double fixed_to_double_slow(long long I, int er, int fn) {
+__device__ __noinline__ double fixed_to_double_slow(F64Sum S, int er, int fn) {
     if (er == kRowNan) return __longlong_as_double(0x7ff8000000000000ll);
-    return ldexp((double)I, er + fn);
+    return ldexp(fixed_to_double(S, 0), er + fn);
 }
 
 // work unit idx: operator, rows, for M2M / L2L the first target cell, and the
@@ -493,13 +527,13 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
             double* orow = a.out + (int64_t)(w.base + row) * a.out_stride;
             for (int c = w.c0; c < w.c1; ++c, ++jacc) {
                 const int N = min(kChunk, a.npad - c * kChunk);
-                const int ng = N / 16, c0 = half * (N / 2);  // groups of 8 columns
+                const int ng = N / 8, c0 = half * (N / 2);  // groups of 4 columns
                 const int n0 = c * kChunk + c0;
                 const int16_t* fe = a.oexp + (int64_t)w.op * a.npad + n0;
-                int4 f[3];
+                int2 f[6];
 #pragma unroll
-                for (int q = 0; q < 3; ++q)
-                    if (q < ng) f[q] = __ldg(reinterpret_cast<const int4*>(fe) + q);
+                for (int q = 0; q < 6; ++q)
+                    if (q < ng) f[q] = __ldg(reinterpret_cast<const int2*>(fe) + q);
                 int ok = 1;
                 if (lane == 0) ok = mbar_wait_or_abort(&accf, jacc & 1, abort_v) ? 1 : 0;
                 ok = __shfl_sync(0xffffffffu, ok, 0);
@@ -509,46 +543,43 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
                     break;
                 }
                 tc_fence_after();
-                long long I[3][8];
+                F64Sum I[6][4];
                 uint32_t big = 0;  // bits 23 and up set by a sum of 2^22 or more
 #pragma unroll
-                for (int q = 0; q < 3; ++q) {
+                for (int q = 0; q < 6; ++q) {
                     if (q >= ng) break;  // uniform
-                    uint32_t s[kDig][8];
+                    uint32_t s[kAcc][4];
 #pragma unroll
-                    for (int d = 0; d < kDig; ++d)
-                        tmem_ld8_nw(tq + (uint32_t)(d * kChunk + c0 + 8 * q), s[d]);
+                    for (int d = 0; d < kAcc; ++d)
+                        tmem_ld4_nw(tq + (uint32_t)(d * kChunk + c0 + 4 * q), s[d]);
                     tmem_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
+                    for (int j = 0; j < 4; ++j) {
                         // s + 1.5 2^23 holds the integer s in its low bits
                         // while |s| < 2^22 (crystals stay below 2^20); the
                         // conversion instruction runs at 16 a clock, the add at 128
-                        uint32_t v[kDig];
+                        uint32_t v[kAcc];
 #pragma unroll
-                        for (int d = 0; d < kDig; ++d) {
+                        for (int d = 0; d < kAcc; ++d) {
                             v[d] = __float_as_uint(__uint_as_float(s[d][j]) + 12582912.f);
                             big |= v[d] ^ 0x4B400000u;
                         }
                         I[q][j] = f64_join(v);
                     }
                     if (__any_sync(0xffffffffu, big >> 23)) {
-                        // (uniform, rare) sums up to 2^24 by conversion
+                        // (uniform, rare) larger sums by conversion
 #pragma unroll 1
-                        for (int j = 0; j < 8; ++j) {
-                            long long S = 0;
+                        for (int j = 0; j < 4; ++j) {
+                            long long S[2] = {0, 0};
 #pragma unroll 1
-                            for (int d = 0; d < kDig - 1; ++d) {
+                            for (int d = 0; d < kAcc; ++d) {
                                 uint32_t x[1];
-                                tmem_ld1(tq + (uint32_t)(d * kChunk + c0 + 8 * q + j), x);
-                                S += (long long)__float2int_rn(__uint_as_float(x[0])) << (40 - 8 * d);
+                                tmem_ld1(tq + (uint32_t)(d * kChunk + c0 + 4 * q + j), x);
+                                S[d >> 2] = S[d >> 2] * 256 + (long long)__float2int_rn(__uint_as_float(x[0]));
                             }
-                            uint32_t x[1];
-                            tmem_ld1(tq + (uint32_t)((kDig - 1) * kChunk + c0 + 8 * q + j), x);
-                            S += ((long long)__float2int_rn(__uint_as_float(x[0])) + 128) >> 8;
 #pragma unroll
-                            for (int jj = 0; jj < 8; ++jj)
-                                if (jj == j) I[q][jj] = S;
+                            for (int jj = 0; jj < 4; ++jj)
+                                if (jj == j) I[q][jj] = f64_sum(S[0], S[1]);
                         }
                         big = 0;
                     }
@@ -556,40 +587,34 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
                 tc_fence_before();
                 mbar_arrive(&acce);  // the issuer may start the next chunk
 #pragma unroll
-                for (int q = 0; q < 3; ++q) {
+                for (int q = 0; q < 6; ++q) {
                     if (q >= ng) break;
                     if (row >= w.rows) continue;
-                    const int fw[4] = {f[q].x, f[q].y, f[q].z, f[q].w};
-                    double v[8];
+                    const int fn[4] = {(int)(int16_t)(f[q].x & 0xffff), f[q].x >> 16,
+                                       (int)(int16_t)(f[q].y & 0xffff), f[q].y >> 16};
+                    double v[4];
                     if (fast) {
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            const int fn = j & 1 ? fw[j >> 1] >> 16 : (int)(int16_t)(fw[j >> 1] & 0xffff);
-                            v[j] = fixed_to_double(I[q][j], er + fn - 50);
-                        }
+                        for (int j = 0; j < 4; ++j) v[j] = fixed_to_double(I[q][j], er + fn[j] - kSumExp);
                     } else {
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            const int fn = j & 1 ? fw[j >> 1] >> 16 : (int)(int16_t)(fw[j >> 1] & 0xffff);
-                            v[j] = fixed_to_double_slow(I[q][j], er, fn - 50);
-                        }
+                        for (int j = 0; j < 4; ++j) v[j] = fixed_to_double_slow(I[q][j], er, fn[j] - kSumExp);
                     }
                     // rows are multiples of 4 doubles apart: whole 32-byte units
-#pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        const int n = n0 + 8 * q + 4 * u;
-                        if (n >= a.ld) break;
-                        double4_32a* o = reinterpret_cast<double4_32a*>(orow + n);
-                        double4_32a r = make_double4_32a(v[4 * u], v[4 * u + 1], v[4 * u + 2], v[4 * u + 3]);
-                        if (MODE == F64_L2L) {
-                            const double4_32a own = *o;
-                            r.x += own.x;
-                            r.y += own.y;
-                            r.z += own.z;
-                            r.w += own.w;
-                        }
-                        *o = r;
+                    const int n = n0 + 4 * q;
+                    if (n >= a.ld) break;
+                    double4_32a* o = reinterpret_cast<double4_32a*>(orow + n);
+                    double4_32a r = make_double4_32a(v[0], v[1], v[2], v[3]);
+                    if (MODE == F64_L2L) {
+                        const double4_32a own = *o;
+                        // the parent's L_0 reaches the child's L_0 only, as L_0 / 2: it has no digits
+                        if (n == 0) r.x += 0.5 * a.up[(int64_t)src * a.ld];
+                        r.x += own.x;
+                        r.y += own.y;
+                        r.z += own.z;
+                        r.w += own.w;
                     }
+                    *o = r;
                 }
             }
         }
@@ -666,8 +691,9 @@ __device__ __forceinline__ void store_digits(const double (&v)[kSliceRegs], int 
     }
 }
 
-// digits of the rows of Y (M or L) of one level's cells
-__global__ void __launch_bounds__(kSliceThreads) k_f64_slice(int level, int P, int ld, int lda,
+// digits of the rows of Y (M or L) of one level's cells, k0 = 1: without their
+// first coefficient
+__global__ void __launch_bounds__(kSliceThreads) k_f64_slice(int level, int k0, int P, int ld, int lda,
                                                              const LevelInfo* linfo,
                                                              const double* __restrict__ Y,
                                                              uint8_t* dig, int* rexp) {
@@ -679,7 +705,7 @@ __global__ void __launch_bounds__(kSliceThreads) k_f64_slice(int level, int P, i
         double v[kSliceRegs];
 #pragma unroll
         for (int r = 0; r < kSliceRegs; ++r)
-            v[r] = lane + 32 * r < P ? Y[(int64_t)g * ld + lane + 32 * r] : 0.0;
+            v[r] = lane + 32 * r >= k0 && lane + 32 * r < P ? Y[(int64_t)g * ld + lane + 32 * r] : 0.0;
         store_digits(v, P, lane, dig + (int64_t)g * kDig * lda, rexp + g);
     }
 }
@@ -870,10 +896,13 @@ cudaError_t m2l_f64_pack(const Workspace& ws) {
     return cudaStreamSynchronize(0);
 }
 
-cudaError_t launch_f64_slice(int64_t n, int l, const double* Y, Workspace& ws, cudaStream_t s) {
-    return launch_pdl(k_f64_slice, dim3(slice_grid(level_cap(n, l))), dim3(kSliceThreads), 0, s, l,
+static cudaError_t slice(int64_t n, int l, int k0, const double* Y, Workspace& ws, cudaStream_t s) {
+    return launch_pdl(k_f64_slice, dim3(slice_grid(level_cap(n, l))), dim3(kSliceThreads), 0, s, l, k0,
                       ws.P, ws.ld, m2l_f64_lda(ws.p), (const LevelInfo*)ws.linfo, Y, ws.f64_dig,
                       ws.f64_rexp);
+}
+cudaError_t launch_f64_slice(int64_t n, int l, const double* M, Workspace& ws, cudaStream_t s) {
+    return slice(n, l, 0, M, ws, s);
 }
 
 cudaError_t launch_f64_m2m(int64_t n, int D, int l, Workspace& ws, cudaStream_t s) {
@@ -893,11 +922,12 @@ cudaError_t launch_f64_m2m(int64_t n, int D, int l, Workspace& ws, cudaStream_t 
 }
 
 cudaError_t launch_f64_l2l(int64_t n, int D, int l, Workspace& ws, cudaStream_t s) {
-    cudaError_t e = launch_f64_slice(n, l - 1, (const double*)ws.L, ws, s);
+    cudaError_t e = slice(n, l - 1, 1, (const double*)ws.L, ws, s);
     if (e != cudaSuccess) return e;
     F64Args a = f64_args(ws);
     a.level = l;
     a.off_parent = dense_layout(D).off[l - 1];
+    a.up = (const double*)ws.L;
     a.out = (double*)ws.L;
     a.out_stride = ws.ld;
     const int64_t items = (level_cap(n, l) / kF64Rows + 8) * a.nch;
