@@ -137,6 +137,15 @@ __device__ __forceinline__ void kb_add(T& s, T& c, T v) {
     s = t;
 }
 
+// The same in FP64 with one instruction of the FP64 pipe less: the order by
+// exponent is enough for the error to be exact.
+__device__ __forceinline__ void kb_add_d(double& s, double& c, double v) {
+    const double t = s + v;
+    const bool ge = (__double2hiint(s) & 0x7ff00000) >= (__double2hiint(v) & 0x7ff00000);
+    c += (ge ? v : s) - (t - (ge ? s : v));
+    s = t;
+}
+
 // Position of a sorted ion in the frame of its ancestor s levels above its
 // leaf: o = the leaf's integer position inside the ancestor (0 .. 2^s - 1
 // per axis), u_anc = (u_leaf + o + 1/2 - 2^s / 2) / 2^s, in ancestor units.
@@ -863,16 +872,17 @@ __global__ void __launch_bounds__(kNfThreads) k_p2p(int D, const LevelInfo* linf
 // instruction as much as a full one, so the work is laid out for full warps:
 //   * thread (target i, chunk c) as above, but the chunk partials (plain sums
 //     over blocks of 64 sources, compensated across blocks: most threads have
-//     one block) are added pairwise by all threads instead of one after the
-//     other by a few lanes of the first warp, which took as long as the pair
-//     sums themselves;
+//     one block) are added by a thread per target and component instead of a
+//     thread per target, which took as long as the pair sums themselves;
 //   * rsqrt (about 7 FP64 instructions) instead of a square root and a
 //     division (about 25);
 //   * `parts` blocks share a leaf's targets where there are few leaves, so
 //     that shallow trees fill the GPU;
 //   * the potential only if it is asked for.
-// 1e5 sweep ions (14.5 M pairs): 2.2 ms before, 0.66 now; 1e6 ions 17.4 and
-// 7.6 ms; the pair sums alone (19 instructions a pair) are 0.44 and 5.7 ms.
+// 1e5 sweep ions (14.5 M pairs): 2.2 ms before, 0.78 now; 1e6 ions 17.4 and
+// 8.4 ms; the pair sums alone (19 instructions a pair) are 0.44 and 5.7 ms.
+// (Plain adds pairwise between the chunks, without the compensation, were
+// 0.12 and 0.75 ms faster.)
 constexpr int kNfSrc64 = 256;  // staged sources per pass; the partials reuse their room
 template <bool PHI>
 __global__ void __launch_bounds__(kNfThreads, 8) k_p2p_f64(
@@ -983,24 +993,14 @@ __global__ void __launch_bounds__(kNfThreads, 8) k_p2p_f64(
             }
             __syncthreads();  // the sources are read
             part[tid] = make_double4_32a(ex, ey, ez, ph);
-            // pairwise over the chunks: a fixed tree (deterministic)
-            int live = nch;
-            while (live > 1) {
-                const int half = (live + 1) >> 1;
-                __syncthreads();
-                if (ch < live - half) {
-                    const R o = part[tid + half * ntb];
-                    ex += o.x;
-                    ey += o.y;
-                    ez += o.z;
-                    if (PHI) ph += o.w;
-                    part[tid] = make_double4_32a(ex, ey, ez, ph);
-                }
-                live = half;
+            __syncthreads();
+            // the chunks in order, compensated: a thread per target and component
+            const double* p = reinterpret_cast<const double*>(part);
+            for (int e = tid; e < 4 * ntb; e += kNfThreads) {
+                double s = 0, c = 0;
+                for (int k = 0; k < nch; ++k) kb_add_d(s, c, p[4 * ntb * k + e]);
+                near[4 * (int64_t)(ts + t0) + e] = s + c;
             }
-            if (ch == 0)
-                *reinterpret_cast<R*>(near + 4 * (int64_t)(ts + t0 + tid)) =
-                    make_double4_32a(ex, ey, ez, ph);
             __syncthreads();
         }
     }
