@@ -224,14 +224,14 @@ cudaError_t upload_ops(fmm_plan_s* pl, const std::vector<double>& m2m, const std
         for (int r = 0; r < P; ++r)
             for (int c = 0; c < P; ++c)
                 tmp[(size_t)o * P * P + (size_t)c * P + r] = (T)m2m[(size_t)o * P * P + (size_t)r * P + c];
-    cudaError_t e = cudaMemcpy(pl->ws.T_m2m, tmp.data(), tmp.size() * sizeof(T), cudaMemcpyHostToDevice);
+    cudaError_t e = upload(pl->ws.T_m2m, tmp.data(), tmp.size() * sizeof(T));
     if (e != cudaSuccess) return e;
     tmp.assign(l2l.begin(), l2l.end());
-    if ((e = cudaMemcpy(pl->ws.T_l2l, tmp.data(), tmp.size() * sizeof(T), cudaMemcpyHostToDevice)) !=
+    if ((e = upload(pl->ws.T_l2l, tmp.data(), tmp.size() * sizeof(T))) !=
         cudaSuccess)
         return e;
     tmp.assign(m2l.begin(), m2l.end());
-    return cudaMemcpy(pl->ws.T_m2l, tmp.data(), tmp.size() * sizeof(T), cudaMemcpyHostToDevice);
+    return upload(pl->ws.T_m2l, tmp.data(), tmp.size() * sizeof(T));
 }
 
 int build_operators(fmm_plan_s* pl) {
@@ -257,7 +257,7 @@ int build_operators(fmm_plan_s* pl) {
         const bool bf16 = pl->precision == PT_MIXED_BF16X3;
         std::vector<unsigned char> packed(m2l_tc_operand_bytes(p, bf16));
         m2l_tc_pack_operands(p, bf16, m2l.data(), m2m.data(), l2l.data(), packed.data());
-        e = cudaMemcpy(pl->ws.T_m2l_tc, packed.data(), packed.size(), cudaMemcpyHostToDevice);
+        e = upload(pl->ws.T_m2l_tc, packed.data(), packed.size());
         if (e != cudaSuccess) return status_from(e);
     }
     return PT_OK;
@@ -278,10 +278,10 @@ int build_rotation_operators(fmm_plan_s* pl) {
                     return PT_ERR_CUDA;
             }
     if (pl->ws.fp64) {
-        e = cudaMemcpy(pl->ws.T_rot, rot.data(), rot.size() * sizeof(double), cudaMemcpyHostToDevice);
+        e = upload(pl->ws.T_rot, rot.data(), rot.size() * sizeof(double));
     } else {
         std::vector<float> rf(rot.begin(), rot.end());
-        e = cudaMemcpy(pl->ws.T_rot, rf.data(), rf.size() * sizeof(float), cudaMemcpyHostToDevice);
+        e = upload(pl->ws.T_rot, rf.data(), rf.size() * sizeof(float));
     }
     return status_from(e);
 }
@@ -444,7 +444,8 @@ static int alloc_pairs(fmm_plan_s* pl) {
         ws.pp_part = nullptr;
         return PT_ERR_OOM;
     }
-    if (!pl->dry && cudaMemset(ws.pp_work, 0, m2l_pp_work_bytes(ws)) != cudaSuccess)
+    if (!pl->dry && (cudaMemset(ws.pp_work, 0, m2l_pp_work_bytes(ws)) != cudaSuccess ||
+                     legacy_done() != cudaSuccess))
         return PT_ERR_CUDA;
     if (!pl->dry && ws.tc_bf16 && m2l_tc_make_part_map(ws) != cudaSuccess) return PT_ERR_CUDA;
     if (!pl->dry && !ws.h_pp_hdr) {
@@ -475,7 +476,8 @@ static int regrow_pairs(fmm_plan_s* pl, int64_t cap) {
     if (!dalloc(pl, ws.pp_work, m2l_pp_work_bytes(ws)) ||
         !dalloc(pl, ws.pp_part, m2l_pp_part_bytes(ws)))
         return PT_ERR_OOM;
-    if (cudaMemset(ws.pp_work, 0, m2l_pp_work_bytes(ws)) != cudaSuccess) return PT_ERR_CUDA;
+    if (cudaMemset(ws.pp_work, 0, m2l_pp_work_bytes(ws)) != cudaSuccess || legacy_done() != cudaSuccess)
+        return PT_ERR_CUDA;
     if (ws.tc_bf16 && m2l_tc_make_part_map(ws) != cudaSuccess) return PT_ERR_CUDA;
     memset(ws.h_pp_hdr, 0, sizeof(M2lPairHdr));
     ++ws.pp_gen;
@@ -524,7 +526,7 @@ static int alloc_tile_slabs(fmm_plan_s* pl) {
         return PT_ERR_OOM;
     }
     if (cudaMemset(work, 0, m2l_tc_work_bytes(ws.tc_tiles_cap, want)) != cudaSuccess ||
-        cudaMemset(part, 0, sizeof(float) * floats) != cudaSuccess) {
+        cudaMemset(part, 0, sizeof(float) * floats) != cudaSuccess || legacy_done() != cudaSuccess) {
         cudaFree(work);
         cudaFree(part);
         return PT_ERR_CUDA;
@@ -794,6 +796,7 @@ struct pt_ensemble_s {
     std::vector<cudaStream_t> br;        // capture-time branch streams
     std::vector<cudaEvent_t> join;
     cudaEvent_t fork = nullptr;
+    cudaEvent_t launched = nullptr;      // after the last launches of the graph
     cudaStream_t cap = nullptr;
     cudaGraphExec_t graph = nullptr;
     std::vector<GraphKey> keys;
@@ -832,7 +835,7 @@ static cudaError_t join_members(pt_ensemble_s* ens, cudaGraph_t g) {
         (e = join_fmm(c)) != cudaSuccess || (e = join_pairs(c)) != cudaSuccess)
         return e;
     return c.host.empty() ? cudaSuccess
-                          : cudaMemcpy(c.dev, c.host.data(), c.host.size(), cudaMemcpyHostToDevice);
+                          : upload(c.dev, c.host.data(), c.host.size());
 }
 
 namespace {
@@ -845,6 +848,7 @@ void free_ensemble(pt_ensemble_s* e) {
     for (cudaEvent_t j : e->join)
         if (j) cudaEventDestroy(j);
     if (e->fork) cudaEventDestroy(e->fork);
+    if (e->launched) cudaEventDestroy(e->launched);
     if (e->cap) cudaStreamDestroy(e->cap);
     if (e->d_members) cudaFree(e->d_members);
     if (e->d_prefix) cudaFree(e->d_prefix);
@@ -1149,6 +1153,7 @@ static int plan_create_impl(int64_t n_max, int p, int leaf_max, int depth, int p
         }
     }
     int r = acquire_ops(pl, tsz * PP);
+    if (r == PT_OK && legacy_done() != cudaSuccess) r = PT_ERR_CUDA;  // the memsets above
     if (r == PT_OK && !ws.T_f64) {
         ws.f64_tc = 0;
         ws.f64_batch = 0;
@@ -1368,7 +1373,8 @@ int pt_ensemble_create(int n_members, const fmm_plan* plans, pt_ensemble* out) {
     e->br.assign(n_members, nullptr);
     e->join.assign(n_members, nullptr);
     bool ok = cudaStreamCreateWithPriority(&e->cap, cudaStreamNonBlocking, prio_high()) == cudaSuccess &&
-              cudaEventCreateWithFlags(&e->fork, cudaEventDisableTiming) == cudaSuccess;
+              cudaEventCreateWithFlags(&e->fork, cudaEventDisableTiming) == cudaSuccess &&
+              cudaEventCreateWithFlags(&e->launched, cudaEventDisableTiming) == cudaSuccess;
     for (int b = 0; ok && b < n_members; ++b)
         ok = cudaStreamCreateWithPriority(&e->br[b], cudaStreamNonBlocking, prio_high()) == cudaSuccess &&
              cudaEventCreateWithFlags(&e->join[b], cudaEventDisableTiming) == cudaSuccess;
@@ -1379,7 +1385,7 @@ int pt_ensemble_create(int n_members, const fmm_plan* plans, pt_ensemble* out) {
     if (ok) {
         std::vector<int*> errs;
         for (fmm_plan_s* pl : e->plans) errs.push_back(pl->ws.err);
-        ok = cudaMemcpy(e->d_errs, errs.data(), sizeof(int*) * errs.size(), cudaMemcpyHostToDevice) ==
+        ok = upload(e->d_errs, errs.data(), sizeof(int*) * errs.size()) ==
              cudaSuccess;
     }
     if (!ok) {
@@ -1436,7 +1442,7 @@ int pt_ensemble_step(pt_ensemble ens, pt_state* states, const pt_trap* traps,
         if (!same) {
             if (ens->graph) {
                 // the joined launches' tables are rewritten below
-                if (cudaDeviceSynchronize() != cudaSuccess) return PT_ERR_CUDA;
+                if (cudaEventSynchronize(ens->launched) != cudaSuccess) return PT_ERR_CUDA;
                 cudaGraphExecDestroy(ens->graph);
                 ens->graph = nullptr;
             }
@@ -1485,6 +1491,7 @@ int pt_ensemble_step(pt_ensemble ens, pt_state* states, const pt_trap* traps,
                 return status_from(e);
             }
         }
+        if ((e = cudaEventRecord(ens->launched, s)) != cudaSuccess) return status_from(e);
         for (int b = 0; b < nm; ++b) {
             fmm_plan_s* pl = ens->plans[b];
             pl->dev_next = step0[b] + s0 + k;

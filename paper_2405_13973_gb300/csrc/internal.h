@@ -291,6 +291,14 @@ cudaError_t m2l_pairs_stats(const Workspace& ws, int64_t* out, cudaStream_t s);
 // this order do not fit), per-device kernel set-up
 int m2l_rot_tile(const Workspace& ws);
 cudaError_t m2l_rot_init();
+// Host memory to the device, there when this returns: a copy from pageable
+// memory may return before its data has arrived, and a kernel on a
+// non-blocking stream does not wait for it (nor for a cudaMemset).
+inline cudaError_t legacy_done() { return cudaStreamSynchronize(cudaStreamLegacy); }
+inline cudaError_t upload(void* dst, const void* src, size_t bytes) {
+    const cudaError_t e = cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
+    return e == cudaSuccess ? legacy_done() : e;
+}
 // ---- FP32 translations on the CUDA cores (m2l_f32.cu) ---------------------------
 size_t m2l_f32_operator_bytes(int p);
 cudaError_t m2l_f32_init();

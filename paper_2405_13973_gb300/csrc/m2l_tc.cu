@@ -1931,7 +1931,7 @@ cudaError_t m2l_join_pair_launches(cudaGraph_t g, void* d_members, int* d_prefix
         hm[k].Mp = args[k].Mp;
         hm[k].hdr = args[k].phdr;
     }
-    if ((e = cudaMemcpy(d_members, hm.data(), sizeof(PairMember) * n, cudaMemcpyHostToDevice)) !=
+    if ((e = upload(d_members, hm.data(), sizeof(PairMember) * n)) !=
         cudaSuccess)
         return e;
     // the joined launch waits for every member's inputs and precedes every
