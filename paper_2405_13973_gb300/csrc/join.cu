@@ -32,6 +32,18 @@ cudaError_t join_table_bytes(cudaGraph_t g, size_t* bytes) {
     return e;
 }
 
+cudaError_t join_smem_limit(const void* joined) {
+    cudaFuncAttributes fa{};
+    int dev = 0, most = 0;
+    cudaError_t e = cudaFuncGetAttributes(&fa, joined);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(joined, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 most - (int)fa.sharedSizeBytes);
+    return e;
+}
+
 cudaError_t join_find(const JoinCtx& c, const void* fn, std::vector<cudaGraphNode_t>& found,
                       std::vector<cudaKernelNodeParams>& kps) {
     std::vector<cudaGraphNode_t> nodes;

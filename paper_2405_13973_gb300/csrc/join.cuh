@@ -50,6 +50,9 @@ cudaError_t join_find(const JoinCtx& c, const void* fn, std::vector<cudaGraphNod
 // predecessor, before every successor of any of them
 cudaError_t join_replace(JoinCtx& c, const std::vector<cudaGraphNode_t>& found,
                          const cudaKernelNodeParams& jp, unsigned cluster);
+// as much dynamic shared memory as the device allows: one limit whatever the
+// ensemble, so that none lowers what another's graph was made with
+cudaError_t join_smem_limit(const void* joined);
 // joins of each translation unit's kernels
 cudaError_t join_push(JoinCtx& c);
 cudaError_t join_tree(JoinCtx& c);
@@ -114,10 +117,7 @@ cudaError_t join_kernel(JoinCtx& c, void (*solo)(A...), unsigned cluster = 1) {
         for (unsigned b = 0; b < d.x * d.y * d.z; ++b) *jb++ = JoinBlock{(int)i, (int)b};
     }
     auto joined = k_joined<Body, THREADS, A...>;
-    if (smem > 48 * 1024 &&
-        (e = cudaFuncSetAttribute(joined, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-            cudaSuccess)
-        return e;
+    if (smem > 0 && (e = join_smem_limit((const void*)joined)) != cudaSuccess) return e;
     const Tuple* da = reinterpret_cast<const Tuple*>(c.dev + at_a);
     const uint4* dd = reinterpret_cast<const uint4*>(c.dev + at_d);
     const JoinBlock* db = reinterpret_cast<const JoinBlock*>(c.dev + at_b);
