@@ -623,10 +623,7 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_f64_mma(const __grid_constan
     __syncthreads();
     if (*abort_v) {
         // drain (bounded): the products in flight and every copy still owed
-        if (tid == 9 * 32) {
-            mma_commit(&drain_bar);
-            mbar_wait(&drain_bar, 0);
-        }
+        if (warp == 9) mma_drain(&drain_bar);
         if (tid == 8 * 32) {
             for (int s = 0; s < kBStages; ++s)
                 if (b_par[s] >= 0) mbar_wait(&fullB[s], (uint32_t)b_par[s]);

@@ -619,9 +619,8 @@ __global__ void __launch_bounds__((TcLayout<MODE, BF16>::kThreads), 1)
     } else if (warp == L::kWarpMma) {
         // ---- MMA issuer.  The whole warp runs the loops on warp-uniform
         // values and one elected lane issues (mbar_wait_warp): issued from a
-        // one-lane branch, the operands of every product were moved to
-        // uniform registers anew and a product of N = 176 took 132 cycles
-        // instead of the tensor core's 88
+        // one-lane branch a product of N = 176 took 132 cycles instead of the
+        // tensor core's 88
         const uint32_t d0 = __shfl_sync(0xffffffffu, tmem, 0);
         // accumulator 0 takes only the leading products hi x hi, the
         // rest (2^-8 / 2^-11 of them and smaller) go to accumulator 1
@@ -1110,10 +1109,7 @@ __global__ void __launch_bounds__((TcLayout<MODE, BF16>::kThreads), 1)
     if (*abort_v) {
         // drain (bounded): the issuer's MMAs in flight and every bulk copy
         // still owed to a stage
-        if (tid == L::kWarpMma * 32) {
-            mma_commit(&drain_bar);
-            mbar_wait(&drain_bar, 0);
-        }
+        if (warp == L::kWarpMma) mma_drain(&drain_bar);
         if (tid == L::kWarpOp * 32) {
             for (int s = 0; s < NS; ++s)
                 if (issued_par[s] >= 0) mbar_wait(&fullB_bar[s], (uint32_t)issued_par[s]);

@@ -256,12 +256,22 @@ __device__ __forceinline__ bool mbar_wait_or_abort(uint64_t* bar, uint32_t parit
 }
 
 // the same for a whole warp, with one answer for all lanes: control flow that
-// depends on it stays warp-uniform (tcgen05.mma takes its operands from
-// uniform registers, and in code that the compiler has to treat as divergent
-// every operand is moved there anew for every instruction)
+// depends on it stays warp-uniform (products issued from a one-lane branch
+// took 100 to 130 cycles each, whatever their size)
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity,
                                                volatile int* abort_flag) {
     return __all_sync(0xffffffffu, mbar_wait_or_abort(bar, parity, abort_flag)) != 0;
+}
+// the issuing warp, whole, waits (bounded) for the products it has issued: a
+// commit covers its own thread's operations, and elect.sync elects the same
+// lane every time, so the lane that issued them commits
+__device__ __forceinline__ void mma_drain(uint64_t* bar) {
+    __syncwarp();
+    if (elect_one()) {
+        mma_commit(bar);
+        mbar_wait(bar, 0);
+    }
+    __syncwarp();
 }
 
 }  // namespace pt
