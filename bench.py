@@ -10,14 +10,16 @@ One benchmark step is one time step of the whole path (drift + root cube,
 octree, upward pass, M2L/L2L, L2P + P2P, kick with photon recoils + drift).
 Timing: W untimed warm-up steps, then K steps each bracketed by CUDA events
 on the launching stream, with a 512 MiB write between steps to flush the
-129 MB L2 (the inputs are smaller than L2).  Prints one JSON line.
+129 MB L2 (the inputs are smaller than L2).  Prints one JSON line, the result
+with its end-to-end measurement; the whole record with the keys named below
+goes to standard error as another.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
                   [--precision fp32|tf32x3|bf16x3|fp64] [--p P] [--p10-steps K10]
                   [--forces N] [--config1-steps K1] [--sweep N1,N2,...]
                   [--ensemble-extra M] [--serve-extra J]
 
-The default line also carries, as extra keys, the 1,000-ion FP64 run
+The default run's record also carries, as extra keys, the 1,000-ion FP64 run
 (1,000 steps at p = 8, oracle timed in the same run: "config1") and the
 single-evaluation sweep over ion counts, orders and precisions with errors
 against the FP64 direct sum ("sweep"), a 256-crystal batched ensemble
@@ -567,6 +569,33 @@ def timed_steps(pt, torch, plan, st, trap, laser, dt, K, flush, profile=True, ke
     return ms, phases
 
 
+def headline(out):
+    """The line that is printed: the result and what it rests on, below 1,500
+    characters.  The whole record goes to standard error."""
+    def short(v):
+        if isinstance(v, dict):
+            return {k: short(x) for k, x in v.items()}
+        return float(f"{v:.6g}") if isinstance(v, float) else v
+
+    def part(key, names):
+        return {k: out[key][k] for k in names if k in out[key]}
+
+    line = {k: out[k] for k in (
+        "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better",
+        "scaling", "vs_baseline", "dtype", "data")}
+    line["config"] = part("config", ("workload", "depth", "m2l_schedule", "l2", "parallelism"))
+    line.update({k: out[k] for k in ("force_err", "latency_ms", "clocks", "gpu_launches")})
+    line["roofline"] = part("roofline", ("kernel", "kernel_ms", "achieved", "peak", "unit", "frac",
+                                         "bound", "traffic"))
+    if "fp64_path" in out:
+        line["fp64_path"] = part("fp64_path", ("value", "ms_per_step", "force_err"))
+    if "cpu_baseline" in out:
+        line["cpu_baseline"] = part("cpu_baseline", ("value", "cores", "kind"))
+    if "e2e" in out:
+        line["e2e"] = part("e2e", ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step"))
+    return short(line)
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -848,7 +877,8 @@ def main():
         out["cpu_baseline"] = run_cpu_baseline(cr)
     plan.close()
     if rank == 0:
-        print(json.dumps(out), flush=True)
+        print(json.dumps(out), file=sys.stderr, flush=True)
+        print(json.dumps(headline(out)), flush=True)
     if dist:
         dist.barrier()
         dist.destroy_process_group()
