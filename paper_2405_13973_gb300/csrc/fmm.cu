@@ -337,7 +337,9 @@ __global__ void __launch_bounds__(kSlotThreads) k_p2m_f64(
 constexpr int kP2mAncIons = 64;
 
 template <typename T>
-__device__ __forceinline__ void k_p2m_anc_body(const BlockId& blk, int D, int lmin, int p, int ld, const LevelInfo* linfo, const uint32_t* __restrict__ code,
+__device__ __forceinline__ void k_p2m_anc_body(
+    const BlockId& blk, int D, int lmin, int p, int ld, const LevelInfo* linfo,
+    const uint32_t* __restrict__ code,
     const int32_t* __restrict__ leaf_start, const int32_t* __restrict__ leaf_of,
     const typename Ion<T>::rec* __restrict__ sorted, T* __restrict__ M, uint16_t* Mp) {
     extern __shared__ unsigned char p2m_smem[];
@@ -393,7 +395,8 @@ __device__ __forceinline__ void k_p2m_anc_body(const BlockId& blk, int D, int lm
     }
 }
 template <typename T>
-__global__ void __launch_bounds__(kP2mThreads) k_p2m_anc(int D, int lmin, int p, int ld, const LevelInfo* linfo, const uint32_t* __restrict__ code,
+__global__ void __launch_bounds__(kP2mThreads) k_p2m_anc(
+    int D, int lmin, int p, int ld, const LevelInfo* linfo, const uint32_t* __restrict__ code,
     const int32_t* __restrict__ leaf_start, const int32_t* __restrict__ leaf_of,
     const typename Ion<T>::rec* __restrict__ sorted, T* __restrict__ M, uint16_t* Mp) {
     k_p2m_anc_body<T>(solo_block(), D, lmin, p, ld, linfo, code, leaf_start, leaf_of, sorted, M, Mp);
@@ -501,7 +504,7 @@ __device__ __forceinline__ void k_shift_rows_body(const BlockId& blk, int l, int
     T* sX = sOp + kShRows * S;                // [CG][K]
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
     const int r0 = (int)blk.x * kShRows;
-    const int oct = MODE == 1 ? (int)(int)blk.y : 0;
+    const int oct = MODE == 1 ? (int)blk.y : 0;
     if (MODE == 0) {
         // Op = T_m2m transposed, [o][c][r]: element (r, t = o P + c) at t P + r
         for (int e = tid; e < K * kShRows; e += kShThreads) {
@@ -526,8 +529,8 @@ __device__ __forceinline__ void k_shift_rows_body(const BlockId& blk, int l, int
         g1 = linfo->oct_start[l][oct + 1];
     }
     const int nch = (g1 - g0 + CG - 1) / CG;
-    const int ch0 = MODE == 0 ? (int)(int)blk.y : (int)(int)blk.z;
-    const int chs = MODE == 0 ? (int)(int)blk.ny : (int)(int)blk.nz;
+    const int ch0 = MODE == 0 ? (int)blk.y : (int)blk.z;
+    const int chs = MODE == 0 ? (int)blk.ny : (int)blk.nz;
     const T* op0 = sOp + w * S;
     const T* op1 = sOp + (w + 8) * S;
     for (int ch = ch0; ch < nch; ch += chs) {
@@ -747,14 +750,14 @@ __device__ __forceinline__ double inv_sqrt<double>(double r2) {
 constexpr int kNfThreads = 128;
 constexpr int kNfSrc = 1024;   // staged sources per pass
 
-template <typename T>
-__device__ __forceinline__ void k_p2p_body(const BlockId& blk, int D, const LevelInfo* linfo, const typename Ion<T>::rec* __restrict__ sorted,
+__device__ __forceinline__ void k_p2p_body(
+    const BlockId& blk, int D, const LevelInfo* linfo, const Ion<float>::rec* __restrict__ sorted,
     const uint32_t* __restrict__ code, const int32_t* __restrict__ cid_leaf,
-    const int32_t* __restrict__ cstart, const int32_t* __restrict__ ccount, T* __restrict__ near) {
-    using R = typename Ion<T>::rec;
+    const int32_t* __restrict__ cstart, const int32_t* __restrict__ ccount, float* __restrict__ near) {
+    using R = Ion<float>::rec;
     __shared__ R src[kNfSrc];
     __shared__ int nb_start[27], nb_count[27], nb_pre[28];
-    __shared__ T part[kNfThreads][4];
+    __shared__ float part[kNfThreads][4];
     const int tid = threadIdx.x;
     const int lim = 1 << D;
     const int g0 = linfo->gbase[D], g1 = linfo->gbase[D + 1];
@@ -793,7 +796,7 @@ __device__ __forceinline__ void k_p2p_body(const BlockId& blk, int D, const Leve
             const int ti = tid % ntb, ch = tid / ntb;
             const bool active = ch < nch;
             const R me = sorted[ts + t0 + ti];
-            T ex = 0, ey = 0, ez = 0, ph = 0, cex = 0, cey = 0, cez = 0, cph = 0;
+            float ex = 0, ey = 0, ez = 0, ph = 0, cex = 0, cey = 0, cez = 0, cph = 0;
             for (int s0 = 0; s0 < ns; s0 += kNfSrc) {    // sources in passes of kNfSrc
                 const int nsb = min(kNfSrc, ns - s0);
                 __syncthreads();
@@ -805,7 +808,7 @@ __device__ __forceinline__ void k_p2p_body(const BlockId& blk, int D, const Leve
                         if (k + step <= 26 && nb_pre[k + step] <= v) k += step;
                     const int dx = k / 9 - 1, dy = (k / 3) % 3 - 1, dz = k % 3 - 1;
                     const int slot = nb_start[k] + (v - nb_pre[k]);
-                    src[j] = Ion<T>::shifted(sorted[slot], dx, dy, dz);
+                    src[j] = Ion<float>::shifted(sorted[slot], dx, dy, dz);
                 }
                 __syncthreads();
                 if (active) {
@@ -814,15 +817,15 @@ __device__ __forceinline__ void k_p2p_body(const BlockId& blk, int D, const Leve
                     // plain sums over blocks of 64 sources, compensated across blocks
                     for (int jb = ch; jb < nsb; jb += 64 * nch) {
                         const int je = min(nsb, jb + 64 * nch);
-                        T px = 0, py = 0, pz = 0, pp = 0;
+                        float px = 0, py = 0, pz = 0, pp = 0;
                         for (int j = jb; j < je; j += nch) {
                             if (j == self) continue;
-                            T rx, ry, rz, q;
-                            Ion<T>::sep_shifted(me, src[j], rx, ry, rz, q);
-                            const T r2 = rx * rx + ry * ry + rz * rz;
-                            const T ir = inv_sqrt<T>(r2);
-                            const T qi = q * ir;
-                            const T q3 = qi * ir * ir;
+                            float rx, ry, rz, q;
+                            Ion<float>::sep_shifted(me, src[j], rx, ry, rz, q);
+                            const float r2 = rx * rx + ry * ry + rz * rz;
+                            const float ir = inv_sqrt<float>(r2);
+                            const float qi = q * ir;
+                            const float q3 = qi * ir * ir;
                             px += q3 * rx;
                             py += q3 * ry;
                             pz += q3 * rz;
@@ -842,7 +845,7 @@ __device__ __forceinline__ void k_p2p_body(const BlockId& blk, int D, const Leve
             __syncthreads();
             if (tid < ntb) {
                 // fixed-order compensated combination of the chunk partials
-                T sx = 0, sy = 0, sz = 0, sp = 0, cx = 0, cy = 0, cz = 0, cp = 0;
+                float sx = 0, sy = 0, sz = 0, sp = 0, cx = 0, cy = 0, cz = 0, cp = 0;
                 for (int c = 0; c < nch; ++c) {
                     const int th = c * ntb + tid;
                     kb_add(sx, cx, part[th][0]);
@@ -850,7 +853,7 @@ __device__ __forceinline__ void k_p2p_body(const BlockId& blk, int D, const Leve
                     kb_add(sz, cz, part[th][2]);
                     kb_add(sp, cp, part[th][3]);
                 }
-                T* o = near + 4 * (int64_t)(ts + t0 + tid);
+                float* o = near + 4 * (int64_t)(ts + t0 + tid);
                 o[0] = sx + cx;
                 o[1] = sy + cy;
                 o[2] = sz + cz;
@@ -861,11 +864,11 @@ __device__ __forceinline__ void k_p2p_body(const BlockId& blk, int D, const Leve
         __syncthreads();
     }
 }
-template <typename T>
-__global__ void __launch_bounds__(kNfThreads) k_p2p(int D, const LevelInfo* linfo, const typename Ion<T>::rec* __restrict__ sorted,
+__global__ void __launch_bounds__(kNfThreads) k_p2p(
+    int D, const LevelInfo* linfo, const Ion<float>::rec* __restrict__ sorted,
     const uint32_t* __restrict__ code, const int32_t* __restrict__ cid_leaf,
-    const int32_t* __restrict__ cstart, const int32_t* __restrict__ ccount, T* __restrict__ near) {
-    k_p2p_body<T>(solo_block(), D, linfo, sorted, code, cid_leaf, cstart, ccount, near);
+    const int32_t* __restrict__ cstart, const int32_t* __restrict__ ccount, float* __restrict__ near) {
+    k_p2p_body(solo_block(), D, linfo, sorted, code, cid_leaf, cstart, ccount, near);
 }
 
 // The same in FP64.  The FP64 units serve two lanes a clock, a warp
@@ -1220,14 +1223,15 @@ __device__ __forceinline__ void l2p_columns8(int p, int j, unsigned gmask, T x, 
 // (equal to the L2L shift into the leaf, which shifts a truncated expansion
 // exactly), saving the last L2L launch.
 template <typename T, int G>
-__device__ __forceinline__ void k_l2p_body(const BlockId& blk, int64_t n, int D, int p, int ld, bool far, int nlev, const RootCube* root,
+__device__ __forceinline__ void k_l2p_body(
+    const BlockId& blk, int64_t n, int D, int p, int ld, bool far, int nlev, const RootCube* root,
     const LevelInfo* linfo, const uint32_t* __restrict__ code, const int32_t* __restrict__ cid,
     const typename Ion<T>::rec* __restrict__ sorted, const int32_t* __restrict__ perm,
     const int32_t* __restrict__ cstart, const int32_t* __restrict__ ccount,
     const T* __restrict__ L, const T* __restrict__ near, double* E, double* phi) {
     pdl_wait();
     const int g0 = linfo->gbase[D], g1 = linfo->gbase[D + 1];
-    if (g0 + (int)(int)blk.x >= g1) return;  // no leaf for this block
+    if (g0 + (int)blk.x >= g1) return;  // no leaf for this block
     constexpr int NL = sizeof(T) == 4 ? 3 : 2;  // levels evaluated at most (shared memory)
     __shared__ T sL[NL][kPmax];
     __shared__ T sD[NL][4][kPmax];  // derived expansions: phi, grad x, grad y, grad z
@@ -1317,12 +1321,14 @@ __device__ __forceinline__ void k_l2p_body(const BlockId& blk, int64_t n, int D,
     }
 }
 template <typename T, int G>
-__global__ void __launch_bounds__(kL2pThreads) k_l2p(int64_t n, int D, int p, int ld, bool far, int nlev, const RootCube* root,
+__global__ void __launch_bounds__(kL2pThreads) k_l2p(
+    int64_t n, int D, int p, int ld, bool far, int nlev, const RootCube* root,
     const LevelInfo* linfo, const uint32_t* __restrict__ code, const int32_t* __restrict__ cid,
     const typename Ion<T>::rec* __restrict__ sorted, const int32_t* __restrict__ perm,
     const int32_t* __restrict__ cstart, const int32_t* __restrict__ ccount,
     const T* __restrict__ L, const T* __restrict__ near, double* E, double* phi) {
-    k_l2p_body<T, G>(solo_block(), n, D, p, ld, far, nlev, root, linfo, code, cid, sorted, perm, cstart, ccount, L, near, E, phi);
+    k_l2p_body<T, G>(solo_block(), n, D, p, ld, far, nlev, root, linfo, code, cid, sorted, perm, cstart,
+                     ccount, L, near, E, phi);
 }
 
 // L2P in FP64 (see k_p2m_f64): a thread per ion, the derived expansions of
@@ -1528,7 +1534,8 @@ __device__ __forceinline__ void l2p_run2(int p, int m, float2 da, float2 db, flo
 }
 
 template <int G>
-__device__ __forceinline__ void k_l2p_f32_body(const BlockId& blk, int64_t n, int D, int p, int ld, int nlev, int emax, const RootCube* root,
+__device__ __forceinline__ void k_l2p_f32_body(
+    const BlockId& blk, int64_t n, int D, int p, int ld, int nlev, int emax, const RootCube* root,
     const uint32_t* __restrict__ code, const int32_t* __restrict__ cid,
     const int32_t* __restrict__ leaf_of, const int32_t* __restrict__ cstart,
     const int32_t* __restrict__ ccount, const Ion<float>::rec* __restrict__ sorted,
@@ -1823,18 +1830,16 @@ __global__ void __launch_bounds__(kNfThreads) k_l2p_anc(
 
 // the near field of `leaves` leaves at most
 template <typename T>
-static void launch_p2p(int D, int64_t leaves, int grid, bool phi, Workspace& ws,
+static void launch_p2p(int D, int64_t leaves, int leaf_grid, bool phi, Workspace& ws,
                        const int32_t* cid_leaf, T* near, cudaStream_t s);
 template <>
-void launch_p2p<float>(int D, int64_t leaves, int grid, bool phi, Workspace& ws,
+void launch_p2p<float>(int D, int64_t, int leaf_grid, bool, Workspace& ws,
                        const int32_t* cid_leaf, float* near, cudaStream_t s) {
-    (void)leaves;
-    (void)phi;
-    k_p2p<float><<<grid, kNfThreads, 0, s>>>(D, ws.linfo, (const Ion<float>::rec*)ws.sorted, ws.code,
+    k_p2p<<<leaf_grid, kNfThreads, 0, s>>>(D, ws.linfo, (const Ion<float>::rec*)ws.sorted, ws.code,
                                              cid_leaf, ws.cstart, ws.ccount, near);
 }
 template <>
-void launch_p2p<double>(int D, int64_t leaves, int grid, bool phi, Workspace& ws,
+void launch_p2p<double>(int D, int64_t leaves, int, bool phi, Workspace& ws,
                         const int32_t* cid_leaf, double* near, cudaStream_t s) {
     // few leaves: several blocks share a leaf's targets, so that a shallow
     // tree (1,000 ions at depth 2: 63 leaves, 223 us with a block per leaf)
@@ -1844,7 +1849,7 @@ void launch_p2p<double>(int D, int64_t leaves, int grid, bool phi, Workspace& ws
     const int64_t want = (int64_t)ws.sms * 4;
     const int parts = (int)(leaves >= want ? 1 : (want + leaves - 1) / leaves);
     const int64_t units = leaves * parts, cap = 152 * 16;
-    grid = (int)(units < cap ? units : cap);
+    const int grid = (int)(units < cap ? units : cap);
     auto k = phi ? k_p2p_f64<true> : k_p2p_f64<false>;
     k<<<grid, kNfThreads, 0, s>>>(D, parts, ws.linfo, (const Ion<double>::rec*)ws.sorted, ws.code,
                                   cid_leaf, ws.cstart, ws.ccount, near);
@@ -2308,7 +2313,7 @@ struct ShiftJoin {
 };
 struct P2pJoin {
     template <class... A>
-    __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const { k_p2p_body<float>(b, a...); }
+    __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const { k_p2p_body(b, a...); }
 };
 struct L2pJoin {
     template <class... A>
@@ -2316,11 +2321,10 @@ struct L2pJoin {
         k_l2p_body<float, 8>(b, a...);
     }
 };
-template <int G>
-struct L2pSlotJoin {
+struct L2pSlotJoin {  // members take one thread an ion
     template <class... A>
     __device__ __forceinline__ void operator()(const BlockId& b, const A&... a) const {
-        k_l2p_f32_body<G>(b, a...);
+        k_l2p_f32_body<1>(b, a...);
     }
 };
 
@@ -2328,10 +2332,9 @@ cudaError_t join_fmm(JoinCtx& c) {
     cudaError_t e = join_kernel<P2mJoin, kP2mThreads, 3>(c, k_p2m<float>);
     if (e == cudaSuccess) e = join_kernel<P2mAncJoin, kP2mThreads, 4>(c, k_p2m_anc<float>);
     if (e == cudaSuccess) e = join_kernel<ShiftJoin, kShThreads, 3>(c, k_shift_rows<float, 0>);
-    if (e == cudaSuccess) e = join_kernel<P2pJoin, kNfThreads, 1>(c, k_p2p<float>);
+    if (e == cudaSuccess) e = join_kernel<P2pJoin, kNfThreads, 1>(c, k_p2p);
     if (e == cudaSuccess) e = join_kernel<L2pJoin, kL2pThreads, 7>(c, k_l2p<float, 8>);
-    if (e == cudaSuccess) e = join_kernel<L2pSlotJoin<4>, l2p_f32_threads(4), 6>(c, k_l2p_f32<4>);
-    if (e == cudaSuccess) e = join_kernel<L2pSlotJoin<1>, l2p_f32_threads(1), 6>(c, k_l2p_f32<1>);
+    if (e == cudaSuccess) e = join_kernel<L2pSlotJoin, l2p_f32_threads(1), 6>(c, k_l2p_f32<1>);
     return e;
 }
 

@@ -278,7 +278,8 @@ __global__ void __launch_bounds__(kPpScanThreads) k_pp_scan(int D, int t0, int t
                                                              int* ocnt, int* ofill, int* obase,
                                                              M2lPairHdr* hdr, M2lPairHdr* host_hdr,
                                                              M2lPairItem* items, int* err) {
-    k_pp_scan_body(solo_block(), D, t0, t1, linfo, slot_cap, rows_cap, item_cap, tcount, tbase, ocnt, ofill, obase, hdr, host_hdr, items, err);
+    k_pp_scan_body(solo_block(), D, t0, t1, linfo, slot_cap, rows_cap, item_cap, tcount, tbase, ocnt,
+                   ofill, obase, hdr, host_hdr, items, err);
 }
 
 // One warp per target: each present offset takes the next position of that

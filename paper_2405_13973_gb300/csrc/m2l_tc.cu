@@ -738,7 +738,7 @@ __global__ void __launch_bounds__((TcLayout<MODE, BF16>::kThreads), 1)
                         for (int q = 0; q < 3; ++q) {
                             const uint16_t* src =
                                 gs >= 0 ? Mp + ((int64_t)gs + q) * a.ld + kc * 32 + c * 8 : Mp;
-                            cp_async16ca(sA + q * a_bytes + off, src, gs >= 0 ? 16u : 0u);
+                            cp_async16(sA + q * a_bytes + off, src, gs >= 0 ? 16u : 0u);
                         }
                     }
                     cp_async_arrive(&fullA_bar[st]);

@@ -70,7 +70,8 @@ __device__ __forceinline__ int leaf_coord(double v, double lo, double side, doub
     return (int)f;
 }
 
-__device__ __forceinline__ void k_keys_body(const BlockId& blk, const double* __restrict__ x, const double* __restrict__ y,
+__device__ __forceinline__ void k_keys_body(const BlockId& blk, const double* __restrict__ x,
+                       const double* __restrict__ y,
                        const double* __restrict__ z, int64_t n, int64_t per, int D,
                        const RootCube* root, uint32_t* key, uint32_t* rank, int32_t* leaf_count) {
     pdl_wait();
@@ -427,11 +428,11 @@ struct CellCompaction {
 // ---------------------------------------------------------------------------
 // 4./6. scatter and per-leaf ordering + gather
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void k_scatter_body(const BlockId& blk, const uint32_t* __restrict__ key, const uint32_t* __restrict__ rank,
+__device__ __forceinline__ void k_scatter_body(const BlockId& blk, const uint32_t* __restrict__ key,
+                          const uint32_t* __restrict__ rank,
                           const int32_t* __restrict__ leaf_start, int64_t n, int32_t* perm_tmp) {
     pdl_wait();
-    for (int64_t i = (int)blk.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)(int)blk.nx * blockDim.x)
+    for (int64_t i = blk.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)blk.nx * blockDim.x)
         perm_tmp[leaf_start[key[i]] + rank[i]] = (int32_t)i;
 }
 __global__ void k_scatter(const uint32_t* __restrict__ key, const uint32_t* __restrict__ rank,
@@ -465,7 +466,8 @@ __device__ __forceinline__ double4_32a make4<double4_32a>(double a, double b, do
 // of k_keys); the leaf's ions are read from the few cache lines the
 // neighbouring threads share.
 template <typename T4>
-__device__ __forceinline__ void k_leaf_gather_body(const BlockId& blk, const double* __restrict__ x, const double* __restrict__ y,
+__device__ __forceinline__ void k_leaf_gather_body(const BlockId& blk, const double* __restrict__ x,
+                              const double* __restrict__ y,
                               const double* __restrict__ z, const double* __restrict__ q, int64_t n,
                               int64_t per, int D, const RootCube* root,
                               const uint32_t* __restrict__ key,
@@ -504,7 +506,8 @@ __global__ void k_leaf_gather(const double* __restrict__ x, const double* __rest
                               const int32_t* __restrict__ cid_leaf,
                               const int32_t* __restrict__ perm_tmp, int32_t* perm,
                               int32_t* slot_of, int32_t* leaf_of, T4* sorted) {
-    k_leaf_gather_body<T4>(solo_block(), x, y, z, q, n, per, D, root, key, leaf_start, cid_leaf, perm_tmp, perm, slot_of, leaf_of, sorted);
+    k_leaf_gather_body<T4>(solo_block(), x, y, z, q, n, per, D, root, key, leaf_start, cid_leaf, perm_tmp,
+                           perm, slot_of, leaf_of, sorted);
 }
 
 // ---------------------------------------------------------------------------
