@@ -1069,8 +1069,19 @@ static int plan_create_impl(int64_t n_max, int p, int leaf_max, int depth, int p
         ws.m2l_pairs = ok ? 1 : 0;
         ws.m2l_rot = ok && ws.fp64 && ws.rot_op_vals > 0 ? 1 : 0;
     }
+    // without memory for the digits, the pool or the operators' digits: the
+    // CUDA-core translations, which need none of them
+    const size_t held = pl->allocs.size();
+    auto drop_f64 = [&]() {
+        for (; pl->allocs.size() > held; pl->allocs.pop_back()) cudaFree(pl->allocs.back());
+        cudaGetLastError();
+        ws.f64_dig = nullptr;
+        ws.f64_rexp = nullptr;
+        if (!ws.m2l_pairs) ws.pp_work = ws.pp_part = nullptr;
+        ws.f64_batch = 0;
+        ws.f64_tc = 0;
+    };
     if (ok && ws.fp64) {
-        const size_t held = pl->allocs.size();
         bool tc = dalloc(pl, ws.f64_dig, m2l_f64_digit_bytes(p, cells)) &&
                   dalloc(pl, ws.f64_rexp, sizeof(int) * cells);
         if (tc && !ws.m2l_pairs) {
@@ -1081,15 +1092,7 @@ static int plan_create_impl(int64_t n_max, int p, int leaf_max, int depth, int p
             tc = alloc_pairs(pl) == PT_OK;
         }
         ws.f64_tc = tc ? 1 : 0;
-        if (!tc) {
-            // no memory for the digits or the pool: the CUDA-core
-            // translations, which need neither
-            for (; pl->allocs.size() > held; pl->allocs.pop_back()) cudaFree(pl->allocs.back());
-            cudaGetLastError();
-            ws.f64_dig = nullptr;
-            ws.f64_rexp = nullptr;
-            ws.f64_batch = 0;
-        }
+        if (!tc) drop_f64();
     }
     if (dry) {
         *dry_bytes = (int64_t)pl->dry_bytes;
@@ -1154,10 +1157,7 @@ static int plan_create_impl(int64_t n_max, int p, int leaf_max, int depth, int p
     }
     int r = acquire_ops(pl, tsz * PP);
     if (r == PT_OK && legacy_done() != cudaSuccess) r = PT_ERR_CUDA;  // the memsets above
-    if (r == PT_OK && !ws.T_f64) {
-        ws.f64_tc = 0;
-        ws.f64_batch = 0;
-    }
+    if (r == PT_OK && ws.f64_tc && !ws.T_f64) drop_f64();
     if (r == PT_OK && ws.m2l_rot && !ws.f64_tc) r = acquire_rotation(pl);
     if (r != PT_OK) {
         free_plan(pl);
