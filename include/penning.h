@@ -159,7 +159,9 @@ int fmm_plan_set_expansion(fmm_plan plan, int mode);
  * PT_M2L_TILES above (the names of the CUDA-core kernels: an FP64 plan whose
  * schedule was never chosen runs the pair work list on the tensor cores, above
  * 262144 ions in batches of targets).  Choosing a schedule, also the default's
- * name, runs it as described here, and allocates what it needs.
+ * name, runs it as described here, and allocates what it needs (rotation: its
+ * operators, built at the first such call of an order); an FP64 plan then does
+ * not go back to the tensor cores, a new one starts there.
  * Errors: PT_ERR_ARG, PT_ERR_UNSUPPORTED (rotation on the tensor-core
  * precisions or beyond p = 16), PT_ERR_OOM, PT_ERR_CUDA. */
 #define PT_M2L_TILES 0

@@ -838,6 +838,19 @@ static cudaError_t join_members(pt_ensemble_s* ens, cudaGraph_t g) {
                           : upload(c.dev, c.host.data(), c.host.size());
 }
 
+// Both kinds of joined launches (others: not for profiled members).  Their
+// tables are a few MB of host memory: no room is an error, no exception.
+static cudaError_t join_launches(pt_ensemble_s* ens, cudaGraph_t g, bool others) {
+    try {
+        const cudaError_t e = others ? join_members(ens, g) : cudaSuccess;
+        if (e != cudaSuccess) return e;
+        return m2l_join_pair_launches(g, ens->d_members, ens->d_prefix, (int)ens->plans.size(),
+                                      &ens->joined);
+    } catch (const std::bad_alloc&) {
+        return cudaErrorMemoryAllocation;
+    }
+}
+
 namespace {
 void free_ensemble(pt_ensemble_s* e) {
     if (!e) return;
@@ -1466,13 +1479,7 @@ int pt_ensemble_step(pt_ensemble ens, pt_state* states, const pt_trap* traps,
             // (profiled members keep their own launches between their events)
             bool profiled = false;
             for (fmm_plan_s* pl : ens->plans) profiled = profiled || pl->profile;
-            if (ens->join_m2l && !profiled && (e = join_members(ens, g)) != cudaSuccess) {
-                cudaGraphDestroy(g);
-                return status_from(e);
-            }
-            if (ens->join_m2l &&
-                (e = m2l_join_pair_launches(g, ens->d_members, ens->d_prefix, nm, &ens->joined)) !=
-                    cudaSuccess) {
+            if (ens->join_m2l && (e = join_launches(ens, g, !profiled)) != cudaSuccess) {
                 cudaGraphDestroy(g);
                 return status_from(e);
             }
