@@ -217,14 +217,14 @@ __global__ void __launch_bounds__(kF32MaxThreads) k_f32_gemm(const __grid_consta
         if (lmore) {
             float* sA = f32_smem + lst * stage_vals;
             float* sB = sA + a_vals;
-            for (int u = tid; u < ROWS * 8; u += nthr) {
-                const int r = u >> 3, q = u & 7;
+            // a thread's 16-byte unit q is the same in all its rows (nthr is a multiple
+            // of 16).  Zeros beyond column P: the rows' padding takes no part,
+            // whatever it holds (a row with a NaN leaves NaN there, below)
+            const int q = tid & 7, col = lk * 32 + 4 * q;
+            const uint32_t bytes = 4u * (uint32_t)max(0, min(4, a.P - col));
+            for (int r = tid >> 3; r < ROWS; r += nthr >> 3) {
                 const float* src = s_src[lbuf][r];
-                // zeros beyond column P: the rows' padding takes no part, whatever it
-                // holds (a row with a NaN leaves NaN there, below)
-                const int left = max(0, min(4, a.P - (lk * 32 + 4 * q)));
-                cp_async16(sA + r * kAStride + 4 * q, src ? src + lk * 32 + 4 * q : a.M,
-                           src ? 4u * (uint32_t)left : 0u);
+                cp_async16(sA + r * kAStride + 4 * q, src ? src + col : a.M, src ? bytes : 0u);
             }
             const int rowq = a.nc / 4;  // 16-byte units per K row
             const float* B = a.ops + (int64_t)f32_op<MODE>(lw, lterm) * a.op_vals +
