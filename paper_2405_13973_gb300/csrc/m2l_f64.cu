@@ -24,15 +24,16 @@
 // products i + j >= 8 left out, below 2^-57 per coefficient: at worst
 // P 2^-53 (1 + 1/16), the bound of P FP64 multiply-adds of values as large as
 // the maxima.  |s_d| <= d 2^14 P (d >= 1; 6 2^14 P for d = 7), so every sum is
-// exact up to p = 12; at p = 16 those from s_4 on could pass 2^24 with nearly every
-// digit at its limit, and would lose their last bit, 2^-42 (crystals reach 2^20).
+// exact up to p = 12; at p = 16 those from s_4 on could pass 2^24 with nearly
+// every digit at its limit, and would lose their last bit, 2^-42 (crystals
+// reach 2^20).
 // Measured against long double, one offset's output row: 1e-16 .. 9e-16 of
 // its norm, FP64 multiply-adds 5e-16 .. 2.6e-15 (p = 4 .. 16, 1 to 100 ions a
-// cell, like and unlike charges); coefficients far below the largest of their row are less
-// exact than by multiply-adds (their error is of the row's size).  Far fields
-// of 1,000 to 60,000 ions, relative error of E: 2.4e-16 .. 7.2e-16, by
-// multiply-adds 3.0e-16 .. 8.8e-16.  Without the products i + j = 7 (28 of
-// them, 5.1 ms for the M2L below) E was off by up to 1.5e-14.
+// cell, like and unlike charges); coefficients far below the largest of their
+// row are less exact than by multiply-adds (their error is of the row's size).
+// Far fields of 427 to 60,000 ions, relative error of E: 2.1e-16 .. 7.2e-16,
+// by multiply-adds 3.0e-16 .. 1.1e-15.  Without the products i + j = 7 (28 of
+// them, 5.1 ms for the M2L below) E was off by up to 2e-14.
 //   * L2L: the parent's L_0, which in a large crystal is many times the rest
 //     of its row, reaches the child's L_0 only; it stays out of the digits and
 //     is added in FP64 (E at depth 4, 12,000 ions, p = 4: 6.1e-16 -> 2.6e-16).
@@ -43,11 +44,11 @@
 // TMEM columns) leave room for two K steps of A in tensor memory (7 digits
 // x 8 columns each).  A comes from tensor memory because with 48 columns a
 // product takes 24 cycles and reading a 4 KB A tile from shared memory 32:
-//   * warps 10..13 (one TMEM lane quarter each) load the rows' digits (one
-//     byte per digit and coefficient: half the bytes of f16, and the digits
-//     of an item, 172 KB at p = 12, are read once per column chunk, mostly
-//     from L1), expand them to f16 (a byte permute into 1024 + d + 128, one
-//     packed subtraction) and store them to tensor memory;
+//   * warps 10..13 (one TMEM lane quarter each) bring the rows' digits by bulk
+//     copies (one byte per digit and coefficient: half the bytes of f16; an
+//     item's, 172 KB at p = 12, once, above p = 12 once per column chunk),
+//     expand them to f16 (a byte permute into 1024 + d + 128, one packed
+//     subtraction) and store them to tensor memory;
 //   * warp 8 brings the operator digits, packed in f16 in the swizzled
 //     K-major shared-memory image, by bulk copies of 32-wide K chunks;
 //   * warp 9 issues the 34 products of a K step;
