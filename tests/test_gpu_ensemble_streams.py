@@ -59,7 +59,7 @@ def test_a_new_graph_does_not_wait_for_other_work():
     torch.cuda.synchronize()
     done = torch.cuda.Event()
     with torch.cuda.stream(other):
-        torch.cuda._sleep(1_000_000_000)  # clock cycles: half a second
+        torch.cuda._sleep(4_000_000_000)  # clock cycles: two seconds
         done.record()
     ens.step(sets[2], traps, None, dts, 1, stream=side)
     waited = done.query()
